@@ -232,3 +232,95 @@ def tolerance(case):
     if kind == "encoder":
         return {"rel": 1.2e-5, "max": 1.2e-4} if f32 else {"rel": 1.2e-2, "max": 6e-2}
     return {"rel": 4e-6, "max": 1e-4} if f32 else {"rel": 2e-2, "max": 0.9}
+
+
+def _phi(x):
+    return torch.where(x > 0, x + 1, torch.exp(torch.clamp(x, max=0.0)))
+
+
+def _slope(x):
+    return torch.where(x > 0, torch.ones_like(x), torch.exp(torch.clamp(x, max=0.0)))
+
+
+def _ones(V):
+    """The values with a column of ones: its sums are the normaliser."""
+    return torch.cat([V, torch.ones_like(V[..., :1])], -1)
+
+
+def _upstream(nd, G):
+    """Gradient of the numerator and of the normaliser from that of the output."""
+    dn, O = nd[..., -1:], nd[..., :-1] / nd[..., -1:]
+    return torch.cat([G, -(G * O).sum(-1, keepdim=True)], -1) / dn
+
+
+def _causal(q, k, V, G=None, St=None, T=128):
+    """O, the final [S | Z] and, with G, the gradients of q, k (features) and V, chunk by chunk."""
+    Vt, N = _ones(V), q.shape[2]
+    St = torch.zeros_like(q[:, :, 0, :, None] * Vt[:, :, 0, None, :]) if St is None else St.clone()
+    nd, gq, gk, gV, Gt = torch.empty_like(Vt), torch.empty_like(q), torch.empty_like(k), torch.empty_like(Vt), None
+    if G is not None:
+        Gt = torch.empty_like(Vt)
+    cuts = [slice(i, min(i + T, N)) for i in range(0, N, T)]
+    for c in cuts:
+        qc, kc, vc = q[:, :, c], k[:, :, c], Vt[:, :, c]
+        nd[:, :, c] = (qc @ kc.mT).tril() @ vc + qc @ St
+        if G is not None:
+            Gt[:, :, c] = _upstream(nd[:, :, c], G[:, :, c])
+            gq[:, :, c] = (Gt[:, :, c] @ vc.mT).tril() @ kc + Gt[:, :, c] @ St.mT
+        St += kc.mT @ vc
+    O = nd[..., :-1] / nd[..., -1:]
+    if G is None:
+        return O, St
+    R = torch.zeros_like(St)
+    for c in reversed(cuts):
+        qc, kc, vc, gc = q[:, :, c], k[:, :, c], Vt[:, :, c], Gt[:, :, c]
+        gk[:, :, c] = (gc @ vc.mT).tril().mT @ qc + vc @ R.mT
+        gV[:, :, c] = (qc @ kc.mT).tril().mT @ gc + kc @ R
+        R += qc.mT @ gc
+    return O, gq, gk, gV[..., :-1]
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits from the formulas of the method."""
+    s = {n: t.double() if torch.is_tensor(t) and t.is_floating_point() else t for n, t in prepare(case, seed).items()}
+    kind = case["kind"]
+    if kind in ("step", "layer"):
+        B, H, D = case["B"], case["H"], case["D"]
+        if kind == "layer":
+            q, k, v = (s["x"] @ s["Wqkv"].mT).view(B, 3, H, D).unbind(1)
+        else:
+            q, k, v = s["q"], s["k"], s["v"]
+        q, k = _phi(q), _phi(k)
+        S, Z = s["S"] + k[..., :, None] * v[..., None, :], s["Z"] + k
+        out = (q[..., None, :] @ S)[..., 0, :] / (q * Z).sum(-1, keepdim=True)
+        if kind == "layer":
+            out = out.reshape(B, H * D) @ s["Wo"].mT + s["x"]
+        return out, S, Z
+    Q, K, V = s["Q"], s["K"], s["V"]
+    if kind == "prefill":
+        O, St = _causal(_phi(Q), _phi(K), V, St=torch.cat([s["S"], s["Z"][..., None]], -1))
+        return O, St[..., :-1], St[..., -1]
+    if kind == "causal":
+        O, gq, gk, gV = _causal(_phi(Q), _phi(K), V, s["G"])
+        return O, gq * _slope(Q), gk * _slope(K), gV
+    if kind == "fourier":
+        W, a = s["W"], s["W"].shape[0] ** -0.5             # sqrt(2 / C): C / 2 frequencies
+        zq, zk = Q @ W.mT, K @ W.mT
+        fq, fk = (a * torch.cat([z.cos(), z.sin()], -1) for z in (zq, zk))
+        O, gq, gk, gV = _causal(fq, fk, V, s["G"])
+        half = W.shape[0]
+        dQ, dK = (a * (z.cos() * g[..., half:] - z.sin() * g[..., :half]) @ W for z, g in ((zq, gq), (zk, gk)))
+        return O, dQ, dK, gV
+    q, k, Vt = _phi(Q), _phi(K), _ones(V)
+    real = torch.ones_like(q[..., :1])
+    if s["lengths"] is not None:        # padded positions: no part in any sum, zeros in every output
+        real = (torch.arange(Q.shape[2], device="cuda") < s["lengths"][:, None]).to(q.dtype)[:, None, :, None].expand_as(real)
+    k = k * real
+    St = k.mT @ (Vt * real)
+    nd = q @ St
+    O = nd[..., :-1] / nd[..., -1:] * real
+    if kind == "encode":
+        return O
+    Gt = _upstream(nd, s["G"]) * real
+    R = (q * real).mT @ Gt
+    return O, Gt @ St.mT * _slope(Q), Vt @ R.mT * _slope(K) * real, (k @ R)[..., :-1]
