@@ -24,8 +24,12 @@
  *  - Supported sizes: D and M multiples of 8 in [8, 128]; B, H >= 1; N >= 0
  *    (N == 0 is a successful no-op).  bf16 problems with D = M in {32, 64} run
  *    on the tensor-core kernels (any N: a last chunk of fewer than 128
- *    positions is handled as padding), everything else on the general
+ *    positions is handled as padding); the causal form of every other problem
+ *    with M <= 64 runs on tensor-core kernels that keep fp32 accuracy (products
+ *    of numbers split into bf16 parts), everything else on the general
  *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.
+ *    The fp32-accurate causal forward takes ws as an option: with less than
+ *    la_workspace_bytes() (or NULL) it does not cut sequences into pieces.
  *  - Return value: LA_OK (0) or a negative la_status.  All argument checks run
  *    on the host before anything is enqueued; a failed check enqueues nothing.
  *    The library never aborts, throws or traps.  la_last_error() returns a

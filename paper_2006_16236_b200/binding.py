@@ -210,6 +210,16 @@ def workspace(p: la_problem, op: int, device) -> torch.Tensor | None:
     return buf
 
 
+def _forward_scratch(p: la_problem, op: int, device) -> torch.Tensor | None:
+    """Scratch of a causal forward call.  The kernels that take bf16 with D = M in {32, 64} share workspace()'s buffer;
+    the others' scratch is optional and was none before, so calls of several streams or threads must not meet in it:
+    it comes from torch's allocator on every call."""
+    if p.dtype == LA_BF16 and p.D == p.M and p.D in (32, 64):
+        return workspace(p, op, device)
+    need = lib().la_workspace_bytes(ctypes.byref(p), op)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
+
+
 def la_workspace_bytes(p: la_problem, op: int) -> int:
     return lib().la_workspace_bytes(ctypes.byref(p), op)
 
@@ -443,12 +453,12 @@ def la_causal_forward(Q, K, V, phi="elu1", eps=0.0, O=None, den=None, S_out=None
     dev = _dev(Q, K, V, O, den, S_out, Z_out, saved, S_in, Z_in, ws, lengths)
     O = torch.empty_like(V) if O is None else O
     if lengths is not None:             # la_causal_forward_varlen: right-padded ragged batch
-        ws = workspace(p, LA_OP_CAUSAL_VARLEN_FORWARD, dev) if ws is None else ws
+        ws = _forward_scratch(p, LA_OP_CAUSAL_VARLEN_FORWARD, dev) if ws is None else ws
         _call(dev, lib().la_causal_forward_varlen, ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(lengths), _ptr(S_in),
               _ptr(Z_in), _ptr(O), _ptr(den), _ptr(S_out), _ptr(Z_out), _ptr(saved), _nbytes(saved), _ptr(ws), _nbytes(ws),
               _stream(dev))
         return O
-    ws = workspace(p, LA_OP_CAUSAL_FORWARD, dev) if ws is None else ws
+    ws = _forward_scratch(p, LA_OP_CAUSAL_FORWARD, dev) if ws is None else ws
     if S_in is None and Z_in is None:
         _call(dev, lib().la_causal_forward, ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(den), _ptr(S_out),
                                        _ptr(Z_out), _ptr(saved), _nbytes(saved), _ptr(ws), _nbytes(ws), _stream(dev))

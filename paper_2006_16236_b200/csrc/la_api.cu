@@ -261,6 +261,8 @@ size_t la_workspace_bytes(const la_problem* p, int32_t op) {
         return tc_supported(*p, full) ? tc_workspace_bytes(*p, full) : general_workspace_bytes(*p, op);
     }
     if (tc_supported(*p, op)) return tc_workspace_bytes(*p, op);
+    if ((op == LA_OP_CAUSAL_FORWARD || op == LA_OP_CAUSAL_BACKWARD) && causal_mma_supported(*p))
+        return causal_mma_workspace(*p, op == LA_OP_CAUSAL_BACKWARD);
     return general_workspace_bytes(*p, op);
 }
 
@@ -480,7 +482,9 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     }
     LA_REQUIRE_PTR(Q); LA_REQUIRE_PTR(K); LA_REQUIRE_PTR(V); LA_REQUIRE_PTR(O);
     LA_OPTIONAL_PTR(saved);
-    if (int rc = check_ws(p, lengths ? LA_OP_CAUSAL_VARLEN_FORWARD : LA_OP_CAUSAL_FORWARD, ws, ws_bytes)) return rc;
+    const bool tc_path = tc_supported(*p, LA_OP_CAUSAL_FORWARD);
+    if (tc_path)        // (the other kernels' workspace is optional: without it a sequence is not cut into pieces)
+        if (int rc = check_ws(p, lengths ? LA_OP_CAUSAL_VARLEN_FORWARD : LA_OP_CAUSAL_FORWARD, ws, ws_bytes)) return rc;
     if (int rc = check_saved(p, saved, saved_bytes)) return rc;
     if (int rc = check_arch()) return rc;
     const TensorBytes tb(*p);
@@ -488,8 +492,10 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     LA_DEBUG_SPAN(den, tb.den); LA_DEBUG_SPAN(S_in, tb.s); LA_DEBUG_SPAN(Z_in, tb.z); LA_DEBUG_SPAN(S_out, tb.s);
     LA_DEBUG_SPAN(Z_out, tb.z); LA_DEBUG_SPAN(lengths, (size_t)p->B * 4); LA_DEBUG_SPAN(ws, ws_bytes);
     LA_DEBUG_SPAN(saved, saved_bytes);
-    if (tc_supported(*p, LA_OP_CAUSAL_FORWARD))
+    if (tc_path)
         return debug_finish(tc::causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, st), stream);
+    if (causal_mma_supported(*p))
+        return debug_finish(causal_mma_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, ws, ws_bytes, st), stream);
     return debug_finish(general_causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, st), stream);
 }
 
@@ -565,6 +571,8 @@ static int causal_backward_common(const la_problem* p, const void* Q, const void
     LA_DEBUG_SPAN(ws, ws_bytes); LA_DEBUG_SPAN(saved, saved_bytes);
     if (tc_supported(*p, LA_OP_CAUSAL_BACKWARD))
         return debug_finish(tc::causal_backward(*p, Q, K, V, lengths, G, sa, saved, dQ, dK, dV, ws, st), stream);
+    if (causal_mma_supported(*p))
+        return debug_finish(causal_mma_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, ws, st), stream);
     return debug_finish(general_causal_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, ws, st), stream);
 }
 

@@ -1,7 +1,8 @@
 // General kernels: any D, M (multiples of 8 up to 128), any N, fp32 or bf16 I/O,
-// fp32 arithmetic on the CUDA cores.  They serve fp32 problems (bf16 tensor-core
-// products cannot hold the fp32 tolerance) and every shape the tensor-core
-// kernels do not cover.  All four are chunked restatements of Algorithm 1 on the
+// fp32 arithmetic on the CUDA cores.  They serve the non-causal form of fp32 problems
+// (plain bf16 tensor-core products cannot hold the fp32 tolerance) and of every shape the
+// tensor-core kernels do not cover, and the causal form with M > 64 (la_causal_mma.cu has
+// the others).  All four are chunked restatements of Algorithm 1 on the
 // values extended by a ones column:
 //     Vt_j = [V_j, 1],   St = [S | Z]  (D x (M+1)),   [num_i | den_i] = phi(Q_i)^T St_i.
 // For a chunk c of T consecutive positions with L the lower-triangular mask,
@@ -191,16 +192,14 @@ size_t smem_floats_backward(int D, int M) {
 // ---------------------------------------------------------------------------
 // Causal forward: one CTA walks one (batch, head) sequence chunk by chunk.
 // ---------------------------------------------------------------------------
-// KD: D = M = KD known at compile time (all tile strides become constants), or 0: any D, M.
-template <typename IO, int KD>
+template <typename IO>
 __global__ void __launch_bounds__(THREADS)
 general_causal_forward_kernel(const IO* __restrict__ Q, const IO* __restrict__ K, const IO* __restrict__ V,
                               const float* __restrict__ S_in, const float* __restrict__ Z_in,
                               IO* __restrict__ O, float* __restrict__ den, float* __restrict__ S_out,
-                              float* __restrict__ Z_out, int64_t Nfull, int D_arg, int M_arg, float eps, int phi,
+                              float* __restrict__ Z_out, int64_t Nfull, int D, int M, float eps, int phi,
                               const int* __restrict__ lengths, int heads) {
     extern __shared__ float smem[];
-    const int D = KD ? KD : D_arg, M = KD ? KD : M_arg;
     const Dims dm = make_dims(D, M);
     float* sq = smem;
     float* sk = sq + T * dm.DS;
@@ -272,15 +271,14 @@ general_causal_forward_kernel(const IO* __restrict__ Q, const IO* __restrict__ K
 // delta_i found in the forward sweep are parked in `aux` ([B,H,N,2] fp32) for
 // the reverse sweep; no per-position state is stored.
 // ---------------------------------------------------------------------------
-template <typename IO, int KD>
+template <typename IO>
 __global__ void __launch_bounds__(THREADS)
 general_causal_backward_kernel(const IO* __restrict__ Q, const IO* __restrict__ K, const IO* __restrict__ V,
                                const IO* __restrict__ G, const StateArgs sa, IO* __restrict__ dQ,
                                IO* __restrict__ dK, IO* __restrict__ dV, float* __restrict__ aux,
-                               int64_t Nfull, int D_arg, int M_arg, float eps, int phi,
+                               int64_t Nfull, int D, int M, float eps, int phi,
                                const int* __restrict__ lengths, int heads) {
     extern __shared__ float smem[];
-    const int D = KD ? KD : D_arg, M = KD ? KD : M_arg;
     const Dims dm = make_dims(D, M);
     float* sq = smem;
     float* sk = sq + T * dm.DS;
@@ -446,6 +444,7 @@ __device__ __forceinline__ int64_t real_end(const int* lengths, int heads, int64
 }
 
 // part[bh][split] = sum over the split's positions of phi(X_i) [Y_i, 1]^T.
+// KD: D = M = KD known at compile time (all tile strides become constants), or 0: any D, M.
 template <typename IO, int KD>
 __global__ void __launch_bounds__(THREADS)
 general_kv_sum_kernel(const IO* __restrict__ X, const IO* __restrict__ Y, float* __restrict__ part,
@@ -666,7 +665,7 @@ template <typename IO>
 static int causal_forward_t(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
                             const float* Z_in, void* O, float* den, float* S_out, float* Z_out, cudaStream_t st) {
     const size_t smem = smem_floats_forward((int)p.D, (int)p.M) * sizeof(float);
-    auto kern = p.D == 64 && p.M == 64 ? general_causal_forward_kernel<IO, 64> : general_causal_forward_kernel<IO, 0>;
+    auto kern = general_causal_forward_kernel<IO>;
     if (int rc = opt_in_smem(kern, smem)) return rc;
     kern<<<(unsigned)(p.B * p.H), THREADS, smem, st>>>((const IO*)Q, (const IO*)K, (const IO*)V, S_in, Z_in, (IO*)O, den,
                                                        S_out, Z_out, p.N, (int)p.D, (int)p.M, p.eps, p.phi, lengths, (int)p.H);
@@ -685,7 +684,7 @@ static int causal_backward_t(const la_problem& p, const void* Q, const void* K, 
                              const void* G, const StateArgs& sa, void* dQ, void* dK, void* dV, void* ws,
                              cudaStream_t st) {
     const size_t smem = smem_floats_backward((int)p.D, (int)p.M) * sizeof(float);
-    auto kern = p.D == 64 && p.M == 64 ? general_causal_backward_kernel<IO, 64> : general_causal_backward_kernel<IO, 0>;
+    auto kern = general_causal_backward_kernel<IO>;
     if (int rc = opt_in_smem(kern, smem)) return rc;
     kern<<<(unsigned)(p.B * p.H), THREADS, smem, st>>>((const IO*)Q, (const IO*)K, (const IO*)V, (const IO*)G, sa,
                                                        (IO*)dQ, (IO*)dK, (IO*)dV, (float*)ws, p.N, (int)p.D,

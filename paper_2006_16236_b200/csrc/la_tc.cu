@@ -20,6 +20,8 @@ void set_plan_override(int pieces, int short_len, int splits) {
     g_override_splits.store(splits, std::memory_order_relaxed);
 }
 
+int causal_pieces_override() { return g_override_pieces.load(std::memory_order_relaxed); }
+
 int sm_count() {
     static thread_local int cached_dev = -1, cached_sms = 148;
     int dev = 0;

@@ -11,9 +11,19 @@ size_t tc_workspace_bytes(const la_problem& p, int op);
 // pieces, parts, piece_begin[], piece_first_part[], part_begin[], launch_order[] (see la_causal_plan)
 int tc_causal_plan(const la_problem& p, int32_t* out, int capacity);
 
+// Causal form at fp32 accuracy on mma.sync (la_causal_mma.cu): M <= 64, any type and feature map.  The forward's
+// workspace is optional (without it a sequence is one piece).
+bool causal_mma_supported(const la_problem& p);
+size_t causal_mma_workspace(const la_problem& p, bool backward);
+int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
+                       const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* ws, size_t ws_bytes, cudaStream_t st);
+int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
+                        const StateArgs& sa, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
+
 namespace tc {
 // process-wide overrides of the automatic plans (see la_plan_override)
 void set_plan_override(int causal_pieces, int causal_short, int linear_splits);
+int causal_pieces_override();        // -1: automatic
 // In all of these: lengths ([B] int32, device, or null) = real positions per batch element of a right-padded
 // ragged batch; saved (or null) = where the forward leaves what the backward pass can reuse.
 size_t causal_forward_workspace(const la_problem& p);

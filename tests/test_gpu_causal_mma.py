@@ -1,0 +1,83 @@
+"""Causal calls at fp32 accuracy on the warp-level tensor instructions: shapes at the edges of their tiles (chunks of
+64 positions, strips of 16, columns padded to 32, 64 or 128), with the sequence whole and cut into pieces, from a state,
+ragged, and without the optional workspace, against the fp64 oracle.
+
+Tolerance (2-norm of the difference over the 2-norm of the result): an operand keeps 24 bits (2^-24), the tensor cores
+truncate a running sum once per 16 terms (2^-23 of it, at most 8 blocks per sum), and the chunks' sums are added in
+fp32: 16 * 2^-23 = 2e-6 bounds fp32 outputs whose terms do not cancel; gradients are differences of terms up to a few
+times their size, so 8e-6.  bf16 outputs end in one rounding: 2^-8."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2006_16236_b200 as la
+from paper_2006_16236_b200.inputs import draw_qkvg
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(autouse=True)
+def _automatic_plans():
+    yield
+    la.la_plan_override()
+
+
+def _close(x, ref, tol, what):
+    x, ref = x.double().cpu().numpy(), np.asarray(ref)
+    scale = np.linalg.norm(ref)
+    assert np.linalg.norm(x - ref) <= tol * scale + 1e-30, (what, np.linalg.norm(x - ref) / scale)
+
+
+@pytest.mark.parametrize("pieces", [-1, 1, 3])
+@pytest.mark.parametrize("N", [2, 16, 63, 64, 65, 200])
+@pytest.mark.parametrize("dims", [(8, 8), (32, 32), (40, 24), (64, 64), (72, 64), (128, 64)], ids=str)
+def test_tiles(dims, N, pieces):
+    D, M = dims
+    for dtype, phi in ((torch.float32, "elu1"), (torch.float32, "identity"), (torch.bfloat16, "identity"), (torch.bfloat16, "elu1")):
+        if dtype == torch.bfloat16 and D == M and D in (32, 64):
+            continue                                    # another kernel's problem
+        Q, K, V, G = draw_qkvg(1, 2, N, D, M, 3 + N, dtype, 1.0)
+        if phi == "identity":                           # features: positive, as the weights of a kernel are
+            Q, K = Q.abs() + 0.1, K.abs() + 0.1
+        la.la_plan_override(pieces)
+        dev = [t.to(DEV) for t in (Q, K, V, G)]
+        eps = 0.5 if N % 2 else 0.0
+        O = la.la_causal_forward(*dev[:3], phi=phi, eps=eps)
+        grads = la.la_causal_backward(*dev, phi=phi, eps=eps)
+        la.la_last_device_status()
+        q, k, v, g = (t.double().numpy() for t in (Q, K, V, G))
+        f32 = dtype == torch.float32
+        _close(O, oracle.linear_attention(q, k, v, causal=True, phi=phi, eps=eps)[0], 2e-6 if f32 else 2 ** -8, "O")
+        for nm, x, ref in zip(("dQ", "dK", "dV"), grads, oracle.linear_attention_backward(q, k, v, g, causal=True, phi=phi, eps=eps)):
+            _close(x, ref, 8e-6 if f32 else 2 ** -8, nm)
+
+
+@pytest.mark.parametrize("pieces", [1, 2, 4])
+def test_state_lengths_and_no_workspace(pieces):
+    B, H, N, D, M = 3, 2, 150, 48, 40
+    lengths = [150, 0, 70]
+    Q, K, V, _ = draw_qkvg(B, H, N, D, M, 5, torch.float32, 1.0)
+    la.la_plan_override(pieces)
+    q, k, v = (t.to(DEV) for t in (Q, K, V))
+    S0 = torch.rand(B, H, D, M, device=DEV)
+    Z0 = torch.rand(B, H, D, device=DEV) + 1
+    S, Z = torch.empty_like(S0), torch.empty_like(Z0)
+    ln = torch.tensor(lengths, dtype=torch.int32, device=DEV)
+    empty = torch.empty(0, dtype=torch.uint8, device=DEV)       # no room for records: one piece, the same sums
+    for ws in (None, empty):
+        O = la.la_causal_forward(q, k, v, S_in=S0, Z_in=Z0, S_out=S, Z_out=Z, lengths=ln, ws=ws)
+        la.la_last_device_status()
+        fk, fq = oracle.feature_map(K.double().numpy()), oracle.feature_map(Q.double().numpy())
+        for b, n in enumerate(lengths):
+            assert not O[b, :, n:].any()
+            St = S0[b].double().cpu().numpy() + np.einsum("hnd,hnm->hdm", fk[b, :, :n], V[b, :, :n].double().numpy())
+            Zt = Z0[b].double().cpu().numpy() + fk[b, :, :n].sum(1)
+            _close(S[b], St, 2e-6, "S_out")
+            _close(Z[b], Zt, 2e-6, "Z_out")
+            if n:
+                w = np.tril(np.einsum("hnd,hjd->hnj", fq[b, :, :n], fk[b, :, :n]))
+                num = w @ V[b, :, :n].double().numpy() + fq[b, :, :n] @ S0[b].double().cpu().numpy()
+                den = w.sum(-1) + np.einsum("hnd,hd->hn", fq[b, :, :n], Z0[b].double().cpu().numpy())
+                _close(O[b, :, :n], num / den[..., None], 2e-6, "O")
