@@ -1,4 +1,4 @@
-"""Thin ctypes binding of the C ABI in include/la.h.
+"""Thin binding of the C ABI in include/la.h: ctypes, and native code for the ordinary call of the hot entry points.
 
 Argument marshalling only: torch supplies device memory and the current
 stream; every step of the computation runs in the CUDA library.  There is no
@@ -103,6 +103,28 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_fast = None
+
+
+def _native():
+    """The native code of the ordinary call (csrc/la_fast.cpp): the same checks and the same library call without the
+    interpreter's part of them (la_recurrent_step 15 -> 4 us a call).  Its functions return NotImplemented, with nothing
+    done, for everything but plain tensors of the right shapes on the current device: the code below each use."""
+    global _fast
+    if _fast is None:
+        lib()
+        from . import _la_fast
+        _fast = _la_fast
+    return _fast
+
+
+def _done(r):
+    """What a native call returned, a status of the library raised as an error."""
+    if type(r) is int:
+        _check(r)
+    return r
+
+
 def _check(rc: int) -> None:
     if rc != 0:
         L = lib()
@@ -202,7 +224,8 @@ def workspace(p: la_problem, op: int, device) -> torch.Tensor | None:
     need = lib().la_workspace_bytes(ctypes.byref(p), op)
     if need == 0:
         return None
-    key = (str(device), op)
+    index = torch.device(device).index
+    key = op * 1024 + (torch.cuda.current_device() if index is None else index)      # (la_fast.cpp uses the same buffers)
     buf = _ws_cache.get(key)
     if buf is None or buf.numel() < need:
         buf = torch.empty(need, dtype=torch.uint8, device=device)
@@ -356,6 +379,9 @@ def la_feature_map_rff_backward(x: torch.Tensor, W: torch.Tensor, dy: torch.Tens
 
 def linear_saved_buffer(Q, V, phi="elu1", eps=0.0):
     """A buffer for what la_linear_attention() keeps for la_linear_attention_backward() (per-split sums over the keys)."""
+    r = _native().new_buffer(Q, V, phi, eps, LA_OP_LINEAR_SAVED)
+    if r is not NotImplemented:
+        return _done(r)
     p = _problem_of(Q, V, phi, eps)
     need = lib().la_workspace_bytes(ctypes.byref(p), LA_OP_LINEAR_SAVED)
     return None if need == 0 else torch.empty(need, dtype=torch.uint8, device=Q.device)
@@ -366,6 +392,9 @@ def la_linear_attention(Q, K, V, phi="elu1", eps=0.0, O=None, den=None, KV=None,
     """Non-causal form.  Returns O; pass preallocated den / KV / Zs tensors to receive them, and a
     linear_saved_buffer() to keep the sums over the keys for the backward pass (la_linear_attention_keep;
     lengths: optional [B] int32 device tensor of a right-padded ragged batch)."""
+    r = _native().linear_forward(Q, K, V, phi, eps, O, den, KV, Zs, ws, saved, lengths, _ws_cache)
+    if r is not NotImplemented:
+        return _done(r)
     p = _problem_of(Q, V, phi, eps)
     _expect(p, Q.dtype, Q=(Q, "qk"), K=(K, "qk"), V=(V, "v"), O=(O, "v"), den=(den, "row"), KV=(KV, "S"), Zs=(Zs, "Z"))
     _buffer("saved", saved), _buffer("ws", ws)
@@ -406,6 +435,9 @@ def la_linear_attention_backward(Q, K, V, G, phi="elu1", eps=0.0, O=None, den=No
                                  dQ=None, dK=None, dV=None, ws=None, saved=None, lengths=None):
     """Gradients of the non-causal form.  saved: what la_linear_attention(..., saved=...) kept for the same
     problem (la_linear_attention_backward_kept); lengths as there.  Returns (dQ, dK, dV)."""
+    r = _native().linear_backward(Q, K, V, G, phi, eps, O, den, dQ, dK, dV, ws, saved, lengths, _ws_cache)
+    if r is not NotImplemented:
+        return _done(r)
     p = _problem_of(Q, V, phi, eps)
     _expect(p, Q.dtype, Q=(Q, "qk"), K=(K, "qk"), V=(V, "v"), G=(G, "v"), O=(O, "v"), den=(den, "row"),
             dQ=(dQ, "qk"), dK=(dK, "qk"), dV=(dV, "v"))
@@ -434,6 +466,9 @@ def _nbytes(t):
 
 def saved_buffer(Q, V, phi="elu1", eps=0.0):
     """A buffer for what la_causal_forward() keeps for la_causal_backward() (None if the problem needs none)."""
+    r = _native().new_buffer(Q, V, phi, eps, LA_OP_CAUSAL_SAVED)
+    if r is not NotImplemented:
+        return _done(r)
     p = _problem_of(Q, V, phi, eps)
     need = lib().la_workspace_bytes(ctypes.byref(p), LA_OP_CAUSAL_SAVED)
     return None if need == 0 else torch.empty(need, dtype=torch.uint8, device=Q.device)
@@ -444,6 +479,9 @@ def la_causal_forward(Q, K, V, phi="elu1", eps=0.0, O=None, den=None, S_out=None
     """Causal form.  Returns O; pass preallocated den / S_out / Z_out tensors to receive them, and a
     saved_buffer() to keep phi(Q), phi(K) for the backward pass.  S_in / Z_in (fp32 [B,H,D,M] / [B,H,D]):
     the state the sequence continues from (la_causal_forward_from)."""
+    r = _native().causal_forward(Q, K, V, phi, eps, O, den, S_out, Z_out, saved, ws, S_in, Z_in, lengths, _ws_cache)
+    if r is not NotImplemented:
+        return _done(r)
     p = _problem_of(Q, V, phi, eps)
     _expect(p, Q.dtype, Q=(Q, "qk"), K=(K, "qk"), V=(V, "v"), O=(O, "v"), den=(den, "row"), S_out=(S_out, "S"),
             Z_out=(Z_out, "Z"), S_in=(S_in, "S"), Z_in=(Z_in, "Z"))
@@ -474,6 +512,10 @@ def la_causal_backward(Q, K, V, G, phi="elu1", eps=0.0, O=None, den=None, saved=
     """Gradients of the causal form; returns (dQ, dK, dV).  With any of the state arguments (fp32 [B,H,D,M] /
     [B,H,D]: the state the forward started from, the upstream gradient of its final state, and tensors that
     receive the gradient of the initial state) the call is la_causal_backward_from."""
+    r = _native().causal_backward(Q, K, V, G, phi, eps, O, den, saved, dQ, dK, dV, ws, S_in, Z_in, dS_out, dZ_out,
+                                  dS_in, dZ_in, lengths, _ws_cache)
+    if r is not NotImplemented:
+        return _done(r)
     p = _problem_of(Q, V, phi, eps)
     _expect(p, Q.dtype, Q=(Q, "qk"), K=(K, "qk"), V=(V, "v"), G=(G, "v"), O=(O, "v"), den=(den, "row"),
             dQ=(dQ, "qk"), dK=(dK, "qk"), dV=(dV, "v"), S_in=(S_in, "S"), Z_in=(Z_in, "Z"), dS_out=(dS_out, "S"),
@@ -505,6 +547,9 @@ def la_causal_backward(Q, K, V, G, phi="elu1", eps=0.0, O=None, den=None, saved=
 
 def la_recurrent_step(q, k, v, S, Z, phi="elu1", eps=0.0, out=None):
     """One decode step: S, Z (fp32) are updated in place; returns out [B,H,M]."""
+    r = _native().recurrent_step(q, k, v, S, Z, phi, eps, out)
+    if r is not NotImplemented:
+        return _done(r)
     if q.dim() != 3 or v.dim() != 3:
         raise ValueError("expected q,k [B,H,D], v [B,H,M], fp32 S [B,H,D,M] and Z [B,H,D]")
     B, H, D = q.shape
@@ -555,6 +600,9 @@ def la_decode_layer_step(x, Wqkv, Wo, S, Z, phi="elu1", eps=0.0, out=None, ws=No
     """One decode step of a whole attention sublayer: x [B,F] -> y [B,F] with F = H*D (bf16, D = M = 64);
     Wqkv [3F,F] and Wo [F,F] are "outputs x inputs" like a linear layer's weight; S [B,H,D,M], Z [B,H,D] (fp32)
     are updated in place.  Returns y = attention(x) W_O + x."""
+    r = _native().decode_layer_step(x, Wqkv, Wo, S, Z, phi, eps, out, ws, _ws_cache)
+    if r is not NotImplemented:
+        return _done(r)
     if S.dim() != 4 or x.dim() != 2:
         raise ValueError("expected x [B,F], fp32 S [B,H,D,M] and Z [B,H,D]")
     B, H, D, M = S.shape

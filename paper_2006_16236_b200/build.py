@@ -1,14 +1,17 @@
-"""Build the CUDA library in-tree: nvcc, sm_100a only, no JIT cache."""
+"""Build the CUDA library (nvcc, sm_100a only, no JIT cache) and the native part of the binding (g++) in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libla.so")
+FAST_SRC = os.path.join(CSRC, "la_fast.cpp")
+FAST = os.path.join(PKG, "_la_fast.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -36,7 +39,24 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         subprocess.run(cmd, check=True)
+    build_fast(force)
     return LIB
+
+
+def build_fast(force: bool = False) -> str:
+    """Compile the native part of the binding against torch's headers; it loads libla.so from its own folder."""
+    header = os.path.join(ROOT, "include", "la.h")
+    if force or not os.path.exists(FAST) or os.path.getmtime(FAST) < max(os.path.getmtime(FAST_SRC), os.path.getmtime(header)):
+        import torch
+        t = os.path.dirname(torch.__file__)
+        include = [os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
+                   sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in include), "-o", FAST, FAST_SRC,
+               "-L", PKG, "-l:libla.so", "-L", os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+               "-Wl,-rpath,$ORIGIN"]
+        subprocess.run(cmd, check=True)
+    return FAST
 
 
 if __name__ == "__main__":
