@@ -63,26 +63,29 @@ __device__ void zero_rows(IO* x, int64_t from, int64_t to, int cols) {       // 
     for (int64_t i = from * cols + threadIdx.x; i < to * cols; i += THREADS) x[i] = from_f32<IO>(0.f);
 }
 
-// Rows d = 16 (warp + 4 i) + g (+ 8) of the running sums, columns e = 8 n + 2 t (+ 1).
+// The running sums of a warp: rows d = 16 strip + g (+ 8), strip = warp (+ 4); with two strips (D <= 32) two warps
+// share one and take half of its columns each.  Columns e = 8 (n0 + n) + 2 t (+ 1).
 template <int DP, int MP>
 struct State {
-    static constexpr int SD = (DP / 16 + WARPS - 1) / WARPS;
-    static __device__ __forceinline__ bool mine(int strip) { return DP % (16 * WARPS) == 0 || strip * 16 < DP; }
-    float s[SD][MP / 8][4];
-    float z[SD][2];
+    static constexpr int STRIPS = DP / 16, SHARE = STRIPS < WARPS ? WARPS / STRIPS : 1, SD = STRIPS < WARPS ? 1 : STRIPS / WARPS;
+    static constexpr int NC = MP / 8 / SHARE;
+    static __device__ __forceinline__ int strip(int i) { return ((int)threadIdx.x >> 5) % STRIPS + WARPS * i; }
+    static __device__ __forceinline__ int n0() { return SHARE == 1 ? 0 : ((int)threadIdx.x >> 5) / STRIPS * NC; }
+    float s[SD][NC][4];
+    float z[SD][2];             // in every warp that shares the strip
 
     __device__ __forceinline__ void init(const Params& p, const float* S0, const float* Z0, const float* rec, int nrec) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+        const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, c0 = n0();
         const int size = p.D * p.M + p.D;
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
-            const int d = (warp + WARPS * i) * 16 + g;
+            const int d = strip(i) * 16 + g;
 #pragma unroll
-            for (int n = 0; n < MP / 8; ++n)
+            for (int n = 0; n < NC; ++n)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     float2 v = make_float2(0.f, 0.f);
-                    if (S0 && d + 8 * h < p.D && n * 8 < p.M) v = load_pair<float>(S0 + (d + 8 * h) * p.M + n * 8 + 2 * t);
+                    if (S0 && d + 8 * h < p.D && (c0 + n) * 8 < p.M) v = load_pair(S0 + (d + 8 * h) * p.M + (c0 + n) * 8 + 2 * t);
                     s[i][n][2 * h] = v.x;
                     s[i][n][2 * h + 1] = v.y;
                 }
@@ -91,11 +94,11 @@ struct State {
             for (int r = 0; r < nrec; ++r) {
                 const float* q = rec + (int64_t)r * size;
 #pragma unroll
-                for (int n = 0; n < MP / 8; ++n)
+                for (int n = 0; n < NC; ++n)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
-                        if (d + 8 * h < p.D && n * 8 < p.M) {
-                            const float2 v = *reinterpret_cast<const float2*>(q + (d + 8 * h) * p.M + n * 8 + 2 * t);
+                        if (d + 8 * h < p.D && (c0 + n) * 8 < p.M) {
+                            const float2 v = *reinterpret_cast<const float2*>(q + (d + 8 * h) * p.M + (c0 + n) * 8 + 2 * t);
                             s[i][n][2 * h] += v.x;
                             s[i][n][2 * h + 1] += v.y;
                         }
@@ -106,38 +109,38 @@ struct State {
         }
     }
     __device__ __forceinline__ void write(const Params& p, float* S1, float* Z1) const {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+        const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, c0 = n0();
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
-            const int d = (warp + WARPS * i) * 16 + g;
+            const int d = strip(i) * 16 + g;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
                 if (d + 8 * h < p.D) {
 #pragma unroll
-                    for (int n = 0; n < MP / 8; ++n)
-                        if (S1 && n * 8 < p.M) store_pair<float>(S1 + (d + 8 * h) * p.M + n * 8 + 2 * t, s[i][n][2 * h], s[i][n][2 * h + 1]);
-                    if (Z1 && t == 0) Z1[d + 8 * h] = z[i][h];
+                    for (int n = 0; n < NC; ++n)
+                        if (S1 && (c0 + n) * 8 < p.M) store_pair<float>(S1 + (d + 8 * h) * p.M + (c0 + n) * 8 + 2 * t, s[i][n][2 * h], s[i][n][2 * h + 1]);
+                    if (Z1 && t == 0 && c0 == 0) Z1[d + 8 * h] = z[i][h];
                 }
         }
     }
     // the operand planes [DP][MP] of the matrix and the vector in fp32
+    template <int NS>
     __device__ __forceinline__ void publish(uint8_t* tile, float* vec) const {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+        const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, c0 = n0();
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
-            const int d = (warp + WARPS * i) * 16 + g;
-            if (!mine(warp + WARPS * i)) break;
+            const int d = strip(i) * 16 + g;
 #pragma unroll
-            for (int n = 0; n < MP / 8; ++n)
+            for (int n = 0; n < NC; ++n)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    uint32_t o[3];
-                    split2<3>(s[i][n][2 * h], s[i][n][2 * h + 1], o);
+                    uint32_t o[NS];
+                    split2<NS>(s[i][n][2 * h], s[i][n][2 * h + 1], o);
 #pragma unroll
-                    for (int k = 0; k < 3; ++k)
-                        *reinterpret_cast<uint32_t*>(tile + k * (DP * MP * 2) + tile_at<MP>(d + 8 * h, n) + t * 4) = o[k];
+                    for (int k = 0; k < NS; ++k)
+                        *reinterpret_cast<uint32_t*>(tile + k * (DP * MP * 2) + tile_at<MP>(d + 8 * h, c0 + n) + t * 4) = o[k];
                 }
-            if (t == 0) {
+            if (t == 0 && c0 == 0) {
                 vec[d] = z[i][0];
                 vec[d + 8] = z[i][1];
             }
@@ -148,17 +151,15 @@ struct State {
     // (a chunk that is not full has zeros in the tiles' other rows)
     template <int NX, int NY, bool ONES>
     __device__ __forceinline__ void update(uint32_t X, uint32_t Y, const uint16_t* wpl) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane & 3;
+        const int lane = threadIdx.x & 31, t = lane & 3, c0 = n0();
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
-            const int strip = warp + WARPS * i;
-            if (!mine(strip)) break;
             uint32_t a[T / 16][NX][4];
             float zs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int b = 0; b < T / 16; ++b)
                 {
-                    load_rows_t<NX, DP>(a[b], X, T * DP * 2, b * 16, strip * 2, lane);
+                    load_rows_t<NX, DP>(a[b], X, T * DP * 2, b * 16, strip(i) * 2, lane);
                     float u[4] = {0.f, 0.f, 0.f, 0.f};
                     if constexpr (ONES) {
 #pragma unroll
@@ -182,12 +183,12 @@ struct State {
             z[i][0] += zs[0];
             z[i][1] += zs[2];
 #pragma unroll
-            for (int n = 0; n < MP / 16; ++n) {
+            for (int n = 0; n < NC / 2; ++n) {
                 Chain c;
 #pragma unroll
                 for (int b = 0; b < T / 16; ++b) {
                         uint32_t y[NY][4];
-                        load_cols_t<NY, MP>(y, Y, T * MP * 2, b * 16, n * 2, lane);
+                        load_cols_t<NY, MP>(y, Y, T * MP * 2, b * 16, c0 + n * 2, lane);
                         c.step<NX, NY>(a[b], y);
                     }
                 c.add_to(s[i][2 * n], s[i][2 * n + 1]);
@@ -196,17 +197,29 @@ struct State {
     }
 };
 
-// planes of the feature-mapped rows (q, k) and of the value rows (V, G): bf16 values have one plane, a bf16 feature
-// map that is the identity too
-template <typename IO, bool MAPPED> constexpr int kFeaturePlanes = sizeof(IO) == 2 && !MAPPED ? 1 : 3;
-template <typename IO> constexpr int kValuePlanes = sizeof(IO) == 2 ? 1 : 3;
+// I/O type and planes of each kind of operand: feature-mapped rows (NQ), value rows V, G (NV), scores (NP), state (NS),
+// q / dn (NR).  Everything computed in fp32 has three planes; bf16 values, and features that are bf16 as given, one.
+struct Fp32 { using IO = float; static constexpr int NQ = 3, NV = 3, NP = 3, NS = 3, NR = 3, BUF = 1; static constexpr bool MAPPED = true; };
+struct Bf16Wide { using IO = __nv_bfloat16; static constexpr int NQ = 3, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1; static constexpr bool MAPPED = true; };
+struct Bf16Features { using IO = __nv_bfloat16; static constexpr int NQ = 1, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1; static constexpr bool MAPPED = false; };
+// bf16 operands throughout (with fp32 sums), as the tcgen05 kernels have them.  BUF = 2: the small tiles are there twice,
+// one barrier per chunk (the other set was last read before the barrier of this chunk).
+struct Bf16 { using IO = __nv_bfloat16; static constexpr int NQ = 1, NV = 1, NP = 1, NS = 1, NR = 1, BUF = 2; static constexpr bool MAPPED = true; };
 
-template <int DP, int MP, int NX, int NY> struct Shared {       // tile X [T][DP], tile Y [T][MP], state planes, vectors
-    static constexpr int X = 0, Y = X + NX * T * DP * 2, S = Y + NY * T * MP * 2, Z = S + 3 * DP * MP * 2,
-                         W = Z + DP * 4, WP = W + T * 4, BYTES = WP + 3 * T * 2;
+template <int DP, int MP, int NX, int NY, int NS> struct Shared {       // tile X [T][DP], tile Y [T][MP], state planes, vectors
+    static constexpr int X = 0, Y = X + NX * T * DP * 2, S = Y + NY * T * MP * 2, Z = S + NS * DP * MP * 2,
+                         W = Z + DP * 4, WP = W + T * 4, BYTES = (WP + 3 * T * 2 + 127) / 128 * 128;
 };
-template <int DP, int MP, int NX, int NY> constexpr int kResident = 3 * (Shared<DP, MP, NX, NY>::BYTES + 1024) <= 227 * 1024 ? 3
-                                                                  : 2 * (Shared<DP, MP, NX, NY>::BYTES + 1024) <= 227 * 1024 ? 2 : 1;
+// CTAs of an SM that the registers are shared out for: as many as shared memory holds, at most `most`
+template <typename Sh, typename C> constexpr int resident(int most) {
+    const int fit = 227 * 1024 / (C::BUF * Sh::BYTES + 1024);
+    return fit < most ? fit : most;
+}
+
+template <typename C, typename Sh>
+__device__ __forceinline__ void flip(uint8_t*& buf, uint8_t* smem) {
+    if constexpr (C::BUF == 2) buf = buf == smem ? smem + Sh::BYTES : smem;
+}
 
 template <typename IO>
 __device__ __forceinline__ void prefetch_rows(const IO* x, int64_t n0, int64_t end, int cols) {
@@ -216,17 +229,21 @@ __device__ __forceinline__ void prefetch_rows(const IO* x, int64_t n0, int64_t e
     for (int64_t o = threadIdx.x * 128; o < rows * cols * (int64_t)sizeof(IO); o += THREADS * 128) prefetch_l2(p + o);
 }
 
+// feature-mapped pairs in registers: bf16 where features have one plane
+template <int NQ> struct FeatureType { using type = float; };
+template <> struct FeatureType<1> { using type = __nv_bfloat16; };
+
 // ---- forward ---------------------------------------------------------------------------------------------------
-template <typename IO, int DP, int MP, bool MAPPED, bool EXACT>
-__global__ void __launch_bounds__(THREADS, (kResident<DP, MP, kFeaturePlanes<IO, MAPPED>, kValuePlanes<IO>> < 2 ? 1 : sizeof(IO) == 4 && DP == 64 ? 2 : kResident<DP, MP, kFeaturePlanes<IO, MAPPED>, kValuePlanes<IO>>))
+template <typename C, int DP, int MP, bool EXACT>
+__global__ void __launch_bounds__(THREADS, (resident<Shared<DP, MP, C::NQ, C::NV, C::NS>, C>(C::NP == 1 ? 4 : sizeof(typename C::IO) == 4 && DP == 64 ? 2 : 3)))
 causal_mma_forward_kernel(const Params p) {
-    constexpr int NQ = kFeaturePlanes<IO, MAPPED>, NV = kValuePlanes<IO>;
-    using Sh = Shared<DP, MP, NQ, NV>;
+    using IO = typename C::IO;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS;
+    using Sh = Shared<DP, MP, NQ, NV, NS>;
     extern __shared__ __align__(128) uint8_t smem[];
-    const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
-    float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
+    uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = sizeof(IO) == 2 && !MAPPED ? LA_PHI_IDENTITY : p.phi;
+    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
     const Range r = range_of(p, blockIdx.y);
     const IO* Q = (const IO*)p.Q + r.bh * p.N * D;
@@ -239,6 +256,8 @@ causal_mma_forward_kernel(const Params p) {
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + r.bh * (p.pieces - 1) * (int64_t)(D * M + D), r.piece);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
+        const uint32_t sK = smem_u32(buf + Sh::X), sV = smem_u32(buf + Sh::Y), sS = smem_u32(buf + Sh::S);
+        float* sZ = reinterpret_cast<float*>(buf + Sh::Z);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         // (the strip with the most blocks left of the diagonal goes round the schedulers)
         const int strip = ((n0 / T) & 1) ? WARPS - 1 - warp : warp, row0 = strip * 16;
@@ -249,37 +268,38 @@ causal_mma_forward_kernel(const Params p) {
             RawTile<IO, T, MP, THREADS> rv;
             rk.load(K + n0 * D, cn, D, pad);
             rv.load(V + n0 * M, cn, M, 0.f);
-            __syncthreads();                    // the planes of the chunk before are no longer read
-            st.publish(smem + Sh::S, sZ);
-            with_phi(phi, [&](auto f) { rk.template store<NQ>(smem + Sh::X, [&](int, float x) { return f(x); }); });
-            rv.template store<NV>(smem + Sh::Y, [](int, float x) { return x; });
+            if constexpr (C::BUF == 1) __syncthreads();         // the planes of the chunk before are no longer read
+            st.template publish<NS>(buf + Sh::S, sZ);
+            with_phi<NQ>(phi, [&](auto f) { rk.template store<NQ>(buf + Sh::X, [&](int, float x) { return f(x); }); });
+            rv.template values<NV>(buf + Sh::Y);
         }
         prefetch_rows(Q, n0 + T, r.end, D);
         prefetch_rows(K, n0 + T, r.end, D);
         prefetch_rows(V, n0 + T, r.end, M);
         __syncthreads();
         if (row0 < cn) {
-            rq.map(phi);
+            RawStrip<typename FeatureType<NQ>::type, DP> fq;
+            rq.template map<NQ>(phi, fq);
             float d0 = 0.f, d1 = 0.f;           // rows g, g + 8: q . Z, then + the scores
 #pragma unroll
             for (int kk = 0; kk < DP / 16; ++kk)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float2 z = *reinterpret_cast<const float2*>(sZ + kk * 16 + h * 8 + 2 * t);
-                    d0 = fmaf(rq.r[kk][2 * h].x, z.x, fmaf(rq.r[kk][2 * h].y, z.y, d0));
-                    d1 = fmaf(rq.r[kk][2 * h + 1].x, z.x, fmaf(rq.r[kk][2 * h + 1].y, z.y, d1));
+                    d0 = fmaf(fq.r[kk][2 * h].lo(), z.x, fmaf(fq.r[kk][2 * h].hi(), z.y, d0));
+                    d1 = fmaf(fq.r[kk][2 * h + 1].lo(), z.x, fmaf(fq.r[kk][2 * h + 1].hi(), z.y, d1));
                 }
             uint32_t qa[DP / 16][NQ][4];
-            rq.template planes<NQ>(qa);
+            fq.template planes<NQ>(qa);
             float o[MP / 8][4];
 #pragma unroll
             for (int n = 0; n < MP / 16; ++n) {
                 Chain c;
 #pragma unroll
                 for (int kk = 0; kk < DP / 16; ++kk) {
-                    uint32_t b[3][4];
-                    load_cols_t<3, MP>(b, sS, DP * MP * 2, kk * 16, n * 2, lane);
-                    c.step<NQ, 3>(qa[kk], b);
+                    uint32_t b[NS][4];
+                    load_cols_t<NS, MP>(b, sS, DP * MP * 2, kk * 16, n * 2, lane);
+                    c.step<NQ, NS>(qa[kk], b);
                 }
                 c.put(o[2 * n], o[2 * n + 1]);
             }
@@ -304,15 +324,22 @@ causal_mma_forward_kernel(const Params p) {
                         if (col + 8 > row) s1[j] = 0.f;
                     }
                 }
-                d0 += (s0[0] + s0[1]) + (s1[0] + s1[1]);
-                d1 += (s0[2] + s0[3]) + (s1[2] + s1[3]);
-                uint32_t pa[3][4];
-                operand_of<3>(pa, s0, s1);
+                uint32_t pa[NP][4];
+                operand_of<NP>(pa, s0, s1);
+                if constexpr (NP == 1) {
+                    float u[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma16816(u, pa[0], 0x3f803f80u, 0x3f803f80u);       // row sums (in every column; lane 0 of a row counts)
+                    d0 += t == 0 ? u[0] : 0.f;
+                    d1 += t == 0 ? u[2] : 0.f;
+                } else {
+                    d0 += (s0[0] + s0[1]) + (s1[0] + s1[1]);
+                    d1 += (s0[2] + s0[3]) + (s1[2] + s1[3]);
+                }
 #pragma unroll
                 for (int n = 0; n < MP / 16; ++n) {
                     uint32_t b[NV][4];
                     load_cols_t<NV, MP>(b, sV, T * MP * 2, jb * 16, n * 2, lane);
-                    block_mma<3, NV>(o[2 * n], o[2 * n + 1], pa, b);
+                    block_mma<NP, NV>(o[2 * n], o[2 * n + 1], pa, b);
                 }
             }
             d0 = quad_sum(d0);
@@ -330,6 +357,7 @@ causal_mma_forward_kernel(const Params p) {
             }
         }
         st.template update<NQ, NV, true>(sK, sV, nullptr);
+        flip<C, Sh>(buf, smem);
     }
     zero_rows(O, r.end, r.hi, M);
     if (den) zero_rows(den, r.end, r.hi, 1);
@@ -355,12 +383,12 @@ struct ReverseRows {
         }
         dl = (int)threadIdx.x < cn ? delta[n0 + threadIdx.x] : 0.f;
     }
-    template <int NV>
+    template <int NR, int NV>
     __device__ __forceinline__ void store(uint8_t* tq, uint8_t* tg, float* w, uint16_t* wpl, int phi) {
 #pragma unroll
         for (int u = 0; u < RawTile<IO, T, DP, THREADS>::GROUPS; ++u) inv[u] = 1.f / inv[u];
-        with_phi(phi, [&](auto f) { rq.template store<3>(tq, [&](int u, float x) { return f(x) * inv[u]; }); });
-        rg.template store<NV>(tg, [](int, float x) { return x; });
+        with_phi<NR>(phi, [&](auto f) { rq.template store<NR>(tq, [&](int u, float x) { return f(x) * inv[u]; }); });
+        rg.template values<NV>(tg);
         if (threadIdx.x < T) {
             w[threadIdx.x] = dl;
             uint32_t o[3];
@@ -371,16 +399,15 @@ struct ReverseRows {
     }
 };
 
-template <typename IO, int DP, int MP, bool MAPPED, bool EXACT, bool REVERSE>
-__global__ void __launch_bounds__(THREADS, 2)
+template <typename C, int DP, int MP, bool EXACT, bool REVERSE>
+__global__ void __launch_bounds__(THREADS, C::NP == 1 ? 4 : 2)
 causal_mma_sum_kernel(const Params p) {
-    constexpr int NX = REVERSE ? 3 : kFeaturePlanes<IO, MAPPED>, NY = kValuePlanes<IO>;
-    using Sh = Shared<DP, MP, NX, NY>;          // (the state planes are not used: the launch asks for less)
+    using IO = typename C::IO;
+    constexpr int NX = REVERSE ? C::NR : C::NQ, NY = C::NV;
+    using Sh = Shared<DP, MP, NX, NY, C::NS>;          // (the state planes are not used: the launch asks for less)
     extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t* base = smem;
-    float* w = reinterpret_cast<float*>(smem + Sh::S);
-    uint16_t* wpl = reinterpret_cast<uint16_t*>(w + T);
-    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = sizeof(IO) == 2 && !MAPPED ? LA_PHI_IDENTITY : p.phi;
+    uint8_t* buf = smem;
+    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
     const Range r = range_of(p, (int)blockIdx.y + (REVERSE ? 1 : 0));
     const IO* X = (const IO*)(REVERSE ? p.Q : p.K) + r.bh * p.N * D;
@@ -390,41 +417,44 @@ causal_mma_sum_kernel(const Params p) {
     State<DP, MP> st;
     st.init(p, nullptr, nullptr, nullptr, 0);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
+        float* w = reinterpret_cast<float*>(buf + Sh::S);
+        uint16_t* wpl = reinterpret_cast<uint16_t*>(w + T);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         if constexpr (REVERSE) {
             ReverseRows<IO, DP, MP> rr;
             rr.load(X, Y, dn, delta, n0, cn, D, M, pad);
-            __syncthreads();
-            rr.template store<NY>(base + Sh::X, base + Sh::Y, w, wpl, phi);
+            if constexpr (C::BUF == 1) __syncthreads();
+            rr.template store<NX, NY>(buf + Sh::X, buf + Sh::Y, w, wpl, phi);
         } else {
             RawTile<IO, T, DP, THREADS> rx;
             RawTile<IO, T, MP, THREADS> ry;
             rx.load(X + n0 * D, cn, D, pad);
             ry.load(Y + n0 * M, cn, M, 0.f);
-            __syncthreads();
-            with_phi(phi, [&](auto f) { rx.template store<NX>(base + Sh::X, [&](int, float x) { return f(x); }); });
-            ry.template store<NY>(base + Sh::Y, [](int, float x) { return x; });
+            if constexpr (C::BUF == 1) __syncthreads();
+            with_phi<NX>(phi, [&](auto f) { rx.template store<NX>(buf + Sh::X, [&](int, float x) { return f(x); }); });
+            ry.template values<NY>(buf + Sh::Y);
         }
         prefetch_rows(X, n0 + T, r.end, D);
         prefetch_rows(Y, n0 + T, r.end, M);
         __syncthreads();
-        st.template update<NX, NY, !REVERSE>(smem_u32(base + Sh::X), smem_u32(base + Sh::Y), wpl);
+        st.template update<NX, NY, !REVERSE>(smem_u32(buf + Sh::X), smem_u32(buf + Sh::Y), wpl);
+        flip<C, Sh>(buf, smem);
     }
     float* dst = p.rec + (r.bh * (p.pieces - 1) + blockIdx.y) * (int64_t)(D * M + D);
     st.write(p, dst, dst + D * M);
 }
 
 // ---- dQ sweep --------------------------------------------------------------------------------------------------
-template <typename IO, int DP, int MP, bool MAPPED, bool EXACT>
-__global__ void __launch_bounds__(THREADS, (kResident<DP, MP, kFeaturePlanes<IO, MAPPED>, kValuePlanes<IO>> < 2 ? 1 : 2))
+template <typename C, int DP, int MP, bool EXACT>
+__global__ void __launch_bounds__(THREADS, (resident<Shared<DP, MP, C::NQ, C::NV, C::NS>, C>(C::NP == 1 ? 4 : 2)))
 causal_mma_dq_kernel(const Params p) {
-    constexpr int NQ = kFeaturePlanes<IO, MAPPED>, NV = kValuePlanes<IO>;
-    using Sh = Shared<DP, MP, NQ, NV>;
+    using IO = typename C::IO;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS;
+    using Sh = Shared<DP, MP, NQ, NV, NS>;
     extern __shared__ __align__(128) uint8_t smem[];
-    const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
-    float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
+    uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = sizeof(IO) == 2 && !MAPPED ? LA_PHI_IDENTITY : p.phi;
+    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
     const Range r = range_of(p, blockIdx.y);
     const IO* Q = (const IO*)p.Q + r.bh * p.N * D;
@@ -439,6 +469,8 @@ causal_mma_dq_kernel(const Params p) {
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + r.bh * (p.pieces - 1) * (int64_t)(D * M + D), r.piece);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
+        const uint32_t sK = smem_u32(buf + Sh::X), sV = smem_u32(buf + Sh::Y), sS = smem_u32(buf + Sh::S);
+        float* sZ = reinterpret_cast<float*>(buf + Sh::Z);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         const int strip = ((n0 / T) & 1) ? WARPS - 1 - warp : warp, row0 = strip * 16;
         uint32_t ga[MP / 16][NV][4];
@@ -449,10 +481,10 @@ causal_mma_dq_kernel(const Params p) {
             rg.load(G + n0 * M, row0, cn, M, 0.f);
             rk.load(K + n0 * D, cn, D, pad);
             rv.load(V + n0 * M, cn, M, 0.f);
-            __syncthreads();
-            st.publish(smem + Sh::S, sZ);
-            with_phi(phi, [&](auto f) { rk.template store<NQ>(smem + Sh::X, [&](int, float x) { return f(x); }); });
-            rv.template store<NV>(smem + Sh::Y, [](int, float x) { return x; });
+            if constexpr (C::BUF == 1) __syncthreads();
+            st.template publish<NS>(buf + Sh::S, sZ);
+            with_phi<NQ>(phi, [&](auto f) { rk.template store<NQ>(buf + Sh::X, [&](int, float x) { return f(x); }); });
+            rv.template values<NV>(buf + Sh::Y);
             rg.template planes<NV>(ga);
         }
         prefetch_rows(Q, n0 + T, r.end, D);
@@ -476,9 +508,9 @@ causal_mma_dq_kernel(const Params p) {
                 Chain c;
 #pragma unroll
                 for (int ee = 0; ee < MP / 16; ++ee) {
-                    uint32_t b[3][4];
-                    load_rows<3, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
-                    c.step<NV, 3>(ga[ee], b);
+                    uint32_t b[NS][4];
+                    load_rows<NS, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
+                    c.step<NV, NS>(ga[ee], b);
                 }
                 c.put(h[2 * n], h[2 * n + 1]);
             }
@@ -511,27 +543,28 @@ causal_mma_dq_kernel(const Params p) {
                     ones[0][0] = ones[0][3] = (2 * t <= g ? 0x3f80u : 0u) | (2 * t + 1 <= g ? 0x3f800000u : 0u);
                     ones[0][2] = 0u;
                 }
-                uint32_t pa[3][4];
-                operand_of<3>(pa, s0, s1);
+                uint32_t pa[NP][4];
+                operand_of<NP>(pa, s0, s1);
 #pragma unroll
                 for (int n = 0; n < DP / 16; ++n) {
                     uint32_t b[NQ][4];
                     load_cols_t<NQ, DP>(b, sK, T * DP * 2, jb * 16, n * 2, lane);
-                    block_mma<3, NQ>(h[2 * n], h[2 * n + 1], pa, b);
+                    block_mma<NP, NQ>(h[2 * n], h[2 * n + 1], pa, b);
                     block_mma<1, NQ>(zc[2 * n], zc[2 * n + 1], ones, b);
                 }
             }
             RawStrip<IO, DP> rq;                // element j of block kk: result column tile 2 kk + j / 2, row g + 8 (j & 1)
             rq.load(Q + n0 * D, row0, cn, D, pad);
-            rq.map(phi);
+            RawStrip<typename FeatureType<NQ>::type, DP> fq;
+            rq.template map<NQ>(phi, fq);
             float qz[2] = {0.f, 0.f}, qh[2] = {0.f, 0.f};
 #pragma unroll
             for (int kk = 0; kk < DP / 16; ++kk)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int n = 2 * kk + (j >> 1), b = j & 1;
-                    qz[b] = fmaf(rq.r[kk][j].x, zc[n][2 * b], fmaf(rq.r[kk][j].y, zc[n][2 * b + 1], qz[b]));
-                    qh[b] = fmaf(rq.r[kk][j].x, h[n][2 * b], fmaf(rq.r[kk][j].y, h[n][2 * b + 1], qh[b]));
+                    qz[b] = fmaf(fq.r[kk][j].lo(), zc[n][2 * b], fmaf(fq.r[kk][j].hi(), zc[n][2 * b + 1], qz[b]));
+                    qh[b] = fmaf(fq.r[kk][j].lo(), h[n][2 * b], fmaf(fq.r[kk][j].hi(), h[n][2 * b + 1], qh[b]));
                 }
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
@@ -543,10 +576,10 @@ causal_mma_dq_kernel(const Params p) {
 #pragma unroll
                     for (int n = 0; n < DP / 8; ++n)
                         if (n * 8 < D) {
-                            const float2 q = rq.r[n >> 1][(n & 1) * 2 + b];
+                            const auto q = fq.r[n >> 1][(n & 1) * 2 + b];
                             store_pair<IO>(dQ + (n0 + row) * D + n * 8 + 2 * t,
-                                           fmaf(-go, zc[n][2 * b], h[n][2 * b]) * inv * phi_slope_from_value(q.x, phi),
-                                           fmaf(-go, zc[n][2 * b + 1], h[n][2 * b + 1]) * inv * phi_slope_from_value(q.y, phi));
+                                           fmaf(-go, zc[n][2 * b], h[n][2 * b]) * inv * phi_slope_from_value(q.lo(), phi),
+                                           fmaf(-go, zc[n][2 * b + 1], h[n][2 * b + 1]) * inv * phi_slope_from_value(q.hi(), phi));
                         }
                     if (t == 0) {
                         dn_all[n0 + row] = dn;
@@ -556,23 +589,22 @@ causal_mma_dq_kernel(const Params p) {
             }
         }
         st.template update<NQ, NV, true>(sK, sV, nullptr);
+        flip<C, Sh>(buf, smem);
     }
     zero_rows(dQ, r.end, r.hi, D);
 }
 
 // ---- dK, dV sweep ----------------------------------------------------------------------------------------------
-template <typename IO, int DP, int MP, bool MAPPED, bool EXACT>
-__global__ void __launch_bounds__(THREADS, (kResident<DP, MP, 3, kValuePlanes<IO>>))
+template <typename C, int DP, int MP, bool EXACT>
+__global__ void __launch_bounds__(THREADS, (resident<Shared<DP, MP, C::NR, C::NV, C::NS>, C>(C::NP == 1 ? 4 : 3)))
 causal_mma_dkv_kernel(const Params p) {
-    constexpr int NQ = kFeaturePlanes<IO, MAPPED>, NV = kValuePlanes<IO>;
-    using Sh = Shared<DP, MP, 3, NV>;
+    using IO = typename C::IO;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, NR = C::NR;
+    using Sh = Shared<DP, MP, NR, NV, NS>;
     extern __shared__ __align__(128) uint8_t smem[];
-    const uint32_t sQ = smem_u32(smem + Sh::X), sG = smem_u32(smem + Sh::Y), sR = smem_u32(smem + Sh::S);
-    float* sr = reinterpret_cast<float*>(smem + Sh::Z);
-    float* sdl = reinterpret_cast<float*>(smem + Sh::W);
-    uint16_t* wpl = reinterpret_cast<uint16_t*>(smem + Sh::WP);
+    uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = sizeof(IO) == 2 && !MAPPED ? LA_PHI_IDENTITY : p.phi;
+    const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
     const Range r = range_of(p, (int)(gridDim.y - 1 - blockIdx.y));
     const IO* Q = (const IO*)p.Q + r.bh * p.N * D;
@@ -589,15 +621,19 @@ causal_mma_dkv_kernel(const Params p) {
             p.rec + (r.bh * (p.pieces - 1) + r.piece) * (int64_t)(D * M + D), p.pieces - 1 - r.piece);
     const int64_t chunks = (r.end - r.lo + T - 1) / T;
     for (int64_t c = chunks - 1; c >= 0; --c) {
+        const uint32_t sQ = smem_u32(buf + Sh::X), sG = smem_u32(buf + Sh::Y), sR = smem_u32(buf + Sh::S);
+        float* sr = reinterpret_cast<float*>(buf + Sh::Z);
+        float* sdl = reinterpret_cast<float*>(buf + Sh::W);
+        uint16_t* wpl = reinterpret_cast<uint16_t*>(buf + Sh::WP);
         const int64_t n0 = r.lo + c * T;
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T), blocks = (cn + 15) / 16;
         const int strip = (c & 1) ? WARPS - 1 - warp : warp, row0 = strip * 16;
         {
             ReverseRows<IO, DP, MP> rr;
             rr.load(Q, G, dn, delta, n0, cn, D, M, pad);
-            __syncthreads();
-            st.publish(smem + Sh::S, sr);
-            rr.template store<NV>(smem + Sh::X, smem + Sh::Y, sdl, wpl, phi);
+            if constexpr (C::BUF == 1) __syncthreads();
+            st.template publish<NS>(buf + Sh::S, sr);
+            rr.template store<NR, NV>(buf + Sh::X, buf + Sh::Y, sdl, wpl, phi);
         }
         if (c > 0) {
             prefetch_rows(Q, n0 - T, r.end, D);
@@ -612,8 +648,9 @@ causal_mma_dkv_kernel(const Params p) {
                 {
                     RawStrip<IO, DP> rk;
                     rk.load(K + n0 * D, row0, cn, D, pad);
-                    rk.map(phi);
-                    rk.template planes<NQ>(ka);
+                    RawStrip<typename FeatureType<NQ>::type, DP> fk;
+                    rk.template map<NQ>(phi, fk);
+                    fk.template planes<NQ>(ka);
                 }
                 float gv[MP / 8][4];
 #pragma unroll
@@ -621,9 +658,9 @@ causal_mma_dkv_kernel(const Params p) {
                     Chain c;
 #pragma unroll
                     for (int kk = 0; kk < DP / 16; ++kk) {
-                        uint32_t b[3][4];
-                        load_cols_t<3, MP>(b, sR, DP * MP * 2, kk * 16, n * 2, lane);
-                        c.step<NQ, 3>(ka[kk], b);
+                        uint32_t b[NS][4];
+                        load_cols_t<NS, MP>(b, sR, DP * MP * 2, kk * 16, n * 2, lane);
+                        c.step<NQ, NS>(ka[kk], b);
                     }
                     c.put(gv[2 * n], gv[2 * n + 1]);
                 }
@@ -634,9 +671,9 @@ causal_mma_dkv_kernel(const Params p) {
                         Chain c;
 #pragma unroll
                         for (int kk = 0; kk < DP / 16; ++kk) {
-                            uint32_t b[3][4];
-                            load_rows<3, DP>(b, sQ, T * DP * 2, ib * 16, kk * 2, lane);
-                            c.step<NQ, 3>(ka[kk], b);
+                            uint32_t b[NR][4];
+                            load_rows<NR, DP>(b, sQ, T * DP * 2, ib * 16, kk * 2, lane);
+                            c.step<NQ, NR>(ka[kk], b);
                         }
                         c.put(s0, s1);
                     }
@@ -648,13 +685,13 @@ causal_mma_dkv_kernel(const Params p) {
                             if (col + 8 < row) s1[j] = 0.f;
                         }
                     }
-                    uint32_t pa[3][4];
-                    operand_of<3>(pa, s0, s1);
+                    uint32_t pa[NP][4];
+                    operand_of<NP>(pa, s0, s1);
 #pragma unroll
                     for (int n = 0; n < MP / 16; ++n) {
                         uint32_t b[NV][4];
                         load_cols_t<NV, MP>(b, sG, T * MP * 2, ib * 16, n * 2, lane);
-                        block_mma<3, NV>(gv[2 * n], gv[2 * n + 1], pa, b);
+                        block_mma<NP, NV>(gv[2 * n], gv[2 * n + 1], pa, b);
                     }
                 }
 #pragma unroll
@@ -686,9 +723,9 @@ causal_mma_dkv_kernel(const Params p) {
                     Chain c;
 #pragma unroll
                     for (int ee = 0; ee < MP / 16; ++ee) {
-                        uint32_t b[3][4];
-                        load_rows<3, MP>(b, sR, DP * MP * 2, n * 16, ee * 2, lane);
-                        c.step<NV, 3>(va[ee], b);
+                        uint32_t b[NS][4];
+                        load_rows<NS, MP>(b, sR, DP * MP * 2, n * 16, ee * 2, lane);
+                        c.step<NV, NS>(va[ee], b);
                     }
                     c.add_to(gk[2 * n], gk[2 * n + 1]);
                 }
@@ -715,18 +752,19 @@ causal_mma_dkv_kernel(const Params p) {
                             if (col + 8 < row) s1[j] = 0.f;
                         }
                     }
-                    uint32_t pa[3][4];
-                    operand_of<3>(pa, s0, s1);
+                    uint32_t pa[NP][4];
+                    operand_of<NP>(pa, s0, s1);
 #pragma unroll
                     for (int n = 0; n < DP / 16; ++n) {
-                        uint32_t b[3][4];
-                        load_cols_t<3, DP>(b, sQ, T * DP * 2, ib * 16, n * 2, lane);
-                        block_mma<3, 3>(gk[2 * n], gk[2 * n + 1], pa, b);
+                        uint32_t b[NR][4];
+                        load_cols_t<NR, DP>(b, sQ, T * DP * 2, ib * 16, n * 2, lane);
+                        block_mma<NP, NR>(gk[2 * n], gk[2 * n + 1], pa, b);
                     }
                 }
                 RawStrip<IO, DP> rk;
                 rk.load(K + n0 * D, row0, cn, D, pad);
-                rk.map(phi);
+                RawStrip<typename FeatureType<NQ>::type, DP> fk;
+                rk.template map<NQ>(phi, fk);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int row = row0 + g + 8 * h;
@@ -734,15 +772,16 @@ causal_mma_dkv_kernel(const Params p) {
 #pragma unroll
                         for (int n = 0; n < DP / 8; ++n)
                             if (n * 8 < D) {
-                                const float2 k = rk.r[n >> 1][(n & 1) * 2 + h];
-                                store_pair<IO>(dK + (n0 + row) * D + n * 8 + 2 * t, gk[n][2 * h] * phi_slope_from_value(k.x, phi),
-                                               gk[n][2 * h + 1] * phi_slope_from_value(k.y, phi));
+                                const auto k = fk.r[n >> 1][(n & 1) * 2 + h];
+                                store_pair<IO>(dK + (n0 + row) * D + n * 8 + 2 * t, gk[n][2 * h] * phi_slope_from_value(k.lo(), phi),
+                                               gk[n][2 * h + 1] * phi_slope_from_value(k.hi(), phi));
                             }
                     }
                 }
             }
         }
-        st.template update<3, NV, false>(sQ, sG, wpl);
+        st.template update<NR, NV, false>(sQ, sG, wpl);
+        flip<C, Sh>(buf, smem);
     }
     zero_rows(dK, r.end, r.hi, D);
     zero_rows(dV, r.end, r.hi, M);
@@ -803,28 +842,26 @@ int launch(void (*kern)(const Params), unsigned bh, unsigned y, int smem, const 
     return LA_OK;
 }
 
-template <typename IO, int DP, int MP, bool MAPPED, bool EXACT> struct Kernels {
-    static constexpr int NQ = kFeaturePlanes<IO, MAPPED>, NV = kValuePlanes<IO>;
+template <typename C, int DP, int MP, bool EXACT> struct Kernels {
+    using Fwd = Shared<DP, MP, C::NQ, C::NV, C::NS>;
+    using Rev = Shared<DP, MP, C::NR, C::NV, C::NS>;
     static int sums(const la_problem& p, const Params& a, bool reverse, cudaStream_t st) {
         if (a.pieces == 1) return LA_OK;
         const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)(a.pieces - 1);
         constexpr int vec = T * 4 + 3 * T * 2;
-        if (reverse) return launch(causal_mma_sum_kernel<IO, DP, MP, MAPPED, EXACT, true>, bh, y, Shared<DP, MP, 3, NV>::S + vec, a, st);
-        return launch(causal_mma_sum_kernel<IO, DP, MP, MAPPED, EXACT, false>, bh, y, Shared<DP, MP, NQ, NV>::S + vec, a, st);
+        if (reverse) return launch(causal_mma_sum_kernel<C, DP, MP, EXACT, true>, bh, y, C::BUF == 2 ? 2 * Rev::BYTES : Rev::S + vec, a, st);
+        return launch(causal_mma_sum_kernel<C, DP, MP, EXACT, false>, bh, y, C::BUF == 2 ? 2 * Fwd::BYTES : Fwd::S + vec, a, st);
     }
     static int forward(const la_problem& p, const Params& a, cudaStream_t st) {
         if (int rc = sums(p, a, false, st)) return rc;
-        return launch(causal_mma_forward_kernel<IO, DP, MP, MAPPED, EXACT>, (unsigned)(p.B * p.H), (unsigned)a.pieces,
-                      Shared<DP, MP, NQ, NV>::BYTES, a, st);
+        return launch(causal_mma_forward_kernel<C, DP, MP, EXACT>, (unsigned)(p.B * p.H), (unsigned)a.pieces, C::BUF * Fwd::BYTES, a, st);
     }
     static int backward(const la_problem& p, const Params& fwd, const Params& rev, cudaStream_t st) {
         if (int rc = sums(p, fwd, false, st)) return rc;
-        if (int rc = launch(causal_mma_dq_kernel<IO, DP, MP, MAPPED, EXACT>, (unsigned)(p.B * p.H), (unsigned)fwd.pieces,
-                            Shared<DP, MP, NQ, NV>::BYTES, fwd, st))
+        if (int rc = launch(causal_mma_dq_kernel<C, DP, MP, EXACT>, (unsigned)(p.B * p.H), (unsigned)fwd.pieces, C::BUF * Fwd::BYTES, fwd, st))
             return rc;
         if (int rc = sums(p, rev, true, st)) return rc;
-        return launch(causal_mma_dkv_kernel<IO, DP, MP, MAPPED, EXACT>, (unsigned)(p.B * p.H), (unsigned)rev.pieces,
-                      Shared<DP, MP, 3, NV>::BYTES, rev, st);
+        return launch(causal_mma_dkv_kernel<C, DP, MP, EXACT>, (unsigned)(p.B * p.H), (unsigned)rev.pieces, C::BUF * Rev::BYTES, rev, st);
     }
 };
 
@@ -832,15 +869,16 @@ template <typename IO, int DP, int MP, bool MAPPED, bool EXACT> struct Kernels {
 template <typename F> int dispatch(const la_problem& p, F f) {
     const bool exact = (p.D == 32 || p.D == 64 || p.D == 128) && p.M == (p.D == 32 ? 32 : 64);
     if (p.dtype == LA_F32) {
-        if (p.D <= 32 && p.M <= 32) return exact ? f(Kernels<float, 32, 32, true, true>()) : f(Kernels<float, 32, 32, true, false>());
-        if (p.D <= 64) return exact ? f(Kernels<float, 64, 64, true, true>()) : f(Kernels<float, 64, 64, true, false>());
-        return f(Kernels<float, 128, 64, true, false>());
+        if (p.D <= 32 && p.M <= 32) return exact ? f(Kernels<Fp32, 32, 32, true>()) : f(Kernels<Fp32, 32, 32, false>());
+        if (p.D <= 64) return exact ? f(Kernels<Fp32, 64, 64, true>()) : f(Kernels<Fp32, 64, 64, false>());
+        return f(Kernels<Fp32, 128, 64, false>());
     }
+    if (p.D == 32 && p.M == 32) return f(Kernels<Bf16, 32, 32, true>());
     if (p.phi == LA_PHI_IDENTITY) {
-        if (p.D <= 64) return f(Kernels<__nv_bfloat16, 64, 64, false, false>());
-        return exact ? f(Kernels<__nv_bfloat16, 128, 64, false, true>()) : f(Kernels<__nv_bfloat16, 128, 64, false, false>());
+        if (p.D <= 64) return f(Kernels<Bf16Features, 64, 64, false>());
+        return exact ? f(Kernels<Bf16Features, 128, 64, true>()) : f(Kernels<Bf16Features, 128, 64, false>());
     }
-    return p.D <= 64 ? f(Kernels<__nv_bfloat16, 64, 64, true, false>()) : f(Kernels<__nv_bfloat16, 128, 64, true, false>());
+    return p.D <= 64 ? f(Kernels<Bf16Wide, 64, 64, false>()) : f(Kernels<Bf16Wide, 128, 64, false>());
 }
 
 }  // namespace
@@ -848,6 +886,14 @@ template <typename F> int dispatch(const la_problem& p, F f) {
 bool causal_mma_supported(const la_problem& p) {
     static const bool disabled = getenv("LA_DISABLE_TC") != nullptr;
     return !disabled && p.M <= 64;
+}
+
+// bf16, D = M = 32, many short sequences: the tcgen05 kernels run one CTA per SM and start up for about three chunks of
+// 128 positions in every sequence, and handle 128 scores per row where D is 32.  Forward + backward, us, tcgen05 /
+// mma.sync: 1024 heads N 784 373 / 287, 2048 x 300 442 / 234, 512 x 512 131 / 102, 512 x 1024 212 / 192; but
+// 512 x 2048 367 / 372, 256 x 512 66 / 70, 128 x 3072 138 / 195.  (D = M = 64: 512 x 512 161 / 265.)
+bool causal_mma_preferred(const la_problem& p) {
+    return p.dtype == LA_BF16 && p.D == 32 && p.M == 32 && p.B * p.H >= 3 * 148 && p.N <= 1024;
 }
 
 size_t causal_mma_workspace(const la_problem& p, bool backward) {

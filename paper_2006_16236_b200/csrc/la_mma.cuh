@@ -43,6 +43,11 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
 template <int NA, int NB>
 __device__ __forceinline__ void block_mma(float (&acc0)[4], float (&acc1)[4], const uint32_t (&a)[NA][4],
                                           const uint32_t (&b)[NB][4]) {
+    if constexpr (NA == 1 && NB == 1) {
+        mma16816(acc0, a[0], b[0][0], b[0][1]);
+        mma16816(acc1, a[0], b[0][2], b[0][3]);
+        return;
+    }
     float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
     constexpr int top = NA + NB - 2 < 2 ? NA + NB - 2 : 2;
 #pragma unroll
@@ -103,18 +108,6 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t (&p)[NP]) {
         p[2] = __byte_perm(__float_as_uint(sx), __float_as_uint(sy), 0x7632);
     }
 }
-// the value of the low / high half of a split pair (exact)
-template <int NP> __device__ __forceinline__ float joined_lo(const uint32_t (&p)[NP][4], int j) {
-    float v = __uint_as_float(p[0][j] << 16);
-    if constexpr (NP == 3) v = (v + __uint_as_float(p[1][j] << 16)) + __uint_as_float(p[2][j] << 16);
-    return v;
-}
-template <int NP> __device__ __forceinline__ float joined_hi(const uint32_t (&p)[NP][4], int j) {
-    float v = __uint_as_float(p[0][j] & 0xffff0000u);
-    if constexpr (NP == 3) v = (v + __uint_as_float(p[1][j] & 0xffff0000u)) + __uint_as_float(p[2][j] & 0xffff0000u);
-    return v;
-}
-
 // A bf16 plane of a shared-memory tile: rows of C columns, the 16-byte group c of row r stored at c ^ (r & 7), so
 // that the eight rows of an ldmatrix fall into different banks (C = 32: two rows per 128 bytes, at c ^ (r / 2 & 3)).
 template <int C> __device__ __forceinline__ uint32_t tile_at(int row, int group) {
@@ -178,10 +171,12 @@ template <> struct Group8<__nv_bfloat16> {
 // What rows and columns that do not exist are read as: a number whose feature is zero.
 __device__ __forceinline__ float pad_value(int phi) { return phi == LA_PHI_IDENTITY ? 0.f : -INFINITY; }
 
-// f(x) over a range of registers with the feature map chosen once
-template <typename F>
+// f(x) over a range of registers with the feature map chosen once; NQ = 1: the values are rounded to bf16 afterwards,
+// the approximate exponential (2^-22) will do
+template <int NQ, typename F>
 __device__ __forceinline__ void with_phi(int phi, F f) {
     if (phi == LA_PHI_IDENTITY) f([](float x) { return x; });
+    else if constexpr (NQ == 1) f([](float x) { const float e = __expf(x); return x > 0.f ? x + 1.f : e; });
     else f([](float x) { const float e = expf(x); return x > 0.f ? x + 1.f : e; });
 }
 
@@ -197,6 +192,20 @@ struct RawTile {
             r[u].fill(pad);
             if (row < cn && c < cols) r[u].load(src + row * cols + c);
         }
+    }
+    // the one plane of bf16 values
+    __device__ __forceinline__ void copy(uint8_t* tile) const {
+        static_assert(sizeof(IO) == 2, "one plane");
+#pragma unroll
+        for (int u = 0; u < GROUPS; ++u) {
+            const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), g = idx % (C / 8);
+            *reinterpret_cast<uint4*>(tile + tile_at<C>(row, g)) = r[u].a;
+        }
+    }
+    template <int NP>
+    __device__ __forceinline__ void values(uint8_t* tile) const {
+        if constexpr (sizeof(IO) == 2) copy(tile);
+        else store<NP>(tile, [](int, float x) { return x; });
     }
     // planes of f(u, x), u the group's index in r
     template <int NP, typename F>
@@ -221,12 +230,7 @@ struct RawTile {
     }
 };
 
-template <typename IO> __device__ __forceinline__ float2 load_pair(const IO* p);
-template <> __device__ __forceinline__ float2 load_pair<float>(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
-template <> __device__ __forceinline__ float2 load_pair<__nv_bfloat16>(const __nv_bfloat16* p) {
-    const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(p));
-    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
+__device__ __forceinline__ float2 load_pair(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
 template <typename IO> __device__ __forceinline__ void store_pair(IO* p, float x, float y);
 template <> __device__ __forceinline__ void store_pair<float>(float* p, float x, float y) { *reinterpret_cast<float2*>(p) = make_float2(x, y); }
 template <> __device__ __forceinline__ void store_pair<__nv_bfloat16>(__nv_bfloat16* p, float x, float y) {
@@ -235,10 +239,33 @@ template <> __device__ __forceinline__ void store_pair<__nv_bfloat16>(__nv_bfloa
 
 // Sixteen rows as A operands straight from global memory: element pairs (row g or g + 8, columns 16 kk + 2t (+ 8)),
 // which are also the positions of the thread's elements in a 16 x C result.
+template <typename IO> struct Pair;
+template <> struct Pair<float> {
+    float2 v;
+    __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float2*>(p)); }
+    __device__ __forceinline__ void fill(float x) { v = make_float2(x, x); }
+    __device__ __forceinline__ float lo() const { return v.x; }
+    __device__ __forceinline__ float hi() const { return v.y; }
+    __device__ __forceinline__ void set(float x, float y) { v = make_float2(x, y); }
+    template <int NP> __device__ __forceinline__ void planes(uint32_t (&p)[NP]) const { split2<NP>(v.x, v.y, p); }
+};
+template <> struct Pair<__nv_bfloat16> {        // as loaded: one plane
+    uint32_t w;
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { w = __ldg(reinterpret_cast<const uint32_t*>(p)); }
+    __device__ __forceinline__ void fill(float x) { w = __byte_perm(__float_as_uint(x), 0u, 0x3232); }
+    __device__ __forceinline__ float lo() const { return __uint_as_float(w << 16); }
+    __device__ __forceinline__ float hi() const { return __uint_as_float(w & 0xffff0000u); }
+    __device__ __forceinline__ void set(float x, float y) { w = pack_rn(x, y); }
+    template <int NP> __device__ __forceinline__ void planes(uint32_t (&p)[NP]) const {
+        static_assert(NP == 1, "a bf16 pair has one plane");
+        p[0] = w;
+    }
+};
+
 template <typename IO, int C>
 struct RawStrip {
     static constexpr int KS = C / 16;
-    float2 r[KS][4];
+    Pair<IO> r[KS][4];
     __device__ __forceinline__ void load(const IO* src, int row0, int cn, int cols, float pad) {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -246,18 +273,18 @@ struct RawStrip {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int row = row0 + g + (j & 1) * 8, c = kk * 16 + t * 2 + (j >> 1) * 8;
-                r[kk][j] = row < cn && c < cols ? load_pair<IO>(src + row * cols + c) : make_float2(pad, pad);
+                r[kk][j].fill(pad);
+                if (row < cn && c < cols) r[kk][j].load(src + row * cols + c);
             }
     }
-    __device__ __forceinline__ void map(int phi) {
-        with_phi(phi, [&](auto f) {
+    // features: as fp32 pairs, or (To = bf16) rounded
+    template <int NQ, typename To>
+    __device__ __forceinline__ void map(int phi, RawStrip<To, C>& out) const {
+        with_phi<NQ>(phi, [&](auto f) {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    r[kk][j].x = f(r[kk][j].x);
-                    r[kk][j].y = f(r[kk][j].y);
-                }
+                for (int j = 0; j < 4; ++j) out.r[kk][j].set(f(r[kk][j].lo()), f(r[kk][j].hi()));
         });
     }
     template <int NP>
@@ -267,7 +294,7 @@ struct RawStrip {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 uint32_t p[NP];
-                split2<NP>(r[kk][j].x, r[kk][j].y, p);
+                r[kk][j].template planes<NP>(p);
 #pragma unroll
                 for (int k = 0; k < NP; ++k) a[kk][k][j] = p[k];
             }

@@ -121,6 +121,7 @@ bool tc_supported(const la_problem& p, int op) {
     if (disabled) return false;
     if (p.dtype != LA_BF16 || p.D != p.M || (p.D != 32 && p.D != 64)) return false;
     if (p.N < 1) return false;      // any length: a last chunk that is not full is handled as padding
+    if ((op == LA_OP_CAUSAL_FORWARD || op == LA_OP_CAUSAL_BACKWARD) && causal_mma_preferred(p)) return false;
     if (p.B * p.H * p.N >= (1LL << 31)) return false;          // TMA coordinates are 32-bit
     return op >= LA_OP_LINEAR_FORWARD && op <= LA_OP_CAUSAL_BACKWARD;
 }

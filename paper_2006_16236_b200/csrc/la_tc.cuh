@@ -14,6 +14,7 @@ int tc_causal_plan(const la_problem& p, int32_t* out, int capacity);
 // Causal form at fp32 accuracy on mma.sync (la_causal_mma.cu): M <= 64, any type and feature map.  The forward's
 // workspace is optional (without it a sequence is one piece).
 bool causal_mma_supported(const la_problem& p);
+bool causal_mma_preferred(const la_problem& p);      // of the problems that both kinds of kernels take
 size_t causal_mma_workspace(const la_problem& p, bool backward);
 int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
                        const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* ws, size_t ws_bytes, cudaStream_t st);

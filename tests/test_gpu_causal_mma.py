@@ -13,6 +13,7 @@ import torch
 import oracle
 import paper_2006_16236_b200 as la
 from paper_2006_16236_b200.inputs import draw_qkvg
+from parity import assert_close
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -81,3 +82,32 @@ def test_state_lengths_and_no_workspace(pieces):
                 num = w @ V[b, :, :n].double().numpy() + fq[b, :, :n] @ S0[b].double().cpu().numpy()
                 den = w.sum(-1) + np.einsum("hnd,hd->hn", fq[b, :, :n], Z0[b].double().cpu().numpy())
                 _close(O[b, :, :n], num / den[..., None], 2e-6, "O")
+
+
+@pytest.mark.parametrize("pieces", [-1, 2])
+@pytest.mark.parametrize("N", [1, 64, 130, 1024])
+def test_many_short_bf16_sequences(N, pieces):
+    """bf16, D = M = 32, at least 444 sequences of at most 1024 positions, whole and ragged, held to the bf16 gates."""
+    B, H, D = 56, 8, 32
+    if N == 1024 and pieces > 0:
+        pytest.skip("covered by the shorter ones")
+    Q, K, V, G = draw_qkvg(B, H, N, D, D, 3 + N, torch.bfloat16, 1.0)
+    la.la_plan_override(pieces)
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    lengths = [N - (5 * b) % N for b in range(B)]
+    for ln in (None, torch.tensor(lengths, dtype=torch.int32, device=DEV)):
+        den = torch.empty(B, H, N, device=DEV)
+        O = la.la_causal_forward(*dev[:3], den=den, lengths=ln)
+        grads = la.la_causal_backward(*dev, lengths=ln)
+        la.la_last_device_status()
+        for b in (0, 1, 17, B - 1):
+            n = N if ln is None else lengths[b]
+            sl = (slice(b, b + 1), slice(0, H, 7), slice(0, n))
+            q, k, v, g = (t[sl].double().numpy() for t in (Q, K, V, G))
+            Or, denr = oracle.linear_attention(q, k, v, causal=True)[:2]
+            assert_close(O[sl], Or, torch.bfloat16, "O")
+            assert_close(den[sl], denr, torch.bfloat16, "den")
+            for nm, x, ref in zip(("dQ", "dK", "dV"), grads, oracle.linear_attention_backward(q, k, v, g, causal=True)):
+                assert_close(x[sl], ref, torch.bfloat16, nm, grad=True)
+                assert not x[b, :, n:].any()
+            assert not O[b, :, n:].any()
