@@ -1,11 +1,11 @@
 // Causal form (Eq. 8-15) at fp32 accuracy on mma.sync (la_mma.cuh): fp32 problems, and bf16 ones of shapes or feature
-// maps that the tcgen05 kernels do not take; M <= 64, any D.
+// maps that the tcgen05 kernels do not take; M <= 64, any D.  Also, with single bf16 planes, many short sequences of
+// D = M = 32 (causal_mma_preferred).
 //
-// A sequence is cut into pieces, one CTA of four warps each; a CTA walks its piece in chunks of T = 64 positions.
-// Per chunk a warp owns a strip of sixteen rows (queries in the forward sweeps, keys in the reverse one) whose
-// operand it loads from global memory into registers, and sixteen rows of the running state per 64 of D, kept in
-// fp32 registers.  The other operands (K | V, or Q / dn | G) and the state before the chunk lie in shared memory as
-// bf16 planes.  Two barriers per chunk: planes free, planes written.
+// A sequence is cut into pieces, one CTA each; a CTA walks its piece in chunks of T = 64 positions.  Per chunk a strip of
+// sixteen rows (queries in the forward sweeps, keys in the reverse one) belongs to a pair of warps, and so do sixteen
+// rows of the running state, kept in fp32 registers.  The operands that all warps read (K | V, or Q / dn | G) and the
+// state before the chunk lie in shared memory as bf16 planes; scores never leave the registers of their warp.
 //
 //   forward   O  = [(q k^T o L) [V | 1] + q [S | Z]],            S += k^T V,  Z += k^T 1
 //   dQ sweep  h  = (G V^T o L) k + G S^T,  Zc = L k + Z,  dn = q . Zc + eps,
@@ -13,10 +13,22 @@
 //   dK, dV    with q^ = q / dn, dl = -G . O:  gV = (q^ k^T o L)^T G + k R,
 //             gk = ((G V^T + dl) o L)^T q^ + V R^T + r,           R += q^^T G,  r += q^^T dl  (chunks last to first)
 //
+// The two warps of a strip share the products: forward, one the state's part and one the scores' part; dQ, one G S^T and
+// L k, one the scores' part; reverse, one dV and one dK.  The partial sums of the first two are added through shared
+// memory (the state planes, once nobody reads them any more).  Two warps per strip at 128 registers keep four warps on
+// a scheduler; one warp per strip at 168 to 255 registers kept two, and the tensor pipe 45 % busy.  Problems with single
+// planes have too little work for that: one warp per strip takes both parts (WPS = 1).
+//
 // Pieces other than the first (last, for the reverse sweep) start from the sum of the records [S | Z] of the pieces
 // before (after) them, which a pre-pass writes to the workspace.
+#include <stdlib.h>
+
+#include <atomic>
+#include <type_traits>
+
 #include "la_mma.cuh"
 #include "la_tc.cuh"
+#include "la_tc_common.cuh"
 
 namespace la {
 namespace {
@@ -24,9 +36,7 @@ namespace {
 using namespace mma;
 
 constexpr int T = 64;
-constexpr int THREADS = 128;
-constexpr int WARPS = THREADS / 32;
-static_assert(T == 16 * WARPS, "one strip of sixteen rows per warp");
+constexpr int STRIPS_T = T / 16;
 
 struct Params {
     const void *Q, *K, *V, *G;
@@ -39,6 +49,7 @@ struct Params {
     const int* lengths;
     int64_t N, piece_len;
     int pieces, heads, D, M, phi;
+    int chained;                 // launched as a programmatic dependent of the kernel before it in the stream
     float eps;
 };
 
@@ -58,17 +69,38 @@ __device__ __forceinline__ Range range_of(const Params& p, int piece) {
     return r;
 }
 
-template <typename IO>
+template <int THREADS, typename IO>
 __device__ void zero_rows(IO* x, int64_t from, int64_t to, int cols) {       // rows from .. to - 1
     for (int64_t i = from * cols + threadIdx.x; i < to * cols; i += THREADS) x[i] = from_f32<IO>(0.f);
 }
 
-// The running sums of a warp: rows d = 16 strip + g (+ 8), strip = warp (+ 4); with two strips (D <= 32) two warps
-// share one and take half of its columns each.  Columns e = 8 (n0 + n) + 2 t (+ 1).
-template <int DP, int MP>
+// u (16 x 8, the same in every column) += A (16 x 16) v, v = elements k0 .. k0 + 15 of a vector held as three planes of
+// LEN elements; smallest partial products first
+template <int NX, int LEN>
+__device__ __forceinline__ void vector_mma(float (&u)[4], const uint32_t (&a)[NX][4], const uint16_t* pl, int k0, int t) {
+    uint32_t w[3][2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        w[k][0] = *reinterpret_cast<const uint32_t*>(pl + k * LEN + k0 + 2 * t);
+        w[k][1] = *reinterpret_cast<const uint32_t*>(pl + k * LEN + k0 + 8 + 2 * t);
+    }
+#pragma unroll
+    for (int sum = 2; sum >= 0; --sum)
+#pragma unroll
+        for (int k = 0; k < NX; ++k)
+            if (sum - k >= 0) mma16816(u, a[k], w[sum - k][0], w[sum - k][1]);
+}
+
+// The running sums of a warp: rows d = 16 strip + g (+ 8), columns e = 8 (n0 + n) + 2 t (+ 1).  The warps share the DP / 16
+// strips out among them: several strips a warp, or several warps a strip with a part of its columns each (at least
+// sixteen: with D = M = 32 and eight warps four of them have none).
+template <int DP, int MP, int WARPS>
 struct State {
-    static constexpr int STRIPS = DP / 16, SHARE = STRIPS < WARPS ? WARPS / STRIPS : 1, SD = STRIPS < WARPS ? 1 : STRIPS / WARPS;
+    static constexpr int STRIPS = DP / 16, WANT = STRIPS < WARPS ? WARPS / STRIPS : 1;
+    static constexpr int SHARE = WANT < MP / 16 ? WANT : MP / 16, SD = STRIPS < WARPS ? 1 : STRIPS / WARPS;
     static constexpr int NC = MP / 8 / SHARE;
+    static constexpr bool ALL = STRIPS * SHARE >= WARPS;
+    static __device__ __forceinline__ bool owner() { return ALL || ((int)threadIdx.x >> 5) < STRIPS * SHARE; }
     static __device__ __forceinline__ int strip(int i) { return ((int)threadIdx.x >> 5) % STRIPS + WARPS * i; }
     static __device__ __forceinline__ int n0() { return SHARE == 1 ? 0 : ((int)threadIdx.x >> 5) / STRIPS * NC; }
     float s[SD][NC][4];
@@ -77,6 +109,7 @@ struct State {
     __device__ __forceinline__ void init(const Params& p, const float* S0, const float* Z0, const float* rec, int nrec) {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, c0 = n0();
         const int size = p.D * p.M + p.D;
+        if (!owner()) return;
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
             const int d = strip(i) * 16 + g;
@@ -110,6 +143,7 @@ struct State {
     }
     __device__ __forceinline__ void write(const Params& p, float* S1, float* Z1) const {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, c0 = n0();
+        if (!owner()) return;
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
             const int d = strip(i) * 16 + g;
@@ -123,10 +157,11 @@ struct State {
                 }
         }
     }
-    // the operand planes [DP][MP] of the matrix and the vector in fp32
+    // the operand planes [DP][MP] of the matrix; the vector in fp32 and as three planes of DP elements
     template <int NS>
-    __device__ __forceinline__ void publish(uint8_t* tile, float* vec) const {
+    __device__ __forceinline__ void publish(uint8_t* tile, float* vec, uint16_t* vpl) const {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, c0 = n0();
+        if (!owner()) return;
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
             const int d = strip(i) * 16 + g;
@@ -141,8 +176,15 @@ struct State {
                         *reinterpret_cast<uint32_t*>(tile + k * (DP * MP * 2) + tile_at<MP>(d + 8 * h, c0 + n) + t * 4) = o[k];
                 }
             if (t == 0 && c0 == 0) {
+                uint32_t o[3];
+                split2<3>(z[i][0], z[i][1], o);
                 vec[d] = z[i][0];
                 vec[d + 8] = z[i][1];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    vpl[k * DP + d] = (uint16_t)o[k];
+                    vpl[k * DP + d + 8] = (uint16_t)(o[k] >> 16);
+                }
             }
         }
     }
@@ -152,34 +194,24 @@ struct State {
     template <int NX, int NY, bool ONES>
     __device__ __forceinline__ void update(uint32_t X, uint32_t Y, const uint16_t* wpl) {
         const int lane = threadIdx.x & 31, t = lane & 3, c0 = n0();
+        if (!owner()) return;
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
             uint32_t a[T / 16][NX][4];
             float zs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int b = 0; b < T / 16; ++b)
-                {
-                    load_rows_t<NX, DP>(a[b], X, T * DP * 2, b * 16, strip(i) * 2, lane);
-                    float u[4] = {0.f, 0.f, 0.f, 0.f};
-                    if constexpr (ONES) {
+            for (int b = 0; b < T / 16; ++b) {
+                load_rows_t<NX, DP>(a[b], X, T * DP * 2, b * 16, strip(i) * 2, lane);
+                float u[4] = {0.f, 0.f, 0.f, 0.f};
+                if constexpr (ONES) {
 #pragma unroll
-                        for (int k = NX - 1; k >= 0; --k) mma16816(u, a[b][k], 0x3f803f80u, 0x3f803f80u);
-                    } else {
-                        uint32_t w[3][2];
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            w[k][0] = *reinterpret_cast<const uint32_t*>(wpl + k * T + b * 16 + 2 * t);
-                            w[k][1] = *reinterpret_cast<const uint32_t*>(wpl + k * T + b * 16 + 8 + 2 * t);
-                        }
-#pragma unroll
-                        for (int sum = 2; sum >= 0; --sum)
-#pragma unroll
-                            for (int k = 0; k < NX; ++k)
-                                if (sum - k >= 0) mma16816(u, a[b][k], w[sum - k][0], w[sum - k][1]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) zs[j] += u[j];
+                    for (int k = NX - 1; k >= 0; --k) mma16816(u, a[b][k], 0x3f803f80u, 0x3f803f80u);
+                } else {
+                    vector_mma<NX, T>(u, a[b], wpl, b * 16, t);
                 }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) zs[j] += u[j];
+            }
             z[i][0] += zs[0];
             z[i][1] += zs[2];
 #pragma unroll
@@ -187,10 +219,10 @@ struct State {
                 Chain c;
 #pragma unroll
                 for (int b = 0; b < T / 16; ++b) {
-                        uint32_t y[NY][4];
-                        load_cols_t<NY, MP>(y, Y, T * MP * 2, b * 16, c0 + n * 2, lane);
-                        c.step<NX, NY>(a[b], y);
-                    }
+                    uint32_t y[NY][4];
+                    load_cols_t<NY, MP>(y, Y, T * MP * 2, b * 16, c0 + n * 2, lane);
+                    c.step<NX, NY>(a[b], y);
+                }
                 c.add_to(s[i][2 * n], s[i][2 * n + 1]);
             }
         }
@@ -199,20 +231,53 @@ struct State {
 
 // I/O type and planes of each kind of operand: feature-mapped rows (NQ), value rows V, G (NV), scores (NP), state (NS),
 // q / dn (NR).  Everything computed in fp32 has three planes; bf16 values, and features that are bf16 as given, one.
-struct Fp32 { using IO = float; static constexpr int NQ = 3, NV = 3, NP = 3, NS = 3, NR = 3, BUF = 1; static constexpr bool MAPPED = true; };
-struct Bf16Wide { using IO = __nv_bfloat16; static constexpr int NQ = 3, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1; static constexpr bool MAPPED = true; };
-struct Bf16Features { using IO = __nv_bfloat16; static constexpr int NQ = 1, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1; static constexpr bool MAPPED = false; };
+struct Fp32 {
+    using IO = float;
+    static constexpr int NQ = 3, NV = 3, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
+    static constexpr bool MAPPED = true;
+};
+struct Bf16Wide {
+    using IO = __nv_bfloat16;
+    static constexpr int NQ = 3, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
+    static constexpr bool MAPPED = true;
+};
+struct Bf16Features {
+    using IO = __nv_bfloat16;
+    static constexpr int NQ = 1, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
+    static constexpr bool MAPPED = false;
+};
+// ... with one warp per strip, at twice the registers: where a machine full of CTAs keeps the schedulers busy anyway, the
+// hand-overs cost more than they give.  Forward + backward, us, one / two warps: fp32 B32 H8 N4096 D64 2690 / 2930,
+// B4 H8 N4096 477 / 472, B1 H8 N1024 122 / 94; Fourier B8 H8 N1000 C128 272 / 288, B1 H8 N4000 343 / 265.
+struct Fp32One : Fp32 { static constexpr int WPS = 1; };
+struct Bf16FeaturesOne : Bf16Features { static constexpr int WPS = 1; };
 // bf16 operands throughout (with fp32 sums), as the tcgen05 kernels have them.  BUF = 2: the small tiles are there twice,
 // one barrier per chunk (the other set was last read before the barrier of this chunk).
-struct Bf16 { using IO = __nv_bfloat16; static constexpr int NQ = 1, NV = 1, NP = 1, NS = 1, NR = 1, BUF = 2; static constexpr bool MAPPED = true; };
-
-template <int DP, int MP, int NX, int NY, int NS> struct Shared {       // tile X [T][DP], tile Y [T][MP], state planes, vectors
-    static constexpr int X = 0, Y = X + NX * T * DP * 2, S = Y + NY * T * MP * 2, Z = S + NS * DP * MP * 2,
-                         W = Z + DP * 4, WP = W + T * 4, BYTES = (WP + 3 * T * 2 + 127) / 128 * 128;
+struct Bf16 {
+    using IO = __nv_bfloat16;
+    static constexpr int NQ = 1, NV = 1, NP = 1, NS = 1, NR = 1, BUF = 2, WPS = 1;
+    static constexpr bool MAPPED = true;
 };
-// CTAs of an SM that the registers are shared out for: as many as shared memory holds, at most `most`
-template <typename Sh, typename C> constexpr int resident(int most) {
-    const int fit = 227 * 1024 / (C::BUF * Sh::BYTES + 1024);
+
+// Shared memory: tiles X [T][DP] and Y [T][MP]; with two warps per strip the tile that holds the strips' own operand
+// (RC columns, NRW planes); the state planes, later the partial results of the strips (EX columns); the vectors.
+template <int WPS, int DP, int MP, int NX, int NY, int NRW, int RC, int NS, int EX> struct Layout {
+    static constexpr int X = 0, Y = X + NX * T * DP * 2, R = Y + NY * T * MP * 2, S = R + (WPS == 2 ? NRW * T * RC * 2 : 0),
+                         PLANES = NS * DP * MP * 2, PART = WPS == 2 ? T * EX * 4 : 0,
+                         Z = S + (PLANES > PART ? PLANES : PART), ZP = Z + DP * 4, W = ZP + 3 * DP * 2, WP = W + T * 4,
+                         BYTES = (WP + 3 * T * 2 + 127) / 128 * 128;
+};
+template <typename C, int DP, int MP> using ForwardLayout = Layout<C::WPS, DP, MP, C::NQ, C::NV, C::NQ, DP, C::NS, MP>;
+template <typename C, int DP, int MP> using DqLayout = Layout<C::WPS, DP, MP, C::NQ, C::NV, C::NV, MP, C::NS, DP>;
+template <typename C, int DP, int MP> using DkvLayout = Layout<C::WPS, DP, MP, C::NR, C::NV, 0, 0, C::NS, 0>;
+template <typename C, int DP, int MP, bool REVERSE>
+using SumLayout = Layout<1, DP, MP, REVERSE ? C::NR : C::NQ, C::NV, 0, 0, 0, 0>;
+
+template <typename C> constexpr int kThreads = 128 * C::WPS;
+// CTAs of an SM that the registers are shared out for: as many as shared memory holds, at most two (or `three_planes`),
+// or four where operands have single planes (1024 sequences of 784: 287 us, five 300, six 330)
+template <typename Sh, typename C> constexpr int resident(int three_planes = 2) {
+    const int fit = 227 * 1024 / (C::BUF * Sh::BYTES + 1024), most = C::NP == 1 ? 4 : three_planes;
     return fit < most ? fit : most;
 }
 
@@ -221,7 +286,37 @@ __device__ __forceinline__ void flip(uint8_t*& buf, uint8_t* smem) {
     if constexpr (C::BUF == 2) buf = buf == smem ? smem + Sh::BYTES : smem;
 }
 
-template <typename IO>
+// named barriers: 1 = the state planes are no longer read; 2 + strip, 6 + strip = hand-overs within a pair of warps
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+    __threadfence_block();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// a strip's partial results between its two warps, whose lanes hold the same positions
+template <int NT8>
+__device__ __forceinline__ void put_part(uint8_t* area, int strip, const float (&x)[NT8][4]) {
+    float4* d = reinterpret_cast<float4*>(area) + strip * NT8 * 32 + (threadIdx.x & 31);
+#pragma unroll
+    for (int n = 0; n < NT8; ++n) d[n * 32] = make_float4(x[n][0], x[n][1], x[n][2], x[n][3]);
+}
+template <int NT8>
+__device__ __forceinline__ void add_part(const uint8_t* area, int strip, float (&x)[NT8][4]) {
+    const float4* d = reinterpret_cast<const float4*>(area) + strip * NT8 * 32 + (threadIdx.x & 31);
+#pragma unroll
+    for (int n = 0; n < NT8; ++n) {
+        const float4 v = d[n * 32];
+        x[n][0] += v.x; x[n][1] += v.y; x[n][2] += v.z; x[n][3] += v.w;
+    }
+}
+template <int NT8> __device__ __forceinline__ void clear(float (&x)[NT8][4]) {
+#pragma unroll
+    for (int n = 0; n < NT8; ++n)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[n][j] = 0.f;
+}
+
+template <int THREADS, typename IO>
 __device__ __forceinline__ void prefetch_rows(const IO* x, int64_t n0, int64_t end, int cols) {
     if (n0 < 0 || n0 >= end) return;
     const int64_t rows = end - n0 < T ? end - n0 : T;
@@ -233,18 +328,54 @@ __device__ __forceinline__ void prefetch_rows(const IO* x, int64_t n0, int64_t e
 template <int NQ> struct FeatureType { using type = float; };
 template <> struct FeatureType<1> { using type = __nv_bfloat16; };
 
+// The A operand of a strip: planes in registers (one warp per strip), or read from a tile block by block (two warps).
+template <int WPS, int NP, int C> struct StripOperand;
+template <int NP, int C> struct StripOperand<1, NP, C> {
+    uint32_t a[C / 16][NP][4];
+    __device__ __forceinline__ const uint32_t (&block(int kk, uint32_t (&)[NP][4]) const)[NP][4] { return a[kk]; }
+};
+template <int NP, int C> struct StripOperand<2, NP, C> {
+    uint32_t tile;
+    int row0, lane;
+    __device__ __forceinline__ const uint32_t (&block(int kk, uint32_t (&f)[NP][4]) const)[NP][4] {
+        load_cols<NP, C>(f, tile, T * C * 2, row0, kk * 2, lane);
+        return f;
+    }
+};
+
+// The strip of a warp.  It alternates with the chunk, so that the strips with the most blocks go round the schedulers, and
+// the second four warps have them the other way round, so that the two warps of a scheduler together have a middling load.
+__device__ __forceinline__ int strip_of(int warp, bool odd) {
+    const int s = warp % STRIPS_T;
+    return odd != (warp >= STRIPS_T) ? STRIPS_T - 1 - s : s;
+}
+
+// zero the scores of a diagonal block: columns right of the row (UPPER: left of it)
+template <bool UPPER>
+__device__ __forceinline__ void mask_diagonal(float (&s0)[4], float (&s1)[4], int g, int t) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int row = g + (j >> 1) * 8, col = 2 * t + (j & 1);
+        if (UPPER ? col < row : col > row) s0[j] = 0.f;
+        if (UPPER ? col + 8 < row : col + 8 > row) s1[j] = 0.f;
+    }
+}
+
 // ---- forward ---------------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(THREADS, (resident<Shared<DP, MP, C::NQ, C::NV, C::NS>, C>(C::NP == 1 ? 4 : sizeof(typename C::IO) == 4 && DP == 64 ? 2 : 3)))
+__global__ void __launch_bounds__(kThreads<C>, (resident<ForwardLayout<C, DP, MP>, C>()))
 causal_mma_forward_kernel(const Params p) {
     using IO = typename C::IO;
-    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS;
-    using Sh = Shared<DP, MP, NQ, NV, NS>;
+    using Sh = ForwardLayout<C, DP, MP>;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, WPS = C::WPS, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const bool state_part = WPS == 1 || warp < STRIPS_T, score_part = WPS == 1 || warp >= STRIPS_T;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
+    wait_for_stream();
+    release_next();
     const Range r = range_of(p, blockIdx.y);
     const IO* Q = (const IO*)p.Q + r.bh * p.N * D;
     const IO* K = (const IO*)p.K + r.bh * p.N * D;
@@ -252,83 +383,64 @@ causal_mma_forward_kernel(const Params p) {
     IO* O = (IO*)p.O + r.bh * p.N * M;
     float* den = p.den ? p.den + r.bh * p.N : nullptr;
 
-    State<DP, MP> st;
+    State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + r.bh * (p.pieces - 1) * (int64_t)(D * M + D), r.piece);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(buf + Sh::X), sV = smem_u32(buf + Sh::Y), sS = smem_u32(buf + Sh::S);
         float* sZ = reinterpret_cast<float*>(buf + Sh::Z);
+        uint16_t* sZp = reinterpret_cast<uint16_t*>(buf + Sh::ZP);
+        float* sden = reinterpret_cast<float*>(buf + Sh::W);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
-        // (the strip with the most blocks left of the diagonal goes round the schedulers)
-        const int strip = ((n0 / T) & 1) ? WARPS - 1 - warp : warp, row0 = strip * 16;
-        RawStrip<IO, DP> rq;
-        rq.load(Q + n0 * D, row0, cn, D, pad);
+        const int strip = strip_of(warp, (n0 / T) & 1), row0 = strip * 16;
+        StripOperand<WPS, NQ, DP> q;
         {
             RawTile<IO, T, DP, THREADS> rk;
             RawTile<IO, T, MP, THREADS> rv;
+            std::conditional_t<WPS == 1, RawStrip<IO, DP>, RawTile<IO, T, DP, THREADS>> rq;
             rk.load(K + n0 * D, cn, D, pad);
             rv.load(V + n0 * M, cn, M, 0.f);
+            if constexpr (WPS == 1) rq.load(Q + n0 * D, row0, cn, D, pad);
+            else rq.load(Q + n0 * D, cn, D, pad);
             if constexpr (C::BUF == 1) __syncthreads();         // the planes of the chunk before are no longer read
-            st.template publish<NS>(buf + Sh::S, sZ);
+            st.template publish<NS>(buf + Sh::S, sZ, sZp);
             with_phi<NQ>(phi, [&](auto f) { rk.template store<NQ>(buf + Sh::X, [&](int, float x) { return f(x); }); });
             rv.template values<NV>(buf + Sh::Y);
-        }
-        prefetch_rows(Q, n0 + T, r.end, D);
-        prefetch_rows(K, n0 + T, r.end, D);
-        prefetch_rows(V, n0 + T, r.end, M);
-        __syncthreads();
-        if (row0 < cn) {
-            RawStrip<typename FeatureType<NQ>::type, DP> fq;
-            rq.template map<NQ>(phi, fq);
-            float d0 = 0.f, d1 = 0.f;           // rows g, g + 8: q . Z, then + the scores
-#pragma unroll
-            for (int kk = 0; kk < DP / 16; ++kk)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float2 z = *reinterpret_cast<const float2*>(sZ + kk * 16 + h * 8 + 2 * t);
-                    d0 = fmaf(fq.r[kk][2 * h].lo(), z.x, fmaf(fq.r[kk][2 * h].hi(), z.y, d0));
-                    d1 = fmaf(fq.r[kk][2 * h + 1].lo(), z.x, fmaf(fq.r[kk][2 * h + 1].hi(), z.y, d1));
-                }
-            uint32_t qa[DP / 16][NQ][4];
-            fq.template planes<NQ>(qa);
-            float o[MP / 8][4];
-#pragma unroll
-            for (int n = 0; n < MP / 16; ++n) {
-                Chain c;
-#pragma unroll
-                for (int kk = 0; kk < DP / 16; ++kk) {
-                    uint32_t b[NS][4];
-                    load_cols_t<NS, MP>(b, sS, DP * MP * 2, kk * 16, n * 2, lane);
-                    c.step<NQ, NS>(qa[kk], b);
-                }
-                c.put(o[2 * n], o[2 * n + 1]);
+            if constexpr (WPS == 1) {
+                RawStrip<typename FeatureType<NQ>::type, DP> fq;
+                rq.template map<NQ>(phi, fq);
+                fq.template planes<NQ>(q.a);
+            } else {
+                with_phi<NQ>(phi, [&](auto f) { rq.template store<NQ>(buf + Sh::R, [&](int, float x) { return f(x); }); });
+                q.tile = smem_u32(buf + Sh::R); q.row0 = row0; q.lane = lane;
             }
+        }
+        prefetch_rows<THREADS>(Q, n0 + T, r.end, D);
+        prefetch_rows<THREADS>(K, n0 + T, r.end, D);
+        prefetch_rows<THREADS>(V, n0 + T, r.end, M);
+        __syncthreads();
+        const bool real = row0 < cn;
+        float o[MP / 8][4], d0 = 0.f, d1 = 0.f;         // rows g, g + 8 of [num | den]; d0, d1 spread over the four lanes
+        auto scores = [&](int from, int to) {           // o += ((q k^T) o L) V, d0, d1 += its row sums, key blocks from .. to
 #pragma unroll 1
-            for (int jb = 0; jb <= strip; ++jb) {
+            for (int jb = from; jb <= to; ++jb) {
                 float s0[4], s1[4];
                 {
                     Chain c;
 #pragma unroll
                     for (int kk = 0; kk < DP / 16; ++kk) {
-                        uint32_t b[NQ][4];
+                        uint32_t b[NQ][4], f[NQ][4];
                         load_rows<NQ, DP>(b, sK, T * DP * 2, jb * 16, kk * 2, lane);
-                        c.step<NQ, NQ>(qa[kk], b);
+                        c.step<NQ, NQ>(q.block(kk, f), b);
                     }
                     c.put(s0, s1);
                 }
-                if (jb == strip) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int row = g + (j >> 1) * 8, col = 2 * t + (j & 1);
-                        if (col > row) s0[j] = 0.f;
-                        if (col + 8 > row) s1[j] = 0.f;
-                    }
-                }
+                if (jb == strip) mask_diagonal<false>(s0, s1, g, t);
                 uint32_t pa[NP][4];
                 operand_of<NP>(pa, s0, s1);
-                if constexpr (NP == 1) {
+                if constexpr (NP == 1) {            // numerator and normaliser see the same rounded scores
                     float u[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma16816(u, pa[0], 0x3f803f80u, 0x3f803f80u);       // row sums (in every column; lane 0 of a row counts)
+                    mma16816(u, pa[0], 0x3f803f80u, 0x3f803f80u);
                     d0 += t == 0 ? u[0] : 0.f;
                     d1 += t == 0 ? u[2] : 0.f;
                 } else {
@@ -342,8 +454,57 @@ causal_mma_forward_kernel(const Params p) {
                     block_mma<NP, NV>(o[2 * n], o[2 * n + 1], pa, b);
                 }
             }
+        };
+        // (long strips: the warp of the state's part takes the first block of scores as well)
+        const bool shared_block = WPS == 2 && strip >= 2;
+        if (state_part) {
+            if (real) {
+#pragma unroll
+                for (int n = 0; n < MP / 16; ++n) {
+                    Chain c;
+#pragma unroll
+                    for (int kk = 0; kk < DP / 16; ++kk) {
+                        uint32_t b[NS][4], f[NQ][4];
+                        load_cols_t<NS, MP>(b, sS, DP * MP * 2, kk * 16, n * 2, lane);
+                        c.step<NQ, NS>(q.block(kk, f), b);
+                    }
+                    c.put(o[2 * n], o[2 * n + 1]);
+                }
+#pragma unroll
+                for (int kk = 0; kk < DP / 16; ++kk) {
+                    float u[4] = {0.f, 0.f, 0.f, 0.f};
+                    uint32_t f[NQ][4];
+                    vector_mma<NQ, DP>(u, q.block(kk, f), sZp, kk * 16, t);
+                    d0 += t == 0 ? u[0] : 0.f;
+                    d1 += t == 0 ? u[2] : 0.f;
+                }
+                if (shared_block) scores(0, 0);
+            }
+            if constexpr (WPS == 2) {
+                bar_sync(1, 128);
+                if (real) {
+                    put_part(buf + Sh::S, strip, o);
+                    d0 = quad_sum(d0);
+                    d1 = quad_sum(d1);
+                    if (t == 0) {
+                        sden[row0 + g] = d0;
+                        sden[row0 + g + 8] = d1;
+                    }
+                    bar_arrive(2 + strip, 64);
+                }
+            }
+        }
+        if (score_part && real) {
+            if constexpr (WPS == 2) clear(o);
+            scores(shared_block ? 1 : 0, strip);
             d0 = quad_sum(d0);
             d1 = quad_sum(d1);
+            if constexpr (WPS == 2) {
+                bar_sync(2 + strip, 64);
+                add_part(buf + Sh::S, strip, o);
+                d0 += sden[row0 + g];
+                d1 += sden[row0 + g + 8];
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int row = row0 + g + 8 * h;
@@ -359,14 +520,14 @@ causal_mma_forward_kernel(const Params p) {
         st.template update<NQ, NV, true>(sK, sV, nullptr);
         flip<C, Sh>(buf, smem);
     }
-    zero_rows(O, r.end, r.hi, M);
-    if (den) zero_rows(den, r.end, r.hi, 1);
+    zero_rows<THREADS>(O, r.end, r.hi, M);
+    if (den) zero_rows<THREADS>(den, r.end, r.hi, 1);
     if (r.piece == p.pieces - 1) st.write(p, p.S1 ? p.S1 + r.bh * D * M : nullptr, p.Z1 ? p.Z1 + r.bh * D : nullptr);
 }
 
 // ---- sums over a piece: the forward records [k^T V | k^T 1], or the reverse ones [q^^T G | q^^T dl] -----------------
 // Reverse tiles: q^ = phi(Q) / dn and the planes of dl, from the parked dn_i, dl_i.
-template <typename IO, int DP, int MP>
+template <typename IO, int DP, int MP, int THREADS>
 struct ReverseRows {
     RawTile<IO, T, DP, THREADS> rq;
     RawTile<IO, T, MP, THREADS> rg;
@@ -400,28 +561,30 @@ struct ReverseRows {
 };
 
 template <typename C, int DP, int MP, bool EXACT, bool REVERSE>
-__global__ void __launch_bounds__(THREADS, C::NP == 1 ? 4 : 2)
+__global__ void __launch_bounds__(kThreads<C>, C::NP == 1 ? 4 : 2)
 causal_mma_sum_kernel(const Params p) {
     using IO = typename C::IO;
-    constexpr int NX = REVERSE ? C::NR : C::NQ, NY = C::NV;
-    using Sh = Shared<DP, MP, NX, NY, C::NS>;          // (the state planes are not used: the launch asks for less)
+    using Sh = SumLayout<C, DP, MP, REVERSE>;
+    constexpr int NX = REVERSE ? C::NR : C::NQ, NY = C::NV, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* buf = smem;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
+    wait_for_stream();
+    release_next();
     const Range r = range_of(p, (int)blockIdx.y + (REVERSE ? 1 : 0));
     const IO* X = (const IO*)(REVERSE ? p.Q : p.K) + r.bh * p.N * D;
     const IO* Y = (const IO*)(REVERSE ? p.G : p.V) + r.bh * p.N * M;
     const float* dn = REVERSE ? p.aux + r.bh * 2 * p.N : nullptr;
     const float* delta = REVERSE ? dn + p.N : nullptr;
-    State<DP, MP> st;
+    State<DP, MP, 4 * C::WPS> st;
     st.init(p, nullptr, nullptr, nullptr, 0);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
-        float* w = reinterpret_cast<float*>(buf + Sh::S);
-        uint16_t* wpl = reinterpret_cast<uint16_t*>(w + T);
+        float* w = reinterpret_cast<float*>(buf + Sh::W);
+        uint16_t* wpl = reinterpret_cast<uint16_t*>(buf + Sh::WP);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         if constexpr (REVERSE) {
-            ReverseRows<IO, DP, MP> rr;
+            ReverseRows<IO, DP, MP, THREADS> rr;
             rr.load(X, Y, dn, delta, n0, cn, D, M, pad);
             if constexpr (C::BUF == 1) __syncthreads();
             rr.template store<NX, NY>(buf + Sh::X, buf + Sh::Y, w, wpl, phi);
@@ -434,8 +597,8 @@ causal_mma_sum_kernel(const Params p) {
             with_phi<NX>(phi, [&](auto f) { rx.template store<NX>(buf + Sh::X, [&](int, float x) { return f(x); }); });
             ry.template values<NY>(buf + Sh::Y);
         }
-        prefetch_rows(X, n0 + T, r.end, D);
-        prefetch_rows(Y, n0 + T, r.end, M);
+        prefetch_rows<THREADS>(X, n0 + T, r.end, D);
+        prefetch_rows<THREADS>(Y, n0 + T, r.end, M);
         __syncthreads();
         st.template update<NX, NY, !REVERSE>(smem_u32(buf + Sh::X), smem_u32(buf + Sh::Y), wpl);
         flip<C, Sh>(buf, smem);
@@ -446,16 +609,19 @@ causal_mma_sum_kernel(const Params p) {
 
 // ---- dQ sweep --------------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(THREADS, (resident<Shared<DP, MP, C::NQ, C::NV, C::NS>, C>(C::NP == 1 ? 4 : 2)))
+__global__ void __launch_bounds__(kThreads<C>, (resident<DqLayout<C, DP, MP>, C>()))
 causal_mma_dq_kernel(const Params p) {
     using IO = typename C::IO;
-    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS;
-    using Sh = Shared<DP, MP, NQ, NV, NS>;
+    using Sh = DqLayout<C, DP, MP>;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, WPS = C::WPS, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const bool state_part = WPS == 1 || warp < STRIPS_T, score_part = WPS == 1 || warp >= STRIPS_T;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
+    wait_for_stream();
+    release_next();
     const Range r = range_of(p, blockIdx.y);
     const IO* Q = (const IO*)p.Q + r.bh * p.N * D;
     const IO* K = (const IO*)p.K + r.bh * p.N * D;
@@ -465,55 +631,64 @@ causal_mma_dq_kernel(const Params p) {
     float* dn_all = p.aux + r.bh * 2 * p.N;
     float* dl_all = dn_all + p.N;
 
-    State<DP, MP> st;
+    State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + r.bh * (p.pieces - 1) * (int64_t)(D * M + D), r.piece);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(buf + Sh::X), sV = smem_u32(buf + Sh::Y), sS = smem_u32(buf + Sh::S);
         float* sZ = reinterpret_cast<float*>(buf + Sh::Z);
+        float* sgo = reinterpret_cast<float*>(buf + Sh::W);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
-        const int strip = ((n0 / T) & 1) ? WARPS - 1 - warp : warp, row0 = strip * 16;
-        uint32_t ga[MP / 16][NV][4];
+        const int strip = strip_of(warp, (n0 / T) & 1), row0 = strip * 16;
+        StripOperand<WPS, NV, MP> ga;
         {
-            RawStrip<IO, MP> rg;
             RawTile<IO, T, DP, THREADS> rk;
             RawTile<IO, T, MP, THREADS> rv;
-            rg.load(G + n0 * M, row0, cn, M, 0.f);
+            std::conditional_t<WPS == 1, RawStrip<IO, MP>, RawTile<IO, T, MP, THREADS>> rg;
             rk.load(K + n0 * D, cn, D, pad);
             rv.load(V + n0 * M, cn, M, 0.f);
+            if constexpr (WPS == 1) rg.load(G + n0 * M, row0, cn, M, 0.f);
+            else rg.load(G + n0 * M, cn, M, 0.f);
             if constexpr (C::BUF == 1) __syncthreads();
-            st.template publish<NS>(buf + Sh::S, sZ);
+            st.template publish<NS>(buf + Sh::S, sZ, reinterpret_cast<uint16_t*>(buf + Sh::ZP));
             with_phi<NQ>(phi, [&](auto f) { rk.template store<NQ>(buf + Sh::X, [&](int, float x) { return f(x); }); });
             rv.template values<NV>(buf + Sh::Y);
-            rg.template planes<NV>(ga);
+            if constexpr (WPS == 1) {
+                rg.template planes<NV>(ga.a);
+            } else {
+                rg.template values<NV>(buf + Sh::R);
+                ga.tile = smem_u32(buf + Sh::R); ga.row0 = row0; ga.lane = lane;
+            }
         }
-        prefetch_rows(Q, n0 + T, r.end, D);
-        prefetch_rows(K, n0 + T, r.end, D);
-        prefetch_rows(V, n0 + T, r.end, M);
-        prefetch_rows(G, n0 + T, r.end, M);
+        prefetch_rows<THREADS>(Q, n0 + T, r.end, D);
+        prefetch_rows<THREADS>(K, n0 + T, r.end, D);
+        prefetch_rows<THREADS>(V, n0 + T, r.end, M);
+        prefetch_rows<THREADS>(G, n0 + T, r.end, M);
         __syncthreads();
+        const bool real = row0 < cn;
         // The first chunk of a sequence goes through twice, the second time with the G_i . O_i it found taken off the
         // scores: where few terms make up a row, h and (q . h / dn) Zc cancel almost entirely (in row 0 completely).
+        // (The state before that chunk is zero: G S^T has no part in it.)
+        const int first_pass = n0 == 0 && !p.S0 ? 0 : 1;
         float c0 = 0.f, c1 = 0.f;               // G_i . O_i of rows g, g + 8, as far as it is known
-        for (int pass = row0 >= cn ? 2 : (n0 == 0 && !p.S0) ? 0 : 1; pass < 2; ++pass) {
-            float h[DP / 8][4], zc[DP / 8][4];
+        float h[DP / 8][4], zc[DP / 8][4];
+        auto ones_block = [&](uint32_t (&ones)[1][4], int jb) {         // the part of L in key block jb
+            ones[0][0] = ones[0][1] = ones[0][2] = ones[0][3] = 0x3f803f80u;
+            if (jb == strip) {
+                ones[0][0] = ones[0][3] = (2 * t <= g ? 0x3f80u : 0u) | (2 * t + 1 <= g ? 0x3f800000u : 0u);
+                ones[0][2] = 0u;
+            }
+        };
+        auto start_zc = [&]() {
 #pragma unroll
             for (int n = 0; n < DP / 8; ++n) {
                 const float2 z = *reinterpret_cast<const float2*>(sZ + n * 8 + 2 * t);
                 zc[n][0] = zc[n][2] = z.x;
                 zc[n][1] = zc[n][3] = z.y;
             }
-#pragma unroll
-            for (int n = 0; n < DP / 16; ++n) {
-                Chain c;
-#pragma unroll
-                for (int ee = 0; ee < MP / 16; ++ee) {
-                    uint32_t b[NS][4];
-                    load_rows<NS, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
-                    c.step<NV, NS>(ga[ee], b);
-                }
-                c.put(h[2 * n], h[2 * n + 1]);
-            }
+        };
+        auto scores = [&]() {                   // h += ((G V^T - c) o L) k; one warp per strip: zc = L k + Z as well
+            if constexpr (WPS == 1) start_zc();
 #pragma unroll 1
             for (int jb = 0; jb <= strip; ++jb) {
                 float s0[4], s1[4];
@@ -521,9 +696,9 @@ causal_mma_dq_kernel(const Params p) {
                     Chain c;
 #pragma unroll
                     for (int ee = 0; ee < MP / 16; ++ee) {
-                        uint32_t b[NV][4];
+                        uint32_t b[NV][4], f[NV][4];
                         load_rows<NV, MP>(b, sV, T * MP * 2, jb * 16, ee * 2, lane);
-                        c.step<NV, NV>(ga[ee], b);
+                        c.step<NV, NV>(ga.block(ee, f), b);
                     }
                     c.put(s0, s1);
                 }
@@ -532,58 +707,117 @@ causal_mma_dq_kernel(const Params p) {
                     s0[j] -= c0; s1[j] -= c0;
                     s0[2 + j] -= c1; s1[2 + j] -= c1;
                 }
-                uint32_t ones[1][4] = {{0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u}};
-                if (jb == strip) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int row = g + (j >> 1) * 8, col = 2 * t + (j & 1);
-                        if (col > row) s0[j] = 0.f;
-                        if (col + 8 > row) s1[j] = 0.f;
-                    }
-                    ones[0][0] = ones[0][3] = (2 * t <= g ? 0x3f80u : 0u) | (2 * t + 1 <= g ? 0x3f800000u : 0u);
-                    ones[0][2] = 0u;
-                }
-                uint32_t pa[NP][4];
+                if (jb == strip) mask_diagonal<false>(s0, s1, g, t);
+                uint32_t pa[NP][4], ones[1][4];
                 operand_of<NP>(pa, s0, s1);
+                if constexpr (WPS == 1) ones_block(ones, jb);
 #pragma unroll
                 for (int n = 0; n < DP / 16; ++n) {
                     uint32_t b[NQ][4];
                     load_cols_t<NQ, DP>(b, sK, T * DP * 2, jb * 16, n * 2, lane);
                     block_mma<NP, NQ>(h[2 * n], h[2 * n + 1], pa, b);
-                    block_mma<1, NQ>(zc[2 * n], zc[2 * n + 1], ones, b);
+                    if constexpr (WPS == 1) block_mma<1, NQ>(zc[2 * n], zc[2 * n + 1], ones, b);
                 }
             }
-            RawStrip<IO, DP> rq;                // element j of block kk: result column tile 2 kk + j / 2, row g + 8 (j & 1)
-            rq.load(Q + n0 * D, row0, cn, D, pad);
-            RawStrip<typename FeatureType<NQ>::type, DP> fq;
-            rq.template map<NQ>(phi, fq);
-            float qz[2] = {0.f, 0.f}, qh[2] = {0.f, 0.f};
-#pragma unroll
-            for (int kk = 0; kk < DP / 16; ++kk)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int n = 2 * kk + (j >> 1), b = j & 1;
-                    qz[b] = fmaf(fq.r[kk][j].lo(), zc[n][2 * b], fmaf(fq.r[kk][j].hi(), zc[n][2 * b + 1], qz[b]));
-                    qh[b] = fmaf(fq.r[kk][j].lo(), h[n][2 * b], fmaf(fq.r[kk][j].hi(), h[n][2 * b + 1], qh[b]));
+        };
+        if (WPS == 2 && score_part) {
+            for (int pass = first_pass; pass < 2; ++pass) {
+                if (real) {
+                    clear(h);
+                    scores();
                 }
+                if (pass == first_pass) bar_sync(1, THREADS);
+                if (real) {
+                    put_part(buf + Sh::S, strip, h);
+                    bar_arrive(2 + strip, 64);
+                    if (pass == 0) {
+                        bar_sync(6 + strip, 64);
+                        c0 = sgo[row0 + g];
+                        c1 = sgo[row0 + g + 8];
+                    }
+                }
+            }
+        }
+        if (state_part) {
+            if (real) {
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const int row = row0 + g + 8 * b;
-                const float dn = quad_sum(qz[b]) + p.eps;
-                const float inv = 1.f / dn, go = (quad_sum(qh[b]) - (b ? c1 : c0) * p.eps) * inv;    // what is left of G_i . O_i
-                (b ? c1 : c0) += go;
-                if (pass == 1 && row < cn) {
+                for (int n = 0; n < DP / 16; ++n) {
+                    Chain c;
 #pragma unroll
-                    for (int n = 0; n < DP / 8; ++n)
-                        if (n * 8 < D) {
-                            const auto q = fq.r[n >> 1][(n & 1) * 2 + b];
-                            store_pair<IO>(dQ + (n0 + row) * D + n * 8 + 2 * t,
-                                           fmaf(-go, zc[n][2 * b], h[n][2 * b]) * inv * phi_slope_from_value(q.lo(), phi),
-                                           fmaf(-go, zc[n][2 * b + 1], h[n][2 * b + 1]) * inv * phi_slope_from_value(q.hi(), phi));
+                    for (int ee = 0; ee < MP / 16; ++ee) {
+                        uint32_t b[NS][4], f[NV][4];
+                        load_rows<NS, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
+                        c.step<NV, NS>(ga.block(ee, f), b);
+                    }
+                    c.put(h[2 * n], h[2 * n + 1]);
+                }
+            }
+            if constexpr (WPS == 2) bar_arrive(1, THREADS);
+            if (real) {
+                if constexpr (WPS == 2) {
+                    start_zc();
+#pragma unroll 1
+                    for (int jb = 0; jb <= strip; ++jb) {
+                        uint32_t ones[1][4];
+                        ones_block(ones, jb);
+#pragma unroll
+                        for (int n = 0; n < DP / 16; ++n) {
+                            uint32_t b[NQ][4];
+                            load_cols_t<NQ, DP>(b, sK, T * DP * 2, jb * 16, n * 2, lane);
+                            block_mma<1, NQ>(zc[2 * n], zc[2 * n + 1], ones, b);
                         }
-                    if (t == 0) {
-                        dn_all[n0 + row] = dn;
-                        dl_all[n0 + row] = b ? -c1 : -c0;
+                    }
+                }
+                for (int pass = first_pass; pass < 2; ++pass) {
+                    if (pass == 1 && first_pass == 0) clear(h);
+                    RawStrip<IO, DP> rq;        // element j of block kk: result column tile 2 kk + j / 2, row g + 8 (j & 1)
+                    if constexpr (WPS == 2) {
+                        rq.load(Q + n0 * D, row0, cn, D, pad);
+                        bar_sync(2 + strip, 64);
+                        add_part(buf + Sh::S, strip, h);
+                    } else {
+                        scores();
+                        rq.load(Q + n0 * D, row0, cn, D, pad);
+                    }
+                    RawStrip<typename FeatureType<NQ>::type, DP> fq;
+                    rq.template map<NQ>(phi, fq);
+                    float qz[2] = {0.f, 0.f}, qh[2] = {0.f, 0.f};
+#pragma unroll
+                    for (int kk = 0; kk < DP / 16; ++kk)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int n = 2 * kk + (j >> 1), b = j & 1;
+                            qz[b] = fmaf(fq.r[kk][j].lo(), zc[n][2 * b], fmaf(fq.r[kk][j].hi(), zc[n][2 * b + 1], qz[b]));
+                            qh[b] = fmaf(fq.r[kk][j].lo(), h[n][2 * b], fmaf(fq.r[kk][j].hi(), h[n][2 * b + 1], qh[b]));
+                        }
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        const int row = row0 + g + 8 * b;
+                        const float dn = quad_sum(qz[b]) + p.eps;
+                        const float inv = 1.f / dn;
+                        const float go = (quad_sum(qh[b]) - (b ? c1 : c0) * p.eps) * inv;    // what is left of G_i . O_i
+                        (b ? c1 : c0) += go;
+                        if (pass == 1 && row < cn) {
+#pragma unroll
+                            for (int n = 0; n < DP / 8; ++n)
+                                if (n * 8 < D) {
+                                    const auto q = fq.r[n >> 1][(n & 1) * 2 + b];
+                                    store_pair<IO>(dQ + (n0 + row) * D + n * 8 + 2 * t,
+                                                   fmaf(-go, zc[n][2 * b], h[n][2 * b]) * inv * phi_slope_from_value(q.lo(), phi),
+                                                   fmaf(-go, zc[n][2 * b + 1], h[n][2 * b + 1]) * inv * phi_slope_from_value(q.hi(), phi));
+                                }
+                            if (t == 0) {
+                                dn_all[n0 + row] = dn;
+                                dl_all[n0 + row] = b ? -c1 : -c0;
+                            }
+                        }
+                    }
+                    if (WPS == 2 && pass == 0) {
+                        if (t == 0) {
+                            sgo[row0 + g] = c0;
+                            sgo[row0 + g + 8] = c1;
+                        }
+                        bar_arrive(6 + strip, 64);
                     }
                 }
             }
@@ -591,21 +825,24 @@ causal_mma_dq_kernel(const Params p) {
         st.template update<NQ, NV, true>(sK, sV, nullptr);
         flip<C, Sh>(buf, smem);
     }
-    zero_rows(dQ, r.end, r.hi, D);
+    zero_rows<THREADS>(dQ, r.end, r.hi, D);
 }
 
 // ---- dK, dV sweep ----------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(THREADS, (resident<Shared<DP, MP, C::NR, C::NV, C::NS>, C>(C::NP == 1 ? 4 : 3)))
+__global__ void __launch_bounds__(kThreads<C>, (resident<DkvLayout<C, DP, MP>, C>(C::WPS == 1 ? 3 : 2)))
 causal_mma_dkv_kernel(const Params p) {
     using IO = typename C::IO;
-    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, NR = C::NR;
-    using Sh = Shared<DP, MP, NR, NV, NS>;
+    using Sh = DkvLayout<C, DP, MP>;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, NR = C::NR, WPS = C::WPS, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const bool v_part = WPS == 1 || warp < STRIPS_T, k_part = WPS == 1 || warp >= STRIPS_T;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
+    wait_for_stream();
+    release_next();
     const Range r = range_of(p, (int)(gridDim.y - 1 - blockIdx.y));
     const IO* Q = (const IO*)p.Q + r.bh * p.N * D;
     const IO* K = (const IO*)p.K + r.bh * p.N * D;
@@ -616,7 +853,7 @@ causal_mma_dkv_kernel(const Params p) {
     const float* dn = p.aux + r.bh * 2 * p.N;
     const float* delta = dn + p.N;
 
-    State<DP, MP> st;           // record i is the sum of piece i + 1
+    State<DP, MP, 4 * WPS> st;           // record i is the sum of piece i + 1
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + (r.bh * (p.pieces - 1) + r.piece) * (int64_t)(D * M + D), p.pieces - 1 - r.piece);
     const int64_t chunks = (r.end - r.lo + T - 1) / T;
@@ -627,164 +864,148 @@ causal_mma_dkv_kernel(const Params p) {
         uint16_t* wpl = reinterpret_cast<uint16_t*>(buf + Sh::WP);
         const int64_t n0 = r.lo + c * T;
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T), blocks = (cn + 15) / 16;
-        const int strip = (c & 1) ? WARPS - 1 - warp : warp, row0 = strip * 16;
+        const int strip = strip_of(warp, c & 1), row0 = strip * 16;
         {
-            ReverseRows<IO, DP, MP> rr;
+            ReverseRows<IO, DP, MP, THREADS> rr;
             rr.load(Q, G, dn, delta, n0, cn, D, M, pad);
             if constexpr (C::BUF == 1) __syncthreads();
-            st.template publish<NS>(buf + Sh::S, sr);
+            st.template publish<NS>(buf + Sh::S, sr, reinterpret_cast<uint16_t*>(buf + Sh::ZP));
             rr.template store<NR, NV>(buf + Sh::X, buf + Sh::Y, sdl, wpl, phi);
         }
         if (c > 0) {
-            prefetch_rows(Q, n0 - T, r.end, D);
-            prefetch_rows(K, n0 - T, r.end, D);
-            prefetch_rows(V, n0 - T, r.end, M);
-            prefetch_rows(G, n0 - T, r.end, M);
+            prefetch_rows<THREADS>(Q, n0 - T, r.end, D);
+            prefetch_rows<THREADS>(K, n0 - T, r.end, D);
+            prefetch_rows<THREADS>(V, n0 - T, r.end, M);
+            prefetch_rows<THREADS>(G, n0 - T, r.end, M);
         }
         __syncthreads();
-        if (row0 < cn) {
+        if (v_part && row0 < cn) {
+            uint32_t ka[DP / 16][NQ][4];
             {
-                uint32_t ka[DP / 16][NQ][4];
-                {
-                    RawStrip<IO, DP> rk;
-                    rk.load(K + n0 * D, row0, cn, D, pad);
-                    RawStrip<typename FeatureType<NQ>::type, DP> fk;
-                    rk.template map<NQ>(phi, fk);
-                    fk.template planes<NQ>(ka);
-                }
-                float gv[MP / 8][4];
-#pragma unroll
-                for (int n = 0; n < MP / 16; ++n) {
-                    Chain c;
-#pragma unroll
-                    for (int kk = 0; kk < DP / 16; ++kk) {
-                        uint32_t b[NS][4];
-                        load_cols_t<NS, MP>(b, sR, DP * MP * 2, kk * 16, n * 2, lane);
-                        c.step<NQ, NS>(ka[kk], b);
-                    }
-                    c.put(gv[2 * n], gv[2 * n + 1]);
-                }
-#pragma unroll 1
-                for (int ib = strip; ib < blocks; ++ib) {
-                    float s0[4], s1[4];
-                    {
-                        Chain c;
-#pragma unroll
-                        for (int kk = 0; kk < DP / 16; ++kk) {
-                            uint32_t b[NR][4];
-                            load_rows<NR, DP>(b, sQ, T * DP * 2, ib * 16, kk * 2, lane);
-                            c.step<NQ, NR>(ka[kk], b);
-                        }
-                        c.put(s0, s1);
-                    }
-                    if (ib == strip) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int row = g + (j >> 1) * 8, col = 2 * t + (j & 1);
-                            if (col < row) s0[j] = 0.f;
-                            if (col + 8 < row) s1[j] = 0.f;
-                        }
-                    }
-                    uint32_t pa[NP][4];
-                    operand_of<NP>(pa, s0, s1);
-#pragma unroll
-                    for (int n = 0; n < MP / 16; ++n) {
-                        uint32_t b[NV][4];
-                        load_cols_t<NV, MP>(b, sG, T * MP * 2, ib * 16, n * 2, lane);
-                        block_mma<NP, NV>(gv[2 * n], gv[2 * n + 1], pa, b);
-                    }
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int row = row0 + g + 8 * h;
-                    if (row < cn) {
-#pragma unroll
-                        for (int n = 0; n < MP / 8; ++n)
-                            if (n * 8 < M) store_pair<IO>(dV + (n0 + row) * M + n * 8 + 2 * t, gv[n][2 * h], gv[n][2 * h + 1]);
-                    }
-                }
-            }
-            {
-                uint32_t va[MP / 16][NV][4];
-                {
-                    RawStrip<IO, MP> rv;
-                    rv.load(V + n0 * M, row0, cn, M, 0.f);
-                    rv.template planes<NV>(va);
-                }
-                float gk[DP / 8][4];
-#pragma unroll
-                for (int n = 0; n < DP / 8; ++n) {
-                    const float2 z = *reinterpret_cast<const float2*>(sr + n * 8 + 2 * t);
-                    gk[n][0] = gk[n][2] = z.x;
-                    gk[n][1] = gk[n][3] = z.y;
-                }
-#pragma unroll
-                for (int n = 0; n < DP / 16; ++n) {
-                    Chain c;
-#pragma unroll
-                    for (int ee = 0; ee < MP / 16; ++ee) {
-                        uint32_t b[NS][4];
-                        load_rows<NS, MP>(b, sR, DP * MP * 2, n * 16, ee * 2, lane);
-                        c.step<NV, NS>(va[ee], b);
-                    }
-                    c.add_to(gk[2 * n], gk[2 * n + 1]);
-                }
-#pragma unroll 1
-                for (int ib = strip; ib < blocks; ++ib) {
-                    const float2 w0 = *reinterpret_cast<const float2*>(sdl + ib * 16 + 2 * t);
-                    const float2 w1 = *reinterpret_cast<const float2*>(sdl + ib * 16 + 8 + 2 * t);
-                    float s0[4] = {w0.x, w0.y, w0.x, w0.y}, s1[4] = {w1.x, w1.y, w1.x, w1.y};
-                    {
-                        Chain c;
-#pragma unroll
-                        for (int ee = 0; ee < MP / 16; ++ee) {
-                            uint32_t b[NV][4];
-                            load_rows<NV, MP>(b, sG, T * MP * 2, ib * 16, ee * 2, lane);
-                            c.step<NV, NV>(va[ee], b);
-                        }
-                        c.add_to(s0, s1);
-                    }
-                    if (ib == strip) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int row = g + (j >> 1) * 8, col = 2 * t + (j & 1);
-                            if (col < row) s0[j] = 0.f;
-                            if (col + 8 < row) s1[j] = 0.f;
-                        }
-                    }
-                    uint32_t pa[NP][4];
-                    operand_of<NP>(pa, s0, s1);
-#pragma unroll
-                    for (int n = 0; n < DP / 16; ++n) {
-                        uint32_t b[NR][4];
-                        load_cols_t<NR, DP>(b, sQ, T * DP * 2, ib * 16, n * 2, lane);
-                        block_mma<NP, NR>(gk[2 * n], gk[2 * n + 1], pa, b);
-                    }
-                }
                 RawStrip<IO, DP> rk;
                 rk.load(K + n0 * D, row0, cn, D, pad);
                 RawStrip<typename FeatureType<NQ>::type, DP> fk;
                 rk.template map<NQ>(phi, fk);
+                fk.template planes<NQ>(ka);
+            }
+            float gv[MP / 8][4];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int row = row0 + g + 8 * h;
-                    if (row < cn) {
+            for (int n = 0; n < MP / 16; ++n) {
+                Chain c;
 #pragma unroll
-                        for (int n = 0; n < DP / 8; ++n)
-                            if (n * 8 < D) {
-                                const auto k = fk.r[n >> 1][(n & 1) * 2 + h];
-                                store_pair<IO>(dK + (n0 + row) * D + n * 8 + 2 * t, gk[n][2 * h] * phi_slope_from_value(k.lo(), phi),
-                                               gk[n][2 * h + 1] * phi_slope_from_value(k.hi(), phi));
-                            }
+                for (int kk = 0; kk < DP / 16; ++kk) {
+                    uint32_t b[NS][4];
+                    load_cols_t<NS, MP>(b, sR, DP * MP * 2, kk * 16, n * 2, lane);
+                    c.step<NQ, NS>(ka[kk], b);
+                }
+                c.put(gv[2 * n], gv[2 * n + 1]);
+            }
+#pragma unroll 1
+            for (int ib = strip; ib < blocks; ++ib) {
+                float s0[4], s1[4];
+                {
+                    Chain c;
+#pragma unroll
+                    for (int kk = 0; kk < DP / 16; ++kk) {
+                        uint32_t b[NR][4];
+                        load_rows<NR, DP>(b, sQ, T * DP * 2, ib * 16, kk * 2, lane);
+                        c.step<NQ, NR>(ka[kk], b);
                     }
+                    c.put(s0, s1);
+                }
+                if (ib == strip) mask_diagonal<true>(s0, s1, g, t);
+                uint32_t pa[NP][4];
+                operand_of<NP>(pa, s0, s1);
+#pragma unroll
+                for (int n = 0; n < MP / 16; ++n) {
+                    uint32_t b[NV][4];
+                    load_cols_t<NV, MP>(b, sG, T * MP * 2, ib * 16, n * 2, lane);
+                    block_mma<NP, NV>(gv[2 * n], gv[2 * n + 1], pa, b);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int row = row0 + g + 8 * h;
+                if (row < cn) {
+#pragma unroll
+                    for (int n = 0; n < MP / 8; ++n)
+                        if (n * 8 < M) store_pair<IO>(dV + (n0 + row) * M + n * 8 + 2 * t, gv[n][2 * h], gv[n][2 * h + 1]);
+                }
+            }
+        }
+        if (k_part && row0 < cn) {
+            uint32_t va[MP / 16][NV][4];
+            {
+                RawStrip<IO, MP> rv;
+                rv.load(V + n0 * M, row0, cn, M, 0.f);
+                rv.template planes<NV>(va);
+            }
+            float gk[DP / 8][4];
+#pragma unroll
+            for (int n = 0; n < DP / 8; ++n) {
+                const float2 z = *reinterpret_cast<const float2*>(sr + n * 8 + 2 * t);
+                gk[n][0] = gk[n][2] = z.x;
+                gk[n][1] = gk[n][3] = z.y;
+            }
+#pragma unroll
+            for (int n = 0; n < DP / 16; ++n) {
+                Chain c;
+#pragma unroll
+                for (int ee = 0; ee < MP / 16; ++ee) {
+                    uint32_t b[NS][4];
+                    load_rows<NS, MP>(b, sR, DP * MP * 2, n * 16, ee * 2, lane);
+                    c.step<NV, NS>(va[ee], b);
+                }
+                c.add_to(gk[2 * n], gk[2 * n + 1]);
+            }
+#pragma unroll 1
+            for (int ib = strip; ib < blocks; ++ib) {
+                const float2 w0 = *reinterpret_cast<const float2*>(sdl + ib * 16 + 2 * t);
+                const float2 w1 = *reinterpret_cast<const float2*>(sdl + ib * 16 + 8 + 2 * t);
+                float s0[4] = {w0.x, w0.y, w0.x, w0.y}, s1[4] = {w1.x, w1.y, w1.x, w1.y};
+                {
+                    Chain c;
+#pragma unroll
+                    for (int ee = 0; ee < MP / 16; ++ee) {
+                        uint32_t b[NV][4];
+                        load_rows<NV, MP>(b, sG, T * MP * 2, ib * 16, ee * 2, lane);
+                        c.step<NV, NV>(va[ee], b);
+                    }
+                    c.add_to(s0, s1);
+                }
+                if (ib == strip) mask_diagonal<true>(s0, s1, g, t);
+                uint32_t pa[NP][4];
+                operand_of<NP>(pa, s0, s1);
+#pragma unroll
+                for (int n = 0; n < DP / 16; ++n) {
+                    uint32_t b[NR][4];
+                    load_cols_t<NR, DP>(b, sQ, T * DP * 2, ib * 16, n * 2, lane);
+                    block_mma<NP, NR>(gk[2 * n], gk[2 * n + 1], pa, b);
+                }
+            }
+            RawStrip<IO, DP> rk;
+            rk.load(K + n0 * D, row0, cn, D, pad);
+            RawStrip<typename FeatureType<NQ>::type, DP> fk;
+            rk.template map<NQ>(phi, fk);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int row = row0 + g + 8 * h;
+                if (row < cn) {
+#pragma unroll
+                    for (int n = 0; n < DP / 8; ++n)
+                        if (n * 8 < D) {
+                            const auto k = fk.r[n >> 1][(n & 1) * 2 + h];
+                            store_pair<IO>(dK + (n0 + row) * D + n * 8 + 2 * t, gk[n][2 * h] * phi_slope_from_value(k.lo(), phi),
+                                           gk[n][2 * h + 1] * phi_slope_from_value(k.hi(), phi));
+                        }
                 }
             }
         }
         st.template update<NR, NV, false>(sQ, sG, wpl);
         flip<C, Sh>(buf, smem);
     }
-    zero_rows(dK, r.end, r.hi, D);
-    zero_rows(dV, r.end, r.hi, M);
+    zero_rows<THREADS>(dK, r.end, r.hi, D);
+    zero_rows<THREADS>(dV, r.end, r.hi, M);
     if (r.piece == 0) st.write(p, p.S1 ? p.S1 + r.bh * D * M : nullptr, p.Z1 ? p.Z1 + r.bh * D : nullptr);
 }
 
@@ -792,7 +1013,7 @@ causal_mma_dkv_kernel(const Params p) {
 struct Plan { int pieces; int64_t len; };
 
 // Pieces per sequence, by the estimated time in units of one chunk of a main kernel (about 10 us alone on an SM).
-// An SM runs two CTAs in 1.25 times the time of one; a CTA's start costs about a chunk, and 0.35 for each record it
+// An SM runs two CTAs in 1.25 times the time of one; a CTA's start costs about a chunk, and 0.2 for each record it
 // sums, of which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk.  Forward +
 // backward in us, fp32, D = M = 64, pieces 1 / 2 / 4 / 8 / 16: B1 H8 N1024 466 / 304 / 172 / 123 / 134;
 // B8 H8 N1024 484 / 324 / 245 / 287 / 381; B16 H8 N2048 963 / 815 / 929 / 913 / 1091;
@@ -813,7 +1034,7 @@ Plan choose_plan(const la_problem& p, bool single) {
         };
         auto cost = [&](int64_t n) {
             const double per = (double)((chunks + n - 1) / n);
-            return (per + 1.0 + 0.175 * (n - 1)) * waves(bh * n) + (n > 1 ? 0.35 * (per + 1.0) * waves(bh * (n - 1)) : 0.0);
+            return (per + 1.0 + 0.1 * (n - 1)) * waves(bh * n) + (n > 1 ? 0.35 * (per + 1.0) * waves(bh * (n - 1)) : 0.0);
         };
         for (int64_t n = 2; n <= 16 && n <= chunks; ++n)
             if (cost(n) < cost(best)) best = n;
@@ -831,51 +1052,71 @@ Params make_params(const la_problem& p, const Plan& pl, const int* lengths) {
     Params a = {};
     a.lengths = lengths;
     a.N = p.N; a.piece_len = pl.len; a.pieces = pl.pieces;
+    // Small grids only, whose CTAs find SMs of their own beside those of the kernel before (fp32 B1 H2 N256 D32: 39 -> 25
+    // us a step); otherwise CTAs that wait on the SMs with room leave the kernel unevenly spread (B32 H8 N4096 D64
+    // backward 2007 -> 2862 us, released at the kernel's end B37 H8 N512 267 -> 328 us).
+    a.chained = 2 * p.B * p.H * pl.pieces <= 148;
     a.heads = (int)p.H; a.D = (int)p.D; a.M = (int)p.M; a.phi = p.phi; a.eps = p.eps;
     return a;
 }
 
-int launch(void (*kern)(const Params), unsigned bh, unsigned y, int smem, const Params& a, cudaStream_t st) {
-    if (smem > 48 * 1024) LA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kern<<<dim3(bh, y), THREADS, smem, st>>>(a);
-    LA_LAUNCHED();
+template <auto KERNEL>
+int launch(int threads, unsigned bh, unsigned y, int smem, const Params& a, cudaStream_t st) {
+    static std::atomic<uint64_t> opted_in{0};           // devices on which the kernel may use that much shared memory
+    if (smem > 48 * 1024)
+        if (int rc = tc::opt_in_smem_once(KERNEL, (uint32_t)smem, opted_in)) return rc;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(bh, y);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = a.chained ? 1 : 0;
+    LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, KERNEL, a));
+    note_launch();
     return LA_OK;
 }
 
 template <typename C, int DP, int MP, bool EXACT> struct Kernels {
-    using Fwd = Shared<DP, MP, C::NQ, C::NV, C::NS>;
-    using Rev = Shared<DP, MP, C::NR, C::NV, C::NS>;
+    static constexpr int THREADS = kThreads<C>, BUF = C::BUF;
     static int sums(const la_problem& p, const Params& a, bool reverse, cudaStream_t st) {
         if (a.pieces == 1) return LA_OK;
         const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)(a.pieces - 1);
-        constexpr int vec = T * 4 + 3 * T * 2;
-        if (reverse) return launch(causal_mma_sum_kernel<C, DP, MP, EXACT, true>, bh, y, C::BUF == 2 ? 2 * Rev::BYTES : Rev::S + vec, a, st);
-        return launch(causal_mma_sum_kernel<C, DP, MP, EXACT, false>, bh, y, C::BUF == 2 ? 2 * Fwd::BYTES : Fwd::S + vec, a, st);
+        if (reverse)
+            return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, true>>(THREADS, bh, y, BUF * SumLayout<C, DP, MP, true>::BYTES, a, st);
+        return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, false>>(THREADS, bh, y, BUF * SumLayout<C, DP, MP, false>::BYTES, a, st);
     }
     static int forward(const la_problem& p, const Params& a, cudaStream_t st) {
         if (int rc = sums(p, a, false, st)) return rc;
-        return launch(causal_mma_forward_kernel<C, DP, MP, EXACT>, (unsigned)(p.B * p.H), (unsigned)a.pieces, C::BUF * Fwd::BYTES, a, st);
+        return launch<causal_mma_forward_kernel<C, DP, MP, EXACT>>(THREADS, (unsigned)(p.B * p.H), (unsigned)a.pieces,
+                      BUF * ForwardLayout<C, DP, MP>::BYTES, a, st);
     }
     static int backward(const la_problem& p, const Params& fwd, const Params& rev, cudaStream_t st) {
+        const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)fwd.pieces;
         if (int rc = sums(p, fwd, false, st)) return rc;
-        if (int rc = launch(causal_mma_dq_kernel<C, DP, MP, EXACT>, (unsigned)(p.B * p.H), (unsigned)fwd.pieces, C::BUF * Fwd::BYTES, fwd, st))
-            return rc;
+        if (int rc = launch<causal_mma_dq_kernel<C, DP, MP, EXACT>>(THREADS, bh, y, BUF * DqLayout<C, DP, MP>::BYTES, fwd, st)) return rc;
         if (int rc = sums(p, rev, true, st)) return rc;
-        return launch(causal_mma_dkv_kernel<C, DP, MP, EXACT>, (unsigned)(p.B * p.H), (unsigned)rev.pieces, C::BUF * Rev::BYTES, rev, st);
+        return launch<causal_mma_dkv_kernel<C, DP, MP, EXACT>>(THREADS, bh, y, BUF * DkvLayout<C, DP, MP>::BYTES, rev, st);
     }
 };
 
 // Tiles are padded to 32, 64 or (D) 128 columns; EXACT: D and M are those sizes.
-template <typename F> int dispatch(const la_problem& p, F f) {
+template <typename F> int dispatch(const la_problem& p, int pieces, F f) {
+    const bool full = p.B * p.H * pieces >= 222;            // one and a half CTAs per SM and more
     const bool exact = (p.D == 32 || p.D == 64 || p.D == 128) && p.M == (p.D == 32 ? 32 : 64);
     if (p.dtype == LA_F32) {
         if (p.D <= 32 && p.M <= 32) return exact ? f(Kernels<Fp32, 32, 32, true>()) : f(Kernels<Fp32, 32, 32, false>());
+        if (exact && p.D == 64 && full) return f(Kernels<Fp32One, 64, 64, true>());
         if (p.D <= 64) return exact ? f(Kernels<Fp32, 64, 64, true>()) : f(Kernels<Fp32, 64, 64, false>());
         return f(Kernels<Fp32, 128, 64, false>());
     }
     if (p.D == 32 && p.M == 32) return f(Kernels<Bf16, 32, 32, true>());
     if (p.phi == LA_PHI_IDENTITY) {
         if (p.D <= 64) return f(Kernels<Bf16Features, 64, 64, false>());
+        if (exact && full) return f(Kernels<Bf16FeaturesOne, 128, 64, true>());
         return exact ? f(Kernels<Bf16Features, 128, 64, true>()) : f(Kernels<Bf16Features, 128, 64, false>());
     }
     return p.D <= 64 ? f(Kernels<Bf16Wide, 64, 64, false>()) : f(Kernels<Bf16Wide, 128, 64, false>());
@@ -909,7 +1150,7 @@ int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const 
     a.Q = Q; a.K = K; a.V = V; a.O = O; a.den = den;
     a.S0 = S_in; a.Z0 = Z_in; a.S1 = S_out; a.Z1 = Z_out;
     a.rec = (float*)ws;
-    return dispatch(p, [&](auto k) { return decltype(k)::forward(p, a, st); });
+    return dispatch(p, pl.pieces, [&](auto k) { return decltype(k)::forward(p, a, st); });
 }
 
 int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
@@ -922,7 +1163,7 @@ int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const
     Params r = f;
     f.S0 = sa.S_in; f.Z0 = sa.Z_in;
     r.S0 = sa.dS_out; r.Z0 = sa.dZ_out; r.S1 = sa.dS_in; r.Z1 = sa.dZ_in;
-    return dispatch(p, [&](auto k) { return decltype(k)::backward(p, f, r, st); });
+    return dispatch(p, pl.pieces, [&](auto k) { return decltype(k)::backward(p, f, r, st); });
 }
 
 }  // namespace la

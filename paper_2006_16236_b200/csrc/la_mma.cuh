@@ -117,7 +117,7 @@ template <int C> __device__ __forceinline__ uint32_t tile_at(int row, int group)
 
 // Lane address patterns of a 16 x 16 block (row, group of eight columns) inside a tile:
 //   Rows: the tile's rows are the rows/columns of the operand (B[n][k] as it lies; A^T[k][m] with .trans)
-//   Cols: the tile's rows are the k index (B[k][n] with .trans)
+//   Cols: the tile's rows are the k index (B[k][n] with .trans) or the rows of A (as it lies)
 __device__ __forceinline__ int rows_row(int lane) { return (lane & 7) + ((lane >> 4) << 3); }
 __device__ __forceinline__ int rows_grp(int lane) { return (lane >> 3) & 1; }
 __device__ __forceinline__ int cols_row(int lane) { return lane & 15; }
@@ -135,6 +135,12 @@ __device__ __forceinline__ void load_rows_t(uint32_t (&f)[NP][4], uint32_t tile,
     const uint32_t a = tile + tile_at<C>(r0 + rows_row(lane), g0 + rows_grp(lane));
 #pragma unroll
     for (int p = 0; p < NP; ++p) ldsm4t(f[p], a + p * pitch);
+}
+template <int NP, int C>
+__device__ __forceinline__ void load_cols(uint32_t (&f)[NP][4], uint32_t tile, uint32_t pitch, int r0, int g0, int lane) {
+    const uint32_t a = tile + tile_at<C>(r0 + cols_row(lane), g0 + cols_grp(lane));
+#pragma unroll
+    for (int p = 0; p < NP; ++p) ldsm4(f[p], a + p * pitch);
 }
 template <int NP, int C>
 __device__ __forceinline__ void load_cols_t(uint32_t (&f)[NP][4], uint32_t tile, uint32_t pitch, int r0, int g0, int lane) {
@@ -319,6 +325,11 @@ __device__ __forceinline__ float quad_sum(float v) {       // over the four lane
     v += __shfl_xor_sync(0xffffffffu, v, 2);
     return v;
 }
+
+// Kernels that follow each other on a stream start early (programmatic dependent launch): nothing of the kernels before
+// is read or written ahead of the wait; the next kernel may be scheduled once every CTA of this one has released it.
+__device__ __forceinline__ void wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
