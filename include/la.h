@@ -24,10 +24,9 @@
  *  - Supported sizes: D and M multiples of 8 in [8, 128]; B, H >= 1; N >= 0
  *    (N == 0 is a successful no-op).  bf16 problems with D = M in {32, 64} run
  *    on the tensor-core kernels (any N: a last chunk of fewer than 128
- *    positions is handled as padding); the causal form of every other problem
- *    with M <= 64 runs on tensor-core kernels that keep fp32 accuracy (products
- *    of numbers split into bf16 parts), everything else on the general
- *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.
+ *    positions is handled as padding); every other problem with M <= 64 runs
+ *    on tensor-core kernels that keep fp32 accuracy (products of numbers split
+ *    into bf16 parts), everything else on the general fp32-arithmetic kernels; results agree within the rounding of the I/O type.
  *    The fp32-accurate causal forward takes ws as an option: with less than
  *    la_workspace_bytes() (or NULL) it does not cut sequences into pieces.
  *  - Return value: LA_OK (0) or a negative la_status.  All argument checks run
@@ -310,7 +309,8 @@ int la_decode_layer_step(const la_problem* p, const void* x, const void* Wqkv, c
  * those LA_NOALLOC_SCRATCH_BYTES until the process exits, used or not.
  *
  *  - The call itself allocates and frees nothing, on the host or the device, and calls no
- *    allocating library routine.  It always runs the general fp32-arithmetic kernels.
+ *    allocating library routine.  It runs the kernels that keep fp32 accuracy, and the
+ *    general fp32-arithmetic kernels for M > 64 or where the sums would not fit the array.
  *    One caveat about the FIRST call on a device: the CUDA runtime loads a library's
  *    device code lazily, and the address look-up of that first call is where the driver
  *    may load this module and place the array in device memory.  That placement is the

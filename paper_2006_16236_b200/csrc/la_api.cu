@@ -256,13 +256,13 @@ size_t la_workspace_bytes(const la_problem* p, int32_t op) {
     if (p->N == 0) return 0;
     if (op == LA_OP_LINEAR_SAVED) op = LA_OP_LINEAR_FORWARD;          // the saved buffer holds what the forward's workspace holds
     if (op == LA_OP_CAUSAL_SAVED) return tc_supported(*p, LA_OP_CAUSAL_BACKWARD) ? tc::causal_saved_bytes(*p) : 0;
-    if (op == LA_OP_LINEAR_VARLEN_FORWARD || op == LA_OP_LINEAR_VARLEN_BACKWARD) {
-        const int full = op == LA_OP_LINEAR_VARLEN_FORWARD ? LA_OP_LINEAR_FORWARD : LA_OP_LINEAR_BACKWARD;
-        return tc_supported(*p, full) ? tc_workspace_bytes(*p, full) : general_workspace_bytes(*p, op);
-    }
+    if (op == LA_OP_LINEAR_VARLEN_FORWARD) op = LA_OP_LINEAR_FORWARD;
+    if (op == LA_OP_LINEAR_VARLEN_BACKWARD) op = LA_OP_LINEAR_BACKWARD;
     if (tc_supported(*p, op)) return tc_workspace_bytes(*p, op);
     if ((op == LA_OP_CAUSAL_FORWARD || op == LA_OP_CAUSAL_BACKWARD) && causal_mma_supported(*p))
         return causal_mma_workspace(*p, op == LA_OP_CAUSAL_BACKWARD);
+    if ((op == LA_OP_LINEAR_FORWARD || op == LA_OP_LINEAR_BACKWARD) && linear_mma_supported(*p))
+        return linear_mma_workspace(*p, op == LA_OP_LINEAR_BACKWARD);
     return general_workspace_bytes(*p, op);
 }
 
@@ -380,6 +380,8 @@ static int linear_forward_common(const la_problem* p, const void* Q, const void*
     cudaStream_t st = (cudaStream_t)stream;
     if (tc_supported(*p, LA_OP_LINEAR_FORWARD))
         return debug_finish(tc::linear_forward(*p, Q, K, V, lengths, O, den, KV, Zs, saved, ws, st), stream);
+    if (linear_mma_supported(*p))
+        return debug_finish(linear_mma_forward(*p, Q, K, V, lengths, O, den, KV, Zs, saved, ws, st), stream);
     return debug_finish(general_linear_forward(*p, Q, K, V, lengths, O, den, KV, Zs, saved, ws, st), stream);
 }
 
@@ -403,6 +405,8 @@ static int linear_backward_common(const la_problem* p, const void* Q, const void
     cudaStream_t st = (cudaStream_t)stream;
     if (tc_supported(*p, LA_OP_LINEAR_BACKWARD))
         return debug_finish(tc::linear_backward(*p, Q, K, V, lengths, saved, G, dQ, dK, dV, ws, st), stream);
+    if (linear_mma_supported(*p))
+        return debug_finish(linear_mma_backward(*p, Q, K, V, lengths, saved, G, dQ, dK, dV, ws, st), stream);
     return debug_finish(general_linear_backward(*p, Q, K, V, lengths, saved, G, dQ, dK, dV, ws, st), stream);
 }
 

@@ -1,8 +1,7 @@
 // General kernels: any D, M (multiples of 8 up to 128), any N, fp32 or bf16 I/O,
-// fp32 arithmetic on the CUDA cores.  They serve the non-causal form of fp32 problems
-// (plain bf16 tensor-core products cannot hold the fp32 tolerance) and of every shape the
-// tensor-core kernels do not cover, and the causal form with M > 64 (la_causal_mma.cu has
-// the others).  All four are chunked restatements of Algorithm 1 on the
+// fp32 arithmetic on the CUDA cores.  They serve problems with M > 64 (la_causal_mma.cu and
+// la_linear_mma.cu have the others that the tcgen05 kernels do not take), and everything
+// with LA_DISABLE_TC.  All four are chunked restatements of Algorithm 1 on the
 // values extended by a ones column:
 //     Vt_j = [V_j, 1],   St = [S | Z]  (D x (M+1)),   [num_i | den_i] = phi(Q_i)^T St_i.
 // For a chunk c of T consecutive positions with L the lower-triangular mask,
@@ -444,13 +443,11 @@ __device__ __forceinline__ int64_t real_end(const int* lengths, int heads, int64
 }
 
 // part[bh][split] = sum over the split's positions of phi(X_i) [Y_i, 1]^T.
-// KD: D = M = KD known at compile time (all tile strides become constants), or 0: any D, M.
-template <typename IO, int KD>
+template <typename IO>
 __global__ void __launch_bounds__(THREADS)
 general_kv_sum_kernel(const IO* __restrict__ X, const IO* __restrict__ Y, float* __restrict__ part,
-                      int64_t N, int64_t split_len, int D_arg, int M_arg, int phi, const int* __restrict__ lengths, int heads) {
+                      int64_t N, int64_t split_len, int D, int M, int phi, const int* __restrict__ lengths, int heads) {
     extern __shared__ float smem[];
-    const int D = KD ? KD : D_arg, M = KD ? KD : M_arg;
     const Dims dm = make_dims(D, M);
     float* sx = smem;
     float* sy = sx + T * dm.DS;
@@ -488,14 +485,13 @@ __device__ void load_reduced_state(float* sSt, const float* part, int nsplit, in
     }
 }
 
-template <typename IO, int KD>
+template <typename IO>
 __global__ void __launch_bounds__(THREADS)
 general_linear_apply_kernel(const IO* __restrict__ Q, const float* __restrict__ part, IO* __restrict__ O,
                             float* __restrict__ den, float* __restrict__ KV, float* __restrict__ Zs,
-                            int nsplit, int64_t N, int64_t split_len, int D_arg, int M_arg, float eps, int phi,
+                            int nsplit, int64_t N, int64_t split_len, int D, int M, float eps, int phi,
                             const int* __restrict__ lengths, int heads) {
     extern __shared__ float smem[];
-    const int D = KD ? KD : D_arg, M = KD ? KD : M_arg;
     const Dims dm = make_dims(D, M);
     float* sq = smem;
     float* snd = sq + T * dm.DS;
@@ -542,14 +538,13 @@ general_linear_apply_kernel(const IO* __restrict__ Q, const float* __restrict__ 
 // Backward, query side: with St = full sum, form Gt_i, write
 // grad phi(Q_i) = St Gt_i (Eq. 13 with the full sum) and accumulate this split's
 // part of Rt = sum_i phi(Q_i) Gt_i^T.
-template <typename IO, int KD>
+template <typename IO>
 __global__ void __launch_bounds__(THREADS)
 general_linear_bwd_q_kernel(const IO* __restrict__ Q, const IO* __restrict__ G,
                             const float* __restrict__ part_s, IO* __restrict__ dQ,
                             float* __restrict__ part_r, int nsplit, int64_t N, int64_t split_len,
-                            int D_arg, int M_arg, float eps, int phi, const int* __restrict__ lengths, int heads) {
+                            int D, int M, float eps, int phi, const int* __restrict__ lengths, int heads) {
     extern __shared__ float smem[];
-    const int D = KD ? KD : D_arg, M = KD ? KD : M_arg;
     const Dims dm = make_dims(D, M);
     float* sq = smem;
     float* sg = sq + T * dm.DS;
@@ -593,14 +588,13 @@ general_linear_bwd_q_kernel(const IO* __restrict__ Q, const IO* __restrict__ G,
 }
 
 // Backward, key/value side: grad phi(K_j) = Rt Vt_j (Eq. 14), grad V_j = (Rt^T phi(K_j))[0:M] (Eq. 15).
-template <typename IO, int KD>
+template <typename IO>
 __global__ void __launch_bounds__(THREADS)
 general_linear_bwd_kv_kernel(const IO* __restrict__ K, const IO* __restrict__ V,
                              const float* __restrict__ part_r, IO* __restrict__ dK, IO* __restrict__ dV,
-                             int nsplit, int64_t N, int64_t split_len, int D_arg, int M_arg, int phi,
+                             int nsplit, int64_t N, int64_t split_len, int D, int M, int phi,
                              const int* __restrict__ lengths, int heads) {
     extern __shared__ float smem[];
-    const int D = KD ? KD : D_arg, M = KD ? KD : M_arg;
     const Dims dm = make_dims(D, M);
     float* sk = smem;
     float* sv = sk + T * dm.DS;
@@ -708,14 +702,14 @@ static int linear_forward_t(const la_problem& p, const void* Q, const void* K, c
     float* part = saved ? (float*)saved : (float*)ws;        // the per-split sums, kept for the backward pass if asked
     {
         const size_t smem = ((size_t)T * (D + 1) + (size_t)T * (M + 1) + state_floats(p)) * sizeof(float);
-        auto kern = D == 64 && M == 64 ? general_kv_sum_kernel<IO, 64> : general_kv_sum_kernel<IO, 0>;
+        auto kern = general_kv_sum_kernel<IO>;
         if (int rc = opt_in_smem(kern, smem)) return rc;
         kern<<<grid, THREADS, smem, st>>>((const IO*)K, (const IO*)V, part, p.N, sp.len, D, M, p.phi, lengths, (int)p.H);
         LA_LAUNCHED();
     }
     {
         const size_t smem = ((size_t)T * (D + 1) + (size_t)T * (M + 1) + state_floats(p)) * sizeof(float);
-        auto kern = D == 64 && M == 64 ? general_linear_apply_kernel<IO, 64> : general_linear_apply_kernel<IO, 0>;
+        auto kern = general_linear_apply_kernel<IO>;
         if (int rc = opt_in_smem(kern, smem)) return rc;
         kern<<<grid, THREADS, smem, st>>>((const IO*)Q, part, (IO*)O, den, KV, Zs, sp.nsplit, p.N, sp.len, D, M,
                                           p.eps, p.phi, lengths, (int)p.H);
@@ -742,14 +736,14 @@ static int linear_backward_t(const la_problem& p, const void* Q, const void* K, 
         part_s = (float*)saved;           // the forward's own sums: nothing to recompute
     } else {
         const size_t smem = ((size_t)T * (D + 1) + (size_t)T * (M + 1) + state_floats(p)) * sizeof(float);
-        auto kern = D == 64 && M == 64 ? general_kv_sum_kernel<IO, 64> : general_kv_sum_kernel<IO, 0>;
+        auto kern = general_kv_sum_kernel<IO>;
         if (int rc = opt_in_smem(kern, smem)) return rc;
         kern<<<grid, THREADS, smem, st>>>((const IO*)K, (const IO*)V, part_s, p.N, sp.len, D, M, p.phi, lengths, (int)p.H);
         LA_LAUNCHED();
     }
     {
         const size_t smem = ((size_t)T * (D + 1) + (size_t)2 * T * (M + 1) + 2 * state_floats(p)) * sizeof(float);
-        auto kern = D == 64 && M == 64 ? general_linear_bwd_q_kernel<IO, 64> : general_linear_bwd_q_kernel<IO, 0>;
+        auto kern = general_linear_bwd_q_kernel<IO>;
         if (int rc = opt_in_smem(kern, smem)) return rc;
         kern<<<grid, THREADS, smem, st>>>((const IO*)Q, (const IO*)G, part_s, (IO*)dQ, part_r, sp.nsplit, p.N,
                                           sp.len, D, M, p.eps, p.phi, lengths, (int)p.H);
@@ -757,7 +751,7 @@ static int linear_backward_t(const la_problem& p, const void* Q, const void* K, 
     }
     {
         const size_t smem = ((size_t)T * (D + 1) + (size_t)T * (M + 1) + state_floats(p)) * sizeof(float);
-        auto kern = D == 64 && M == 64 ? general_linear_bwd_kv_kernel<IO, 64> : general_linear_bwd_kv_kernel<IO, 0>;
+        auto kern = general_linear_bwd_kv_kernel<IO>;
         if (int rc = opt_in_smem(kern, smem)) return rc;
         kern<<<grid, THREADS, smem, st>>>((const IO*)K, (const IO*)V, part_r, (IO*)dK, (IO*)dV, sp.nsplit, p.N,
                                           sp.len, D, M, p.phi, lengths, (int)p.H);

@@ -12,6 +12,7 @@
 #include <mutex>
 
 #include "la_common.cuh"
+#include "la_tc.cuh"
 
 namespace la {
 namespace {
@@ -58,7 +59,9 @@ extern "C" int la_linear_attention_noalloc(const la_problem* p, const void* Q, c
     if ((den && !aligned16(den)) || (KV && !aligned16(KV)) || (Zs && !aligned16(Zs)))
         return fail(LA_ERR_INVALID_ARG, "den, KV and Zs must be 16-byte aligned");
 
-    const size_t need = general_workspace_bytes(*p, LA_OP_LINEAR_FORWARD);
+    // the kernels of la_linear_attention() for problems off the tcgen05 kernels, where their sums fit the array
+    const bool mma = linear_mma_supported(*p) && linear_mma_workspace(*p, false) <= (size_t)LA_NOALLOC_SCRATCH_BYTES;
+    const size_t need = mma ? linear_mma_workspace(*p, false) : general_workspace_bytes(*p, LA_OP_LINEAR_FORWARD);
     if (need > (size_t)LA_NOALLOC_SCRATCH_BYTES)
         return fail(LA_ERR_WORKSPACE,
                     "this problem needs %zu bytes of scratch but the built-in array holds %zu: use "
@@ -70,5 +73,6 @@ extern "C" int la_linear_attention_noalloc(const la_problem* p, const void* Q, c
     if (int rc = scratch_for_current_device(&scratch)) return rc;
     // Every partial sum the second kernel reads is written by the first one in the same call,
     // so nothing in the array has to start at zero.
+    if (mma) return linear_mma_forward(*p, Q, K, V, nullptr, O, den, KV, Zs, nullptr, scratch, (cudaStream_t)stream);
     return general_linear_forward(*p, Q, K, V, nullptr, O, den, KV, Zs, nullptr, scratch, (cudaStream_t)stream);
 }

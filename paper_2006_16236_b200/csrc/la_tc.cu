@@ -21,6 +21,7 @@ void set_plan_override(int pieces, int short_len, int splits) {
 }
 
 int causal_pieces_override() { return g_override_pieces.load(std::memory_order_relaxed); }
+int linear_splits_override() { return g_override_splits.load(std::memory_order_relaxed); }
 
 int sm_count() {
     static thread_local int cached_dev = -1, cached_sms = 148;

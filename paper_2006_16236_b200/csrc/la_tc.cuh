@@ -21,10 +21,20 @@ int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const 
 int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
                         const StateArgs& sa, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
 
+// Non-causal form at fp32 accuracy on mma.sync (la_linear_mma.cu): M <= 64, any type and feature map; saved (or null):
+// where the forward leaves its sums and the backward finds them.
+bool linear_mma_supported(const la_problem& p);
+size_t linear_mma_workspace(const la_problem& p, bool backward);
+int linear_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O, float* den,
+                       float* KV, float* Zs, void* saved, void* ws, cudaStream_t st);
+int linear_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* saved,
+                        const void* G, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
+
 namespace tc {
 // process-wide overrides of the automatic plans (see la_plan_override)
 void set_plan_override(int causal_pieces, int causal_short, int linear_splits);
 int causal_pieces_override();        // -1: automatic
+int linear_splits_override();
 // In all of these: lengths ([B] int32, device, or null) = real positions per batch element of a right-padded
 // ragged batch; saved (or null) = where the forward leaves what the backward pass can reuse.
 size_t causal_forward_workspace(const la_problem& p);

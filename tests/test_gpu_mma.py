@@ -1,4 +1,4 @@
-"""Causal calls at fp32 accuracy on the warp-level tensor instructions: shapes at the edges of their tiles (chunks of
+"""Calls at fp32 accuracy on the warp-level tensor instructions: shapes at the edges of their tiles (chunks of
 64 positions, strips of 16, columns padded to 32, 64 or 128), with the sequence whole and cut into pieces, from a state,
 ragged, and without the optional workspace, against the fp64 oracle.
 
@@ -111,3 +111,47 @@ def test_many_short_bf16_sequences(N, pieces):
                 assert_close(x[sl], ref, torch.bfloat16, nm, grad=True)
                 assert not x[b, :, n:].any()
             assert not O[b, :, n:].any()
+
+
+@pytest.mark.parametrize("splits", [-1, 1, 3])
+@pytest.mark.parametrize("N", [1, 16, 63, 64, 65, 400])
+@pytest.mark.parametrize("dims", [(8, 8), (32, 32), (40, 24), (64, 64), (72, 64), (128, 64)], ids=str)
+def test_noncausal_tiles(dims, N, splits):
+    """The non-causal form on the same products: strips, splits, a ragged batch with an empty sequence, kept sums."""
+    D, M = dims
+    for dtype, phi in ((torch.float32, "elu1"), (torch.float32, "identity"), (torch.bfloat16, "identity"), (torch.bfloat16, "elu1")):
+        if dtype == torch.bfloat16 and D == M and D in (32, 64):
+            continue                                    # another kernel's problem
+        Q, K, V, G = draw_qkvg(3, 2, N, D, M, 3 + N, dtype, 1.0)
+        if phi == "identity":
+            Q, K = Q.abs() + 0.1, K.abs() + 0.1
+        la.la_plan_override(-1, -1, splits)
+        dev = [t.to(DEV) for t in (Q, K, V, G)]
+        eps = 0.5 if N % 2 else 0.0
+        lengths = [N, 0, (N + 1) // 2]
+        for ln in (None, torch.tensor(lengths, dtype=torch.int32, device=DEV)):
+            saved = la.linear_saved_buffer(dev[0], dev[2], phi=phi)
+            den = torch.empty(3, 2, N, device=DEV)
+            O = la.la_linear_attention(*dev[:3], phi=phi, eps=eps, lengths=ln, saved=saved, den=den)
+            grads = la.la_linear_attention_backward(*dev, phi=phi, eps=eps, lengths=ln, saved=saved)
+            plain = la.la_linear_attention_backward(*dev, phi=phi, eps=eps, lengths=ln)
+            la.la_last_device_status()
+            assert all(torch.equal(a, b) for a, b in zip(grads, plain))
+            f32 = dtype == torch.float32
+            for b in range(3):
+                n = N if ln is None else lengths[b]
+                assert not O[b, :, n:].any() and not den[b, :, n:].any() and not any(x[b, :, n:].any() for x in grads)
+                if n == 0:
+                    continue
+                sl = (slice(b, b + 1), slice(None), slice(0, n))
+                q, k, v, g = (t[sl].double().numpy() for t in (Q, K, V, G))
+                Or, denr = oracle.linear_attention(q, k, v, causal=False, phi=phi, eps=eps)[:2]
+                _close(O[sl], Or, 2e-6 if f32 else 2 ** -8, "O")
+                _close(den[sl], denr, 2e-6, "den")
+                if n == 1 and not eps:
+                    continue                            # dQ and dK are analytically zero
+                # (one key: O = V dn' / (dn' + eps), so that of dQ's and dK's terms only their eps / dn is left)
+                left = eps / (np.abs(denr).max() + eps) if n == 1 else 1.0
+                for nm, x, ref in zip(("dQ", "dK", "dV"), grads,
+                                      oracle.linear_attention_backward(q, k, v, g, causal=False, phi=phi, eps=eps)):
+                    _close(x[sl], ref, (8e-6 if f32 else 2 ** -8) / (left if f32 else 1.0), nm)
