@@ -150,14 +150,18 @@ __device__ __forceinline__ void load_cols_t(uint32_t (&f)[NP][4], uint32_t tile,
 }
 
 // ---- global memory -> registers -> operand planes ------------------------------------------------------------
+// Ordinary loads throughout, not __ldg: a kernel that was launched as a programmatic dependent is resident while the kernel
+// before it still writes what it will read (the state of the piece before, the features of a map).  The read-only path asks
+// for data that nobody writes while the kernel runs, and the compiler may move such a load ahead of griddepcontrol.wait.
+
 // A group of eight consecutive elements of a row.
 template <typename IO> struct Group8;
 template <> struct Group8<float> {
     float4 a, b;
     __device__ __forceinline__ void fill(float v) { a = b = make_float4(v, v, v, v); }
     __device__ __forceinline__ void load(const float* p) {
-        a = __ldg(reinterpret_cast<const float4*>(p));
-        b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+        a = *reinterpret_cast<const float4*>(p);
+        b = reinterpret_cast<const float4*>(p)[1];
     }
     __device__ __forceinline__ void get(float (&x)[8]) const {
         x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
@@ -166,7 +170,7 @@ template <> struct Group8<float> {
 template <> struct Group8<__nv_bfloat16> {
     uint4 a;
     __device__ __forceinline__ void fill(float v) { const uint32_t w = __byte_perm(__float_as_uint(v), 0u, 0x3232); a = make_uint4(w, w, w, w); }
-    __device__ __forceinline__ void load(const __nv_bfloat16* p) { a = __ldg(reinterpret_cast<const uint4*>(p)); }
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { a = *reinterpret_cast<const uint4*>(p); }
     __device__ __forceinline__ void get(float (&x)[8]) const {
         const uint32_t w[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
@@ -236,7 +240,7 @@ struct RawTile {
     }
 };
 
-__device__ __forceinline__ float2 load_pair(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
+__device__ __forceinline__ float2 load_pair(const float* p) { return *reinterpret_cast<const float2*>(p); }
 template <typename IO> __device__ __forceinline__ void store_pair(IO* p, float x, float y);
 template <> __device__ __forceinline__ void store_pair<float>(float* p, float x, float y) { *reinterpret_cast<float2*>(p) = make_float2(x, y); }
 template <> __device__ __forceinline__ void store_pair<__nv_bfloat16>(__nv_bfloat16* p, float x, float y) {
@@ -248,7 +252,7 @@ template <> __device__ __forceinline__ void store_pair<__nv_bfloat16>(__nv_bfloa
 template <typename IO> struct Pair;
 template <> struct Pair<float> {
     float2 v;
-    __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float2*>(p)); }
+    __device__ __forceinline__ void load(const float* p) { v = *reinterpret_cast<const float2*>(p); }
     __device__ __forceinline__ void fill(float x) { v = make_float2(x, x); }
     __device__ __forceinline__ float lo() const { return v.x; }
     __device__ __forceinline__ float hi() const { return v.y; }
@@ -257,7 +261,7 @@ template <> struct Pair<float> {
 };
 template <> struct Pair<__nv_bfloat16> {        // as loaded: one plane
     uint32_t w;
-    __device__ __forceinline__ void load(const __nv_bfloat16* p) { w = __ldg(reinterpret_cast<const uint32_t*>(p)); }
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { w = *reinterpret_cast<const uint32_t*>(p); }
     __device__ __forceinline__ void fill(float x) { w = __byte_perm(__float_as_uint(x), 0u, 0x3232); }
     __device__ __forceinline__ float lo() const { return __uint_as_float(w << 16); }
     __device__ __forceinline__ float hi() const { return __uint_as_float(w & 0xffff0000u); }

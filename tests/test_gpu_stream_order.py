@@ -135,3 +135,37 @@ def test_training_step_replayed_from_a_cuda_graph(name):
         for a, b, nm in zip(want, (O, dQ, dK, dV), ("O", "dQ", "dK", "dV")):
             assert torch.equal(a, b), f"{name}: {nm} of a graph replay differs from the eager call"
     la.la_last_device_status()
+
+
+@pytest.mark.parametrize("D,H", [(32, 2), (64, 4)])
+def test_small_fp32_calls_that_feed_each_other(D, H):
+    """The kernels of small fp32 problems start as programmatic dependents of whatever is in front of them, another call's
+    included: the state goes from piece to piece of a prompt between two pairs of buffers, outputs and gradients go
+    straight into the next call as its inputs, and nothing is synchronised.  Same bits as with a wait after every call."""
+    B, N, T = 1, 200, 12
+    g = torch.Generator().manual_seed(11)
+    Q, K, V, G = (torch.randn((B, H, T * N, D), generator=g).to(DEV) for _ in range(4))
+    pieces = [[t[:, :, i * N:(i + 1) * N].contiguous() for t in (Q, K, V, G)] for i in range(T)]
+
+    def run(synced):
+        def gap():
+            if synced:
+                torch.cuda.synchronize()
+        S = [torch.zeros((B, H, D, D), device=DEV) for _ in range(2)]
+        Z = [torch.zeros((B, H, D), device=DEV) for _ in range(2)]
+        q, k, v, o = (torch.empty_like(pieces[0][0]) for _ in range(4))
+        out = []
+        for i, (a, b, c, d) in enumerate(pieces):
+            q.copy_(a); k.copy_(b); v.copy_(c); gap()
+            la.la_causal_forward(q, k, v, O=o, S_in=S[i & 1], Z_in=Z[i & 1], S_out=S[~i & 1], Z_out=Z[~i & 1]); gap()
+            dq, dk, dv = la.la_causal_backward(q, k, o, d, S_in=S[i & 1], Z_in=Z[i & 1]); gap()
+            e = la.la_linear_attention(dq, dk, dv); gap()
+            out += [o.clone(), dq, dk, dv, e, *la.la_linear_attention_backward(q, k, e, dv)]; gap()
+        torch.cuda.synchronize()
+        return out + S + Z
+
+    want = run(True)
+    for _ in range(4):
+        for i, (a, b) in enumerate(zip(want, run(False), strict=True)):
+            assert torch.equal(a, b), i
+    la.la_last_device_status()
