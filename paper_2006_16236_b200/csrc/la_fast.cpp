@@ -14,9 +14,8 @@
 #include <ATen/PythonTorchFunctionTLS.h>
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
-
-#include <exception>
 
 #include "la.h"
 
@@ -162,16 +161,12 @@ template <typename F> int unlocked(F f) {
     return rc;
 }
 
-template <typename F> PyObject* guarded(F f) {      // no C++ exception leaves this file
-    try {
-        return f();
-    } catch (const std::exception& e) {
-        if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
-    } catch (...) {
-        if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, "unknown C++ exception");
-        return nullptr;
-    }
+// No C++ exception leaves this file: it becomes the Python exception that torch's own functions raise (an allocation that
+// fails is a torch.OutOfMemoryError, which programs catch to go on with a smaller batch).
+template <typename F> PyObject* guarded(F f) {
+    HANDLE_TH_ERRORS
+    return f();
+    END_HANDLE_TH_ERRORS
 }
 
 PyObject* three(Out& a, Out& b, Out& c) {

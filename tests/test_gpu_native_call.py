@@ -72,3 +72,28 @@ def test_same_errors_and_outputs_in_place():
         la.la_causal_forward(Q, Q, V, eps=-1.0)
     with pytest.raises(la.LaError):
         la.la_causal_forward(Q, Q, V, S_in=torch.zeros(1, 2, 32, 32, device=DEV))
+
+
+def test_an_allocation_that_fails_is_an_out_of_memory_error():
+    """Outputs and scratch are allocated in native code; a program that catches torch.OutOfMemoryError to go on with a
+    smaller batch has to see that type.  The failure is the allocator's: it is told to hold no more than it already does."""
+    n = lambda *s, dt=torch.float32: torch.zeros(s, device=DEV, dtype=dt)
+    Q, Qb = n(1, 8, 65536, 16), n(1, 8, 65536, 64, dt=torch.bfloat16)       # 33 and 67 MB: no block of that size is kept
+    q, S, Z = n(32768, 8, 32), n(32768, 8, 32, 32), n(32768, 8, 32)
+    x, W, Wo = n(32768, 512, dt=torch.bfloat16), n(1536, 512, dt=torch.bfloat16), n(512, 512, dt=torch.bfloat16)
+    Sl, Zl = n(32768, 8, 64, 64), n(32768, 8, 64)
+    calls = [lambda: la.la_causal_forward(Q, Q, Q), lambda: la.la_causal_backward(Q, Q, Q, Q),
+             lambda: la.la_linear_attention(Q, Q, Q), lambda: la.la_linear_attention_backward(Q, Q, Q, Q),
+             lambda: la.la_recurrent_step(q, q, q, S, Z), lambda: la.la_decode_layer_step(x, W, Wo, Sl, Zl),
+             lambda: la.saved_buffer(Qb, Qb)]
+    binding._ws_cache.clear()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    torch.cuda.set_per_process_memory_fraction(0.0)
+    try:
+        for call in calls:
+            with pytest.raises(torch.OutOfMemoryError):
+                call()
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert torch.isfinite(la.la_causal_forward(Q, Q, Q)).all()
