@@ -113,7 +113,11 @@ def _native():
     global _fast
     if _fast is None:
         lib()
-        from . import _la_fast
+        try:
+            from . import _la_fast
+        except ImportError as e:
+            raise RuntimeError(f"the native part of the binding (_la_fast.so) cannot be loaded ({e}): run "
+                               "`python -m paper_2006_16236_b200.build` (there is no fallback path)") from e
         _fast = _la_fast
     return _fast
 

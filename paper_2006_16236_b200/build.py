@@ -43,16 +43,29 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def _built_for() -> str:
+    """What the native part of the binding was compiled against, a string that it carries."""
+    import torch
+    return f"built for torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _fast_stale() -> bool:
+    """Missing, older than its sources, or compiled against another torch or Python."""
+    if not os.path.exists(FAST) or os.path.getmtime(FAST) < max(map(os.path.getmtime, (FAST_SRC, os.path.join(ROOT, "include", "la.h")))):
+        return True
+    with open(FAST, "rb") as f:
+        return _built_for().encode() + b"\0" not in f.read()
+
+
 def build_fast(force: bool = False) -> str:
     """Compile the native part of the binding against torch's headers; it loads libla.so from its own folder."""
-    header = os.path.join(ROOT, "include", "la.h")
-    if force or not os.path.exists(FAST) or os.path.getmtime(FAST) < max(os.path.getmtime(FAST_SRC), os.path.getmtime(header)):
+    if force or _fast_stale():
         import torch
         t = os.path.dirname(torch.__file__)
         include = [os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
                    sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
         cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in include), "-o", FAST, FAST_SRC,
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DLA_BUILT_FOR="{_built_for()}"', *(f"-I{d}" for d in include), "-o", FAST, FAST_SRC,
                "-L", PKG, "-l:libla.so", "-L", os.path.join(t, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
                "-Wl,-rpath,$ORIGIN"]
         subprocess.run(cmd, check=True)

@@ -365,7 +365,8 @@ PyObject* new_buffer(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
 #define LA_METHOD(f) {#f, (PyCFunction)(void (*)(void))f, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {LA_METHOD(recurrent_step), LA_METHOD(decode_layer_step), LA_METHOD(causal_forward), LA_METHOD(causal_backward),
                          LA_METHOD(linear_forward), LA_METHOD(linear_backward), LA_METHOD(new_buffer), {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_la_fast", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+// (build.py looks for this string in the file: built against another torch or Python it is built again)
+PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_la_fast", LA_BUILT_FOR, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 

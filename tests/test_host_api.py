@@ -214,6 +214,24 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
         binding.lib()
 
 
+def test_missing_native_part_fails_loudly(L, monkeypatch):
+    import sys
+    monkeypatch.setattr(binding, "_fast", None)
+    monkeypatch.delattr(la, "_la_fast", raising=False)
+    monkeypatch.setitem(sys.modules, "paper_2006_16236_b200._la_fast", None)       # as if the file were not there
+    with pytest.raises(RuntimeError, match="paper_2006_16236_b200.build.*no fallback"):
+        binding._native()
+
+
+def test_native_part_of_another_torch_or_python_is_built_again(L, monkeypatch, tmp_path):
+    assert not build._fast_stale()
+    data = open(build.FAST, "rb").read()
+    other = tmp_path / "other.so"
+    other.write_bytes(data.replace(torch.__version__.encode(), b"0" * len(torch.__version__)))
+    monkeypatch.setattr(build, "FAST", str(other))
+    assert build._fast_stale()
+
+
 def test_plan_override_is_an_explicit_call(L):
     p = la.make_problem(4, 16, 18 * 128, 64, 64, la.LA_BF16)
     auto = la.la_causal_plan(p)
