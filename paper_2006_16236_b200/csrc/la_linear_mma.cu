@@ -128,10 +128,12 @@ linear_mma_dq_kernel(const Params p) {
     IO* dQ = (IO*)p.dQ + r.bh * p.N * D;
     float* dn_all = p.aux + r.bh * 2 * p.N;
     float* dl_all = dn_all + p.N;
+    const int4 stamp = p.stamp ? *reinterpret_cast<const int4*>(p.stamp) : plan_stamp(p);        // (on its way beside the records)
     {
         State<DP, MP, THREADS / 32> st;
         load_state<C>(st, p, r.bh, smem);
     }
+    if (other_plan(p, stamp)) return;
     for (int64_t n0 = r.lo + 16 * warp; n0 < r.end; n0 += 16 * (THREADS / 32)) {
         const int cn = (int)(r.end - n0 < 16 ? r.end - n0 : 16);
         RawStrip<IO, DP> rq;            // element j of block kk: result column tile 2 kk + j / 2, row g + 8 (j & 1)
@@ -210,10 +212,12 @@ linear_mma_dkv_kernel(const Params p) {
     const IO* V = (const IO*)p.V + r.bh * p.N * M;
     IO* dK = (IO*)p.dK + r.bh * p.N * D;
     IO* dV = (IO*)p.dV + r.bh * p.N * M;
+    const int4 stamp = p.stamp ? *reinterpret_cast<const int4*>(p.stamp) : plan_stamp(p);
     {
         State<DP, MP, THREADS / 32> st;
         load_state<C>(st, p, r.bh, smem);
     }
+    if (other_plan(p, stamp)) return;
     for (int64_t n0 = r.lo + 16 * warp; n0 < r.end; n0 += 16 * (THREADS / 32)) {
         const int cn = (int)(r.end - n0 < 16 ? r.end - n0 : 16);
         RawStrip<typename FeatureType<NQ>::type, DP> fk;
@@ -350,7 +354,7 @@ bool linear_mma_supported(const la_problem& p) {
 }
 
 size_t linear_mma_workspace(const la_problem& p, bool backward) {
-    if (!backward) return record_bytes(p);
+    if (!backward) return kStampBytes + record_bytes(p);
     return 2 * record_bytes(p) + (((size_t)(p.B * p.H) * (size_t)p.N * 2 * sizeof(float) + 15) & ~(size_t)15);
 }
 
@@ -358,7 +362,8 @@ int linear_mma_forward(const la_problem& p, const void* Q, const void* K, const 
                        float* KV, float* Zs, void* saved, void* ws, cudaStream_t st) {
     Params a = make_params(p, lengths);
     a.Q = Q; a.K = K; a.V = V; a.O = O; a.den = den; a.S1 = KV; a.Z1 = Zs;
-    a.rec = saved ? (float*)saved : (float*)ws;          // kept for the backward pass if asked
+    a.stamp = saved ? (int*)saved : (int*)ws;            // kept for the backward pass if asked
+    a.rec = (float*)((char*)a.stamp + kStampBytes);
     return dispatch(p, [&](auto k) { return decltype(k)::forward(p, a, st); });
 }
 
@@ -366,8 +371,13 @@ int linear_mma_backward(const la_problem& p, const void* Q, const void* K, const
                         const void* G, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st) {
     Params f = make_params(p, lengths);
     f.Q = Q; f.K = K; f.V = V; f.G = G; f.dQ = dQ; f.dK = dK; f.dV = dV;
+    if (saved) {
+        f.stamp = (int*)saved;
+        f.status = device_status_ptr();
+        if (!f.status) return fail(LA_ERR_CUDA, "device status word unavailable");
+    }
     Params r = f;
-    f.rec = saved ? (float*)saved : (float*)ws;
+    f.rec = saved ? (float*)((char*)saved + kStampBytes) : (float*)ws;
     r.rec = (float*)((char*)ws + record_bytes(p));
     f.aux = r.aux = (float*)((char*)ws + 2 * record_bytes(p));
     return dispatch(p, [&](auto k) { return decltype(k)::backward(p, f, r, saved != nullptr, st); });

@@ -29,6 +29,8 @@ struct Params {
     int64_t N, piece_len;
     int pieces, heads, D, M, phi;
     int chained;                 // launched as a programmatic dependent of the kernel before it in the stream
+    int* stamp;                  // kept sums (or null): the plan they were written under, see plan_stamp()
+    int* status;                 // device status word (with stamp)
     float eps;
 };
 
@@ -46,6 +48,19 @@ __device__ __forceinline__ Range range_of(const Params& p, int piece) {
         if (len < r.end) r.end = len < r.lo ? r.lo : len;
     }
     return r;
+}
+
+// Kept sums start with the plan they were written under.  A backward pass that would cut the sequences in another way
+// (la_plan_override() in between) would add up the wrong records: it reports that and writes no gradient.
+constexpr int kStampBytes = 16;
+__device__ __forceinline__ int4 plan_stamp(const Params& p) {
+    return make_int4(0x4c414d4d, p.pieces, (int)(p.piece_len / T), p.D * 256 + p.M);
+}
+__device__ __forceinline__ bool other_plan(const Params& p, const int4& found) {
+    const int4 mine = plan_stamp(p);
+    if (found.x == mine.x && found.y == mine.y && found.z == mine.z && found.w == mine.w) return false;
+    if (threadIdx.x == 0) atomicOr(p.status, sm100::kStatusPlanMismatch);
+    return true;
 }
 
 template <int THREADS, typename IO>
@@ -334,6 +349,7 @@ causal_mma_sum_kernel(const Params p) {
     const IO* Y = (const IO*)(REVERSE ? p.G : p.V) + r.bh * p.N * M;
     const float* dn = REVERSE ? p.aux + r.bh * 2 * p.N : nullptr;
     const float* delta = REVERSE ? dn + p.N : nullptr;
+    if (!REVERSE && p.stamp && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *reinterpret_cast<int4*>(p.stamp) = plan_stamp(p);
     State<DP, MP, 4 * C::WPS> st;
     st.init(p, nullptr, nullptr, nullptr, 0);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {

@@ -42,6 +42,12 @@ namespace {
 //   forward sums (sum kernel)            : A' = sum k'_j V_j^T, a' = sum k'_j, ysum = sum V_j,        w0 unused
 //   reverse sums (backward-Q apply pass) : A' = sum qh'_i G_i^T, a' = sum qh'_i dl_i, ysum = sum G_i / dn_i, w0 = sum dl_i / dn_i
 constexpr int kRecFloats = kDim * kDim + kDim + kDim + 8;
+// The last four words of the first record: the split plan it was written under.  A backward pass that is given kept
+// records and would split the sequences in another way (la_plan_override() in between) reports that and writes nothing.
+constexpr int kRecStamp = kRecFloats - 4;
+__device__ __forceinline__ int4 split_stamp(int nseg, int chunks_per_seg, int dim) {
+    return make_int4(0x4c414c53, nseg, chunks_per_seg, dim);
+}
 
 __device__ __forceinline__ float elu_fast(float x) {      // elu(x) = phi(x) - 1
     float e;
@@ -161,6 +167,8 @@ linear_sum_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     grid_dependency_wait();
     allow_dependent_launch();
     LA_TRACE_CTA(g_trace_lin, 1);
+    if (blockIdx.x == 0 && tid == kLsThreads - 1)
+        *reinterpret_cast<int4*>(prm.records + kRecStamp) = split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
     // Ragged batch: only `real` rows of this split exist; chunks behind them are skipped and the rows behind
     // them in the last chunk are zeroed after the load (at least one chunk runs, so that the record is written
     // from an accumulator that holds zeros and not from one that was never started).
@@ -319,6 +327,7 @@ struct ApParams {
     float* state_out;           // forward: KV [BH][64][64] (optional)
     float* vec_out;             // forward: Zs [BH][64] (optional)
     const int* lengths;         // [B] real positions per batch element (right-padded ragged batch), or null
+    const float* kept;          // backward: the forward's kept records, whose stamp has to be this plan's, or null
     int heads;
     int* status;
     int64_t N;
@@ -410,6 +419,11 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         grid_dependency_wait();
         allow_dependent_launch();
     }
+    bool mismatch = false;      // (the same for every thread)
+    if (kHasY && prm.kept) {
+        const int4 a = *reinterpret_cast<const int4*>(prm.kept + kRecStamp), b = split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
+        mismatch = a.x != b.x || a.y != b.y || a.z != b.z || a.w != b.w;
+    }
     // state of this head: add the split records (fp32), remove the column means, round the
     // centred remainder to a bf16 operand tile.  Scratch: the output staging tiles, free until the first epilogue.
     {
@@ -495,7 +509,11 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
     volatile int* abort_flag = &bars->abort_flag;
     LA_TRACE_CTA(g_trace_lin, 5);
 
-    if (warp == 8) {
+    if (kHasY && mismatch) {    // nothing is started; the tiles requested above have to arrive before the CTA may leave
+        if (tid == 0) atomicOr(prm.status, kStatusPlanMismatch);
+        if (warp == 8 && lane == 0)
+            for (int c = 0; c < min(L, kApStages); ++c) mbar_wait(&bars->full[c], 0, prm.status, kStatusTmaTimeout);
+    } else if (warp == 8) {
         if (lane == 0) {
             #pragma unroll 1
             for (int c = kApStages; c < L; ++c) {
@@ -955,12 +973,14 @@ int linear_backward(const la_problem& p, const void* Q, const void* K, const voi
     ApParams a = {};
     a.early = saved ? 0 : 1;    // the first kernel of the call with saved records, else behind the sum kernel
     a.lengths = lengths;
+    a.kept = (const float*)saved;
     a.records = rec_s;
     a.out0 = (__nv_bfloat16*)dQ;
     a.rec_out = rec_r;          // the reverse sums of Q / dn and G are formed by the same pass
     if (int rc = launch_apply<kApplyBackwardQ>(p, sg, mQ, mG, a, st)) return rc;
     ApParams b = {};
     b.lengths = lengths;
+    b.kept = (const float*)saved;
     b.records = rec_r;
     b.out0 = (__nv_bfloat16*)dK;
     b.out1 = (__nv_bfloat16*)dV;

@@ -157,6 +157,35 @@ def test_backward_refuses_a_saved_buffer_of_another_plan(plan_override):
     assert_close(dV[sl], rv, torch.bfloat16, "dV", grad=True)
 
 
+@pytest.mark.parametrize("dtype,D,M", [(torch.bfloat16, 64, 64), (torch.float32, 64, 64), (torch.float32, 40, 24),
+                                       (torch.bfloat16, 128, 64)])
+def test_noncausal_backward_refuses_kept_sums_of_another_plan(plan_override, dtype, D, M):
+    """The same of the non-causal form: the kept sums carry the splits they were formed over."""
+    if os.environ.get("LA_DEBUG"):
+        pytest.skip("in checked mode the call itself reads the status and raises; this test reads it afterwards")
+    Q, K, V, G = draw_qkvg(2, 3, 2100, D, M, seed=79, dtype=dtype, scale=0.5)
+    Qd, Kd, Vd, Gd = gpu(Q, K, V, G)
+    plan_override(linear_splits=4)
+    saved = la.linear_saved_buffer(Qd, Vd)
+    la.la_linear_attention(Qd, Kd, Vd, saved=saved)
+    for splits in (2, 3, -1):
+        plan_override(linear_splits=splits)
+        if splits < 0:
+            saved = torch.cat([saved, torch.zeros_like(saved).repeat(64)])      # large enough under any plan
+        dQ, dK, dV = torch.full_like(Qd, 7.0), torch.full_like(Kd, 7.0), torch.full_like(Vd, 7.0)
+        la.la_linear_attention_backward(Qd, Kd, Vd, Gd, saved=saved, dQ=dQ, dK=dK, dV=dV)
+        with pytest.raises(la.LaError) as e:
+            la.la_last_device_status()
+        assert e.value.status == -1 and "plan" in str(e.value)
+        assert all(torch.all(t == 7.0) for t in (dQ, dK, dV))       # nothing was written
+        la.la_last_device_status()              # the flag is cleared, the context usable
+    plan_override(linear_splits=4)
+    grads = la.la_linear_attention_backward(Qd, Kd, Vd, Gd, saved=saved)
+    la.la_last_device_status()
+    for nm, x, ref in zip(("dQ", "dK", "dV"), grads, oracle.linear_attention_backward(Q, K, V, G, False)):
+        assert_close(x, ref, dtype, nm, grad=True)
+
+
 @pytest.mark.parametrize("causal", [True, False])
 @pytest.mark.parametrize("dtype", DTYPES)
 def test_eps_and_identity_feature_map(causal, dtype):
