@@ -318,8 +318,9 @@ causal_mma_dq_kernel(const Params p) {
         const bool real = row0 < cn;
         // The first chunk of a sequence goes through twice, the second time with the G_i . O_i it found taken off the
         // scores: where few terms make up a row, h and (q . h / dn) Zc cancel almost entirely (in row 0 completely).
-        // (The state before that chunk is zero: G S^T has no part in it.)
-        const int first_pass = n0 == 0 && !p.S0 ? 0 : 1;
+        // (A state it continues from may be zero as well and is treated alike, its part of h included, by single warps;
+        // pairs have overwritten its planes by then and go through twice only where it has no part.)
+        const int first_pass = n0 == 0 && (WPS == 1 || !p.S0) ? 0 : 1;
         float c0 = 0.f, c1 = 0.f;               // G_i . O_i of rows g, g + 8, as far as it is known
         float h[DP / 8][4], zc[DP / 8][4];
         auto ones_block = [&](uint32_t (&ones)[1][4], int jb) {         // the part of L in key block jb
@@ -388,20 +389,21 @@ causal_mma_dq_kernel(const Params p) {
                 }
             }
         }
-        if (state_part) {
-            if (real) {
+        auto state_product = [&]() {            // h = G S^T
 #pragma unroll
-                for (int n = 0; n < DP / 16; ++n) {
-                    Chain c;
+            for (int n = 0; n < DP / 16; ++n) {
+                Chain c;
 #pragma unroll
-                    for (int ee = 0; ee < MP / 16; ++ee) {
-                        uint32_t b[NS][4], f[NV][4];
-                        load_rows<NS, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
-                        c.step<NV, NS>(ga.block(ee, f), b);
-                    }
-                    c.put(h[2 * n], h[2 * n + 1]);
+                for (int ee = 0; ee < MP / 16; ++ee) {
+                    uint32_t b[NS][4], f[NV][4];
+                    load_rows<NS, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
+                    c.step<NV, NS>(ga.block(ee, f), b);
                 }
+                c.put(h[2 * n], h[2 * n + 1]);
             }
+        };
+        if (state_part) {
+            if (WPS == 2 && real) state_product();
             if constexpr (WPS == 2) bar_arrive(1, THREADS);
             if (real) {
                 if constexpr (WPS == 2) {
@@ -419,7 +421,19 @@ causal_mma_dq_kernel(const Params p) {
                     }
                 }
                 for (int pass = first_pass; pass < 2; ++pass) {
-                    if (pass == 1 && first_pass == 0) clear(h);
+                    if constexpr (WPS == 1) {
+                        state_product();
+                        if (pass > first_pass) {            // the second time: take G_i . O_i off the state's part too
+#pragma unroll
+                            for (int n = 0; n < DP / 8; ++n) {
+                                const float2 z = *reinterpret_cast<const float2*>(sZ + n * 8 + 2 * t);
+                                h[n][0] = fmaf(-c0, z.x, h[n][0]); h[n][1] = fmaf(-c0, z.y, h[n][1]);
+                                h[n][2] = fmaf(-c1, z.x, h[n][2]); h[n][3] = fmaf(-c1, z.y, h[n][3]);
+                            }
+                        }
+                    } else if (pass > first_pass) {
+                        clear(h);
+                    }
                     RawStrip<IO, DP> rq;        // element j of block kk: result column tile 2 kk + j / 2, row g + 8 (j & 1)
                     if constexpr (WPS == 2) {
                         rq.load(Q + n0 * D, row0, cn, D, pad);

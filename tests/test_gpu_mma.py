@@ -113,6 +113,22 @@ def test_many_short_bf16_sequences(N, pieces):
             assert not O[b, :, n:].any()
 
 
+@pytest.mark.parametrize("N", [1, 17, 64, 130])
+@pytest.mark.parametrize("B,dtype,phi,D,M", [(56, torch.bfloat16, "elu1", 32, 32), (28, torch.float32, "elu1", 64, 64),
+                                             (28, torch.bfloat16, "identity", 128, 64)])
+def test_a_zero_state_changes_nothing(B, dtype, phi, D, M, N):
+    """A sequence that is trained in pieces may start from a state of zeros: the same results bit for bit as from none
+    (the first rows, whose gradients cancel almost entirely, above all).  One warp per strip: at least 222 CTAs."""
+    dev = [t.to(DEV) for t in draw_qkvg(B, 8, N, D, M, 3 + N, dtype, 1.0)]
+    if phi == "identity":
+        dev[0], dev[1] = dev[0].abs() + 0.1, dev[1].abs() + 0.1
+    state = {"S_in": torch.zeros(B, 8, D, M, device=DEV), "Z_in": torch.zeros(B, 8, D, device=DEV)}
+    plain = (la.la_causal_forward(*dev[:3], phi=phi), *la.la_causal_backward(*dev, phi=phi))
+    from_zero = (la.la_causal_forward(*dev[:3], phi=phi, **state), *la.la_causal_backward(*dev, phi=phi, **state))
+    la.la_last_device_status()
+    assert all(torch.equal(a, b) for a, b in zip(plain, from_zero))
+
+
 @pytest.mark.parametrize("splits", [-1, 1, 3])
 @pytest.mark.parametrize("N", [1, 16, 63, 64, 65, 400])
 @pytest.mark.parametrize("dims", [(8, 8), (32, 32), (40, 24), (64, 64), (72, 64), (128, 64)], ids=str)
