@@ -289,6 +289,8 @@ KERNEL_ALG_BYTES = {
     "causal_bwd_dkv_kernel": lambda d, e: 6 * d * e + 8,        # Q, K, V, G, dn, dl in; dK, dV out
     "linear_apply_kernel": None,                                # three variants share the name: not ranked
 }
+for _tc, _mma in (("fwd", "forward"), ("bwd_dq", "dq"), ("bwd_dkv", "dkv")):       # the same work on mma.sync
+    KERNEL_ALG_BYTES[f"causal_mma_{_mma}_kernel"] = KERNEL_ALG_BYTES[f"causal_{_tc}_kernel"]
 
 
 def bench_attention(la, w, dev, steps, warmup, world, rank, pk, do_e2e=True, from_state=False):
@@ -340,7 +342,7 @@ def bench_attention(la, w, dev, steps, warmup, world, rank, pk, do_e2e=True, fro
         tied = [r for r in ranked if r[0] >= 0.98 * top]
         _, dom, dom_ms = max(tied, key=lambda r: KERNEL_ALG_BYTES[r[1]](w.D, elem_bytes(w)))
         dom_bytes = KERNEL_ALG_BYTES[dom](w.D, elem_bytes(w)) * th
-    else:                       # general kernels: one kernel per call
+    else:                       # no kernel with a byte count of its own (non-causal, general kernels): the longer call as a whole
         dom = ("la_causal_" if w.kind == "causal" else "la_linear_attention_") + ("backward" if bwd_ms >= fwd_ms else "forward")
         dom_ms = max(bwd_ms, fwd_ms)
         dom_bytes = algorithmic_bytes(w, "bwd" if bwd_ms >= fwd_ms else "fwd")

@@ -458,7 +458,9 @@ long long la_kernel_launches(void);
  * la_profile_enable(0) stops recording.  la_profile_read() waits for the recorded events and
  * returns the mean duration in milliseconds and the number of launches of one kernel:
  * 0 causal_fwd_kernel, 1 causal_bwd_dq_kernel, 2 causal_bwd_dkv_kernel, 3 segment_sum_kernel,
- * 4 projection_gemm_kernel, 5 linear_sum_kernel, 6 linear_apply_kernel, 7 recurrent_step_kernel.
+ * 4 projection_gemm_kernel, 5 linear_sum_kernel, 6 linear_apply_kernel, 7 recurrent_step_kernel, and of
+ * the kernels on mma.sync 8 causal_mma_forward_kernel, 9 causal_mma_dq_kernel, 10 causal_mma_dkv_kernel,
+ * 11 causal_mma_sum_kernel (both forms), 12 linear_mma_apply_kernel (three variants).
  * Not thread-safe; meant for a benchmark's single launching thread.
  */
 int la_profile_enable(int on);

@@ -290,11 +290,13 @@ def la_profile_enable(on: bool) -> None:
 def la_profile_read() -> dict:
     """{kernel name: (mean ms per launch, launches)} for every kernel recorded since la_profile_enable(True)."""
     out = {}
-    for k in range(8):
+    k = 0
+    while name := lib().la_profile_kernel_name(k).decode():
         ms, n = ctypes.c_double(), ctypes.c_int()
         _check(lib().la_profile_read(k, ctypes.byref(ms), ctypes.byref(n)))
         if n.value:
-            out[lib().la_profile_kernel_name(k).decode()] = (ms.value, n.value)
+            out[name] = (ms.value, n.value)
+        k += 1
     return out
 
 

@@ -243,7 +243,9 @@ int la_profile_read(int kernel, double* mean_ms, int* launches) {
 const char* la_profile_kernel_name(int kernel) {
     static const char* names[kProfCount] = {"causal_fwd_kernel", "causal_bwd_dq_kernel", "causal_bwd_dkv_kernel",
                                             "segment_sum_kernel", "projection_gemm_kernel", "linear_sum_kernel",
-                                            "linear_apply_kernel", "recurrent_step_kernel"};
+                                            "linear_apply_kernel", "recurrent_step_kernel", "causal_mma_forward_kernel",
+                                            "causal_mma_dq_kernel", "causal_mma_dkv_kernel", "causal_mma_sum_kernel",
+                                            "linear_mma_apply_kernel"};
     return kernel >= 0 && kernel < kProfCount ? names[kernel] : "";
 }
 

@@ -731,20 +731,20 @@ template <typename C, int DP, int MP, bool EXACT> struct Kernels {
         if (a.pieces == 1) return LA_OK;
         const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)(a.pieces - 1);
         if (reverse)
-            return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, true>>(THREADS, bh, y, BUF * SumLayout<C, DP, MP, true>::BYTES, a, st);
-        return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, false>>(THREADS, bh, y, BUF * SumLayout<C, DP, MP, false>::BYTES, a, st);
+            return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, true>>(kProfMmaSum, THREADS, bh, y, BUF * SumLayout<C, DP, MP, true>::BYTES, a, st);
+        return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, false>>(kProfMmaSum, THREADS, bh, y, BUF * SumLayout<C, DP, MP, false>::BYTES, a, st);
     }
     static int forward(const la_problem& p, const Params& a, cudaStream_t st) {
         if (int rc = sums(p, a, false, st)) return rc;
-        return launch<causal_mma_forward_kernel<C, DP, MP, EXACT>>(THREADS, (unsigned)(p.B * p.H), (unsigned)a.pieces,
+        return launch<causal_mma_forward_kernel<C, DP, MP, EXACT>>(kProfMmaForward, THREADS, (unsigned)(p.B * p.H), (unsigned)a.pieces,
                       BUF * ForwardLayout<C, DP, MP>::BYTES, a, st);
     }
     static int backward(const la_problem& p, const Params& fwd, const Params& rev, cudaStream_t st) {
         const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)fwd.pieces;
         if (int rc = sums(p, fwd, false, st)) return rc;
-        if (int rc = launch<causal_mma_dq_kernel<C, DP, MP, EXACT>>(THREADS, bh, y, BUF * DqLayout<C, DP, MP>::BYTES, fwd, st)) return rc;
+        if (int rc = launch<causal_mma_dq_kernel<C, DP, MP, EXACT>>(kProfMmaDq, THREADS, bh, y, BUF * DqLayout<C, DP, MP>::BYTES, fwd, st)) return rc;
         if (int rc = sums(p, rev, true, st)) return rc;
-        return launch<causal_mma_dkv_kernel<C, DP, MP, EXACT>>(THREADS, bh, y, BUF * DkvLayout<C, DP, MP>::BYTES, rev, st);
+        return launch<causal_mma_dkv_kernel<C, DP, MP, EXACT>>(kProfMmaDkv, THREADS, bh, y, BUF * DkvLayout<C, DP, MP>::BYTES, rev, st);
     }
 };
 

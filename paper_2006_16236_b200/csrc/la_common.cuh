@@ -44,7 +44,8 @@ void note_launch();
 // Indices are part of the C ABI (la_profile_read); no-ops unless profiling is switched on.
 enum ProfKernel {
     kProfCausalFwd = 0, kProfCausalBwdDq = 1, kProfCausalBwdDkv = 2, kProfSegmentSum = 3, kProfProjection = 4,
-    kProfLinearSum = 5, kProfLinearApply = 6, kProfRecurrent = 7, kProfCount = 8
+    kProfLinearSum = 5, kProfLinearApply = 6, kProfRecurrent = 7, kProfMmaForward = 8, kProfMmaDq = 9, kProfMmaDkv = 10,
+    kProfMmaSum = 11, kProfMmaApply = 12, kProfCount = 13
 };
 void prof_begin(int kernel, cudaStream_t st);
 void prof_end(int kernel, cudaStream_t st);

@@ -381,7 +381,7 @@ causal_mma_sum_kernel(const Params p) {
 }
 
 template <auto KERNEL>
-inline int launch(int threads, unsigned bh, unsigned y, int smem, const Params& a, cudaStream_t st) {
+inline int launch(ProfKernel prof, int threads, unsigned bh, unsigned y, int smem, const Params& a, cudaStream_t st) {
     static std::atomic<uint64_t> opted_in{0};           // devices on which the kernel may use that much shared memory
     if (smem > 48 * 1024)
         if (int rc = tc::opt_in_smem_once(KERNEL, (uint32_t)smem, opted_in)) return rc;
@@ -395,8 +395,10 @@ inline int launch(int threads, unsigned bh, unsigned y, int smem, const Params& 
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = a.chained ? 1 : 0;
+    prof_begin(prof, st);
     LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, KERNEL, a));
     note_launch();
+    prof_end(prof, st);
     return LA_OK;
 }
 

@@ -129,6 +129,26 @@ def test_a_zero_state_changes_nothing(B, dtype, phi, D, M, N):
     assert all(torch.equal(a, b) for a, b in zip(plain, from_zero))
 
 
+def test_every_launch_can_be_profiled():
+    """la_profile_enable() brackets every main kernel, these ones included."""
+    dev = [t.to(DEV) for t in draw_qkvg(56, 8, 96, 32, 32, 1, torch.bfloat16, 1.0)]
+    f32 = [t[:2].float().contiguous() for t in dev]
+    la.la_plan_override(2, -1, -1)
+    want = {"causal_mma_forward_kernel": 2, "causal_mma_dq_kernel": 1, "causal_mma_dkv_kernel": 1, "causal_mma_sum_kernel": 6,
+            "linear_mma_apply_kernel": 3}
+    la.la_profile_enable(True)
+    try:
+        la.la_causal_forward(*dev[:3])          # two pieces: sums, forward
+        la.la_causal_backward(*dev)             # sums, dQ, reverse sums, dK and dV
+        la.la_causal_forward(*f32[:3], ws=torch.empty(0, dtype=torch.uint8, device=DEV))        # no room for pieces: one kernel
+        la.la_linear_attention(*f32[:3])
+        la.la_linear_attention_backward(*f32, saved=None)
+        got = {k: n for k, (_, n) in la.la_profile_read().items()}
+    finally:
+        la.la_profile_enable(False)
+    assert got == want
+
+
 @pytest.mark.parametrize("splits", [-1, 1, 3])
 @pytest.mark.parametrize("N", [1, 16, 63, 64, 65, 400])
 @pytest.mark.parametrize("dims", [(8, 8), (32, 32), (40, 24), (64, 64), (72, 64), (128, 64)], ids=str)
