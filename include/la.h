@@ -27,6 +27,10 @@
  *    positions is handled as padding); every other problem with M <= 64 runs
  *    on tensor-core kernels that keep fp32 accuracy (products of numbers split
  *    into bf16 parts), everything else on the general fp32-arithmetic kernels; results agree within the rounding of the I/O type.
+ *    Finite numbers keep their value on these kernels; an infinity in Q, K, V or G acts like a NaN
+ *    (its products with split numbers are sums of infinities of both signs), so that results that
+ *    fp32 arithmetic would make infinite may be NaN.  Rows that a length excludes are never read.
+ *    Features of -Inf keys and queries under LA_PHI_ELU1 are zero as everywhere.
  *    The fp32-accurate causal forward takes ws as an option: with less than
  *    la_workspace_bytes() (or NULL) it does not cut sequences into pieces.
  *  - Return value: LA_OK (0) or a negative la_status.  All argument checks run

@@ -96,10 +96,18 @@ __device__ __forceinline__ uint32_t pack_rn(float x, float y) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(y), "f"(x));
     return r;
 }
+__device__ __forceinline__ uint32_t pack_rn_finite(float x, float y) {        // numbers beyond the largest bf16 become that
+    uint32_t r;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(y), "f"(x));
+    return r;
+}
 template <int NP>
 __device__ __forceinline__ void split2(float x, float y, uint32_t (&p)[NP]) {
-    p[0] = pack_rn(x, y);
-    if constexpr (NP == 3) {
+    if constexpr (NP == 1) {
+        p[0] = pack_rn(x, y);
+    } else {
+        // (finite: an fp32 number above 3.39e38 keeps its value, the rest of it in plane 1; an infinity becomes a NaN)
+        p[0] = pack_rn_finite(x, y);
         // (both differences are exact; the rounding of plane 0 leaves planes 1 and 2 with a sign of their own, so
         // that the dropped partial products have no common sign and truncating them costs no bias)
         const float rx = x - __uint_as_float(p[0] << 16), ry = y - __uint_as_float(p[0] & 0xffff0000u);

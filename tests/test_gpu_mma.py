@@ -129,6 +129,26 @@ def test_a_zero_state_changes_nothing(B, dtype, phi, D, M, N):
     assert all(torch.equal(a, b) for a, b in zip(plain, from_zero))
 
 
+@pytest.mark.parametrize("D,M", [(32, 32), (64, 64), (72, 40)])
+def test_the_largest_numbers_keep_their_value(D, M):
+    """fp32 numbers above the largest bf16 (3.39e38) are finite and stay what they are; keys of minus infinity have no
+    weight, whatever finite values lie beside them."""
+    B, H, N = 2, 2, 70
+    g = torch.Generator().manual_seed(4)
+    top = torch.finfo(torch.float32).max
+    K = torch.full((B, H, N, D), -torch.inf)
+    K[:, :, ::7] = torch.rand((B, H, 10, D), generator=g) - 8          # ten keys, weights that add up to less than one
+    Q = torch.rand((B, H, N, D), generator=g) - 6
+    V = top * (1 - torch.rand((B, H, N, M), generator=g) * 2 ** -10) * 2.0 ** -torch.randint(0, 3, (1, H, 1, M), generator=g)
+    q, k, v = (t.double().numpy() for t in (Q, K, V))
+    dev = [t.to(DEV) for t in (Q, K, V)]
+    for causal, call in ((True, la.la_causal_forward), (False, la.la_linear_attention)):
+        O = call(*dev)
+        la.la_last_device_status()
+        assert torch.isfinite(O).all()
+        _close(O, oracle.linear_attention(q, k, v, causal=causal)[0], 2e-6, f"O {causal}")
+
+
 def test_every_launch_can_be_profiled():
     """la_profile_enable() brackets every main kernel, these ones included."""
     dev = [t.to(DEV) for t in draw_qkvg(56, 8, 96, 32, 32, 1, torch.bfloat16, 1.0)]
