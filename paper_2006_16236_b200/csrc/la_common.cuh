@@ -62,6 +62,12 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
     return __float2bfloat16_rn(x);
 }
 
+// What an earlier kernel of the stream may have written, read by a kernel that can start as a programmatic dependent: an
+// ordinary load, not __ldg.  Such a kernel is resident while the one before it still writes, and the read-only path asks
+// for data that nobody writes while the kernel runs (the compiler may move such a load ahead of griddepcontrol.wait).
+// For the same reason the pointers have no __restrict__ next to their const.
+template <typename T> __device__ __forceinline__ T load_global(const T* p) { return *p; }
+
 // ---- feature map, Eq. 7 ------------------------------------------------------
 // phi(x) = x + 1 for x > 0, exp(x) otherwise; identity mode passes x through.
 __device__ __forceinline__ float phi_apply(float x, int phi) {

@@ -132,6 +132,10 @@ projection_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
         const __nv_bfloat16* res = prm.res ? prm.res + (int64_t)row * prm.out_cols + n0 % prm.out_cols : nullptr;
         #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
+            uint4 r[4];                 // the residual, requested ahead of the accumulator
+#pragma unroll
+            for (int cc = 0; cc < 4; ++cc)
+                r[cc] = res && row < prm.rows ? load_global(reinterpret_cast<const uint4*>(res + h * 32 + cc * 8)) : make_uint4(0u, 0u, 0u, 0u);
             uint32_t v[32];
             tmem_ld32(tmem + lane_base + h * 32, v);
             tmem_ld_wait();
@@ -140,8 +144,7 @@ projection_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
                 for (int cc = 0; cc < 4; ++cc) {
                     float add[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                     if (res) {
-                        const uint4 r = __ldg(reinterpret_cast<const uint4*>(res + h * 32 + cc * 8));
-                        const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
+                        const uint32_t rw[4] = {r[cc].x, r[cc].y, r[cc].z, r[cc].w};
 #pragma unroll
                         for (int j = 0; j < 4; ++j) { add[2 * j] = bf16_lo(rw[j]); add[2 * j + 1] = bf16_hi(rw[j]); }
                     }

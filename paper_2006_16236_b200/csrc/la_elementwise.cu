@@ -282,7 +282,7 @@ int launch_poly2_map_backward(const void* x, const void* dy, void* dx, int64_t r
 // is all the traffic of this kernel, streams in while that projection runs.
 template <typename T, int D, int M, bool kEarlyState = false>
 __global__ void __launch_bounds__(128)
-recurrent_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
+recurrent_step_kernel(const T* q, const T* k, const T* v,       // (written by the kernel in front, see load_global())
                       float* __restrict__ S, float* __restrict__ Z, T* __restrict__ out,
                       float eps, int phi) {
     constexpr int TPR = M / 4;        // threads per state row (one float4 each)
@@ -309,6 +309,16 @@ recurrent_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T*
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // All loads of the step in one batch, the vectors ahead of the state, which takes longest and is wanted last: B256 H8
+    // D64 11.2 us a step; with q, k, Z and v loaded where they are used, behind the state's loads, 14.1.
+    T kx = from_f32<T>(0.f), qx = kx, vx = kx;
+    float zx = 0.f;
+    if (tid < D) {
+        kx = k[bh * D + tid];
+        qx = q[bh * D + tid];
+        zx = Z[bh * D + tid];
+    }
+    if (tid < M) vx = v[bh * M + tid];
     if (!kEarlyState) {
 #pragma unroll
         for (int p = 0; p < PASSES; ++p) s[p] = Sp[(r0 + p * RPP) * TPR + c4];
@@ -316,15 +326,15 @@ recurrent_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T*
 
     float zq = 0.f;
     if (tid < D) {
-        float kd = phi_apply(to_f32<T>(k[bh * D + tid]), phi);
-        float qd = phi_apply(to_f32<T>(q[bh * D + tid]), phi);
-        float z = Z[bh * D + tid] + kd;
+        float kd = phi_apply(to_f32<T>(kx), phi);
+        float qd = phi_apply(to_f32<T>(qx), phi);
+        float z = zx + kd;
         Z[bh * D + tid] = z;
         sk[tid] = kd;
         sq[tid] = qd;
         zq = qd * z;
     }
-    if (tid < M) sv[tid] = to_f32<T>(v[bh * M + tid]);
+    if (tid < M) sv[tid] = to_f32<T>(vx);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) zq += __shfl_xor_sync(0xffffffffu, zq, off);
     if (lane == 0) sden[warp] = zq;

@@ -184,7 +184,7 @@ causal_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
         int want[kPlanStampInts];
         plan_stamp(plan, prm.dim, want);
 #pragma unroll
-        for (int i = 0; i < kPlanStampInts; ++i) mismatch = mismatch || __ldg(prm.stamp + i) != want[i];
+        for (int i = 0; i < kPlanStampInts; ++i) mismatch |= load_global(prm.stamp + i) != want[i];
     }
 
     if (mismatch) {             // the same for every thread: nothing is started, the CTA leaves through the common exit
@@ -813,8 +813,8 @@ causal_bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
             const int s = i % kKvStages;
             const int64_t row = chunk_row(i) + t;
             const bool pad = kVarlen && i == 0 && t >= tail_rows;       // (a padded row may lie past the sequence's N)
-            const float inv = pad ? 1.f : 1.f / __ldg(prm.dn + row);
-            const float delta = pad ? 0.f : __ldg(prm.dl + row);
+            const float inv = pad ? 1.f : 1.f / load_global(prm.dn + row);
+            const float delta = pad ? 0.f : load_global(prm.dl + row);
             if (!mbar_wait(&bars->full[s], (i / kKvStages) & 1, prm.status, kStatusTmaTimeout)) { *abort_flag = 1; break; }
             if (*abort_flag) break;
             if (t == 0) LA_TRACE(g_trace_dkv, i, 5);

@@ -424,7 +424,7 @@ __device__ __forceinline__ void sum_records16(const float* rec, int part_lo, int
                                               const float* base = nullptr) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {      // `base` (16 floats, 16-byte aligned, or null): the value the sum starts from
-        const float4 b = base ? __ldg(reinterpret_cast<const float4*>(base) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 b = base ? load_global(reinterpret_cast<const float4*>(base) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
         acc[4 * j] = b.x; acc[4 * j + 1] = b.y; acc[4 * j + 2] = b.z; acc[4 * j + 3] = b.w;
     }
 #pragma unroll 1
@@ -435,7 +435,7 @@ __device__ __forceinline__ void sum_records16(const float* rec, int part_lo, int
             const bool on = p + u < part_hi;
             const float4* src = reinterpret_cast<const float4*>(rec + (int64_t)(on ? p + u : p) * kStateFloats + offset);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) a[u][j] = on ? __ldg(src + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int j = 0; j < 4; ++j) a[u][j] = on ? load_global(src + j) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -452,7 +452,7 @@ __device__ __forceinline__ float sum_records1(const float* rec, int part_lo, int
     for (int p = part_lo; p < part_hi; p += 4) {
         float a[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) a[u] = p + u < part_hi ? __ldg(rec + (int64_t)(p + u) * kStateFloats + offset) : 0.f;
+        for (int u = 0; u < 4; ++u) a[u] = p + u < part_hi ? load_global(rec + (int64_t)(p + u) * kStateFloats + offset) : 0.f;
 #pragma unroll
         for (int u = 0; u < 4; ++u) z += a[u];
     }
@@ -486,7 +486,7 @@ __device__ __forceinline__ void state_init(uint32_t tmem_state, int quad, int la
                        sm100::pack_bf16x2(acc[cc * 8 + 4], acc[cc * 8 + 5]), sm100::pack_bf16x2(acc[cc * 8 + 6], acc[cc * 8 + 7]));
         }
     }
-    const float z = (owner ? sum_records1(rec, part_lo, part_hi, kDim * kDim + d_row) : 0.f) + (in_row ? __ldg(z_in + d_row) : 0.f);
+    const float z = (owner ? sum_records1(rec, part_lo, part_hi, kDim * kDim + d_row) : 0.f) + (in_row ? load_global(z_in + d_row) : 0.f);
     uint32_t zz[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) zz[j] = __float_as_uint(z);
@@ -596,9 +596,9 @@ __device__ __noinline__ void state_add_given(uint32_t tmem_state, int quad, int 
     float4 given[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-        given[j] = (in_row && s_in && j * 4 < dim) ? __ldg(reinterpret_cast<const float4*>(s_in + d_row * dim) + j)
+        given[j] = (in_row && s_in && j * 4 < dim) ? load_global(reinterpret_cast<const float4*>(s_in + d_row * dim) + j)
                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float z_given = (in_row && z_in) ? __ldg(z_in + d_row) : 0.f;
+    const float z_given = (in_row && z_in) ? load_global(z_in + d_row) : 0.f;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         uint32_t v[16];

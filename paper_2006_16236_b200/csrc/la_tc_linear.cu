@@ -441,7 +441,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
                 for (int u = 0; u < kPer; ++u) {        // independent loads: all in flight together
                     const int idx = tid + u * kApThreads;
                     if (idx < kDim * kDim / 4) {
-                        const float4 a = __ldg(src + idx);
+                        const float4 a = load_global(src + idx);
                         acc[u].x += a.x; acc[u].y += a.y; acc[u].z += a.z; acc[u].w += a.w;
                     }
                 }
@@ -454,7 +454,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         }
         if (tid < 2 * kDim + 1) {       // a' (64), ysum (64), w0 (1)
             float z = 0.f;
-            for (int n = 0; n < prm.nseg; ++n) z += __ldg(rec + (int64_t)n * kRecFloats + kDim * kDim + tid);
+            for (int n = 0; n < prm.nseg; ++n) z += load_global(rec + (int64_t)n * kRecFloats + kDim * kDim + tid);
             if (tid < kDim) sA[tid] = z;
             else if (tid < 2 * kDim) sNu[tid - kDim] = z;
             else sScal[1] = z;

@@ -184,8 +184,8 @@ segment_sum_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
             const bool pad = kVarlen && c == L - 1 && t >= span.tail_rows;      // (a padded row may lie past the sequence's N)
             float inv = 1.f, delta = 0.f;
             if (scaled && !pad) {
-                inv = 1.f / __ldg(prm.dn + row);
-                delta = __ldg(prm.dl + row);
+                inv = 1.f / load_global(prm.dn + row);
+                delta = load_global(prm.dl + row);
             }
             if (!mbar_wait(&bars->full[s], (c / kSumStages) & 1, prm.status, kStatusTmaTimeout)) { *abort_flag = 1; break; }
             if (*abort_flag) break;

@@ -17,6 +17,24 @@ def _code(name):
     return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
 
 
-@pytest.mark.parametrize("name", ["la_mma.cuh", "la_mma_sweep.cuh", "la_causal_mma.cu", "la_linear_mma.cu"])
+READ_ONLY = r"__ldg\s*\(|ld\.global\.nc|const \w+\s*\*\s*__restrict__"
+
+
+@pytest.mark.parametrize("name", ["la_mma.cuh", "la_mma_sweep.cuh", "la_causal_mma.cu", "la_linear_mma.cu", "la_tc_common.cuh",
+                                  "la_tc_causal_fwd.cu", "la_tc_causal_bwd.cu", "la_tc_segment.cu", "la_tc_linear.cu",
+                                  "la_decode_layer.cu", "la_sm100.cuh"])
 def test_no_read_only_loads(name):
-    assert not re.findall(r"__ldg\s*\(|ld\.global\.nc|__restrict__", _code(name))
+    assert not re.findall(READ_ONLY, _code(name))
+
+
+def test_the_chained_kernel_of_the_elementwise_file():
+    code = _code("la_elementwise.cu")
+    kernels = {re.search(r"(\w+_kernel)\(", k).group(1): k for k in code.split("__global__")[1:]}
+    chained = [n for n, k in kernels.items() if "griddepcontrol.wait" in k]
+    assert chained == ["recurrent_step_kernel"]
+    assert not re.findall(READ_ONLY, kernels[chained[0]].split("template")[0])
+
+
+def test_no_other_file_launches_programmatic_dependents():
+    known = {"la_mma_sweep.cuh", "la_tc_common.cuh", "la_elementwise.cu"}       # where the launch attribute is set
+    assert {n for n in os.listdir(CSRC) if "ProgrammaticStreamSerialization" in _code(n)} == known
