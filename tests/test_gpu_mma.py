@@ -113,6 +113,56 @@ def test_many_short_bf16_sequences(N, pieces):
             assert not O[b, :, n:].any()
 
 
+@pytest.mark.parametrize("pieces", [1, 3])
+@pytest.mark.parametrize("N", [1, 63, 65, 200])
+@pytest.mark.parametrize("B,dtype,phi,D,M", [(28, torch.float32, "elu1", 64, 64), (28, torch.bfloat16, "identity", 128, 64),
+                                             (56, torch.bfloat16, "elu1", 32, 32)])
+def test_one_warp_per_strip(B, dtype, phi, D, M, N, pieces):
+    """The kernels of full grids (at least 222 CTAs; the last ones also of many short sequences): short last chunks, whole and
+    cut into pieces, ragged, from a state and with state gradients, against the oracle on sampled heads.  Tolerances as above,
+    8e-6 also for the fp32 state gradients; single planes are held to the bf16 gates."""
+    H, eps = 8, 0.5 if N % 2 else 0.0
+    Q, K, V, G = draw_qkvg(B, H, N, D, M, 7 + N, dtype, 1.0)
+    if phi == "identity":
+        Q, K = Q.abs() + 0.1, K.abs() + 0.1
+    g = torch.Generator().manual_seed(N)
+    S0, Z0 = torch.randn((B, H, D, M), generator=g), torch.rand((B, H, D), generator=g) * 4 + 1
+    dS, dZ = torch.randn((B, H, D, M), generator=g) * 0.05, torch.randn((B, H, D), generator=g) * 0.05
+    lengths = [N - (7 * b) % (N + 1) for b in range(B)]
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    S0d, Z0d, dSd, dZd = (t.to(DEV) for t in (S0, Z0, dS, dZ))
+    la.la_plan_override(pieces)
+
+    def check(x, ref, what, state=False):
+        if D == 32:
+            assert_close(x, ref, dtype, what, grad=True)
+        else:
+            tight = dtype == torch.float32 or state
+            _close(x, ref, (8e-6 if what[0] == "d" else 2e-6) if tight else 2 ** -8, what)
+
+    for ln in (None, torch.tensor(lengths, dtype=torch.int32, device=DEV)):
+        S1, Z1, dS0, dZ0 = (torch.empty_like(t) for t in (S0d, Z0d, S0d, Z0d))
+        kw = {"phi": phi, "eps": eps, "lengths": ln, "S_in": S0d, "Z_in": Z0d}
+        O = la.la_causal_forward(*dev[:3], S_out=S1, Z_out=Z1, **kw)
+        grads = la.la_causal_backward(*dev, dS_out=dSd, dZ_out=dZd, dS_in=dS0, dZ_in=dZ0, **kw)
+        la.la_last_device_status()
+        for b in (0, 1, 10, B - 1):
+            n = N if ln is None else lengths[b]
+            assert not O[b, :, n:].any() and not any(x[b, :, n:].any() for x in grads)
+            hs = (slice(b, b + 1), slice(0, H, 7))
+            sl = (*hs, slice(0, n))
+            q, k, v, gg = (t[sl].double().numpy() for t in (Q, K, V, G))
+            st = [t[hs].double().numpy() for t in (S0, Z0, dS, dZ)]
+            Or, _, Sr, Zr = oracle.causal_from_state(q, k, v, st[0], st[1], phi, eps)
+            rq, rk, rv, rS, rZ = oracle.causal_backward_from_state(q, k, v, st[0], st[1], gg, st[2], st[3], phi, eps)
+            check(S1[hs], Sr, "S_out", True), check(Z1[hs], Zr, "Z_out", True)
+            check(dS0[hs], rS, "dS_in", True), check(dZ0[hs], rZ, "dZ_in", True)
+            if n:
+                check(O[sl], Or, "O")
+                for nm, x, ref in zip(("dQ", "dK", "dV"), grads, (rq, rk, rv)):
+                    check(x[sl], ref, nm)
+
+
 @pytest.mark.parametrize("N", [1, 17, 64, 130])
 @pytest.mark.parametrize("B,dtype,phi,D,M", [(56, torch.bfloat16, "elu1", 32, 32), (28, torch.float32, "elu1", 64, 64),
                                              (28, torch.bfloat16, "identity", 128, 64)])

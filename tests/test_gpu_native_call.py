@@ -97,3 +97,45 @@ def test_an_allocation_that_fails_is_an_out_of_memory_error():
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert torch.isfinite(la.la_causal_forward(Q, Q, Q)).all()
+
+
+class _Sub(torch.Tensor):
+    pass
+
+
+def test_what_is_not_ordinary_goes_to_the_python_code():
+    """A tensor subclass, an active function mode: the native functions decline, nothing done, and the call still works."""
+    from torch.overrides import TorchFunctionMode
+
+    class Mode(TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            return func(*args, **(kwargs or {}))
+
+    Q = torch.randn(1, 2, 40, 32, device=DEV)
+    want = la.la_causal_forward(Q, Q, Q)
+    native = lambda q: binding._native().linear_forward(q, q, q, "elu1", 0.0, None, None, None, None, None, None, None, {})
+    launches = la.la_kernel_launches()
+    assert native(Q.as_subclass(_Sub)) is NotImplemented
+    with Mode():
+        assert native(Q) is NotImplemented
+    assert native(Q[:, :, ::2]) is NotImplemented and native(Q.half()) is NotImplemented and native(Q.cpu()) is NotImplemented
+    assert la.la_kernel_launches() == launches
+    assert torch.equal(la.la_causal_forward(Q.as_subclass(_Sub), Q, Q), want)
+    with Mode():
+        assert torch.equal(la.la_causal_forward(Q, Q, Q), want)
+
+
+def test_the_current_stream_is_the_one_that_runs():
+    """The call is enqueued on the stream that is current, behind what is already there, and on no other."""
+    Q = torch.randn(1, 2, 300, 32, device=DEV)
+    want = la.la_causal_forward(Q, Q, Q)
+    side, q, O = torch.cuda.Stream(), torch.zeros_like(Q), torch.empty_like(Q)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)           # about 10 ms
+        q.copy_(Q)
+        la.la_causal_forward(q, q, q, O=O)
+        assert not side.query()
+    assert torch.cuda.default_stream().query()
+    side.synchronize()
+    assert torch.equal(O, want)

@@ -186,10 +186,11 @@ def test_noncausal_backward_refuses_kept_sums_of_another_plan(plan_override, dty
         assert_close(x, ref, dtype, nm, grad=True)
 
 
+@pytest.mark.parametrize("M", [16, 80])        # fp32-accurate mma.sync kernels; general kernels
 @pytest.mark.parametrize("causal", [True, False])
 @pytest.mark.parametrize("dtype", DTYPES)
-def test_eps_and_identity_feature_map(causal, dtype):
-    B, H, N, D, M = 2, 2, 96, 32, 16
+def test_eps_and_identity_feature_map(causal, dtype, M):
+    B, H, N, D = 2, 2, 96, 32
     Q, K, V, G = draw_qkvg(B, H, N, D, M, seed=77, dtype=torch.float32)
     Q, K = (Q.abs() + 0.1).to(dtype), (K.abs() + 0.1).to(dtype)      # already "feature-mapped"
     V, G = V.to(dtype), G.to(dtype)
@@ -270,10 +271,10 @@ def test_prefill_then_decode_handoff():
 
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("shape", [(2, 3, 100, 16, 48), (1, 2, 31, 64, 64), (2, 2, 640, 32, 32), (1, 4, 384, 64, 64),
-                                   (4, 16, 18 * 128, 64, 64), (2, 8, 1000, 64, 64)])
+                                   (4, 16, 18 * 128, 64, 64), (2, 8, 1000, 64, 64), (2, 3, 100, 40, 72), (1, 2, 65, 128, 96)])
 def test_causal_forward_from_a_state(shape, dtype):
-    """The recurrence of Eq. 16-20 started from a given S_0, Z_0 (general kernels and, for bf16 D = M in
-    {32, 64}, the tensor-core kernel, with several pieces per sequence at the larger shapes)."""
+    """The recurrence of Eq. 16-20 started from a given S_0, Z_0 (bf16 D = M in {32, 64}: tcgen05 kernel, with several
+    pieces per sequence at the larger shapes; other M <= 64: mma.sync kernels; M > 64: general kernels)."""
     B, H, N, D, M = shape
     Q, K, V, _ = draw_qkvg(B, H, N, D, M, seed=sum(shape) + 1, dtype=dtype, with_grad=False)
     g = torch.Generator().manual_seed(5)
@@ -323,7 +324,7 @@ def test_chunked_prefill_then_decode(dtype, D, chunks):
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("keep", [False, True], ids=["recompute", "saved"])
 @pytest.mark.parametrize("shape", [(2, 3, 100, 16, 48), (1, 2, 31, 64, 64), (2, 2, 640, 32, 32), (4, 16, 18 * 128, 64, 64),
-                                   (2, 8, 1000, 64, 64)])
+                                   (2, 8, 1000, 64, 64), (2, 3, 100, 40, 72), (1, 2, 65, 128, 96)])
 def test_causal_backward_from_a_state(shape, keep, dtype):
     """Algorithm 1 (backward) with the forward sum started from [S_0 | Z_0] and the reverse sum from an upstream
     gradient of the final state; the gradient of the initial state is what the reverse sum ends with."""
@@ -339,7 +340,7 @@ def test_causal_backward_from_a_state(shape, keep, dtype):
     dZ0 = torch.empty((B, H, D), device=DEV)
     saved = la.saved_buffer(Qd, Vd) if keep else None
     if keep and saved is None:
-        pytest.skip("no saved buffer for problems on the general kernels")
+        pytest.skip("no saved buffer for problems off the tcgen05 kernels")
     if keep:
         la.la_causal_forward(Qd, Kd, Vd, S_in=S0d, Z_in=Z0d, saved=saved)
     dQ, dK, dV = la.la_causal_backward(Qd, Kd, Vd, Gd, saved=saved, S_in=S0d, Z_in=Z0d, dS_out=dSNd, dZ_out=dZNd,
@@ -409,7 +410,8 @@ def test_right_padded_causal_batches_need_no_mask(dtype, D, N):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
-@pytest.mark.parametrize("shape,lengths", [((3, 2, 100, 16, 48), [100, 37, 1]), ((4, 2, 517, 64, 64), [517, 0, 300, 129]),
+@pytest.mark.parametrize("shape,lengths", [((3, 2, 100, 16, 48), [100, 37, 1]), ((3, 2, 100, 40, 72), [100, 37, 1]),
+                                           ((4, 2, 300, 128, 96), [300, 0, 131, 128]), ((4, 2, 517, 64, 64), [517, 0, 300, 129]),
                                            ((2, 4, 1024, 64, 64), [1024, 700]),
                                            ((5, 2, 2048, 64, 64), [2048, 0, 129, 1500, 1024]),
                                            ((3, 2, 512, 32, 32), [512, 130, 1])])
@@ -417,7 +419,8 @@ def test_noncausal_ragged_batches(shape, lengths, dtype):
     """Right-padded sequences of different lengths (key-padding mask): every sequence equals the oracle run on
     its own length, sums included, and everything is zero on the padding whatever the tensors hold there
     (not even numbers).  The bf16 cases with D = M in {32, 64} run the tensor-core
-    kernels, whose splits end inside, at and before a sequence's end; the others the general kernels."""
+    kernels, whose splits end inside, at and before a sequence's end; those with M > 64 the general kernels, the others the
+    fp32-accurate mma.sync kernels."""
     B, H, N, D, M = shape
     Q, K, V, G = draw_qkvg(B, H, N, D, M, seed=sum(shape) + 4, dtype=dtype)
     for b, n in enumerate(lengths):
@@ -553,14 +556,14 @@ def test_rff_attention_end_to_end(causal):
 def test_poly2_attention_end_to_end(shape, signed, causal, dtype):
     """Queries and keys -> features on the device -> attention with the identity map; gradients through both
     steps.  D = 8 gives C = 64: in bf16 the tensor-core kernels; D = 5 (C = 25 padded to 32, M = 24) the
-    general ones.  The features are a stored tensor of the I/O type: the device's must equal the oracle's,
+    fp32-accurate mma.sync ones.  The features are a stored tensor of the I/O type: the device's must equal the oracle's,
     rounded once, bit for bit, and the attention step is judged on those, like every other input.  Against the
     exact kernel (q.k)^2 on the N x N matrix the fp32 path meets the fp32 gate; in bf16 the 2^-9 rounding
     of each stored feature is what remains (a weight (q.k)^2 is a sum of D^2 products that cancel), which
     no kernel downstream can remove: only a loose bound is asserted there.
     Signed queries and keys give signed features, and a weight that is small against the products it sums
-    (the first causal rows above all).  The general kernels (fp32 arithmetic) hold the usual gates there; the
-    tensor-core kernels round scores and state to bf16, an error relative to the products and not to their
+    (the first causal rows above all).  The kernels at fp32 accuracy hold the usual gates there; the
+    tcgen05 kernels round scores and state to bf16, an error relative to the products and not to their
     sum: for signed features in bf16 they are held to 0.15, and to the usual gates for features of one sign."""
     B, H, N, D, M = shape
     Q, K, V, G = draw_qkvg(B, H, N, D, M, seed=sum(shape) + causal, dtype=dtype)
@@ -634,7 +637,7 @@ def test_causal_workloads_full_size(name, keep):
     den = torch.empty((w.B, w.H, w.N), device=DEV)
     saved = la.saved_buffer(Qd, Vd) if keep else None      # what a training step keeps for the backward pass
     if keep and saved is None:
-        pytest.skip("this problem runs the general kernels, which keep nothing")
+        pytest.skip("this problem does not run the tcgen05 kernels: nothing is kept")
     O = la.la_causal_forward(Qd, Kd, Vd, den=den, saved=saved)
     dQ, dK, dV = la.la_causal_backward(Qd, Kd, Vd, Gd, O=O, den=den, saved=saved)
     la.la_last_device_status()
@@ -721,10 +724,11 @@ def test_noncausal_workload_full_size():
 
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("shape,lengths", [((2, 3, 512, 64, 64), None), ((3, 2, 1024, 64, 64), [1024, 130, 700]),
-                                           ((2, 2, 200, 16, 24), None), ((2, 2, 200, 16, 24), [200, 77])])
+                                           ((2, 2, 200, 16, 24), None), ((2, 2, 200, 16, 24), [200, 77]),
+                                           ((2, 2, 200, 128, 96), None), ((2, 2, 200, 40, 72), [200, 77])])
 def test_noncausal_saved_sums_give_identical_results(shape, lengths, dtype):
     """What the non-causal forward keeps for the backward pass (the per-split sums over the keys) changes no bit
-    of either call's results, on the tensor-core and on the general kernels, full-length and ragged; and the
+    of either call's results, on the tensor-core and (M > 64) on the general kernels, full-length and ragged; and the
     forward leaves its workspace alone when it is given a saved buffer."""
     B, H, N, D, M = shape
     Q, K, V, G = gpu(*draw_qkvg(B, H, N, D, M, seed=sum(shape) + 9, dtype=dtype))
@@ -866,7 +870,8 @@ def _poison_padding(tensors, lengths):
 
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("shape,lengths", [
-    ((4, 2, 100, 16, 48), [100, 37, 1, 0]),                       # general kernels, ragged chunk tails
+    ((4, 2, 100, 16, 48), [100, 37, 1, 0]),                       # mma.sync kernels, ragged chunk tails
+    ((4, 2, 100, 40, 72), [100, 37, 1, 0]),                       # general kernels, the same
     ((3, 2, 384, 64, 64), [384, 129, 300]),                       # bf16: the tensor-core shapes
     ((6, 4, 1024, 64, 64), [1024, 0, 1, 128, 641, 900]),          # whole chunks, a chunk boundary, nothing at all
     ((2, 32, 2304, 64, 64), [2304, 1000]),                        # B*H = 64: sequences cut into pieces with a pre-pass
@@ -921,16 +926,17 @@ def test_causal_ragged_batches(shape, lengths, dtype):
         assert_close(out1[sl], oracle.attention_quadratic(*longer, True)[:, :, n], dtype, f"decode after prefill, length {n}")
 
 
-def test_causal_ragged_batch_from_a_state_with_state_gradients():
+@pytest.mark.parametrize("dtype,D,M", [(torch.bfloat16, 64, 64), (torch.float32, 48, 40), (torch.float32, 40, 72),
+                                       (torch.bfloat16, 128, 96)])      # tcgen05, mma.sync, general, general
+def test_causal_ragged_batch_from_a_state_with_state_gradients(dtype, D, M):
     """The ragged calls with every state argument: the sequences continue from S_0, Z_0, the upstream gradient
     of the state at each sequence's own end comes in, the gradient of the initial state goes out."""
-    B, H, N, D = 3, 2, 512, 64
+    B, H, N = 3, 2, 512
     lengths = [512, 200, 77]
-    dtype = torch.bfloat16
-    Q, K, V, G = draw_qkvg(B, H, N, D, D, seed=410, dtype=dtype)
+    Q, K, V, G = draw_qkvg(B, H, N, D, M, seed=410, dtype=dtype)
     g = torch.Generator().manual_seed(411)
-    S0, Z0 = torch.randn((B, H, D, D), generator=g) * 3.0, torch.rand((B, H, D), generator=g) * 4.0 + 1.0
-    dS, dZ = torch.randn((B, H, D, D), generator=g) * 0.05, torch.randn((B, H, D), generator=g) * 0.05
+    S0, Z0 = torch.randn((B, H, D, M), generator=g) * 3.0, torch.rand((B, H, D), generator=g) * 4.0 + 1.0
+    dS, dZ = torch.randn((B, H, D, M), generator=g) * 0.05, torch.randn((B, H, D), generator=g) * 0.05
     Qd, Kd, Vd, Gd, S0d, Z0d, dSd, dZd = gpu(Q, K, V, G, S0, Z0, dS, dZ)
     ln = torch.tensor(lengths, dtype=torch.int32, device=DEV)
     S1, Z1 = torch.empty_like(S0d), torch.empty_like(Z0d)
