@@ -76,9 +76,10 @@ def test_same_errors_and_outputs_in_place():
 
 def test_an_allocation_that_fails_is_an_out_of_memory_error():
     """Outputs and scratch are allocated in native code; a program that catches torch.OutOfMemoryError to go on with a
-    smaller batch has to see that type.  The failure is the allocator's: it is told to hold no more than it already does."""
+    smaller batch has to see that type.  The failure is the allocator's: it is told to hold no more than it already does,
+    and what it keeps free is taken first."""
     n = lambda *s, dt=torch.float32: torch.zeros(s, device=DEV, dtype=dt)
-    Q, Qb = n(1, 8, 65536, 16), n(1, 8, 65536, 64, dt=torch.bfloat16)       # 33 and 67 MB: no block of that size is kept
+    Q, Qb = n(1, 8, 65536, 16), n(1, 8, 65536, 64, dt=torch.bfloat16)       # outputs of 33 MB and more
     q, S, Z = n(32768, 8, 32), n(32768, 8, 32, 32), n(32768, 8, 32)
     x, W, Wo = n(32768, 512, dt=torch.bfloat16), n(1536, 512, dt=torch.bfloat16), n(512, 512, dt=torch.bfloat16)
     Sl, Zl = n(32768, 8, 64, 64), n(32768, 8, 64)
@@ -90,12 +91,17 @@ def test_an_allocation_that_fails_is_an_out_of_memory_error():
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     torch.cuda.set_per_process_memory_fraction(0.0)
+    taken = []
     try:
+        with pytest.raises(torch.OutOfMemoryError):
+            while True:
+                taken.append(torch.empty(Q.nbytes, dtype=torch.uint8, device=DEV))
         for call in calls:
             with pytest.raises(torch.OutOfMemoryError):
                 call()
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
+    del taken
     assert torch.isfinite(la.la_causal_forward(Q, Q, Q)).all()
 
 
