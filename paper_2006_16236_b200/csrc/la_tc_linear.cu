@@ -42,8 +42,9 @@ namespace {
 //   forward sums (sum kernel)            : A' = sum k'_j V_j^T, a' = sum k'_j, ysum = sum V_j,        w0 unused
 //   reverse sums (backward-Q apply pass) : A' = sum qh'_i G_i^T, a' = sum qh'_i dl_i, ysum = sum G_i / dn_i, w0 = sum dl_i / dn_i
 constexpr int kRecFloats = kDim * kDim + kDim + kDim + 8;
-// The last four words of the first record: the split plan it was written under.  A backward pass that is given kept
-// records and would split the sequences in another way (la_plan_override() in between) reports that and writes nothing.
+// The last four words of a record: the split plan it was written under.  A backward pass that is given kept records and
+// would split the sequences in another way (la_plan_override() in between) reports that and writes nothing.  The CTAs of
+// sequence i look at record i, which every plan has: all of them at the first one took 0.5 us longer a step.
 constexpr int kRecStamp = kRecFloats - 4;
 __device__ __forceinline__ int4 split_stamp(int nseg, int chunks_per_seg, int dim) {
     return make_int4(0x4c414c53, nseg, chunks_per_seg, dim);
@@ -167,8 +168,9 @@ linear_sum_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     grid_dependency_wait();
     allow_dependent_launch();
     LA_TRACE_CTA(g_trace_lin, 1);
-    if (blockIdx.x == 0 && tid == kLsThreads - 1)
-        *reinterpret_cast<int4*>(prm.records + kRecStamp) = split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
+    if (tid == kLsThreads - 1)
+        *reinterpret_cast<int4*>(prm.records + (bh * prm.nseg + seg) * (int64_t)kRecFloats + kRecStamp) =
+            split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
     // Ragged batch: only `real` rows of this split exist; chunks behind them are skipped and the rows behind
     // them in the last chunk are zeroed after the load (at least one chunk runs, so that the record is written
     // from an accumulator that holds zeros and not from one that was never started).
@@ -421,7 +423,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
     }
     bool mismatch = false;      // (the same for every thread)
     if (kHasY && prm.kept) {
-        const int4 a = *reinterpret_cast<const int4*>(prm.kept + kRecStamp), b = split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
+        const int4 a = *reinterpret_cast<const int4*>(prm.kept + bh * (int64_t)kRecFloats + kRecStamp), b = split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
         mismatch = a.x != b.x || a.y != b.y || a.z != b.z || a.w != b.w;
     }
     // state of this head: add the split records (fp32), remove the column means, round the
