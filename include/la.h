@@ -23,10 +23,13 @@
  *  - Outputs must not alias inputs (S and Z of la_recurrent_step are in-out).
  *  - Supported sizes: D and M multiples of 8 in [8, 128]; B, H >= 1; N >= 0
  *    (N == 0 is a successful no-op).  bf16 problems with D = M in {32, 64} run
- *    on the tensor-core kernels (any N: a last chunk of fewer than 128
- *    positions is handled as padding); every other problem with M <= 64 runs
- *    on tensor-core kernels that keep fp32 accuracy (products of numbers split
- *    into bf16 parts), everything else on the general fp32-arithmetic kernels; results agree within the rounding of the I/O type.
+ *    on the tcgen05 kernels (any N: a last chunk of fewer than 128 positions is
+ *    handled as padding), but causal ones of many short sequences (D = M = 32,
+ *    B*H >= 444, N <= 1024) on mma.sync kernels with bf16 operands; every other
+ *    problem with M <= 64 runs on mma.sync kernels that keep fp32 accuracy
+ *    (products of numbers split into bf16 parts), everything else on the general
+ *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.
+ *    Only the tcgen05 kernels have a la_causal_plan() and a causal saved buffer.
  *    Finite numbers keep their value on these kernels; an infinity in Q, K, V or G acts like a NaN
  *    (its products with split numbers are sums of infinities of both signs), so that results that
  *    fp32 arithmetic would make infinite may be NaN.  Rows that a length excludes are never read.
@@ -212,7 +215,7 @@ int la_linear_attention_backward_kept(const la_problem* p, const void* Q, const 
  * paper's autograd function keeps phi(Q), phi(K): the mapped queries and keys and the
  * per-segment sums of the forward pre-pass.  Its layout is private to the library; it is
  * valid for la_causal_backward() with the same problem, Q, K and V until overwritten.  The
- * size is 0 for problems that run the general kernels (pass NULL, or any pointer).
+ * size is 0 for problems that do not run the tcgen05 kernels (pass NULL, or any pointer).
  */
 int la_causal_forward(const la_problem* p, const void* Q, const void* K, const void* V,
                       void* O, float* den, float* S_out, float* Z_out,
@@ -366,12 +369,12 @@ const char* la_last_error(void);
 int la_last_device_status(void* stream);
 
 /*
- * How the tensor-core causal kernels cut the sequences of problem p (a diagnostic, no counterpart
+ * How the tcgen05 causal kernels cut the sequences of problem p (a diagnostic, no counterpart
  * in the paper; host only, nothing is enqueued).  A sequence of N / 128 chunks is cut into pieces,
  * one CTA of a main kernel each, launched in the order the function reports, so that B*H*pieces
  * CTAs keep all SMs busy; every piece is cut into pre-pass parts whose sums give a piece its
  * starting state.  Writes up to `capacity` 32-bit integers to `out` (host memory) and returns how
- * many the full description has, or 0 when p does not run the tensor-core kernels, or a negative
+ * many the full description has, or 0 when p does not run the tcgen05 kernels, or a negative
  * status:  out = { pieces, parts,
  *                  piece_begin[0..pieces]  (chunk index; piece_begin[pieces] = N / 128),
  *                  piece_first_part[0..pieces],
@@ -383,7 +386,7 @@ int la_causal_plan(const la_problem* p, int32_t* out, int capacity);
 
 /*
  * Overrides of the automatic plans, for A/B checks and tests (no counterpart in the paper; host only).
- * causal_pieces: equal pieces per sequence in the causal kernels; causal_short: length in chunks of the
+ * causal_pieces: equal pieces per sequence in the causal kernels (tcgen05 and mma.sync); causal_short: length in chunks of the
  * short middle piece (0: none); linear_splits: splits per sequence in the non-causal kernels.  -1 leaves a
  * choice automatic; la_plan_override(-1, -1, -1) restores the defaults.  The setting is process-wide and
  * read by every later call, la_workspace_bytes() and la_causal_plan() included: change it only between

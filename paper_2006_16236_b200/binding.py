@@ -108,7 +108,7 @@ _fast = None
 
 def _native():
     """The native code of the ordinary call (csrc/la_fast.cpp): the same checks and the same library call without the
-    interpreter's part of them (la_recurrent_step 15 -> 4 us a call).  Its functions return NotImplemented, with nothing
+    interpreter's part of them (la_recurrent_step 15.3 -> 4.4 us a call).  Its functions return NotImplemented, with nothing
     done, for everything but plain tensors of the right shapes on the current device: the code below each use."""
     global _fast
     if _fast is None:
@@ -238,9 +238,10 @@ def workspace(p: la_problem, op: int, device) -> torch.Tensor | None:
 
 
 def _forward_scratch(p: la_problem, op: int, device) -> torch.Tensor | None:
-    """Scratch of a causal forward call.  The kernels that take bf16 with D = M in {32, 64} share workspace()'s buffer;
-    the others' scratch is optional and was none before, so calls of several streams or threads must not meet in it:
-    it comes from torch's allocator on every call."""
+    """Scratch of a causal forward call (la_fast.cpp does the same).  bf16 calls with D = M in {32, 64} share workspace()'s
+    buffer, whichever kernels they run (the short ones that leave the tcgen05 kernels need none unless a plan override
+    cuts them); the others' scratch is optional, and calls of several streams or threads must not meet in it: it comes
+    from torch's allocator on every call."""
     if p.dtype == LA_BF16 and p.D == p.M and p.D in (32, 64):
         return workspace(p, op, device)
     need = lib().la_workspace_bytes(ctypes.byref(p), op)
@@ -256,8 +257,8 @@ def la_kernel_launches() -> int:
 
 
 def la_causal_plan(p: la_problem):
-    """How the tensor-core causal kernels cut the sequences of p: a dict of plain lists, or None when p runs
-    the general kernels.  Host only."""
+    """How the tcgen05 causal kernels cut the sequences of p: a dict of plain lists, or None when p runs
+    other kernels.  Host only."""
     n = lib().la_causal_plan(ctypes.byref(p), None, 0)
     if n < 0:
         _check(n)

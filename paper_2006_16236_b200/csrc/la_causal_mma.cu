@@ -681,7 +681,8 @@ struct Plan { int pieces; int64_t len; };
 // sums, of which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk.  Forward +
 // backward in us, fp32, D = M = 64, pieces 1 / 2 / 4 / 8 / 16: B1 H8 N1024 466 / 304 / 172 / 123 / 134;
 // B8 H8 N1024 484 / 324 / 245 / 287 / 381; B16 H8 N2048 963 / 815 / 929 / 913 / 1091;
-// B32 H8 N4096 2632 / 3318 / 3219 / 3215 / 3645.
+// B32 H8 N4096 2632 / 3318 / 3219 / 3215 / 3645.  At most sixteen: the estimate is checked up to N = 4096 only (for few
+// sequences much longer than that it would want more), and it knows nothing of the single-plane kernels' four CTAs per SM.
 Plan choose_plan(const la_problem& p, bool single) {
     const int64_t chunks = (p.N + T - 1) / T, bh = p.B * p.H;
     int64_t best = 1;
@@ -748,7 +749,8 @@ template <typename C, int DP, int MP, bool EXACT> struct Kernels {
     }
 };
 
-// Tiles are padded to 32, 64 or (D) 128 columns; EXACT: D and M are those sizes.
+// Tiles are padded to 32, 64 or (D) 128 columns; EXACT: D and M are those sizes.  One warp per strip was measured, and is
+// instantiated, at the exact sizes only; padded ones take two whatever the grid.
 template <typename F> int dispatch(const la_problem& p, int pieces, F f) {
     const bool full = p.B * p.H * pieces >= 222;            // one and a half CTAs per SM and more
     const bool exact = (p.D == 32 || p.D == 64 || p.D == 128) && p.M == (p.D == 32 ? 32 : 64);

@@ -1,6 +1,6 @@
 // la_linear_attention_noalloc: the non-causal forward for callers that cannot allocate.
 //
-// The general non-causal kernels split every (batch, head) sequence over several CTAs
+// The non-causal kernels split every (batch, head) sequence over several CTAs
 // and need scratch memory for the per-split partial sums of phi(K)^T [V | 1].  The
 // regular entry point takes that scratch from the caller.  Some callers have no way to
 // provide it: code running inside a framework's memory-planning phase or under a memory

@@ -90,7 +90,7 @@ def test_causal_plan_of_the_bench_workload(L):
     pb = plan["piece_begin"]
     short = pb[2] - pb[1]
     assert 8 <= short <= 16 and abs((pb[1] - pb[0]) - (pb[3] - pb[2])) <= 1
-    # problems that run the general kernels have no plan
+    # problems off the tcgen05 kernels have no plan
     assert la.la_causal_plan(la.make_problem(1, 2, 256, 32, 32, la.LA_F32)) is None
     assert la.la_causal_plan(la.make_problem(1, 2, 256, 64, 48, la.LA_BF16)) is None
     # a length that is not a multiple of the chunk: the last chunk is partial
@@ -126,7 +126,7 @@ def test_bad_arguments_are_rejected_on_the_host(L):
     args = [ctypes.byref(p), ok, ok, ok, null, null, ok, null, 0, ok, ok, ok]
     assert L.la_causal_backward(*args, null, 0, null) == -3
     assert L.la_causal_backward(*args, ok, need - 1, null) == -3
-    # the optional saved buffer: a short or misaligned one is refused; problems on the general kernels need none
+    # the optional saved buffer: a short or misaligned one is refused; problems off the tcgen05 kernels need none
     pb = _p(dtype_code=binding.LA_BF16, N=256, D=64, M=64)
     keep = la.la_workspace_bytes(pb, binding.LA_OP_CAUSAL_SAVED)
     assert keep >= 2 * 256 * 64 * 2 * pb.B * pb.H
