@@ -136,20 +136,20 @@ causal_mma_forward_kernel(const Params p) {
             else rq.load(Q + n0 * D, cn, D, pad);
             if constexpr (C::BUF == 1) __syncthreads();         // the planes of the chunk before are no longer read
             st.template publish<NS>(buf + Sh::S, sZ, sZp);
-            with_phi<NQ>(phi, [&](auto f) { rk.template store<NQ>(buf + Sh::X, [&](int, float x) { return f(x); }); });
+            rk.template features<NQ>(buf + Sh::X, phi);
             rv.template values<NV>(buf + Sh::Y);
             if constexpr (WPS == 1) {
                 RawStrip<typename FeatureType<NQ>::type, DP> fq;
                 rq.template map<NQ>(phi, fq);
                 fq.template planes<NQ>(q.a);
             } else {
-                with_phi<NQ>(phi, [&](auto f) { rq.template store<NQ>(buf + Sh::R, [&](int, float x) { return f(x); }); });
+                rq.template features<NQ>(buf + Sh::R, phi);
                 q.tile = smem_u32(buf + Sh::R); q.row0 = row0; q.lane = lane;
             }
         }
-        prefetch_rows<THREADS>(Q, n0 + T, r.end, D);
-        prefetch_rows<THREADS>(K, n0 + T, r.end, D);
-        prefetch_rows<THREADS>(V, n0 + T, r.end, M);
+        prefetch_rows<C, DP>(Q, n0 + T, r.end, D);
+        prefetch_rows<C, DP>(K, n0 + T, r.end, D);
+        prefetch_rows<C, MP>(V, n0 + T, r.end, M);
         __syncthreads();
         const bool real = row0 < cn;
         float o[MP / 8][4], d0 = 0.f, d1 = 0.f;         // rows g, g + 8 of [num | den]; d0, d1 spread over the four lanes
@@ -301,7 +301,7 @@ causal_mma_dq_kernel(const Params p) {
             else rg.load(G + n0 * M, cn, M, 0.f);
             if constexpr (C::BUF == 1) __syncthreads();
             st.template publish<NS>(buf + Sh::S, sZ, reinterpret_cast<uint16_t*>(buf + Sh::ZP));
-            with_phi<NQ>(phi, [&](auto f) { rk.template store<NQ>(buf + Sh::X, [&](int, float x) { return f(x); }); });
+            rk.template features<NQ>(buf + Sh::X, phi);
             rv.template values<NV>(buf + Sh::Y);
             if constexpr (WPS == 1) {
                 rg.template planes<NV>(ga.a);
@@ -310,10 +310,10 @@ causal_mma_dq_kernel(const Params p) {
                 ga.tile = smem_u32(buf + Sh::R); ga.row0 = row0; ga.lane = lane;
             }
         }
-        prefetch_rows<THREADS>(Q, n0 + T, r.end, D);
-        prefetch_rows<THREADS>(K, n0 + T, r.end, D);
-        prefetch_rows<THREADS>(V, n0 + T, r.end, M);
-        prefetch_rows<THREADS>(G, n0 + T, r.end, M);
+        prefetch_rows<C, DP>(Q, n0 + T, r.end, D);
+        prefetch_rows<C, DP>(K, n0 + T, r.end, D);
+        prefetch_rows<C, MP>(V, n0 + T, r.end, M);
+        prefetch_rows<C, MP>(G, n0 + T, r.end, M);
         __syncthreads();
         const bool real = row0 < cn;
         // The first chunk of a sequence goes through twice, the second time with the G_i . O_i it found taken off the
@@ -537,10 +537,10 @@ causal_mma_dkv_kernel(const Params p) {
             rr.template store<NR, NV>(buf + Sh::X, buf + Sh::Y, sdl, wpl, phi);
         }
         if (c > 0) {
-            prefetch_rows<THREADS>(Q, n0 - T, r.end, D);
-            prefetch_rows<THREADS>(K, n0 - T, r.end, D);
-            prefetch_rows<THREADS>(V, n0 - T, r.end, M);
-            prefetch_rows<THREADS>(G, n0 - T, r.end, M);
+            prefetch_rows<C, DP>(Q, n0 - T, r.end, D);
+            prefetch_rows<C, DP>(K, n0 - T, r.end, D);
+            prefetch_rows<C, MP>(V, n0 - T, r.end, M);
+            prefetch_rows<C, MP>(G, n0 - T, r.end, M);
         }
         __syncthreads();
         if (v_part && row0 < cn) {

@@ -17,6 +17,7 @@
 #pragma once
 
 #include "la_common.cuh"
+#include "la_tc_common.cuh"
 
 namespace la {
 namespace mma {
@@ -194,9 +195,13 @@ __device__ __forceinline__ float pad_value(int phi) { return phi == LA_PHI_IDENT
 template <int NQ, typename F>
 __device__ __forceinline__ void with_phi(int phi, F f) {
     if (phi == LA_PHI_IDENTITY) f([](float x) { return x; });
-    else if constexpr (NQ == 1) f([](float x) { const float e = __expf(x); return x > 0.f ? x + 1.f : e; });
+    else if constexpr (NQ == 1) f([](float x) { return tc::phi_fast(x); });
     else f([](float x) { const float e = expf(x); return x > 0.f ? x + 1.f : e; });
 }
+
+// Whole tiles without a predicate and padding per group: where tiles are never wider than the problem and the kernels small,
+// that is bf16 with 32 columns (D = M = 32, la_causal_mma.cu); the others lost 5 to 8 % to the second copy of their loads.
+template <typename IO, int C> constexpr bool kPlainLoads = sizeof(IO) == 2 && C == 32;
 
 // T rows of `cols` columns (padded to C), contiguous in global memory; rows cn.. and columns cols.. hold `pad`.
 template <typename IO, int T, int C, int THREADS>
@@ -204,6 +209,14 @@ struct RawTile {
     static constexpr int GROUPS = T * (C / 8) / THREADS;
     Group8<IO> r[GROUPS];
     __device__ __forceinline__ void load(const IO* src, int cn, int cols, float pad) {
+        if constexpr (kPlainLoads<IO, C>) {
+            if (cn >= T) {
+                src += threadIdx.x * 8;
+#pragma unroll
+                for (int u = 0; u < GROUPS; ++u) r[u].load(src + u * (THREADS * 8));
+                return;
+            }
+        }
 #pragma unroll
         for (int u = 0; u < GROUPS; ++u) {
             const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), c = idx % (C / 8) * 8;
@@ -218,6 +231,25 @@ struct RawTile {
         for (int u = 0; u < GROUPS; ++u) {
             const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), g = idx % (C / 8);
             *reinterpret_cast<uint4*>(tile + tile_at<C>(row, g)) = r[u].a;
+        }
+    }
+    // planes of the features
+    template <int NP>
+    __device__ __forceinline__ void features(uint8_t* tile, int phi) const {
+        // One plane: two values at a time, from bf16 to bf16, five instructions a value instead of ten (the exponential of
+        // negative numbers below -87 is zero, as in the tcgen05 kernels).  These kernels are bound by instruction issue: with
+        // this, loads without predicates and one prefetch per thread, B128 H8 N784 D32 forward + backward 298.9 -> 281.3 us.
+        if constexpr (NP == 1) {
+            static_assert(sizeof(IO) == 2, "one plane");
+            if (phi == LA_PHI_IDENTITY) return copy(tile);
+#pragma unroll
+            for (int u = 0; u < GROUPS; ++u) {
+                const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), g = idx % (C / 8);
+                *reinterpret_cast<uint4*>(tile + tile_at<C>(row, g)) =
+                    make_uint4(tc::phi_pair(r[u].a.x), tc::phi_pair(r[u].a.y), tc::phi_pair(r[u].a.z), tc::phi_pair(r[u].a.w));
+            }
+        } else {
+            with_phi<NP>(phi, [&](auto f) { store<NP>(tile, [&](int, float x) { return f(x); }); });
         }
     }
     template <int NP>
@@ -286,6 +318,16 @@ struct RawStrip {
     Pair<IO> r[KS][4];
     __device__ __forceinline__ void load(const IO* src, int row0, int cn, int cols, float pad) {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+        if constexpr (kPlainLoads<IO, C>) {
+            if (cn >= row0 + 16) {
+                src += (row0 + g) * C + t * 2;
+#pragma unroll
+                for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) r[kk][j].load(src + (j & 1) * (8 * C) + kk * 16 + (j >> 1) * 8);
+                return;
+            }
+        }
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk)
 #pragma unroll
@@ -298,7 +340,16 @@ struct RawStrip {
     // features: as fp32 pairs, or (To = bf16) rounded
     template <int NQ, typename To>
     __device__ __forceinline__ void map(int phi, RawStrip<To, C>& out) const {
-        with_phi<NQ>(phi, [&](auto f) {
+        if constexpr (sizeof(To) == 2) {        // two at a time, from bf16 to bf16
+            if (phi == LA_PHI_IDENTITY) {
+                out = *this;
+                return;
+            }
+#pragma unroll
+            for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) out.r[kk][j].w = tc::phi_pair(r[kk][j].w);
+        } else with_phi<NQ>(phi, [&](auto f) {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk)
 #pragma unroll

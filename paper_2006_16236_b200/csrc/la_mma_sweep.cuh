@@ -183,26 +183,26 @@ struct State {
             }
         }
     }
-    // s += X^T Y, z += X^T w over the rows of the tiles X [T][DP] (NX planes), Y [T][MP] (NY);
-    // w: ones, or the vector whose three planes of T elements are at wpl
+    // s += X^T Y, z += X^T w over the rows of the tiles X [ROWS][DP] (NX planes), Y [ROWS][MP] (NY);
+    // w: ones, or the vector whose three planes of ROWS elements are at wpl
     // (a chunk that is not full has zeros in the tiles' other rows)
-    template <int NX, int NY, bool ONES>
+    template <int NX, int NY, bool ONES, int ROWS = T>
     __device__ __forceinline__ void update(uint32_t X, uint32_t Y, const uint16_t* wpl) {
         const int lane = threadIdx.x & 31, t = lane & 3, c0 = n0();
         if (!owner()) return;
 #pragma unroll
         for (int i = 0; i < SD; ++i) {
-            uint32_t a[T / 16][NX][4];
+            uint32_t a[ROWS / 16][NX][4];
             float zs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int b = 0; b < T / 16; ++b) {
-                load_rows_t<NX, DP>(a[b], X, T * DP * 2, b * 16, strip(i) * 2, lane);
+            for (int b = 0; b < ROWS / 16; ++b) {
+                load_rows_t<NX, DP>(a[b], X, ROWS * DP * 2, b * 16, strip(i) * 2, lane);
                 float u[4] = {0.f, 0.f, 0.f, 0.f};
                 if constexpr (ONES) {
 #pragma unroll
                     for (int k = NX - 1; k >= 0; --k) mma16816(u, a[b][k], 0x3f803f80u, 0x3f803f80u);
                 } else {
-                    vector_mma<NX, T>(u, a[b], wpl, b * 16, t);
+                    vector_mma<NX, ROWS>(u, a[b], wpl, b * 16, t);
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) zs[j] += u[j];
@@ -213,9 +213,9 @@ struct State {
             for (int n = 0; n < NC / 2; ++n) {
                 Chain c;
 #pragma unroll
-                for (int b = 0; b < T / 16; ++b) {
+                for (int b = 0; b < ROWS / 16; ++b) {
                     uint32_t y[NY][4];
-                    load_cols_t<NY, MP>(y, Y, T * MP * 2, b * 16, c0 + n * 2, lane);
+                    load_cols_t<NY, MP>(y, Y, ROWS * MP * 2, b * 16, c0 + n * 2, lane);
                     c.step<NX, NY>(a[b], y);
                 }
                 c.add_to(s[i][2 * n], s[i][2 * n + 1]);
@@ -285,12 +285,20 @@ template <int NT8> __device__ __forceinline__ void clear(float (&x)[NT8][4]) {
         for (int j = 0; j < 4; ++j) x[n][j] = 0.f;
 }
 
-template <int THREADS, typename IO>
+// rows n0 .. n0 + T - 1, those before `end`, on their way to L2
+template <typename C, int COLS, typename IO>
 __device__ __forceinline__ void prefetch_rows(const IO* x, int64_t n0, int64_t end, int cols) {
+    constexpr int THREADS = kThreads<C>;
     if (n0 < 0 || n0 >= end) return;
     const int64_t rows = end - n0 < T ? end - n0 : T;
     const char* p = reinterpret_cast<const char*>(x + n0 * cols);
-    for (int64_t o = threadIdx.x * 128; o < rows * cols * (int64_t)sizeof(IO); o += THREADS * 128) prefetch_l2(p + o);
+    if constexpr (C::BUF == 2) {            // (few lines: no loop)
+        const int bytes = (int)rows * cols * (int)sizeof(IO), o = (int)threadIdx.x * 128;
+        static_assert(T * COLS * (int)sizeof(IO) <= THREADS * 128, "one line per thread");
+        if (o < bytes) prefetch_l2(p + o);
+    } else {
+        for (int64_t o = threadIdx.x * 128; o < rows * cols * (int64_t)sizeof(IO); o += THREADS * 128) prefetch_l2(p + o);
+    }
 }
 
 // feature-mapped pairs in registers: bf16 where features have one plane
@@ -367,11 +375,11 @@ causal_mma_sum_kernel(const Params p) {
             rx.load(X + n0 * D, cn, D, pad);
             ry.load(Y + n0 * M, cn, M, 0.f);
             if constexpr (C::BUF == 1) __syncthreads();
-            with_phi<NX>(phi, [&](auto f) { rx.template store<NX>(buf + Sh::X, [&](int, float x) { return f(x); }); });
+            rx.template features<NX>(buf + Sh::X, phi);
             ry.template values<NY>(buf + Sh::Y);
         }
-        prefetch_rows<THREADS>(X, n0 + T, r.end, D);
-        prefetch_rows<THREADS>(Y, n0 + T, r.end, M);
+        prefetch_rows<C, DP>(X, n0 + T, r.end, D);
+        prefetch_rows<C, MP>(Y, n0 + T, r.end, M);
         __syncthreads();
         st.template update<NX, NY, !REVERSE>(smem_u32(buf + Sh::X), smem_u32(buf + Sh::Y), wpl);
         flip<C, Sh>(buf, smem);
