@@ -29,6 +29,9 @@
  *    problem with M <= 64 runs on mma.sync kernels that keep fp32 accuracy
  *    (products of numbers split into bf16 parts), everything else on the general
  *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.
+ *    Few short sequences (D = M in {32, 64}, or 128 features to 64 values; some
+ *    hundred positions to 2048) take one launch of a kernel with a thread-block
+ *    cluster per sequence instead; sizes of buffers and plans are unaffected.
  *    Only the tcgen05 kernels have a la_causal_plan() and a causal saved buffer.
  *    Finite numbers keep their value on these kernels; an infinity in Q, K, V or G acts like a NaN
  *    (its products with split numbers are sums of infinities of both signs), so that results that

@@ -30,6 +30,18 @@ int linear_mma_forward(const la_problem& p, const void* Q, const void* K, const 
 int linear_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* saved,
                         const void* G, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
 
+// Short sequences in one launch (la_cluster.cu): ahead of the other kernels where these say so.  saved (or null): filled for
+// the tcgen05 backward kernels.
+bool causal_cluster_forward_preferred(const la_problem& p);
+bool causal_cluster_backward_preferred(const la_problem& p);
+int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
+                           const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, cudaStream_t st);
+int causal_cluster_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
+                            const StateArgs& sa, void* dQ, void* dK, void* dV, cudaStream_t st);
+bool linear_cluster_preferred(const la_problem& p);
+int linear_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O, float* den,
+                           float* KV, float* Zs, void* saved, cudaStream_t st);
+
 namespace tc {
 // process-wide overrides of the automatic plans (see la_plan_override)
 void set_plan_override(int causal_pieces, int causal_short, int linear_splits);
@@ -39,6 +51,8 @@ int linear_splits_override();
 // ragged batch; saved (or null) = where the forward leaves what the backward pass can reuse.
 size_t causal_forward_workspace(const la_problem& p);
 size_t causal_saved_bytes(const la_problem& p);
+// the part of a saved buffer that a kernel of its own writes: the forward pre-pass's records
+int causal_keep_records(const la_problem& p, const void* K, const void* V, const int* lengths, void* saved, cudaStream_t st);
 int causal_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
                    const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, void* ws,
                    cudaStream_t st);
@@ -47,6 +61,7 @@ int causal_backward(const la_problem& p, const void* Q, const void* K, const voi
                     const StateArgs& sa, const void* saved, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
 size_t linear_forward_workspace(const la_problem& p);
 size_t linear_backward_workspace(const la_problem& p);
+int linear_keep_sums(const la_problem& p, const void* K, const void* V, const int* lengths, void* saved, cudaStream_t st);
 int linear_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O,
                    float* den, float* KV, float* Zs, void* saved, void* ws, cudaStream_t st);
 int linear_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths,

@@ -560,6 +560,17 @@ size_t causal_forward_workspace(const la_problem& p) {
 
 size_t causal_saved_bytes(const la_problem& p) { return saved_layout(p, choose_plan(p)).bytes; }
 
+int causal_keep_records(const la_problem& p, const void* K, const void* V, const int* lengths, void* saved, cudaStream_t st) {
+    const CausalPlan pl = choose_plan(p);
+    const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
+    const bool ragged = ragged_problem(p, lengths);
+    CUtensorMap mK, mV;
+    if (int rc = encode_attention_map(&mK, K, ragged, seqs, n, kChunk, (int)p.D)) return rc;
+    if (int rc = encode_attention_map(&mV, V, ragged, seqs, n, kChunk, (int)p.D)) return rc;
+    return segment_states(p, pl, mK, mV, nullptr, nullptr, (float*)((char*)saved + saved_layout(p, pl).records), /*reverse=*/false,
+                          p.phi == LA_PHI_ELU1, st, lengths);
+}
+
 int causal_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
                    const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, void* ws,
                    cudaStream_t st) {

@@ -935,6 +935,14 @@ size_t linear_backward_workspace(const la_problem& p) {
     return 2 * linear_forward_workspace(p);
 }
 
+int linear_keep_sums(const la_problem& p, const void* K, const void* V, const int* lengths, void* saved, cudaStream_t st) {
+    const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
+    CUtensorMap mK, mV;
+    if (int rc = encode_attention_map(&mK, K, p.N % kChunk != 0, seqs, n, kChunk, (int)p.D)) return rc;
+    if (int rc = encode_attention_map(&mV, V, p.N % kChunk != 0, seqs, n, kChunk, (int)p.D)) return rc;
+    return launch_sums(p, choose_splits(p), mK, mV, lengths, (float*)saved, st);
+}
+
 int linear_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O,
                    float* den, float* KV, float* Zs, void* saved, void* ws, cudaStream_t st) {
     const Segmentation sg = choose_splits(p);

@@ -1,0 +1,131 @@
+"""Short sequences in one launch (a thread-block cluster per sequence): lengths at the edges of a CTA's rows and of the cluster,
+ragged, from a state and with state gradients, and the bidirectional forward pass, against the fp64 oracle.
+
+Tolerances (2-norm of the difference over the 2-norm of the result) as for the other kernels on these instructions: fp32 2e-6
+where terms do not cancel (16 * 2^-23), 8e-6 for gradients; bf16 D = M calls are held to the gates of tests/parity.py, bf16
+features of 128 columns to one rounding of the output, 2^-8 (their states stay in fp32)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2006_16236_b200 as la
+from paper_2006_16236_b200.inputs import draw_qkvg
+from parity import assert_close
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+SIZES = {torch.float32: [1, 16, 63, 64, 65, 130, 1000, 1024], torch.bfloat16: [1, 63, 64, 128, 129, 300, 1024, 1025, 2048]}
+CAUSAL = [(torch.float32, "elu1", 32, 32), (torch.float32, "identity", 64, 64), (torch.bfloat16, "elu1", 64, 64),
+          (torch.bfloat16, "elu1", 32, 32), (torch.bfloat16, "identity", 128, 64)]
+
+
+def _close(x, ref, tol, what):
+    x, ref = x.double().cpu().numpy(), np.asarray(ref)
+    assert np.linalg.norm(x - ref) <= tol * np.linalg.norm(ref) + 1e-30, (what, np.linalg.norm(x - ref) / np.linalg.norm(ref))
+
+
+@pytest.mark.parametrize("dtype,phi,D,M,N", [(*c, n) for c in CAUSAL for n in SIZES[c[0]] if c[2] != 128 or n <= 1024])
+def test_causal(dtype, phi, D, M, N):
+    B, H, eps = 3, 1, 0.5 if N % 2 else 0.0
+    Q, K, V, G = draw_qkvg(B, H, N, D, M, 11 + N, dtype, 1.0)
+    if phi == "identity":                               # features: positive, as the weights of a kernel are
+        Q, K = Q.abs() + 0.1, K.abs() + 0.1
+    g = torch.Generator().manual_seed(N)
+    S0, Z0 = torch.randn((B, H, D, M), generator=g), torch.rand((B, H, D), generator=g) * 4 + 1
+    dS, dZ = torch.randn((B, H, D, M), generator=g) * 0.05, torch.randn((B, H, D), generator=g) * 0.05
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    S0d, Z0d, dSd, dZd = (t.to(DEV) for t in (S0, Z0, dS, dZ))
+
+    def check(x, ref, what, state=False):
+        if dtype == torch.bfloat16 and D == M:
+            assert_close(x, ref, dtype, what, grad=what[0] == "d")
+        else:
+            _close(x, ref, (8e-6 if what[0] == "d" else 2e-6) if dtype == torch.float32 or state else 2 ** -8, what)
+
+    for lengths in (None, [N, N // 2, 0]):
+        ln = None if lengths is None else torch.tensor(lengths, dtype=torch.int32, device=DEV)
+        for state in (False, True):
+            S1, Z1, dS0, dZ0 = (torch.full_like(t, 7.0) for t in (S0d, Z0d, S0d, Z0d))
+            den = torch.empty(B, H, N, device=DEV)
+            kw = {"phi": phi, "eps": eps, "lengths": ln, **({"S_in": S0d, "Z_in": Z0d} if state else {})}
+            O = la.la_causal_forward(*dev[:3], den=den, S_out=S1, Z_out=Z1, **kw)
+            grads = la.la_causal_backward(*dev, **kw, **({"dS_out": dSd, "dZ_out": dZd, "dS_in": dS0, "dZ_in": dZ0} if state else {}))
+            la.la_last_device_status()
+            for b in range(B):
+                n = N if lengths is None else lengths[b]
+                assert not O[b, :, n:].any() and not den[b, :, n:].any() and not any(x[b, :, n:].any() for x in grads)
+                sl = (slice(b, b + 1), slice(None), slice(0, n))
+                q, k, v, gg = (t[sl].double().numpy() for t in (Q, K, V, G))
+                st = [(t[b:b + 1] if state else torch.zeros_like(t[b:b + 1])).double().numpy() for t in (S0, Z0, dS, dZ)]
+                Or, denr, Sr, Zr = oracle.causal_from_state(q, k, v, st[0], st[1], phi, eps)
+                rq, rk, rv, rS, rZ = oracle.causal_backward_from_state(q, k, v, st[0], st[1], gg, st[2], st[3], phi, eps)
+                if n or state:
+                    check(S1[b:b + 1], Sr, "S_out", True), check(Z1[b:b + 1], Zr, "Z_out", True)
+                if state:
+                    check(dS0[b:b + 1], rS, "dS_in", True), check(dZ0[b:b + 1], rZ, "dZ_in", True)
+                if n:
+                    check(O[sl], Or, "O"), check(den[sl], denr, "O den", True)
+                    for nm, x, ref in zip(("dQ", "dK", "dV"), grads, (rq, rk, rv)):
+                        check(x[sl], ref, nm)
+
+
+@pytest.mark.parametrize("phi", ["elu1", "identity"])
+@pytest.mark.parametrize("N", [1, 64, 127, 128, 129, 1000, 2048, 2049, 4500])
+@pytest.mark.parametrize("D", [32, 64])
+def test_bidirectional_forward(D, N, phi):
+    B, H = 3, 1
+    Q, K, V, _ = draw_qkvg(B, H, N, D, D, 5 + N, torch.bfloat16, 0.125)
+    if phi == "identity":
+        Q, K = Q.abs() + 0.9, K.abs() + 0.9
+    dev = [t.to(DEV) for t in (Q, K, V)]
+    for lengths in ([N] * B, [N, N // 2 + 1, 0]):
+        den, S, Z = torch.empty(B, H, N, device=DEV), torch.empty(B, H, D, D, device=DEV), torch.empty(B, H, D, device=DEV)
+        ln = None if lengths[-1] else torch.tensor(lengths, dtype=torch.int32, device=DEV)
+        O = la.la_linear_attention(*dev, phi=phi, lengths=ln, den=den, KV=S, Zs=Z)
+        la.la_last_device_status()
+        for b, n in enumerate(lengths):
+            sl = (slice(b, b + 1), slice(None), slice(0, n))
+            assert not O[b, :, n:].any() and not den[b, :, n:].any()
+            if not n:
+                assert not S[b].any() and not Z[b].any()
+                continue
+            q, k, v = (t[sl].double().numpy() for t in (Q, K, V))
+            Or, denr = oracle.linear_attention(q, k, v, causal=False, phi=phi)[:2]
+            fk = oracle.feature_map(k) if phi == "elu1" else k
+            assert_close(O[sl], Or, torch.bfloat16, "O")
+            assert_close(den[sl], denr, torch.bfloat16, "den")
+            assert_close(S[b:b + 1], np.einsum("bhnd,bhnm->bhdm", fk, v), torch.bfloat16, "KV")
+            assert_close(Z[b:b + 1], fk.sum(2), torch.bfloat16, "Zs")
+
+
+@pytest.mark.parametrize("D", [32, 64])
+@pytest.mark.parametrize("N", [300, 1024, 1025, 2048])
+def test_training_steps_follow_each_other(N, D):
+    """Steps with and without a saved buffer, enqueued one behind the other on data that changes in between without any host
+    synchronisation: the same bits every time, and the forward's do not depend on the buffer."""
+    sets = [[t.to(DEV) for t in draw_qkvg(1, 4, N, D, D, seed, torch.bfloat16, 1.0)] for seed in (1, 2)]
+    buf = [torch.empty_like(t) for t in sets[0]]
+    saved = la.saved_buffer(buf[0], buf[2])
+    sums = la.linear_saved_buffer(buf[0], buf[2])
+
+    def step(i):
+        for b, t in zip(buf, sets[i % 2]):
+            b.copy_(t)
+        out = [la.la_causal_forward(*buf[:3], saved=saved if i % 4 < 2 else None)]
+        out += la.la_causal_backward(*buf, saved=saved if i % 4 < 2 else None)
+        out.append(la.la_linear_attention(*buf[:3], saved=sums if i % 4 < 2 else None))
+        out += la.la_linear_attention_backward(*buf, saved=sums if i % 4 < 2 else None)
+        return out
+
+    steps = [step(i) for i in range(12)]
+    la.la_last_device_status()
+    for i in range(4, 12):
+        assert all(torch.equal(a, b) for a, b in zip(steps[i], steps[i % 4])), i
+    for i in (0, 1):                            # (the causal dK and dV agree to rounding only, where the buffer is used)
+        assert torch.equal(steps[i][0], steps[i + 2][0]) and torch.equal(steps[i][1], steps[i + 2][1])
+        assert all(torch.equal(a, b) for a, b in zip(steps[i][4:], steps[i + 2][4:]))
+    q, k, v, g = (t.double().cpu().numpy() for t in sets[0])
+    assert_close(steps[0][0], oracle.linear_attention(q, k, v, causal=True)[0], torch.bfloat16, "O")
+    for nm, x, ref in zip(("dQ", "dK", "dV"), steps[0][1:4], oracle.linear_attention_backward(q, k, v, g, causal=True)):
+        assert_close(x, ref, torch.bfloat16, nm, grad=True)
