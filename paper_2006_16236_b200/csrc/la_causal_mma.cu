@@ -95,7 +95,7 @@ __device__ __forceinline__ void mask_diagonal(float (&s0)[4], float (&s1)[4], in
 
 // ---- forward ---------------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(kThreads<C>, (resident<ForwardLayout<C, DP, MP>, C>()))
+__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<ForwardLayout<C, DP, MP>, C>()))
 causal_mma_forward_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = ForwardLayout<C, DP, MP>;
@@ -259,7 +259,7 @@ causal_mma_forward_kernel(const Params p) {
 
 // ---- dQ sweep --------------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(kThreads<C>, (resident<DqLayout<C, DP, MP>, C>()))
+__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DqLayout<C, DP, MP>, C>()))
 causal_mma_dq_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = DqLayout<C, DP, MP>;
@@ -494,7 +494,7 @@ causal_mma_dq_kernel(const Params p) {
 
 // ---- dK, dV sweep ----------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(kThreads<C>, (resident<DkvLayout<C, DP, MP>, C>(C::WPS == 1 ? 3 : 2)))
+__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DkvLayout<C, DP, MP>, C>(C::WPS == 1 ? 3 : 2)))
 causal_mma_dkv_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = DkvLayout<C, DP, MP>;
@@ -677,12 +677,15 @@ causal_mma_dkv_kernel(const Params p) {
 struct Plan { int pieces; int64_t len; };
 
 // Pieces per sequence, by the estimated time in units of one chunk of a main kernel (about 10 us alone on an SM).
-// An SM runs two CTAs in 1.25 times the time of one; a CTA's start costs about a chunk, and 0.2 for each record it
-// sums, of which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk.  Forward +
-// backward in us, fp32, D = M = 64, pieces 1 / 2 / 4 / 8 / 16: B1 H8 N1024 466 / 304 / 172 / 123 / 134;
-// B8 H8 N1024 484 / 324 / 245 / 287 / 381; B16 H8 N2048 963 / 815 / 929 / 913 / 1091;
-// B32 H8 N4096 2632 / 3318 / 3219 / 3215 / 3645.  At most sixteen: the estimate is checked up to N = 4096 only (for few
-// sequences much longer than that it would want more), and it knows nothing of the single-plane kernels' four CTAs per SM.
+// fp32 D = M = 64 and Fourier features, whose kernels leave an SM little to gain from a second CTA (0.9 of the time of the two one
+// after the other; a pre-pass costs 0.16 per chunk and 1.3), forward + backward in us at the pieces of the other rule / of
+// this one (B x H x N: pieces): fp32 4x8x1000 8: 163 / 4: 150, 16x8x256 2: 132 / 1: 108, 16x8x2000 2: 829 / 1: 765, 2x8x4096 16: 306 /
+// 8: 283; Fourier 3x8x2666 11: 290 / 6: 233, 4x8x1500 8: 227 / 4: 195, 8x8x500 4: 152 / 2: 133, 16x8x1000 2: 380 / 1: 349.  The others:
+// an SM runs two CTAs in 1.25 times the time of one; a CTA's start costs about a chunk, and 0.2 for each record it sums, of
+// which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk (fp32 D = M = 32, B4 H8 N2000,
+// pieces 1 / 4 / 8 / 12 / 16: 353 / 141 / 113 / 131 / 119; B22 H8 N3316 903 / 732 / 749 / 733 / 757).  At most sixteen: the estimates
+// are checked up to N = 4096 only (for few sequences much longer than that they would want more), and they know nothing of the
+// single-plane kernels' four CTAs per SM.
 Plan choose_plan(const la_problem& p, bool single) {
     const int64_t chunks = (p.N + T - 1) / T, bh = p.B * p.H;
     int64_t best = 1;
@@ -693,12 +696,18 @@ Plan choose_plan(const la_problem& p, bool single) {
         best = forced < chunks ? forced : chunks;
         if (best > 1024) best = 1024;
     } else {
-        auto waves = [](int64_t ctas) {
+        const bool wide = p.dtype == LA_F32 ? p.D == 64 && p.M == 64 : p.phi == LA_PHI_IDENTITY && p.D == 128 && p.M == 64;
+        auto waves = [&](int64_t ctas) {
             const int64_t sm = (ctas + 147) / 148;
+            if (wide) return sm == 1 ? 1.0 : 0.9 * (double)sm;
             return 1.25 * (double)(sm / 2) + (double)(sm % 2);
         };
         auto cost = [&](int64_t n) {
             const double per = (double)((chunks + n - 1) / n);
+            if (wide) {
+                const int64_t cut = (chunks + (int64_t)per - 1) / (int64_t)per;         // pieces that this makes
+                return (per + 0.5 + 0.1 * (cut - 1)) * waves(bh * cut) + (cut > 1 ? 0.16 * per * waves(bh * (cut - 1)) + 1.3 : 0.0);
+            }
             return (per + 1.0 + 0.1 * (n - 1)) * waves(bh * n) + (n > 1 ? 0.35 * (per + 1.0) * waves(bh * (n - 1)) : 0.0);
         };
         for (int64_t n = 2; n <= 16 && n <= chunks; ++n)
@@ -753,10 +762,12 @@ template <typename C, int DP, int MP, bool EXACT> struct Kernels {
 // instantiated, at the exact sizes only; padded ones take two whatever the grid.
 template <typename F> int dispatch(const la_problem& p, int pieces, F f) {
     const bool full = p.B * p.H * pieces >= 222;            // one and a half CTAs per SM and more
+    const bool few = p.B * p.H * pieces <= 148;
     const bool exact = (p.D == 32 || p.D == 64 || p.D == 128) && p.M == (p.D == 32 ? 32 : 64);
     if (p.dtype == LA_F32) {
         if (p.D <= 32 && p.M <= 32) return exact ? f(Kernels<Fp32, 32, 32, true>()) : f(Kernels<Fp32, 32, 32, false>());
         if (exact && p.D == 64 && full) return f(Kernels<Fp32One, 64, 64, true>());
+        if (exact && p.D == 64 && few) return f(Kernels<Fp32Alone, 64, 64, true>());
         if (p.D <= 64) return exact ? f(Kernels<Fp32, 64, 64, true>()) : f(Kernels<Fp32, 64, 64, false>());
         return f(Kernels<Fp32, 128, 64, false>());
     }
@@ -764,6 +775,7 @@ template <typename F> int dispatch(const la_problem& p, int pieces, F f) {
     if (p.phi == LA_PHI_IDENTITY) {
         if (p.D <= 64) return f(Kernels<Bf16Features, 64, 64, false>());
         if (exact && full) return f(Kernels<Bf16FeaturesOne, 128, 64, true>());
+        if (exact && few) return f(Kernels<Bf16FeaturesAlone, 128, 64, true>());
         return exact ? f(Kernels<Bf16Features, 128, 64, true>()) : f(Kernels<Bf16Features, 128, 64, false>());
     }
     return p.D <= 64 ? f(Kernels<Bf16Wide, 64, 64, false>()) : f(Kernels<Bf16Wide, 128, 64, false>());

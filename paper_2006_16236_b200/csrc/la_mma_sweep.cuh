@@ -229,29 +229,34 @@ struct State {
 struct Fp32 {
     using IO = float;
     static constexpr int NQ = 3, NV = 3, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
-    static constexpr bool MAPPED = true;
+    static constexpr bool MAPPED = true, ALONE = false;
 };
 struct Bf16Wide {
     using IO = __nv_bfloat16;
     static constexpr int NQ = 3, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
-    static constexpr bool MAPPED = true;
+    static constexpr bool MAPPED = true, ALONE = false;
 };
 struct Bf16Features {
     using IO = __nv_bfloat16;
     static constexpr int NQ = 1, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
-    static constexpr bool MAPPED = false;
+    static constexpr bool MAPPED = false, ALONE = false;
 };
 // ... with one warp per strip, at twice the registers: where a machine full of CTAs keeps the schedulers busy anyway, the
 // hand-overs cost more than they give.  Forward + backward, us, one / two warps: fp32 B32 H8 N4096 D64 2690 / 2930,
 // B4 H8 N4096 477 / 472, B1 H8 N1024 122 / 94; Fourier B8 H8 N1000 C128 272 / 288, B1 H8 N4000 343 / 265.
 struct Fp32One : Fp32 { static constexpr int WPS = 1; };
 struct Bf16FeaturesOne : Bf16Features { static constexpr int WPS = 1; };
+// ... and with an SM to itself: a grid of at most 148 CTAs has that anyway, and the backward kernels then have 255 registers
+// instead of 128 and up to 2.2 KB spilled.  Forward + backward, us, before / after: Fourier B1 H8 N4000 C128 282 / 234, B3 H8
+// N2666 341 / 327; fp32 D = 64 B1 H8 N2000 110 / 100, B16 H8 N100 67 / 59 (but 160 CTAs, B20 H8 N99, 95 / 100).
+struct Fp32Alone : Fp32 { static constexpr bool ALONE = true; };
+struct Bf16FeaturesAlone : Bf16Features { static constexpr bool ALONE = true; };
 // bf16 operands throughout (with fp32 sums), as the tcgen05 kernels have them.  BUF = 2: the small tiles are there twice,
 // one barrier per chunk (the other set was last read before the barrier of this chunk).
 struct Bf16 {
     using IO = __nv_bfloat16;
     static constexpr int NQ = 1, NV = 1, NP = 1, NS = 1, NR = 1, BUF = 2, WPS = 1;
-    static constexpr bool MAPPED = true;
+    static constexpr bool MAPPED = true, ALONE = false;
 };
 
 // Shared memory: tiles X [T][DP] and Y [T][MP]; with two warps per strip the tile that holds the strips' own operand
