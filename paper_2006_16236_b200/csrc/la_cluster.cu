@@ -596,7 +596,7 @@ causal_cluster_backward_kernel(const BackwardParams p) {
     };
     clear(zc);
     if (real && first) {
-        rq.template map<NQ>(phi, fq);
+        rq.template map<NQ, false>(phi, fq);
 #pragma unroll 1
         for (int jb = 0; jb <= strip; ++jb) {                   // zc = L k
             uint32_t ones[1][4] = {{0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u}};
@@ -830,7 +830,7 @@ causal_cluster_backward_kernel(const BackwardParams p) {
             c.add_to(acc[2 * n], acc[2 * n + 1]);
         }
         RawStrip<typename FeatureType<NQ>::type, DP> fk;
-        rk.template map<NQ>(phi, fk);
+        rk.template map<NQ, false>(phi, fk);        // (as the tile has them)
         IO* dK = (IO*)p.dK + base * DP;
 #pragma unroll
         for (int n = 0; n < DP / 8; ++n) {

@@ -191,11 +191,15 @@ template <> struct Group8<__nv_bfloat16> {
 __device__ __forceinline__ float pad_value(int phi) { return phi == LA_PHI_IDENTITY ? 0.f : -INFINITY; }
 
 // f(x) over a range of registers with the feature map chosen once; NQ = 1: the values are rounded to bf16 afterwards,
-// the approximate exponential (2^-22) will do
+// the approximate exponential (2^-21, the square of that of half the number: no feature that bf16 holds is lost) will do
 template <int NQ, typename F>
 __device__ __forceinline__ void with_phi(int phi, F f) {
     if (phi == LA_PHI_IDENTITY) f([](float x) { return x; });
-    else if constexpr (NQ == 1) f([](float x) { return tc::phi_fast(x); });
+    else if constexpr (NQ == 1) f([](float x) {
+        float e;
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * 0.72134752044448170f));
+        return x > 0.f ? x + 1.f : e * e;
+    });
     else f([](float x) { const float e = expf(x); return x > 0.f ? x + 1.f : e; });
 }
 
@@ -236,9 +240,9 @@ struct RawTile {
     // planes of the features
     template <int NP>
     __device__ __forceinline__ void features(uint8_t* tile, int phi) const {
-        // One plane: two values at a time, from bf16 to bf16, five instructions a value instead of ten (the exponential of
-        // negative numbers below -87 is zero, as in the tcgen05 kernels).  These kernels are bound by instruction issue: with
-        // this, loads without predicates and one prefetch per thread, B128 H8 N784 D32 forward + backward 298.9 -> 281.3 us.
+        // One plane: two values at a time, from bf16 to bf16, five and a half instructions a value instead of ten.  These kernels
+        // are bound by instruction issue: with this, loads without predicates and one prefetch per thread, B128 H8 N784 D32
+        // forward + backward 298.9 -> 283 us.
         if constexpr (NP == 1) {
             static_assert(sizeof(IO) == 2, "one plane");
             if (phi == LA_PHI_IDENTITY) return copy(tile);
@@ -246,7 +250,7 @@ struct RawTile {
             for (int u = 0; u < GROUPS; ++u) {
                 const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), g = idx % (C / 8);
                 *reinterpret_cast<uint4*>(tile + tile_at<C>(row, g)) =
-                    make_uint4(tc::phi_pair(r[u].a.x), tc::phi_pair(r[u].a.y), tc::phi_pair(r[u].a.z), tc::phi_pair(r[u].a.w));
+                    make_uint4(tc::phi_pair<true>(r[u].a.x), tc::phi_pair<true>(r[u].a.y), tc::phi_pair<true>(r[u].a.z), tc::phi_pair<true>(r[u].a.w));
             }
         } else {
             with_phi<NP>(phi, [&](auto f) { store<NP>(tile, [&](int, float x) { return f(x); }); });
@@ -338,7 +342,7 @@ struct RawStrip {
             }
     }
     // features: as fp32 pairs, or (To = bf16) rounded
-    template <int NQ, typename To>
+    template <int NQ, bool kSubnormal = true, typename To>
     __device__ __forceinline__ void map(int phi, RawStrip<To, C>& out) const {
         if constexpr (sizeof(To) == 2) {        // two at a time, from bf16 to bf16
             if (phi == LA_PHI_IDENTITY) {
@@ -348,7 +352,7 @@ struct RawStrip {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) out.r[kk][j].w = tc::phi_pair(r[kk][j].w);
+                for (int j = 0; j < 4; ++j) out.r[kk][j].w = tc::phi_pair<kSubnormal>(r[kk][j].w);
         } else with_phi<NQ>(phi, [&](auto f) {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk)

@@ -216,17 +216,26 @@ __device__ __forceinline__ float phi_fast(float x) {
 // conversion gives), the two products with log2 e are one packed fp32 multiply, and each half
 // takes the exponential where its sign bit is set (a byte permute that replicates the sign
 // bits builds the mask; -0 takes 2^0 = 1 = 0 + 1).  Bit-identical to phi_fast per element.
+// kSubnormal: the exponential as the square of that of half the number, one packed multiply more: features
+// below the smallest normal number (x below -87.3) are not zero but what bf16 holds of them.
+template <bool kSubnormal = false>
 __device__ __forceinline__ uint32_t phi_pair(uint32_t w) {
     uint32_t lin, mask, ex, res;
     asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(lin) : "r"(w), "r"(0x3F803F80u));
     uint64_t xx, tt, cc;
     asm("mov.b64 %0, {%1, %2};" : "=l"(xx) : "r"(w << 16), "r"(w & 0xFFFF0000u));
-    asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(1.4426950408889634f));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(kSubnormal ? 0.72134752044448170f : 1.4426950408889634f));
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(tt) : "l"(xx), "l"(cc));
     float t0, t1, e0, e1;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(tt));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(t0));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(t1));
+    if constexpr (kSubnormal) {
+        uint64_t ee;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(ee) : "f"(e0), "f"(e1));
+        asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(tt) : "l"(ee));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(e0), "=f"(e1) : "l"(tt));
+    }
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(ex) : "f"(e1), "f"(e0));
     asm("prmt.b32 %0, %1, %1, 0xBB99;" : "=r"(mask) : "r"(w));
     asm("lop3.b32 %0, %1, %2, %3, 0xCA;" : "=r"(res) : "r"(mask), "r"(ex), "r"(lin));    // mask ? ex : lin

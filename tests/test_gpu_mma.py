@@ -199,6 +199,35 @@ def test_the_largest_numbers_keep_their_value(D, M):
         _close(O, oracle.linear_attention(q, k, v, causal=causal)[0], 2e-6, f"O {causal}")
 
 
+@pytest.mark.parametrize("N", [1, 16, 63, 64, 100])
+def test_features_below_the_smallest_normal_number(N):
+    """Short bf16 sequences whose keys all lie where exp(x) is below 2^-126: their weights are small numbers like any other.
+    The reference takes the features as bf16 holds them (multiples of 2^-133); queries are large enough that scores are normal
+    numbers.  2-norms: operands (q, scores, state) and result are each rounded to bf16, 2^-9, so 2^-7 for O and den; the
+    gradients are differences of terms of about twice their size, 2^-6."""
+    B, H, D = 56, 8, 32
+    g = torch.Generator().manual_seed(N)
+    Q = (torch.rand((B, H, N, D), generator=g) * 20 + 40).bfloat16()
+    K = (torch.randint(0, 4, (B, H, N, D), generator=g) * -0.5 - 87.5).bfloat16()          # -87.5 .. -89
+    V, G = (torch.randn((B, H, N, D), generator=g).bfloat16() for _ in range(2))
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    den = torch.empty(B, H, N, device=DEV)
+    O = la.la_causal_forward(*dev[:3], den=den)
+    grads = la.la_causal_backward(*dev)
+    la.la_last_device_status()
+    sl = (slice(0, B, 55), slice(0, H, 7))
+    q, k, v, gg = (t[sl].double().numpy() for t in (Q, K, V, G))
+    fq, fk = q + 1, np.round(np.exp(k) * 2.0 ** 133) * 2.0 ** -133
+    fq = torch.from_numpy(fq).bfloat16().double().numpy()
+    Or, denr = oracle.linear_attention(fq, fk, v, causal=True, phi="identity")[:2]
+    _close(O[sl], Or, 2 ** -7, "O")
+    _close(den[sl].double() * 2.0 ** 120, denr * 2.0 ** 120, 2 ** -7, "den")
+    rq, rk, rv = oracle.linear_attention_backward(fq, fk, v, gg, causal=True, phi="identity")
+    for nm, x, ref in zip(("dQ", "dK", "dV"), grads, (rq, rk * fk, rv)):           # slopes: 1 and the feature itself
+        if N > 1 or nm == "dV":                                                     # (one key: the others are analytically zero)
+            _close(x[sl], ref, 2 ** -6, nm)
+
+
 def test_every_launch_can_be_profiled():
     """la_profile_enable() brackets every main kernel, these ones included."""
     dev = [t.to(DEV) for t in draw_qkvg(56, 8, 96, 32, 32, 1, torch.bfloat16, 1.0)]
