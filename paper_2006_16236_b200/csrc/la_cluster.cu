@@ -116,28 +116,31 @@ __device__ __forceinline__ void running_sums(const Exchange& x, const float* S0,
     const Inbox<DP, MP> in(smem_u32(x.inbox));
     const int R = in.R, slot = in.slot();
     in.template for_own_rows<THREADS>(reinterpret_cast<const float*>(x.inbox), [&](int d, int e, const float* from) {
-        float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (S0) run = *reinterpret_cast<const float4*>(S0 + d * MP + e);
+        // (the given state, often much larger than the sums, is added to each of them and not a term that they start with: one
+        // rounding of its size instead of sixteen)
+        float4 run = make_float4(0.f, 0.f, 0.f, 0.f), s0 = run;
+        if (S0) s0 = *reinterpret_cast<const float4*>(S0 + d * MP + e);
         const uint32_t tile = x.tile + tile_at<MP>(d, e / 8) + e % 8 * 2;
 #pragma unroll 4
         for (int i = 0; i < R; ++i) {
             const int c = ORDER == kBefore ? i : R - 1 - i;
             const float4 v = *reinterpret_cast<const float4*>(from + c * slot);
-            give_planes<NS, DP, MP>(tile, run, c);
+            give_planes<NS, DP, MP>(tile, make_float4(run.x + s0.x, run.y + s0.y, run.z + s0.z, run.w + s0.w), c);
             run.x += v.x; run.y += v.y; run.z += v.z; run.w += v.w;
         }
-        if (S1) *reinterpret_cast<float4*>(S1 + d * MP + e) = run;
+        if (S1) *reinterpret_cast<float4*>(S1 + d * MP + e) = make_float4(run.x + s0.x, run.y + s0.y, run.z + s0.z, run.w + s0.w);
     }, [&](int d, int c, const float* from) {
         const int before = ORDER == kBefore ? c : R - 1 - c;           // CTAs ahead of c
-        float run = Z0 ? Z0[d] : 0.f;
+        const float z0 = Z0 ? Z0[d] : 0.f;
+        float run = 0.f;
 #pragma unroll 4
         for (int i = 0; i < before; ++i) run += from[(ORDER == kBefore ? i : R - 1 - i) * slot];
         uint32_t o[3];
-        split2<3>(run, 0.f, o);
-        peer_store(address_in(x.vec + d * 4, c), run);
+        split2<3>(run + z0, 0.f, o);
+        peer_store(address_in(x.vec + d * 4, c), run + z0);
 #pragma unroll
         for (int k = 0; k < 3; ++k) asm volatile("st.shared::cluster.b16 [%0], %1;" ::"r"(address_in(x.vpl + (k * DP + d) * 2, c)), "h"((uint16_t)o[k]) : "memory");
-        if (Z1 && before == R - 1) Z1[d] = run + from[c * slot];
+        if (Z1 && before == R - 1) Z1[d] = (run + from[c * slot]) + z0;
     });
 }
 
@@ -818,7 +821,9 @@ causal_cluster_backward_kernel(const BackwardParams p) {
     }
     if (real && !first) {
 #pragma unroll
-        for (int n = 0; n < DP / 16; ++n) {                     // V R^T + r
+        for (int n = 0; n < DP / 16; ++n) {                     // V R^T + r (which often cancel), then the scores' part
+            const float2 z0 = load_pair(sZ + n * 16 + 2 * t), z1 = load_pair(sZ + n * 16 + 8 + 2 * t);
+            float s0[4] = {z0.x, z0.y, z0.x, z0.y}, s1[4] = {z1.x, z1.y, z1.x, z1.y};
             Chain c;
 #pragma unroll
             for (int ee = 0; ee < MP / 16; ++ee) {
@@ -827,21 +832,25 @@ causal_cluster_backward_kernel(const BackwardParams p) {
                 load_rows<NS, MP>(b, sS, DP * MP * 2, n * 16, ee * 2, lane);
                 c.template step<NV, NS>(a, b);
             }
-            c.add_to(acc[2 * n], acc[2 * n + 1]);
+            c.add_to(s0, s1);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[2 * n][j] += s0[j];
+                acc[2 * n + 1][j] += s1[j];
+            }
         }
         RawStrip<typename FeatureType<NQ>::type, DP> fk;
         rk.template map<NQ, false>(phi, fk);        // (as the tile has them)
         IO* dK = (IO*)p.dK + base * DP;
 #pragma unroll
         for (int n = 0; n < DP / 8; ++n) {
-            const float2 z = *reinterpret_cast<const float2*>(sZ + n * 8 + 2 * t);
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
                 const int row = row0 + g + 8 * b;
                 const auto k = fk.r[n >> 1][(n & 1) * 2 + b];
                 if (row < r.cn)
-                    store_pair<IO>(dK + row * DP + n * 8 + 2 * t, (acc[n][2 * b] + z.x) * phi_slope_from_value(k.lo(), phi),
-                                   (acc[n][2 * b + 1] + z.y) * phi_slope_from_value(k.hi(), phi));
+                    store_pair<IO>(dK + row * DP + n * 8 + 2 * t, acc[n][2 * b] * phi_slope_from_value(k.lo(), phi),
+                                   acc[n][2 * b + 1] * phi_slope_from_value(k.hi(), phi));
             }
         }
     }

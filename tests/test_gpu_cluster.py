@@ -129,3 +129,34 @@ def test_training_steps_follow_each_other(N, D):
     assert_close(steps[0][0], oracle.linear_attention(q, k, v, causal=True)[0], torch.bfloat16, "O")
     for nm, x, ref in zip(("dQ", "dK", "dV"), steps[0][1:4], oracle.linear_attention_backward(q, k, v, g, causal=True)):
         assert_close(x, ref, torch.bfloat16, nm, grad=True)
+
+
+@pytest.mark.parametrize("dtype,N", [(torch.float32, 1000), (torch.bfloat16, 1024)])
+@pytest.mark.parametrize("D", [32, 64])
+def test_a_large_state_is_rounded_once(D, N, dtype):
+    """A state, or the gradient of one, much larger than what a call adds to it: the sum is rounded once at its size (2^-24 of
+    the result).  The sums themselves are held to 2e-6 of their terms' size, in the backward pass of bf16, whose q / dn is
+    rounded, to 2^-8."""
+    B, H = 1, 2
+    Q, K, V, G = draw_qkvg(B, H, N, D, D, 21, dtype, 1.0)
+    Q, K = Q.abs() + 0.1, K.abs() + 0.1
+    g = torch.Generator().manual_seed(22)
+    S0, Z0 = (torch.randn((B, H, D, D), generator=g) + 4) * 1e5, (torch.rand((B, H, D), generator=g) + 1) * 1e6
+    S0d, Z0d, q, k, v, gg = (t.to(DEV) for t in (S0, Z0, Q, K, V, G))
+    S1, Z1, dS, dZ = (torch.empty_like(t) for t in (S0d, Z0d, S0d, Z0d))
+    la.la_causal_forward(q, k, v, phi="identity", S_in=S0d, Z_in=Z0d, S_out=S1, Z_out=Z1)
+    la.la_causal_backward(q, k, v, gg, phi="identity", dS_out=S0d, dZ_out=Z0d, dS_in=dS, dZ_in=dZ)
+    la.la_last_device_status()
+    Q, K, V, G = (t.double().numpy() for t in (Q, K, V, G))
+    O, den = oracle.linear_attention(Q, K, V, causal=True, phi="identity")[:2]
+    qn, dl = Q / den[..., None], -(G * O).sum(-1, keepdims=True)
+
+    def check(x, x0, a, b, tol, what):
+        ref = x0.double().numpy() + np.einsum("bhnd,bhnm->bhdm", a, b).reshape(x0.shape)
+        size = np.einsum("bhnd,bhnm->bhdm", abs(a), abs(b)).reshape(x0.shape)
+        err = abs(x.double().cpu().numpy() - ref) / (2.0 ** -24 * 1.001 * abs(ref) + tol * size)
+        assert err.max() <= 1, (what, err.max())
+
+    ones, tol = np.ones_like(dl), 2e-6 if dtype == torch.float32 else 2.0 ** -8
+    check(S1, S0, K, V, 2e-6, "S_out"), check(Z1, Z0, K, ones, 2e-6, "Z_out")
+    check(dS, S0, qn, G, tol, "dS_in"), check(dZ, Z0, qn, dl, tol, "dZ_in")
