@@ -291,6 +291,8 @@ KERNEL_ALG_BYTES = {
 }
 for _tc, _mma in (("fwd", "forward"), ("bwd_dq", "dq"), ("bwd_dkv", "dkv")):       # the same work on mma.sync
     KERNEL_ALG_BYTES[f"causal_mma_{_mma}_kernel"] = KERNEL_ALG_BYTES[f"causal_{_tc}_kernel"]
+KERNEL_ALG_BYTES["causal_cluster_forward_kernel"] = KERNEL_ALG_BYTES["causal_fwd_kernel"]
+KERNEL_ALG_BYTES["causal_cluster_backward_kernel"] = lambda d, e: 7 * d * e        # Q, K, V, G in; dQ, dK, dV out
 
 
 def bench_attention(la, w, dev, steps, warmup, world, rank, pk, do_e2e=True, from_state=False):

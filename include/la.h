@@ -470,7 +470,9 @@ long long la_kernel_launches(void);
  * 0 causal_fwd_kernel, 1 causal_bwd_dq_kernel, 2 causal_bwd_dkv_kernel, 3 segment_sum_kernel,
  * 4 projection_gemm_kernel, 5 linear_sum_kernel, 6 linear_apply_kernel, 7 recurrent_step_kernel, and of
  * the kernels on mma.sync 8 causal_mma_forward_kernel, 9 causal_mma_dq_kernel, 10 causal_mma_dkv_kernel,
- * 11 causal_mma_sum_kernel (both forms), 12 linear_mma_apply_kernel (three variants).
+ * 11 causal_mma_sum_kernel (both forms), 12 linear_mma_apply_kernel (three variants), and of those with a
+ * thread-block cluster per sequence 13 causal_cluster_forward_kernel, 14 causal_cluster_backward_kernel (all
+ * gradients), 15 linear_cluster_forward_kernel.
  * Not thread-safe; meant for a benchmark's single launching thread.
  */
 int la_profile_enable(int on);

@@ -1148,14 +1148,14 @@ ClusterParams cluster_params(const la_problem& p, const int* lengths) {
 template <typename C, int DP, int MP, int STRIPS, int WPS>
 int launch_forward(const la_problem& p, const ClusterParams& a, cudaStream_t st) {
     constexpr int T = 16 * STRIPS;
-    return launch_cluster<causal_cluster_forward_kernel<C, DP, MP, STRIPS, WPS>>(kProfMmaForward, 32 * STRIPS * WPS, (unsigned)((p.N + T - 1) / T),
+    return launch_cluster<causal_cluster_forward_kernel<C, DP, MP, STRIPS, WPS>>(kProfClusterForward, 32 * STRIPS * WPS, (unsigned)((p.N + T - 1) / T),
                                                                                  (unsigned)(p.B * p.H), ForwardShared<C, DP, MP, STRIPS>::BYTES,
                                                                                  ForwardShared<C, DP, MP, STRIPS>::BYTES, a, st);
 }
 template <typename C, int DP, int MP, int STRIPS>
 int launch_backward(const la_problem& p, const BackwardParams& a, cudaStream_t st) {
     constexpr int T = 16 * STRIPS;
-    return launch_cluster<causal_cluster_backward_kernel<C, DP, MP, STRIPS>>(kProfMmaDq, 64 * STRIPS, (unsigned)((p.N + T - 1) / T),
+    return launch_cluster<causal_cluster_backward_kernel<C, DP, MP, STRIPS>>(kProfClusterBackward, 64 * STRIPS, (unsigned)((p.N + T - 1) / T),
                                                                              (unsigned)(p.B * p.H), BackwardShared<C, DP, MP, STRIPS>::BYTES,
                                                                              BackwardShared<C, DP, MP, STRIPS>::BYTES, a, st);
 }
@@ -1164,7 +1164,7 @@ int launch_linear(const la_problem& p, ClusterParams a, cudaStream_t st) {
     constexpr int T = 16 * STRIPS;
     const int64_t tiles = (p.N + T - 1) / T, per = (tiles + kMaxCluster - 1) / kMaxCluster;
     a.piece_len = per * T;
-    return launch_cluster<linear_cluster_forward_kernel<DP, STRIPS>>(kProfMmaApply, 32 * STRIPS, (unsigned)((tiles + per - 1) / per),
+    return launch_cluster<linear_cluster_forward_kernel<DP, STRIPS>>(kProfClusterLinear, 32 * STRIPS, (unsigned)((tiles + per - 1) / per),
                                                                           (unsigned)(p.B * p.H), per > 1 ? LinearShared<DP, STRIPS>::BYTES : LinearShared<DP, STRIPS>::STAGE,
                                                                      LinearShared<DP, STRIPS>::BYTES, a, st);
 }

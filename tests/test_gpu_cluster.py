@@ -160,3 +160,23 @@ def test_a_large_state_is_rounded_once(D, N, dtype):
     ones, tol = np.ones_like(dl), 2e-6 if dtype == torch.float32 else 2.0 ** -8
     check(S1, S0, K, V, 2e-6, "S_out"), check(Z1, Z0, K, ones, 2e-6, "Z_out")
     check(dS, S0, qn, G, tol, "dS_in"), check(dZ, Z0, qn, dl, tol, "dZ_in")
+
+
+def kernels_of(call):
+    """The library's kernels that a call launches, with how often."""
+    la.la_profile_enable(True)
+    try:
+        call()
+        la.la_last_device_status()
+        return {k: n for k, (_, n) in la.la_profile_read().items()}
+    finally:
+        la.la_profile_enable(False)
+
+
+def test_these_kernels_are_profiled_under_their_own_names():
+    Q, K, V, G = (t.to(DEV) for t in draw_qkvg(1, 2, 500, 64, 64, 1, torch.bfloat16, 1.0))
+    assert kernels_of(lambda: la.la_causal_forward(Q, K, V)) == {"causal_cluster_forward_kernel": 1}
+    assert kernels_of(lambda: la.la_causal_backward(Q, K, V, G)) == {"causal_cluster_backward_kernel": 1}
+    assert kernels_of(lambda: la.la_linear_attention(Q, K, V)) == {"linear_cluster_forward_kernel": 1}
+    saved = la.linear_saved_buffer(Q, V)
+    assert kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved)) == {"linear_sum_kernel": 1, "linear_cluster_forward_kernel": 1}
