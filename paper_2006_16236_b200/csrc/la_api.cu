@@ -381,7 +381,7 @@ static int linear_forward_common(const la_problem* p, const void* Q, const void*
     LA_DEBUG_SPAN(den, tb.den); LA_DEBUG_SPAN(KV, tb.s); LA_DEBUG_SPAN(Zs, tb.z);
     LA_DEBUG_SPAN(lengths, (size_t)p->B * 4); LA_DEBUG_SPAN(ws, ws_bytes); LA_DEBUG_SPAN(saved, saved_bytes);
     cudaStream_t st = (cudaStream_t)stream;
-    if (linear_cluster_preferred(*p))
+    if (linear_cluster_preferred(*p, st))
         return debug_finish(linear_cluster_forward(*p, Q, K, V, lengths, O, den, KV, Zs, saved, st), stream);
     if (tc_supported(*p, LA_OP_LINEAR_FORWARD))
         return debug_finish(tc::linear_forward(*p, Q, K, V, lengths, O, den, KV, Zs, saved, ws, st), stream);
@@ -501,7 +501,7 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     LA_DEBUG_SPAN(den, tb.den); LA_DEBUG_SPAN(S_in, tb.s); LA_DEBUG_SPAN(Z_in, tb.z); LA_DEBUG_SPAN(S_out, tb.s);
     LA_DEBUG_SPAN(Z_out, tb.z); LA_DEBUG_SPAN(lengths, (size_t)p->B * 4); LA_DEBUG_SPAN(ws, ws_bytes);
     LA_DEBUG_SPAN(saved, saved_bytes);
-    if (causal_cluster_forward_preferred(*p))
+    if (causal_cluster_forward_preferred(*p, st))
         return debug_finish(causal_cluster_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, tc_path ? saved : nullptr, st), stream);
     if (tc_path)
         return debug_finish(tc::causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, st), stream);
@@ -580,10 +580,10 @@ static int causal_backward_common(const la_problem* p, const void* Q, const void
     LA_DEBUG_SPAN(S_in, tb.s); LA_DEBUG_SPAN(Z_in, tb.z); LA_DEBUG_SPAN(dS_out, tb.s); LA_DEBUG_SPAN(dZ_out, tb.z);
     LA_DEBUG_SPAN(dS_in, tb.s); LA_DEBUG_SPAN(dZ_in, tb.z); LA_DEBUG_SPAN(lengths, (size_t)p->B * 4);
     LA_DEBUG_SPAN(ws, ws_bytes); LA_DEBUG_SPAN(saved, saved_bytes);
-    if (causal_cluster_backward_preferred(*p))
+    if (causal_cluster_backward_preferred(*p, (cudaStream_t)stream))
         return debug_finish(causal_cluster_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, st), stream);
     if (tc_supported(*p, LA_OP_CAUSAL_BACKWARD))
-        return debug_finish(tc::causal_backward(*p, Q, K, V, lengths, G, sa, saved, dQ, dK, dV, ws, st), stream);
+        return debug_finish(tc::causal_backward(*p, Q, K, V, lengths, G, sa, causal_cluster_backward_size(*p) ? nullptr : saved, dQ, dK, dV, ws, st), stream);
     if (causal_mma_supported(*p))
         return debug_finish(causal_mma_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, ws, st), stream);
     return debug_finish(general_causal_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, ws, st), stream);

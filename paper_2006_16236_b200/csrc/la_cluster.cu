@@ -1112,8 +1112,10 @@ linear_cluster_forward_kernel(const ClusterParams p) {
 }
 
 // ---- host ------------------------------------------------------------------------------------------------------
-template <auto KERNEL, typename P>
-int launch_cluster(ProfKernel prof, int threads, unsigned ctas, unsigned bh, int smem, int most_smem, const P& a, cudaStream_t st) {
+struct ClusterShape { int threads; unsigned ctas, bh; int smem, most_smem; };
+
+template <auto KERNEL>
+int opt_in(int most_smem) {
     static std::atomic<uint64_t> opted_in{0};           // devices on which the kernel may use that much shared memory and 16 CTAs
     int dev = 0;
     LA_CUDA_TRY(cudaGetDevice(&dev));
@@ -1123,13 +1125,42 @@ int launch_cluster(ProfKernel prof, int threads, unsigned ctas, unsigned bh, int
         LA_CUDA_TRY(cudaFuncSetAttribute(KERNEL, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         opted_in.fetch_or(bit, std::memory_order_release);
     }
-    cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = tc::chained_launch(1, (unsigned)threads, (size_t)smem, st, attr);
-    cfg.gridDim = dim3(ctas, bh);
+    return LA_OK;
+}
+
+cudaLaunchConfig_t cluster_launch(const ClusterShape& s, cudaStream_t st, cudaLaunchAttribute (&attr)[2]) {
+    cudaLaunchConfig_t cfg = tc::chained_launch(1, (unsigned)s.threads, (size_t)s.smem, st, attr);
+    cfg.gridDim = dim3(s.ctas, s.bh);
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = ctas;
+    attr[1].val.clusterDim.x = s.ctas;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
+    return cfg;
+}
+
+// How many clusters the context of the stream runs at once: 0 where none has room (a cluster of sixteen CTAs needs them all in one
+// GPC; a context that is limited to some SMs of the device may not have that).  Asked at every call, since it depends on
+// the stream: 0.2 us.
+template <auto KERNEL>
+int64_t clusters_at_once(const ClusterShape& s, cudaStream_t st) {
+    if (opt_in<KERNEL>(s.most_smem) != LA_OK) return 0;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_launch(s, st, attr);
+    cfg.attrs = attr + 1;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, KERNEL, &cfg) != cudaSuccess) {
+        cudaGetLastError();         // not an error of the caller's: the other kernels take the problem
+        return 0;
+    }
+    return n;
+}
+
+template <auto KERNEL, typename P>
+int launch_cluster(ProfKernel prof, const ClusterShape& s, const P& a, cudaStream_t st) {
+    if (int rc = opt_in<KERNEL>(s.most_smem)) return rc;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_launch(s, st, attr);
     prof_begin(prof, st);
     LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, KERNEL, a));
     note_launch();
@@ -1145,29 +1176,57 @@ ClusterParams cluster_params(const la_problem& p, const int* lengths) {
     return a;
 }
 
-template <typename C, int DP, int MP, int STRIPS, int WPS>
-int launch_forward(const la_problem& p, const ClusterParams& a, cudaStream_t st) {
-    constexpr int T = 16 * STRIPS;
-    return launch_cluster<causal_cluster_forward_kernel<C, DP, MP, STRIPS, WPS>>(kProfClusterForward, 32 * STRIPS * WPS, (unsigned)((p.N + T - 1) / T),
-                                                                                 (unsigned)(p.B * p.H), ForwardShared<C, DP, MP, STRIPS>::BYTES,
-                                                                                 ForwardShared<C, DP, MP, STRIPS>::BYTES, a, st);
+template <typename C, int DP, int MP, int STRIPS, int WPS> struct Forward {
+    static constexpr int T = 16 * STRIPS, BYTES = ForwardShared<C, DP, MP, STRIPS>::BYTES;
+    static ClusterShape shape(const la_problem& p) {
+        return {32 * STRIPS * WPS, (unsigned)((p.N + T - 1) / T), (unsigned)(p.B * p.H), BYTES, BYTES};
+    }
+    static int64_t at_once(const la_problem& p, cudaStream_t st) {
+        return clusters_at_once<causal_cluster_forward_kernel<C, DP, MP, STRIPS, WPS>>(shape(p), st);
+    }
+    static int launch(const la_problem& p, const ClusterParams& a, cudaStream_t st) {
+        return launch_cluster<causal_cluster_forward_kernel<C, DP, MP, STRIPS, WPS>>(kProfClusterForward, shape(p), a, st);
+    }
+};
+template <typename C, int DP, int MP> struct Backward {
+    static constexpr int STRIPS = 4, T = 16 * STRIPS, BYTES = BackwardShared<C, DP, MP, STRIPS>::BYTES;
+    static ClusterShape shape(const la_problem& p) {
+        return {64 * STRIPS, (unsigned)((p.N + T - 1) / T), (unsigned)(p.B * p.H), BYTES, BYTES};
+    }
+    static int64_t at_once(const la_problem& p, cudaStream_t st) {
+        return clusters_at_once<causal_cluster_backward_kernel<C, DP, MP, STRIPS>>(shape(p), st);
+    }
+    static int launch(const la_problem& p, const BackwardParams& a, cudaStream_t st) {
+        return launch_cluster<causal_cluster_backward_kernel<C, DP, MP, STRIPS>>(kProfClusterBackward, shape(p), a, st);
+    }
+};
+template <int DP> struct Linear {
+    static constexpr int STRIPS = 8, T = 16 * STRIPS;
+    static int64_t tiles_per_cta(const la_problem& p) { return ((p.N + T - 1) / T + kMaxCluster - 1) / kMaxCluster; }
+    static ClusterShape shape(const la_problem& p) {
+        const int64_t tiles = (p.N + T - 1) / T, per = tiles_per_cta(p);
+        return {32 * STRIPS, (unsigned)((tiles + per - 1) / per), (unsigned)(p.B * p.H),
+                per > 1 ? LinearShared<DP, STRIPS>::BYTES : LinearShared<DP, STRIPS>::STAGE, LinearShared<DP, STRIPS>::BYTES};
+    }
+    static int64_t at_once(const la_problem& p, cudaStream_t st) { return clusters_at_once<linear_cluster_forward_kernel<DP, STRIPS>>(shape(p), st); }
+    static int launch(const la_problem& p, ClusterParams a, cudaStream_t st) {
+        a.piece_len = tiles_per_cta(p) * T;
+        return launch_cluster<linear_cluster_forward_kernel<DP, STRIPS>>(kProfClusterLinear, shape(p), a, st);
+    }
+};
+
+// the kernel of a problem that has one
+template <typename F> auto with_forward(const la_problem& p, F f) {
+    if (p.D == 128) return f(Forward<Bf16Features, 128, 64, 4, 2>());
+    if (p.dtype == LA_F32) return p.D == 32 ? f(Forward<Fp32, 32, 32, 4, 2>()) : f(Forward<Fp32, 64, 64, 4, 2>());
+    return p.D == 32 ? f(Forward<Bf16, 32, 32, 8, 1>()) : f(Forward<Bf16, 64, 64, 8, 1>());
 }
-template <typename C, int DP, int MP, int STRIPS>
-int launch_backward(const la_problem& p, const BackwardParams& a, cudaStream_t st) {
-    constexpr int T = 16 * STRIPS;
-    return launch_cluster<causal_cluster_backward_kernel<C, DP, MP, STRIPS>>(kProfClusterBackward, 64 * STRIPS, (unsigned)((p.N + T - 1) / T),
-                                                                             (unsigned)(p.B * p.H), BackwardShared<C, DP, MP, STRIPS>::BYTES,
-                                                                             BackwardShared<C, DP, MP, STRIPS>::BYTES, a, st);
+template <typename F> auto with_backward(const la_problem& p, F f) {
+    if (p.D == 128) return f(Backward<Bf16Features, 128, 64>());
+    if (p.dtype == LA_F32) return p.D == 32 ? f(Backward<Fp32, 32, 32>()) : f(Backward<Fp32, 64, 64>());
+    return p.D == 32 ? f(Backward<Bf16, 32, 32>()) : f(Backward<Bf16, 64, 64>());
 }
-template <int DP, int STRIPS>
-int launch_linear(const la_problem& p, ClusterParams a, cudaStream_t st) {
-    constexpr int T = 16 * STRIPS;
-    const int64_t tiles = (p.N + T - 1) / T, per = (tiles + kMaxCluster - 1) / kMaxCluster;
-    a.piece_len = per * T;
-    return launch_cluster<linear_cluster_forward_kernel<DP, STRIPS>>(kProfClusterLinear, 32 * STRIPS, (unsigned)((tiles + per - 1) / per),
-                                                                          (unsigned)(p.B * p.H), per > 1 ? LinearShared<DP, STRIPS>::BYTES : LinearShared<DP, STRIPS>::STAGE,
-                                                                     LinearShared<DP, STRIPS>::BYTES, a, st);
-}
+template <typename F> auto with_linear(const la_problem& p, F f) { return p.D == 32 ? f(Linear<32>()) : f(Linear<64>()); }
 
 int64_t tiles_of(const la_problem& p, int rows) { return (p.N + rows - 1) / rows; }
 
@@ -1193,26 +1252,31 @@ bool square(const la_problem& p) { return p.D == p.M && (p.D == 32 || p.D == 64)
 //     50.3 / 34.3, 1x8x600 66.6 / 36.1, 1x8x1000 77.2 / 69.8 (seven clusters of sixteen run at once), 3x12x300 80.9 / 69.5, 16x8x256
 //     132 / 136
 //   and with the 128 Fourier features 1x8x1000 165 / 105, 8x8x142 114 / 98, 8x8x500 188 / 201
-bool causal_cluster_forward_preferred(const la_problem& p) {
+bool causal_cluster_forward_preferred(const la_problem& p, cudaStream_t st) {
     if (!enabled() || tc::causal_pieces_override() >= 0 || !(square(p) || fourier(p))) return false;
     const bool f32 = p.dtype == LA_F32;
     const int64_t tiles = tiles_of(p, f32 || fourier(p) ? 64 : 128), ctas = tiles * p.B * p.H;
-    if (f32 || fourier(p)) return tiles > 1 && tiles <= kMaxCluster && ctas <= (p.D == 32 ? 296 : 192);
-    return tiles > 2 && tiles <= kMaxCluster && (ctas <= (p.D == 32 ? 296 : tiles > 3 ? 200 : 148) || (tiles >= 8 && ctas <= 512));
+    const bool size = f32 || fourier(p) ? tiles > 1 && tiles <= kMaxCluster && ctas <= (p.D == 32 ? 296 : 192)
+                                        : tiles > 2 && tiles <= kMaxCluster && (ctas <= (p.D == 32 ? 296 : tiles > 3 ? 200 : 148) || (tiles >= 8 && ctas <= 512));
+    return size && with_forward(p, [&](auto k) { return decltype(k)::at_once(p, st); }) > 0;
 }
-bool causal_cluster_backward_preferred(const la_problem& p) {
+bool causal_cluster_backward_size(const la_problem& p) {
     if (!enabled() || tc::causal_pieces_override() >= 0 || !(square(p) || fourier(p))) return false;
     const int64_t tiles = tiles_of(p, 64);
     return tiles > (p.dtype == LA_BF16 && p.D == 64 ? 4 : 1) && tiles <= kMaxCluster && tiles * p.B * p.H <= (p.D == 32 ? 296 : 192);
 }
+bool causal_cluster_backward_preferred(const la_problem& p, cudaStream_t st) {
+    return causal_cluster_backward_size(p) && with_backward(p, [&](auto k) { return decltype(k)::at_once(p, st); }) > 0;
+}
 // Without a buffer for the sums / encoder forward + backward with one, whose sums need a kernel of their own: D = 64 1x8x64 12.1 / 8.3,
 // 1x8x1000 14.3 / 9.6 and 38.5 / 36.7, 1x8x2000 16.2 / 13.3 but 42.6 / 43.8, 4x8x1000 15.8 / 17.2; D = 32 1x8x1000 14.1 / 5.9 and
 // 37.8 / 31.7, 16x8x300 17.6 / 12.6, 8x8x777 19.2 / 13.8, 16x8x1000 26.0 / 26.9, 1x8x8192 22.7 / 16.0, 4x8x4096 26.1 / 28.9
-bool linear_cluster_preferred(const la_problem& p) {
+bool linear_cluster_preferred(const la_problem& p, cudaStream_t st) {
     if (!enabled() || tc::linear_splits_override() >= 0 || p.dtype != LA_BF16 || !square(p) || p.N < 1) return false;
     const int64_t tiles = tiles_of(p, 128);
-    if (p.D == 64) return tiles <= 12 && tiles * p.B * p.H <= 148;
-    return tiles <= kMaxCluster ? tiles * p.B * p.H <= 448 : tiles <= 4 * kMaxCluster && kMaxCluster * p.B * p.H <= 148;
+    const bool size = p.D == 64 ? tiles <= 12 && tiles * p.B * p.H <= 148
+                      : tiles <= kMaxCluster ? tiles * p.B * p.H <= 448 : tiles <= 4 * kMaxCluster && kMaxCluster * p.B * p.H <= 148;
+    return size && with_linear(p, [&](auto k) { return decltype(k)::at_once(p, st); }) > 0;
 }
 
 int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
@@ -1220,13 +1284,13 @@ int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, co
     ClusterParams a = cluster_params(p, lengths);
     a.Q = Q; a.K = K; a.V = V; a.O = O; a.den = den;
     a.S0 = S_in; a.Z0 = Z_in; a.S1 = S_out; a.Z1 = Z_out;
-    if (saved) {                // what the tcgen05 backward pass would find there, if that is the one to come
+    if (saved) {                // what the tcgen05 backward pass finds there, where that is the one to come
         const tc::CausalPlan pl = tc::choose_plan(p);
         const tc::SavedLayout l = tc::saved_layout(p, pl);
         char* sv = (char*)saved;
         a.stamp = (int*)(sv + l.stamp);
         if (p.phi == LA_PHI_ELU1) { a.keep_q = sv + l.phiq; a.keep_k = sv + l.phik; }
-        if (!causal_cluster_backward_preferred(p)) {
+        if (!causal_cluster_backward_size(p)) {
             tc::plan_stamp(pl, (int)p.D, a.stamp_value);
             if (pl.npieces() > 1) {
                 if (int rc = tc::causal_keep_records(p, K, V, lengths, saved, st)) return rc;
@@ -1234,9 +1298,7 @@ int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, co
             }
         }
     }
-    if (p.D == 128) return launch_forward<Bf16Features, 128, 64, 4, 2>(p, a, st);
-    if (p.dtype == LA_F32) return p.D == 32 ? launch_forward<Fp32, 32, 32, 4, 2>(p, a, st) : launch_forward<Fp32, 64, 64, 4, 2>(p, a, st);
-    return p.D == 32 ? launch_forward<Bf16, 32, 32, 8, 1>(p, a, st) : launch_forward<Bf16, 64, 64, 8, 1>(p, a, st);
+    return with_forward(p, [&](auto k) { return decltype(k)::launch(p, a, st); });
 }
 
 int causal_cluster_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
@@ -1245,9 +1307,7 @@ int causal_cluster_backward(const la_problem& p, const void* Q, const void* K, c
     static_cast<ClusterParams&>(a) = cluster_params(p, lengths);
     a.Q = Q; a.K = K; a.V = V; a.G = G; a.dQ = dQ; a.dK = dK; a.dV = dV;
     a.S0 = sa.S_in; a.Z0 = sa.Z_in; a.R0 = sa.dS_out; a.r0 = sa.dZ_out; a.R1 = sa.dS_in; a.r1 = sa.dZ_in;
-    if (p.D == 128) return launch_backward<Bf16Features, 128, 64, 4>(p, a, st);
-    if (p.dtype == LA_F32) return p.D == 32 ? launch_backward<Fp32, 32, 32, 4>(p, a, st) : launch_backward<Fp32, 64, 64, 4>(p, a, st);
-    return p.D == 32 ? launch_backward<Bf16, 32, 32, 4>(p, a, st) : launch_backward<Bf16, 64, 64, 4>(p, a, st);
+    return with_backward(p, [&](auto k) { return decltype(k)::launch(p, a, st); });
 }
 
 int linear_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O, float* den,
@@ -1258,7 +1318,7 @@ int linear_cluster_forward(const la_problem& p, const void* Q, const void* K, co
         if (int rc = tc::linear_keep_sums(p, K, V, lengths, saved, st)) return rc;
         a.late = 1;
     }
-    return p.D == 32 ? launch_linear<32, 8>(p, a, st) : launch_linear<64, 8>(p, a, st);
+    return with_linear(p, [&](auto k) { return decltype(k)::launch(p, a, st); });
 }
 
 }  // namespace la

@@ -30,15 +30,18 @@ int linear_mma_forward(const la_problem& p, const void* Q, const void* K, const 
 int linear_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* saved,
                         const void* G, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
 
-// Short sequences in one launch (la_cluster.cu): ahead of the other kernels where these say so.  saved (or null): filled for
-// the tcgen05 backward kernels.
-bool causal_cluster_forward_preferred(const la_problem& p);
-bool causal_cluster_backward_preferred(const la_problem& p);
+// Short sequences in one launch (la_cluster.cu): ahead of the other kernels where these say so, by the problem's size and by
+// whether the context of the stream has room for such a cluster.  saved (or null): filled for the tcgen05 backward kernels,
+// except where the size alone says that a cluster does the backward pass: no kernel reads the buffer there, also where the stream
+// of the backward call turns out to have no room.
+bool causal_cluster_forward_preferred(const la_problem& p, cudaStream_t st);
+bool causal_cluster_backward_size(const la_problem& p);
+bool causal_cluster_backward_preferred(const la_problem& p, cudaStream_t st);
 int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
                            const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, cudaStream_t st);
 int causal_cluster_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
                             const StateArgs& sa, void* dQ, void* dK, void* dV, cudaStream_t st);
-bool linear_cluster_preferred(const la_problem& p);
+bool linear_cluster_preferred(const la_problem& p, cudaStream_t st);
 int linear_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O, float* den,
                            float* KV, float* Zs, void* saved, cudaStream_t st);
 

@@ -180,3 +180,58 @@ def test_these_kernels_are_profiled_under_their_own_names():
     assert kernels_of(lambda: la.la_linear_attention(Q, K, V)) == {"linear_cluster_forward_kernel": 1}
     saved = la.linear_saved_buffer(Q, V)
     assert kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved)) == {"linear_sum_kernel": 1, "linear_cluster_forward_kernel": 1}
+
+
+@pytest.fixture(scope="module")
+def small_context():
+    """A stream whose context has eight of the device's SMs: no room for a cluster of more than eight CTAs."""
+    cu = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(r):
+        assert r[0] == cu.CUresult.CUDA_SUCCESS, r[0]
+        return r[1] if len(r) == 2 else r[1:]
+
+    torch.zeros(1, device=DEV)
+    dev = ok(cu.cuDeviceGet(0))
+    sms = ok(cu.cuDeviceGetDevResource(dev, cu.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM))
+    groups, _, _ = ok(cu.cuDevSmResourceSplitByCount(1, sms, 0, 8))
+    ctx = ok(cu.cuGreenCtxCreate(ok(cu.cuDevResourceGenerateDesc(groups, 1)), dev, cu.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    # (kept for the life of the process: the allocator remembers the stream)
+    return torch.cuda.ExternalStream(int(ok(cu.cuGreenCtxStreamCreate(ctx, cu.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))))
+
+
+@pytest.mark.parametrize("dtype,phi,D,M,N", [(torch.bfloat16, "elu1", 64, 64, 1030), (torch.bfloat16, "elu1", 32, 32, 1030),
+                                             (torch.bfloat16, "elu1", 32, 32, 600), (torch.bfloat16, "elu1", 64, 64, 600),
+                                             (torch.float32, "elu1", 64, 64, 600), (torch.float32, "elu1", 32, 32, 600),
+                                             (torch.bfloat16, "identity", 128, 64, 600)])
+def test_a_context_without_room_for_a_cluster(small_context, dtype, phi, D, M, N):
+    """The other kernels take the problem: same results to the usual tolerances, with a saved buffer too, whichever of the two
+    calls of a step ran where there was room."""
+    Q, K, V, G = draw_qkvg(1, 2, N, D, M, 31, dtype, 1.0 if D != 32 else 0.5)
+    if phi == "identity":
+        Q, K = Q.abs() + 0.1, K.abs() + 0.1
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    q, k, v, g = (t.double().numpy() for t in (Q, K, V, G))
+    Or, grads = oracle.linear_attention(q, k, v, causal=True, phi=phi)[0], oracle.linear_attention_backward(q, k, v, g, causal=True, phi=phi)
+    Ob = oracle.linear_attention(q, k, v, causal=False, phi=phi)[0]
+    streams = {"here": torch.cuda.current_stream(), "there": small_context}
+    torch.cuda.synchronize()
+    for f, b in (("there", "there"), ("here", "there"), ("there", "here")):
+        saved = la.saved_buffer(dev[0], dev[2], phi=phi)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(streams[f]):
+            if f == "there" and N > 1024:
+                n0 = la.la_kernel_launches()
+                la.la_causal_forward(*dev[:3], phi=phi)
+                assert la.la_kernel_launches() > n0 + 1
+            O = la.la_causal_forward(*dev[:3], phi=phi, saved=saved)
+            E = la.la_linear_attention(*dev[:3], phi=phi)
+            la.la_last_device_status()
+        with torch.cuda.stream(streams[b]):
+            out = la.la_causal_backward(*dev, phi=phi, saved=saved)
+            la.la_last_device_status()
+        for x, ref, nm in ((O, Or, "O"), (E, Ob, "E"), *zip(out, grads, ("dQ", "dK", "dV"))):
+            if D == M and dtype == torch.bfloat16:
+                assert_close(x, ref, dtype, f"{nm}, forward {f}, backward {b}", grad=nm[0] == "d")
+            else:
+                _close(x, ref, (8e-6 if nm[0] == "d" else 2e-6) if dtype == torch.float32 else 2 ** -7, nm)
