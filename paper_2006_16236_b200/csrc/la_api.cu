@@ -501,7 +501,7 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     LA_DEBUG_SPAN(den, tb.den); LA_DEBUG_SPAN(S_in, tb.s); LA_DEBUG_SPAN(Z_in, tb.z); LA_DEBUG_SPAN(S_out, tb.s);
     LA_DEBUG_SPAN(Z_out, tb.z); LA_DEBUG_SPAN(lengths, (size_t)p->B * 4); LA_DEBUG_SPAN(ws, ws_bytes);
     LA_DEBUG_SPAN(saved, saved_bytes);
-    if (causal_cluster_forward_preferred(*p, st))
+    if (causal_cluster_forward_preferred(*p, tc_path && saved, S_in != nullptr, st))
         return debug_finish(causal_cluster_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, tc_path ? saved : nullptr, st), stream);
     if (tc_path)
         return debug_finish(tc::causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, st), stream);

@@ -1264,34 +1264,57 @@ bool square(const la_problem& p) { return p.D == p.M && (p.D == 32 || p.D == 64)
 
 }  // namespace
 
-// Which problems: those that one wave of CTAs holds, or little more.  us, the other kernels / these, B x H x N:
-//   forward, bf16 (128 positions a CTA): up to 256 positions the tcgen05 kernel is one launch too (D = 64 1x8x128 5.1 / 9.4);
-//     D = 64: 1x8x600 16.7 / 8.5, 1x8x2048 22.2 / 11.7, 3x12x300 10.0 / 8.5, 16x8x300 13.9 / 21.5, 8x8x1000 28.6 / 23.1, 4x8x2048
-//     31.0 / 29.7, 16x8x1000 23.8 / 45; D = 32: 1x8x600 14.6 / 4.9, 3x12x300 8.1 / 5.2, 16x8x300 9.5 / 11.2, 8x8x1000 23.4 / 14.0
-//     (many CTAs pay only where the other kernel has many pieces to sum)
-//   backward (64 positions a CTA), bf16, from a saved buffer: D = 32 1x8x128 9.8 / 8.4, 1x8x1000 25.8 / 11.1, 8x8x250 15.2 / 10.0,
-//     2x8x1000 26.5 / 20.2; D = 64 1x8x128 10.3 / 14.4, 8x8x250 15.9 / 20.3, 2x8x500 24.6 / 18.9, 3x12x300 21.1 / 20.9, 2x8x1000
-//     27.6 / 34.5
-//   forward + backward, fp32 (64 a CTA): one CTA per sequence is no gain (1x2x64 D = 32 15.8 / 17.9); D = 32 1x2x256 26.3 / 17.8,
-//     1x8x1000 41.2 / 26.8, 8x8x250 45.5 / 31.5, 2x8x1000 55.4 / 47.2, 16x8x256 65.6 / 60.8, 4x8x1000 68.3 / 82.6; D = 64 1x2x256
-//     50.3 / 34.3, 1x8x600 66.6 / 36.1, 1x8x1000 77.2 / 69.8 (seven clusters of sixteen run at once), 3x12x300 80.9 / 69.5, 16x8x256
-//     132 / 136
-//   and with the 128 Fourier features 1x8x1000 165 / 105, 8x8x142 114 / 98, 8x8x500 188 / 201
-bool causal_cluster_forward_preferred(const la_problem& p, cudaStream_t st) {
+// Which problems: those that one wave of clusters holds (clusters_at_once(): on a whole B200 with two CTAs per SM 148 of 2 CTAs, 93 of
+// 3, 71 of 4, 45 of 6, 33 of 8, 26 of 10, 21 of 12, 14 of 14 to 16; with one 74, 45, 33, 22, 15, 11, 7, 7), or little more.
+// us of GPU time, the other kernels / these, B x H x N:
+//   forward, bf16 (128 positions a CTA, two CTAs per SM): up to 256 positions the tcgen05 kernel is one launch too (D = 64 1x8x128
+//     5.1 / 9.4).  D = 64: 1x8x600 16.4 / 7.7, 6x8x500 15.4 / 10.9, 1x8x2048 18.8 / 11.3; three tiles with CTAs that share an SM 5x8x384
+//     8.8 / 8.0, but 6x8x300 10.0 / 10.4, 6x8x384 9.0 / 10.8 (from a state, which costs the other kernel 3, 12.1 / 11.1); a second wave
+//     pays from eight tiles on (2x8x2048 22.7 / 18.1, 6x8x1024 21.4 / 20.8, 3x8x2048 23.2 / 21.8), a third does not (4x8x2048 27.4 / 29.0).
+//     D = 32: 1x8x600 14.2 / 4.5, 10x8x300 8.3 / 5.9 but 12x8x300, a second wave, 8.2 / 8.9; 9x8x512 16.6 / 8.8, 8x8x1000 20.8 / 11.3
+//   ... with a saved buffer whose records the tcgen05 backward kernels take, their pre-pass being on top: D = 64 6x8x500 15.9 / 13.2,
+//     4x8x1000 20.6 / 20.2, but in two waves 6x8x1024 22.1 / 25.1, 8x8x1000 24.8 / 31.9, 4x8x2048 28.4 / 36.4 (forward + backward 73.0 /
+//     85.0); D = 32 5x8x1024 19.5 / 14.8, 3x8x2048 21.1 / 19.0, 5x8x1536 22.2 / 22.4, 4x8x2048 24.4 / 24.8 (without the buffer 23.8 / 16.6)
+//   backward (64 positions a CTA), bf16: D = 32 4x8x576 34.4 / 18.5, 6x8x384 18.2 / 18.0, but 9x8x256, two chunks of the other kernel,
+//     14.9 / 15.9; D = 64 4x8x320 25.1 / 19.6, 1x8x1024 34.9 / 19.9, 2x8x704 35.7 / 20.3; 1x8x128 10.3 / 14.4
+//   fp32 (64 a CTA): one CTA per sequence is no gain (1x2x64 D = 32 15.8 / 17.9).  D = 64, one CTA per SM, forward and backward: 9x8x128 14.4 / 10.8
+//     and 36.7 / 23.4, 4x8x256 15.9 / 10.8 and 38.3 / 24.1, 1x6x1000 19.8 / 11.1 and 44.6 / 24.6; in two waves, the second well filled
+//     4x8x384 23.3 / 21.2 and 55.8 / 46.1, 7x8x192 19.3 / 20.3 and 49.5 / 44.9, 12x8x128 16.3 / 19.8 and 44.7 / 44.1, or not 6x8x192
+//     15.5 / 19.9 and 37.3 / 44.5, 3x8x384 16.3 / 20.7 and 38.0 / 45.2, 1x8x700 18.2 / 20.5 and 40.5 / 45.6.  D = 32, two CTAs: 5x8x384
+//     11.1 / 8.0 and 25.8 / 18.2; in two waves 12x8x192 10.6 / 12.1 and 25.5 / 28.3, 3x8x768 12.6 / 14.2 and 30.7 / 30.0, but these
+//     calls are bound by the host, two launches for one and six: 14.5 / 12.6 and 34.1 / 28.5, 16.7 / 14.4 and 39.2 / 31.1
+//   and with the 128 Fourier features, forward + backward 1x8x1000 130 / 75, 8x8x142 79 / 68, 3x8x512 117 / 73; 8x8x500 188 / 201
+int64_t waves(const la_problem& p, int64_t at_once) { return at_once > 0 ? (p.B * p.H + at_once - 1) / at_once : INT64_MAX; }
+// fp32, D = M = 64: one wave, or two of which the second is at least a fifth full
+bool well_filled(const la_problem& p, int64_t at_once) {
+    const int64_t w = waves(p, at_once);
+    return w == 1 || (w == 2 && 5 * p.B * p.H >= 6 * at_once);
+}
+
+// saved: with a buffer for the tcgen05 backward kernels; state: from a given state
+bool causal_cluster_forward_preferred(const la_problem& p, bool saved, bool state, cudaStream_t st) {
     if (!enabled() || tc::causal_pieces_override() >= 0 || !(square(p) || fourier(p))) return false;
-    const bool f32 = p.dtype == LA_F32;
-    const int64_t tiles = tiles_of(p, f32 || fourier(p) ? 64 : 128), ctas = tiles * p.B * p.H;
-    const bool size = f32 || fourier(p) ? tiles > 1 && tiles <= kMaxCluster && ctas <= (p.D == 32 ? 296 : 192)
-                                        : tiles > 2 && tiles <= kMaxCluster && (ctas <= (p.D == 32 ? 296 : tiles > 3 ? 200 : 148) || (tiles >= 8 && ctas <= 512));
-    return size && with_forward(p, [&](auto k) { return decltype(k)::at_once(p, st); }) > 0;
+    const bool exact = p.dtype == LA_F32 || fourier(p);
+    const int64_t tiles = tiles_of(p, exact ? 64 : 128), ctas = tiles * p.B * p.H;
+    if (tiles <= (exact ? 1 : 2) || tiles > kMaxCluster || ctas > 512) return false;
+    const int64_t at_once = with_forward(p, [&](auto k) { return decltype(k)::at_once(p, st); }), w = waves(p, at_once);
+    if (at_once == 0) return false;
+    if (exact && p.D == 64) return ctas <= 192 && well_filled(p, at_once) && (w == 1 || tiles > 2);
+    if (exact) return ctas <= (p.D == 32 ? 296 : 192);
+    if (p.D == 32) return (ctas <= 296 && (tiles > 3 || w == 1)) || tiles >= 8;
+    const bool records = saved && !causal_cluster_backward_size(p);
+    return ctas <= (tiles > 3 ? 200 : state ? 148 : 132) || (tiles >= 8 && w <= (records ? 1 : 2));
 }
 bool causal_cluster_backward_size(const la_problem& p) {
     if (!enabled() || tc::causal_pieces_override() >= 0 || !(square(p) || fourier(p))) return false;
-    const int64_t tiles = tiles_of(p, 64);
-    return tiles > (p.dtype == LA_BF16 && p.D == 64 ? 4 : 1) && tiles <= kMaxCluster && tiles * p.B * p.H <= (p.D == 32 ? 296 : 192);
+    const bool bf16 = p.dtype == LA_BF16;
+    const int64_t tiles = tiles_of(p, 64), ctas = tiles * p.B * p.H;
+    return tiles > (bf16 && p.D == 64 ? 4 : 1) && tiles <= kMaxCluster && ctas <= (p.D == 32 ? (bf16 && tiles == 4 ? 256 : 296) : 192);
 }
 bool causal_cluster_backward_preferred(const la_problem& p, cudaStream_t st) {
-    return causal_cluster_backward_size(p) && with_backward(p, [&](auto k) { return decltype(k)::at_once(p, st); }) > 0;
+    if (!causal_cluster_backward_size(p)) return false;
+    const int64_t at_once = with_backward(p, [&](auto k) { return decltype(k)::at_once(p, st); });
+    return at_once > 0 && (p.dtype == LA_BF16 || p.D == 32 || well_filled(p, at_once));
 }
 // Without a buffer for the sums / encoder forward + backward with one, whose sums need a kernel of their own: D = 64 1x8x64 12.1 / 8.3,
 // 1x8x1000 14.3 / 9.6 and 38.5 / 36.7, 1x8x2000 16.2 / 13.3 but 42.6 / 43.8, 4x8x1000 15.8 / 17.2; D = 32 1x8x1000 14.1 / 5.9 and

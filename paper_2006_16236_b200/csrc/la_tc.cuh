@@ -34,7 +34,7 @@ int linear_mma_backward(const la_problem& p, const void* Q, const void* K, const
 // whether the context of the stream has room for such a cluster.  saved (or null): filled for the tcgen05 backward kernels,
 // except where the size alone says that a cluster does the backward pass: no kernel reads the buffer there, also where the stream
 // of the backward call turns out to have no room.
-bool causal_cluster_forward_preferred(const la_problem& p, cudaStream_t st);
+bool causal_cluster_forward_preferred(const la_problem& p, bool saved, bool state, cudaStream_t st);
 bool causal_cluster_backward_size(const la_problem& p);
 bool causal_cluster_backward_preferred(const la_problem& p, cudaStream_t st);
 int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,

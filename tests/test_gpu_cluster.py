@@ -235,3 +235,42 @@ def test_a_context_without_room_for_a_cluster(small_context, dtype, phi, D, M, N
                 assert_close(x, ref, dtype, f"{nm}, forward {f}, backward {b}", grad=nm[0] == "d")
             else:
                 _close(x, ref, (8e-6 if nm[0] == "d" else 2e-6) if dtype == torch.float32 else 2 ** -7, nm)
+
+
+SUM, FWD, MMA = "segment_sum_kernel", "causal_fwd_kernel", "causal_mma_forward_kernel"
+CLUSTER, GRADIENTS = "causal_cluster_forward_kernel", "causal_cluster_backward_kernel"
+
+
+@pytest.mark.parametrize("dtype,D,BHN,state,saved,want", [
+    (torch.bfloat16, 64, (6, 8, 1024), False, False, {CLUSTER}),               # two waves ...
+    (torch.bfloat16, 64, (6, 8, 1024), False, True, {SUM, FWD}),               # ... are none with the records on top
+    (torch.bfloat16, 64, (6, 8, 500), False, True, {SUM, CLUSTER}),            # one wave is, beside the pre-pass
+    (torch.bfloat16, 64, (4, 8, 2048), False, False, {SUM, FWD}),              # three waves
+    (torch.bfloat16, 64, (2, 8, 384), False, False, {CLUSTER}),                # three tiles, an SM each ...
+    (torch.bfloat16, 64, (6, 8, 384), False, False, {FWD}),                    # ... or shared ...
+    (torch.bfloat16, 64, (6, 8, 384), True, False, {CLUSTER}),                 # ... from a state
+    (torch.bfloat16, 64, (1, 8, 256), False, False, {FWD}),
+    (torch.bfloat16, 32, (7, 8, 300), False, False, {CLUSTER}),
+    (torch.bfloat16, 32, (7, 14, 300), False, False, {FWD}),                   # a second wave of three tiles
+    (torch.bfloat16, 32, (5, 8, 1024), False, True, {SUM, CLUSTER}),
+    (torch.float32, 64, (4, 8, 128), False, False, {CLUSTER}),
+    (torch.float32, 64, (12, 8, 128), False, False, {MMA}),                    # a second wave of two tiles
+    (torch.float32, 64, (4, 8, 64), False, False, {MMA}),
+    (torch.float32, 32, (12, 8, 192), False, False, {CLUSTER})], ids=str)
+def test_which_kernel_takes_a_forward_pass(dtype, D, BHN, state, saved, want):
+    B, H, N = BHN
+    Q, K, V = (torch.zeros(B, H, N, D, dtype=dtype, device=DEV) for _ in range(3))
+    kw = {"S_in": torch.zeros(B, H, D, D, device=DEV), "Z_in": torch.zeros(B, H, D, device=DEV)} if state else {}
+    names = kernels_of(lambda: la.la_causal_forward(Q, K, V, saved=la.saved_buffer(Q, V) if saved else None, **kw))
+    assert set(names) - {"causal_mma_sum_kernel"} == want
+
+
+@pytest.mark.parametrize("dtype,D,BHN,cluster", [
+    (torch.bfloat16, 64, (1, 8, 257), True), (torch.bfloat16, 64, (1, 8, 256), False), (torch.bfloat16, 64, (1, 12, 1024), True),
+    (torch.bfloat16, 64, (1, 13, 1024), False), (torch.bfloat16, 32, (8, 8, 256), True), (torch.bfloat16, 32, (9, 8, 256), False),
+    (torch.bfloat16, 32, (6, 8, 384), True), (torch.bfloat16, 32, (1, 8, 64), False), (torch.float32, 64, (4, 8, 128), True),
+    (torch.float32, 64, (12, 8, 128), True), (torch.float32, 64, (20, 1, 256), True), (torch.float32, 64, (10, 8, 128), False)], ids=str)
+def test_which_kernel_takes_a_backward_pass(dtype, D, BHN, cluster):
+    Q, K, V, G = (torch.zeros(*BHN, D, dtype=dtype, device=DEV) for _ in range(4))
+    names = kernels_of(lambda: la.la_causal_backward(Q, K, V, G))
+    assert (set(names) == {GRADIENTS}) if cluster else (len(names) > 1 and GRADIENTS not in names)
