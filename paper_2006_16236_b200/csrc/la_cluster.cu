@@ -1316,15 +1316,19 @@ bool causal_cluster_backward_preferred(const la_problem& p, cudaStream_t st) {
     const int64_t at_once = with_backward(p, [&](auto k) { return decltype(k)::at_once(p, st); });
     return at_once > 0 && (p.dtype == LA_BF16 || p.D == 32 || well_filled(p, at_once));
 }
-// Without a buffer for the sums / encoder forward + backward with one, whose sums need a kernel of their own: D = 64 1x8x64 12.1 / 8.3,
-// 1x8x1000 14.3 / 9.6 and 38.5 / 36.7, 1x8x2000 16.2 / 13.3 but 42.6 / 43.8, 4x8x1000 15.8 / 17.2; D = 32 1x8x1000 14.1 / 5.9 and
-// 37.8 / 31.7, 16x8x300 17.6 / 12.6, 8x8x777 19.2 / 13.8, 16x8x1000 26.0 / 26.9, 1x8x8192 22.7 / 16.0, 4x8x4096 26.1 / 28.9
+// GPU us without a buffer for the sums / encoder forward + backward with one, whose sums need a kernel of their own (results do not
+// depend on the buffer, so neither does the rule: where the two disagree a training step loses less than an encoder gains): D = 64 1x8x64
+// 11.5 / 8.1 and 27.2 / 27.0, 1x8x1000 14.2 / 9.3 and 37.1 / 34.6, 4x8x384 15.4 / 8.8 and 40.8 / 36.0, 1x12x1500 16.1 / 14.2 and 40.5 / 41.8,
+// 18x8x100 13.2 / 8.6 and 32.1 / 36.5; D = 32 1x8x1000 13.9 / 5.9 and 36.5 / 30.3, 56x8x128 42.0 / 12.2 and 101 / 90, 4x8x1024 15.0 / 8.0 and
+// 38.2 / 39.3, 8x8x777 18.9 / 13.5 and 48.8 / 51.7, 3x8x1800 18.5 / 14.4 and 46.6 / 51.6, but in three waves 4x8x1700 18.3 / 20.2 and 49.0 /
+// 59.0.  More than a tile per CTA: 1x8x4096 18.6 / 10.4 and 47.8 / 48.1, 1x8x8192 22.1 / 15.7 and 58.9 / 62.8, 4x8x4096 26.1 / 28.9
 bool linear_cluster_preferred(const la_problem& p, cudaStream_t st) {
     if (!enabled() || tc::linear_splits_override() >= 0 || p.dtype != LA_BF16 || !square(p) || p.N < 1) return false;
     const int64_t tiles = tiles_of(p, 128);
-    const bool size = p.D == 64 ? tiles <= 12 && tiles * p.B * p.H <= 148
-                      : tiles <= kMaxCluster ? tiles * p.B * p.H <= 448 : tiles <= 4 * kMaxCluster && kMaxCluster * p.B * p.H <= 148;
-    return size && with_linear(p, [&](auto k) { return decltype(k)::at_once(p, st); }) > 0;
+    if (p.D == 64 ? tiles > 12 || tiles * p.B * p.H > 148
+                  : tiles <= kMaxCluster ? tiles * p.B * p.H > 448 : tiles > 4 * kMaxCluster || kMaxCluster * p.B * p.H > 148) return false;
+    const int64_t at_once = with_linear(p, [&](auto k) { return decltype(k)::at_once(p, st); });
+    return waves(p, at_once) <= 2;
 }
 
 int causal_cluster_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,

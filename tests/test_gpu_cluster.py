@@ -274,3 +274,14 @@ def test_which_kernel_takes_a_backward_pass(dtype, D, BHN, cluster):
     Q, K, V, G = (torch.zeros(*BHN, D, dtype=dtype, device=DEV) for _ in range(4))
     names = kernels_of(lambda: la.la_causal_backward(Q, K, V, G))
     assert (set(names) == {GRADIENTS}) if cluster else (len(names) > 1 and GRADIENTS not in names)
+
+
+@pytest.mark.parametrize("D,BHN,cluster", [(64, (1, 8, 1536), True), (64, (1, 8, 1537), False), (64, (18, 8, 128), True), (64, (19, 8, 128), False),
+                                           (32, (56, 8, 128), True), (32, (57, 8, 128), False), (32, (4, 8, 1700), False), (32, (3, 8, 2048), True),
+                                           (32, (1, 8, 8192), True), (32, (1, 8, 8193), False), (32, (2, 8, 2049), False)], ids=str)
+def test_which_kernel_takes_a_bidirectional_forward_pass(D, BHN, cluster):
+    Q, K, V = (torch.zeros(*BHN, D, dtype=torch.bfloat16, device=DEV) for _ in range(3))
+    want = {"linear_cluster_forward_kernel"} if cluster else {"linear_sum_kernel", "linear_apply_kernel"}
+    assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V))) == want
+    saved = la.linear_saved_buffer(Q, V)
+    assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved))) == want | {"linear_sum_kernel"}
