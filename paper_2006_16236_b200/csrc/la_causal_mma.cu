@@ -676,11 +676,29 @@ causal_mma_dkv_kernel(const Params p) {
 // ---- host ------------------------------------------------------------------------------------------------------
 struct Plan { int pieces; int64_t len; };
 
-// Pieces per sequence, by the estimated time in units of one chunk of a main kernel (about 10 us alone on an SM).
-// fp32 D = M = 64 and Fourier features, whose kernels leave an SM little to gain from a second CTA (0.9 of the time of the two one
-// after the other; a pre-pass costs 0.16 per chunk and 1.3), forward + backward in us at the pieces of the other rule / of
-// this one (B x H x N: pieces): fp32 4x8x1000 8: 163 / 4: 150, 16x8x256 2: 132 / 1: 108, 16x8x2000 2: 829 / 1: 765, 2x8x4096 16: 306 /
-// 8: 283; Fourier 3x8x2666 11: 290 / 6: 233, 4x8x1500 8: 227 / 4: 195, 8x8x500 4: 152 / 2: 133, 16x8x1000 2: 380 / 1: 349.  The others:
+// The estimates of choose_plan() for kernels that leave an SM little to gain from a second CTA, in units of one chunk of the main
+// kernels (forward and backward together, 21.8 us in fp32 and 19.4 with Fourier features) of a CTA that has an SM to itself: their time
+// with 1 to 5 CTAs per SM (uneven: with two on some, 149 to 221) and for each of more, a CTA's start and what each record costs it, the
+// pre-pass's time per chunk, its start, and its time for each CTA per SM.  An odd CTA out has its SM to itself at the end, so that 3 and 5
+// are hardly less than 4 and 6.  Chosen over forced pieces of 8 to 352 sequences of 2 to 64 chunks: 0.5 % above the best number of pieces in the mean
+// where the other rule is 5.3 % (fp32) and 10.6 % (Fourier) above it, and never slower than that one by more than 8 and 4 %.  us, forward +
+// backward, at the pieces of the other rule / of this one (B x H x N: pieces): fp32 4x8x1416 8: 207 / 4: 198, 15x8x2354 2: 953 / 1: 824;
+// Fourier 3x8x1999 11: 241 / 6: 188, 13x8x1271 5: 441 / 1: 402, 23x8x405 1: 316 / 2: 271.
+struct WideCosts { double sms[5], uneven, more_sms, start, record, sum, sum_start, sum_sms; };
+constexpr WideCosts kFp32Costs = {{1.0, 1.86, 3.44, 3.85, 7.19}, 1.92, 0.91, 0.34, 0.12, 0.18, 1.03, 0.58};
+constexpr WideCosts kFourierCosts = {{1.0, 1.9, 3.33, 3.64, 5.0}, 2.39, 0.92, 0.85, 0.2, 0.17, 1.22, 0.45};
+
+double wide_cost(const WideCosts& w, int64_t bh, int64_t chunks, int64_t n) {
+    const int64_t per = (chunks + n - 1) / n, cut = (chunks + per - 1) / per;        // cut: the pieces that this makes
+    auto sms = [&](int64_t pieces) { return (bh * pieces + 147) / 148; };
+    const int64_t m = sms(cut);
+    double t = ((double)per + w.start + w.record * (double)(cut - 1)) * (m == 2 && bh * cut < 222 ? w.uneven : m <= 5 ? w.sms[m - 1] : w.more_sms * (double)m);
+    if (cut > 1) t += w.sum * (double)per * (sms(cut - 1) == 1 ? 1.0 : w.sum_sms * (double)sms(cut - 1)) + w.sum_start;
+    return t;
+}
+
+// Pieces per sequence, by the estimated time: fp32 D = M = 64 and Fourier features as above; the others in units of one chunk of a main
+// kernel (about 10 us alone on an SM):
 // an SM runs two CTAs in 1.25 times the time of one; a CTA's start costs about a chunk, and 0.2 for each record it sums, of
 // which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk (fp32 D = M = 32, B4 H8 N2000,
 // pieces 1 / 4 / 8 / 12 / 16: 353 / 141 / 113 / 131 / 119; B22 H8 N3316 903 / 732 / 749 / 733 / 757).  At most sixteen: the estimates
@@ -697,17 +715,13 @@ Plan choose_plan(const la_problem& p, bool single) {
         if (best > 1024) best = 1024;
     } else {
         const bool wide = p.dtype == LA_F32 ? p.D == 64 && p.M == 64 : p.phi == LA_PHI_IDENTITY && p.D == 128 && p.M == 64;
-        auto waves = [&](int64_t ctas) {
+        auto waves = [](int64_t ctas) {
             const int64_t sm = (ctas + 147) / 148;
-            if (wide) return sm == 1 ? 1.0 : 0.9 * (double)sm;
             return 1.25 * (double)(sm / 2) + (double)(sm % 2);
         };
         auto cost = [&](int64_t n) {
+            if (wide) return wide_cost(p.dtype == LA_F32 ? kFp32Costs : kFourierCosts, bh, chunks, n);
             const double per = (double)((chunks + n - 1) / n);
-            if (wide) {
-                const int64_t cut = (chunks + (int64_t)per - 1) / (int64_t)per;         // pieces that this makes
-                return (per + 0.5 + 0.1 * (cut - 1)) * waves(bh * cut) + (cut > 1 ? 0.16 * per * waves(bh * (cut - 1)) + 1.3 : 0.0);
-            }
             return (per + 1.0 + 0.1 * (n - 1)) * waves(bh * n) + (n > 1 ? 0.35 * (per + 1.0) * waves(bh * (n - 1)) : 0.0);
         };
         for (int64_t n = 2; n <= 16 && n <= chunks; ++n)
