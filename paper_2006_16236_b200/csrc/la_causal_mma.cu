@@ -678,21 +678,23 @@ struct Plan { int pieces; int64_t len; };
 
 // The estimates of choose_plan() for kernels that leave an SM little to gain from a second CTA, in units of one chunk of the main
 // kernels (forward and backward together, 21.8 us in fp32 and 19.4 with Fourier features) of a CTA that has an SM to itself: their time
-// with 1 to 5 CTAs per SM (uneven: with two on some, 149 to 221) and for each of more, a CTA's start and what each record costs it, the
-// pre-pass's time per chunk, its start, and its time for each CTA per SM.  An odd CTA out has its SM to itself at the end, so that 3 and 5
-// are hardly less than 4 and 6.  Chosen over forced pieces of 8 to 352 sequences of 2 to 64 chunks: 0.5 % above the best number of pieces in the mean
-// where the other rule is 5.3 % (fp32) and 10.6 % (Fourier) above it, and never slower than that one by more than 8 and 4 %.  us, forward +
-// backward, at the pieces of the other rule / of this one (B x H x N: pieces): fp32 4x8x1416 8: 207 / 4: 198, 15x8x2354 2: 953 / 1: 824;
-// Fourier 3x8x1999 11: 241 / 6: 188, 13x8x1271 5: 441 / 1: 402, 23x8x405 1: 316 / 2: 271.
-struct WideCosts { double sms[5], uneven, more_sms, start, record, sum, sum_start, sum_sms; };
-constexpr WideCosts kFp32Costs = {{1.0, 1.86, 3.44, 3.85, 7.19}, 1.92, 0.91, 0.34, 0.12, 0.18, 1.03, 0.58};
-constexpr WideCosts kFourierCosts = {{1.0, 1.9, 3.33, 3.64, 5.0}, 2.39, 0.92, 0.85, 0.2, 0.17, 1.22, 0.45};
+// with 1 to 5 CTAs per SM (uneven: with two on some, 149 to 221), for each of more, and for an odd one among those; a CTA's start
+// and what each record costs it; the pre-pass's time per chunk, its start, and its time for each CTA per SM.  A CTA left over has its SM
+// to itself, so that 3 and 5 are hardly less than 4 and 6.  Chosen over forced pieces of 8 to 352 sequences of 2 to 64 chunks: 0.5 % above
+// the best number of pieces in the mean where the other rule is 5.3 % (fp32) and 10.6 % (Fourier) above it, and slower than that one in
+// 7 of 460 and 9 of 350 cases, by 6 and 4 % at most.  us, forward + backward, at the pieces of the other rule / of this one (B x H x N:
+// pieces): fp32 4x8x1416 8: 207 / 4: 198, 15x8x2354 2: 953 / 1: 824; Fourier 3x8x1999 11: 241 / 6: 188, 13x8x1271 5: 441 / 1: 402, 23x8x405
+// 1: 316 / 2: 271.
+struct WideCosts { double sms[5], uneven, more_sms, odd, start, record, sum, sum_start, sum_sms; };
+constexpr WideCosts kFp32Costs = {{1.0, 1.86, 3.44, 3.8, 5.5}, 1.92, 0.94, 1.7, 0.34, 0.12, 0.18, 1.03, 0.58};
+constexpr WideCosts kFourierCosts = {{1.0, 1.9, 3.33, 3.64, 5.0}, 2.39, 0.92, 0.92, 0.85, 0.2, 0.17, 1.22, 0.45};
 
 double wide_cost(const WideCosts& w, int64_t bh, int64_t chunks, int64_t n) {
     const int64_t per = (chunks + n - 1) / n, cut = (chunks + per - 1) / per;        // cut: the pieces that this makes
     auto sms = [&](int64_t pieces) { return (bh * pieces + 147) / 148; };
     const int64_t m = sms(cut);
-    double t = ((double)per + w.start + w.record * (double)(cut - 1)) * (m == 2 && bh * cut < 222 ? w.uneven : m <= 5 ? w.sms[m - 1] : w.more_sms * (double)m);
+    double t = (double)per + w.start + w.record * (double)(cut - 1);
+    t *= m == 2 && bh * cut < 222 ? w.uneven : m <= 5 ? w.sms[m - 1] : w.more_sms * (double)(m - m % 2) + w.odd * (double)(m % 2);
     if (cut > 1) t += w.sum * (double)per * (sms(cut - 1) == 1 ? 1.0 : w.sum_sms * (double)sms(cut - 1)) + w.sum_start;
     return t;
 }
@@ -708,13 +710,13 @@ Plan choose_plan(const la_problem& p, bool single) {
     const int64_t chunks = (p.N + T - 1) / T, bh = p.B * p.H;
     int64_t best = 1;
     const int forced = tc::causal_pieces_override();
+    const bool wide = p.dtype == LA_F32 ? p.D == 64 && p.M == 64 : p.phi == LA_PHI_IDENTITY && p.D == 128 && p.M == 64;
     if (single) {
         best = 1;
     } else if (forced > 0) {
         best = forced < chunks ? forced : chunks;
         if (best > 1024) best = 1024;
-    } else {
-        const bool wide = p.dtype == LA_F32 ? p.D == 64 && p.M == 64 : p.phi == LA_PHI_IDENTITY && p.D == 128 && p.M == 64;
+    } else if (!(wide && bh >= 222 && bh <= 296)) {          // (two CTAs on an SM as they are: one piece was the best of 112 measured sizes of 2 to 64 chunks)
         auto waves = [](int64_t ctas) {
             const int64_t sm = (ctas + 147) / 148;
             return 1.25 * (double)(sm / 2) + (double)(sm % 2);

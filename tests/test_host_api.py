@@ -50,6 +50,16 @@ def test_workspace_sizes_are_independent_of_n_times_d_times_m(L):
     assert la.la_workspace_bytes(la.make_problem(1, 1, 128, 256, 64, 0), 3) == 0   # invalid -> 0
 
 
+@pytest.mark.parametrize("dt,phi,D,BHN,pieces", [
+    # Fourier features and fp32 D = 64: what was measured best of neighbouring counts, an odd number of CTAs per SM among them
+    (binding.LA_BF16, 1, 128, (30, 8, 2072), 1), (binding.LA_BF16, 1, 128, (13, 8, 1271), 1), (binding.LA_BF16, 1, 128, (10, 8, 639), 1),
+    (binding.LA_BF16, 1, 128, (22, 8, 1500), 3), (binding.LA_BF16, 1, 128, (3, 8, 2666), 6), (binding.LA_F32, 0, 64, (26, 8, 2027), 4),
+    (binding.LA_F32, 0, 64, (15, 8, 2354), 1), (binding.LA_F32, 0, 64, (2, 8, 4096), 8), (binding.LA_F32, 0, 64, (32, 8, 4096), 1)], ids=str)
+def test_pieces_of_the_fp32_accurate_causal_kernels(L, dt, phi, D, BHN, pieces):
+    p = la.make_problem(*BHN, D, 64, dt, phi)
+    assert la.la_workspace_bytes(p, binding.LA_OP_CAUSAL_FORWARD) == BHN[0] * BHN[1] * (pieces - 1) * D * 65 * 4
+
+
 def _p(**kw):
     base = dict(B=1, H=1, N=128, D=64, M=64, dtype_code=binding.LA_F32)
     base.update(kw)
