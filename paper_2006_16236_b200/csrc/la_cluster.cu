@@ -93,6 +93,29 @@ template <int DP, int MP> struct Inbox {
     }
 };
 
+// Four numbers, in packed pairs (an addition of two is one instruction)
+struct Four {
+    sm100::f32x2 a, b;
+    __device__ __forceinline__ Four() : a(0), b(0) {}
+    __device__ __forceinline__ Four(const float* p) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        a = sm100::pair(v.x, v.y);
+        b = sm100::pair(v.z, v.w);
+    }
+    __device__ __forceinline__ Four operator+(const Four& y) const {
+        Four r;
+        r.a = sm100::add2(a, y.a);
+        r.b = sm100::add2(b, y.b);
+        return r;
+    }
+    __device__ __forceinline__ float4 get() const {
+        float4 v;
+        sm100::unpair(a, v.x, v.y);
+        sm100::unpair(b, v.z, v.w);
+        return v;
+    }
+};
+
 // Four numbers of a state's matrix as operand planes, for CTA c.
 template <int NS, int DP, int MP>
 __device__ __forceinline__ void give_planes(uint32_t tile, const float4& v, int c) {
@@ -118,17 +141,17 @@ __device__ __forceinline__ void running_sums(const Exchange& x, const float* S0,
     in.template for_own_rows<THREADS>(reinterpret_cast<const float*>(x.inbox), [&](int d, int e, const float* from) {
         // (the given state, often much larger than the sums, is added to each of them and not a term that they start with: one
         // rounding of its size instead of sixteen)
-        float4 run = make_float4(0.f, 0.f, 0.f, 0.f), s0 = run;
-        if (S0) s0 = *reinterpret_cast<const float4*>(S0 + d * MP + e);
+        Four run, s0;
+        if (S0) s0 = Four(S0 + d * MP + e);
         const uint32_t tile = x.tile + tile_at<MP>(d, e / 8) + e % 8 * 2;
 #pragma unroll 4
         for (int i = 0; i < R; ++i) {
             const int c = ORDER == kBefore ? i : R - 1 - i;
-            const float4 v = *reinterpret_cast<const float4*>(from + c * slot);
-            give_planes<NS, DP, MP>(tile, make_float4(run.x + s0.x, run.y + s0.y, run.z + s0.z, run.w + s0.w), c);
-            run.x += v.x; run.y += v.y; run.z += v.z; run.w += v.w;
+            const Four v(from + c * slot);
+            give_planes<NS, DP, MP>(tile, (run + s0).get(), c);
+            run = run + v;
         }
-        if (S1) *reinterpret_cast<float4*>(S1 + d * MP + e) = make_float4(run.x + s0.x, run.y + s0.y, run.z + s0.z, run.w + s0.w);
+        if (S1) *reinterpret_cast<float4*>(S1 + d * MP + e) = (run + s0).get();
     }, [&](int d, int c, const float* from) {
         const int before = ORDER == kBefore ? c : R - 1 - c;           // CTAs ahead of c
         const float z0 = Z0 ? Z0[d] : 0.f;
