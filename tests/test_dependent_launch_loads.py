@@ -20,9 +20,11 @@ def _code(name):
 READ_ONLY = r"__ldg\s*\(|ld\.global\.nc|const \w+\s*\*\s*__restrict__"
 
 
-@pytest.mark.parametrize("name", ["la_mma.cuh", "la_mma_sweep.cuh", "la_causal_mma.cu", "la_linear_mma.cu", "la_tc_common.cuh",
-                                  "la_tc_causal_fwd.cu", "la_tc_causal_bwd.cu", "la_tc_segment.cu", "la_tc_linear.cu",
-                                  "la_decode_layer.cu", "la_sm100.cuh"])
+NO_READ_ONLY_LOADS = ["la_mma.cuh", "la_mma_sweep.cuh", "la_causal_mma.cu", "la_linear_mma.cu", "la_tc_common.cuh", "la_tc_causal_fwd.cu",
+                      "la_tc_causal_bwd.cu", "la_tc_segment.cu", "la_tc_linear.cu", "la_decode_layer.cu", "la_sm100.cuh", "la_cluster.cu", "la_common.cuh", "la_tc.cuh"]
+
+
+@pytest.mark.parametrize("name", NO_READ_ONLY_LOADS)
 def test_no_read_only_loads(name):
     assert not re.findall(READ_ONLY, _code(name))
 
@@ -38,3 +40,8 @@ def test_the_chained_kernel_of_the_elementwise_file():
 def test_no_other_file_launches_programmatic_dependents():
     known = {"la_mma_sweep.cuh", "la_tc_common.cuh", "la_elementwise.cu"}       # where the launch attribute is set
     assert {n for n in os.listdir(CSRC) if "ProgrammaticStreamSerialization" in _code(n)} == known
+    by_helper = {n for n in os.listdir(CSRC) if re.search(r"\bchained_launch\s*\(", _code(n))}
+    assert by_helper == {"la_tc_common.cuh", "la_cluster.cu", "la_decode_layer.cu", "la_tc_causal_bwd.cu", "la_tc_causal_fwd.cu", "la_tc_linear.cu",
+                         "la_tc_segment.cu"}
+    waits = {n for n in os.listdir(CSRC) if re.search(r"\b(grid_dependency_wait|wait_for_stream)\s*\(|griddepcontrol\.wait", _code(n))}
+    assert waits - {"la_elementwise.cu"} <= set(NO_READ_ONLY_LOADS)

@@ -38,16 +38,30 @@ def _untouched(tails):
         assert bool((tail == MARK).all()), f"{nm}: something was stored behind the tensor's end"
 
 
+@pytest.fixture
+def tcgen05(request):
+    """Whether the calls are kept to the tcgen05 kernels: plans that are forced, to pieces and splits as the automatic ones
+    choose about, leave out the kernels with a cluster per sequence that would take short problems."""
+    yield request.param
+    la.la_plan_override()
+
+
+ROUTES = pytest.mark.parametrize("tcgen05", [False, True], ids=["automatic", "tcgen05"], indirect=True)
+CLUSTER, TC = {"causal_cluster_forward_kernel", "causal_cluster_backward_kernel"}, {"causal_fwd_kernel", "causal_bwd_dq_kernel", "causal_bwd_dkv_kernel"}
+
 SHAPES = [(2, 3, 100, 64), (2, 3, 129, 64), (1, 5, 200, 32), (2, 8, 784, 32), (3, 2, 1000, 64), (1, 70, 700, 64),
           (2, 2, 1, 64), (1, 3, 127, 32), (1, 2, 2, 32)]
 
 
 @pytest.mark.parametrize("keep", [False, True], ids=["recompute", "saved"])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "B%d_H%d_N%d_D%d" % s)
-def test_causal_any_length(shape, keep):
+@ROUTES
+def test_causal_any_length(tcgen05, shape, keep):
     B, H, N, D = shape
     p = la.make_problem(B, H, N, D, D, la.LA_BF16)
     assert la.la_causal_plan(p) is not None, "this shape is meant to run the tensor-core kernels"
+    if tcgen05:
+        la.la_plan_override(causal_pieces=min(3, (N + 127) // 128))
     Q, K, V, G = draw_qkvg(B, H, N, D, D, 7 + N, torch.bfloat16, 1.0)
     tails = {}
     dev = {}
@@ -61,9 +75,13 @@ def test_causal_any_length(shape, keep):
     Z, tails["Z"] = _front((B, H, D), torch.float32)
     saved = la.saved_buffer(dev["Q"], dev["V"]) if keep else None
     kw = {"saved": saved} if keep else {}
+    la.la_profile_enable(True)
     la.la_causal_forward(dev["Q"], dev["K"], dev["V"], O=outs["O"], den=den, S_out=S, Z_out=Z, **kw)
     la.la_causal_backward(dev["Q"], dev["K"], dev["V"], dev["G"], dQ=outs["dQ"], dK=outs["dK"], dV=outs["dV"], **kw)
     la.la_last_device_status()
+    names = set(la.la_profile_read()) - {"segment_sum_kernel"}
+    la.la_profile_enable(False)
+    assert names == TC if tcgen05 else names <= TC | CLUSTER
     _untouched(tails)
     q, k, v, g = (t.double().numpy() for t in (Q, K, V, G))
     O_ref, den_ref = oracle.linear_attention(q, k, v, causal=True)[:2]
@@ -78,8 +96,11 @@ def test_causal_any_length(shape, keep):
 
 
 @pytest.mark.parametrize("shape", SHAPES[:5] + SHAPES[6:], ids=lambda s: "B%d_H%d_N%d_D%d" % s)
-def test_noncausal_any_length(shape):
+@ROUTES
+def test_noncausal_any_length(tcgen05, shape):
     B, H, N, D = shape
+    if tcgen05:
+        la.la_plan_override(linear_splits=min(3, (N + 127) // 128))
     Q, K, V, G = draw_qkvg(B, H, N, D, D, 11 + N, torch.bfloat16, 0.5)
     tails, dev, outs = {}, {}, {}
     for nm, t in zip("QKVG", (Q, K, V, G)):
@@ -93,7 +114,7 @@ def test_noncausal_any_length(shape):
     la.la_last_device_status()
     names = set(la.la_profile_read())
     la.la_profile_enable(False)
-    assert "linear_apply_kernel" in names, names
+    assert names == {"linear_sum_kernel", "linear_apply_kernel"} | (set() if tcgen05 else {"linear_cluster_forward_kernel"}), names
     _untouched(tails)
     q, k, v, g = (t.double().numpy() for t in (Q, K, V, G))
     O_ref, den_ref = oracle.linear_attention(q, k, v, causal=False)[:2]
@@ -104,8 +125,11 @@ def test_noncausal_any_length(shape):
 
 
 @pytest.mark.parametrize("causal", [False, True])
-def test_lengths_inside_a_batch_whose_own_length_is_odd(causal):
+@ROUTES
+def test_lengths_inside_a_batch_whose_own_length_is_odd(tcgen05, causal):
     """Both kinds of raggedness at once: N = 700 and per-sequence lengths below it (one of them 0, one of them N)."""
+    if tcgen05:
+        la.la_plan_override(causal_pieces=3, linear_splits=3)
     B, H, N, D = 4, 2, 700, 64
     lengths = [700, 0, 333, 129]
     Q, K, V, G = draw_qkvg(B, H, N, D, D, 5, torch.bfloat16, 1.0)

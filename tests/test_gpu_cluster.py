@@ -27,7 +27,21 @@ def _close(x, ref, tol, what):
 
 @pytest.mark.parametrize("dtype,phi,D,M,N", [(*c, n) for c in CAUSAL for n in SIZES[c[0]] if c[2] != 128 or n <= 1024])
 def test_causal(dtype, phi, D, M, N):
-    B, H, eps = 3, 1, 0.5 if N % 2 else 0.0
+    causal_against_the_oracle(dtype, phi, D, M, N, 3, 1)
+
+
+@pytest.mark.parametrize("dtype,phi,D,M", CAUSAL + [(torch.float32, "elu1", 64, 64), (torch.float32, "identity", 32, 32),
+                                                    (torch.bfloat16, "identity", 64, 64), (torch.bfloat16, "identity", 32, 32)])
+def test_causal_with_several_heads(dtype, phi, D, M):
+    """The lengths of a ragged batch belong to its sequences, each of several heads; both feature maps of every kernel."""
+    causal_against_the_oracle(dtype, phi, D, M, 500, 3, 2)
+    Q, K, V = (torch.zeros(3, 2, 500, c, dtype=dtype, device=DEV) + 1 for c in (D, D, M))
+    assert set(kernels_of(lambda: la.la_causal_forward(Q, K, V, phi=phi))) == {"causal_cluster_forward_kernel"}
+    assert set(kernels_of(lambda: la.la_causal_backward(Q, K, V, V, phi=phi))) == {"causal_cluster_backward_kernel"}
+
+
+def causal_against_the_oracle(dtype, phi, D, M, N, B, H):
+    eps = 0.5 if N % 2 else 0.0
     Q, K, V, G = draw_qkvg(B, H, N, D, M, 11 + N, dtype, 1.0)
     if phi == "identity":                               # features: positive, as the weights of a kernel are
         Q, K = Q.abs() + 0.1, K.abs() + 0.1
@@ -285,3 +299,16 @@ def test_which_kernel_takes_a_bidirectional_forward_pass(D, BHN, cluster):
     assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V))) == want
     saved = la.linear_saved_buffer(Q, V)
     assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved))) == want | {"linear_sum_kernel"}
+
+
+@pytest.mark.parametrize("dtype,phi,D,M", CAUSAL)
+def test_a_zero_state_changes_nothing(dtype, phi, D, M):
+    """A sequence may start from a state of zeros: the same results bit for bit as from none."""
+    dev = [t.to(DEV) for t in draw_qkvg(2, 2, 500, D, M, 3, dtype, 1.0)]
+    if phi == "identity":
+        dev[0], dev[1] = dev[0].abs() + 0.1, dev[1].abs() + 0.1
+    state = {"S_in": torch.zeros(2, 2, D, M, device=DEV), "Z_in": torch.zeros(2, 2, D, device=DEV)}
+    plain = (la.la_causal_forward(*dev[:3], phi=phi), *la.la_causal_backward(*dev, phi=phi))
+    from_zero = (la.la_causal_forward(*dev[:3], phi=phi, **state), *la.la_causal_backward(*dev, phi=phi, **state))
+    la.la_last_device_status()
+    assert all(torch.equal(a, b) for a, b in zip(plain, from_zero))

@@ -116,9 +116,11 @@ def test_many_short_bf16_sequences(N, pieces):
 @pytest.mark.parametrize("pieces", [1, 3])
 @pytest.mark.parametrize("N", [1, 63, 65, 200])
 @pytest.mark.parametrize("B,dtype,phi,D,M", [(28, torch.float32, "elu1", 64, 64), (28, torch.bfloat16, "identity", 128, 64),
-                                             (56, torch.bfloat16, "elu1", 32, 32)])
+                                             (56, torch.bfloat16, "elu1", 32, 32),
+                                             (20, torch.float32, "elu1", 64, 64), (20, torch.bfloat16, "identity", 128, 64)])
 def test_one_warp_per_strip(B, dtype, phi, D, M, N, pieces):
-    """The kernels of full grids (at least 222 CTAs; the last ones also of many short sequences): short last chunks, whole and
+    """The kernels of full grids (at least 222 CTAs; the third also of many short sequences; the last two, in one piece, the kernels
+    with two warps per strip of 149 to 221 CTAs, which neither smaller grids nor full ones take): short last chunks, whole and
     cut into pieces, ragged, from a state and with state gradients, against the oracle on sampled heads.  Tolerances as above,
     8e-6 also for the fp32 state gradients; single planes are held to the bf16 gates."""
     H, eps = 8, 0.5 if N % 2 else 0.0

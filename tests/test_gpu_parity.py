@@ -272,10 +272,15 @@ def test_prefill_then_decode_handoff():
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("shape", [(2, 3, 100, 16, 48), (1, 2, 31, 64, 64), (2, 2, 640, 32, 32), (1, 4, 384, 64, 64),
                                    (4, 16, 18 * 128, 64, 64), (2, 8, 1000, 64, 64), (2, 3, 100, 40, 72), (1, 2, 65, 128, 96)])
-def test_causal_forward_from_a_state(shape, dtype):
+@pytest.mark.parametrize("pieces", [-1, 3])
+def test_causal_forward_from_a_state(plan_override, pieces, shape, dtype):
     """The recurrence of Eq. 16-20 started from a given S_0, Z_0 (bf16 D = M in {32, 64}: tcgen05 kernel, with several
-    pieces per sequence at the larger shapes; other M <= 64: mma.sync kernels; M > 64: general kernels)."""
+    pieces per sequence at the larger shapes; other M <= 64: mma.sync kernels; M > 64: general kernels).  With three
+    pieces the short sequences, which a cluster of CTAs takes otherwise, go there too."""
     B, H, N, D, M = shape
+    if pieces > 0 and N < 300:
+        pytest.skip("the same kernels")
+    plan_override(causal_pieces=pieces)
     Q, K, V, _ = draw_qkvg(B, H, N, D, M, seed=sum(shape) + 1, dtype=dtype, with_grad=False)
     g = torch.Generator().manual_seed(5)
     S0 = torch.randn((B, H, D, M), generator=g) * 3.0
@@ -325,10 +330,14 @@ def test_chunked_prefill_then_decode(dtype, D, chunks):
 @pytest.mark.parametrize("keep", [False, True], ids=["recompute", "saved"])
 @pytest.mark.parametrize("shape", [(2, 3, 100, 16, 48), (1, 2, 31, 64, 64), (2, 2, 640, 32, 32), (4, 16, 18 * 128, 64, 64),
                                    (2, 8, 1000, 64, 64), (2, 3, 100, 40, 72), (1, 2, 65, 128, 96)])
-def test_causal_backward_from_a_state(shape, keep, dtype):
+@pytest.mark.parametrize("pieces", [-1, 3])
+def test_causal_backward_from_a_state(plan_override, pieces, shape, keep, dtype):
     """Algorithm 1 (backward) with the forward sum started from [S_0 | Z_0] and the reverse sum from an upstream
     gradient of the final state; the gradient of the initial state is what the reverse sum ends with."""
     B, H, N, D, M = shape
+    if pieces > 0 and N < 300:
+        pytest.skip("the same kernels")
+    plan_override(causal_pieces=pieces)
     Q, K, V, G = draw_qkvg(B, H, N, D, M, seed=sum(shape) + 2, dtype=dtype)
     g = torch.Generator().manual_seed(6)
     S0 = torch.randn((B, H, D, M), generator=g) * 3.0
@@ -676,7 +685,7 @@ def test_results_are_repeatable_bit_for_bit(name):
                 assert torch.equal(a, b), f"{name}: {nm} differs between repeats"
 
 
-@pytest.mark.parametrize("shape", [(2, 2, 1024, 64), (1, 3, 384, 32), (3, 50, 2048, 64)])
+@pytest.mark.parametrize("shape", [(2, 2, 1024, 64), (1, 3, 384, 32), (3, 50, 2048, 64), (2, 2, 1100, 64), (1, 3, 1100, 32), (6, 4, 1024, 64)])
 def test_saved_buffer_matches_recomputation(shape):
     """The forward's saved phi(Q), phi(K) are the bf16 feature maps of Q and K, the forward's own result
     does not depend on saving them, dQ (whose operands are identical on both paths) is bit-identical, and
@@ -697,9 +706,16 @@ def test_saved_buffer_matches_recomputation(shape):
         ref = oracle.feature_map(x.double().cpu().numpy())
         err = (got.double().cpu().numpy() - ref) / ref
         assert abs(err).max() <= 2.0 ** -8, abs(err).max()
+    la.la_profile_enable(True)
     g0 = la.la_causal_backward(Q, K, V, G)
     g1 = la.la_causal_backward(Q, K, V, G, saved=saved)
     la.la_last_device_status()
+    names = la.la_profile_read()
+    la.la_profile_enable(False)
+    # (up to 192 tiles of 64, 296 at D = 32, a cluster per sequence does the backward pass and has no use for the buffer)
+    tiles = (N + 63) // 64
+    reads = tiles > 16 or tiles * B * H > (192 if D == 64 else 296)
+    assert ("causal_bwd_dq_kernel" in names) == reads and ("causal_cluster_backward_kernel" in names) != reads
     assert torch.equal(g0[0], g1[0]), "dQ differs"
     for a, b, nm in zip(g0[1:], g1[1:], "KV"):
         ref = a.double().cpu().numpy()
@@ -927,11 +943,14 @@ def test_causal_ragged_batches(shape, lengths, dtype):
 
 
 @pytest.mark.parametrize("dtype,D,M", [(torch.bfloat16, 64, 64), (torch.float32, 48, 40), (torch.float32, 40, 72),
-                                       (torch.bfloat16, 128, 96)])      # tcgen05, mma.sync, general, general
-def test_causal_ragged_batch_from_a_state_with_state_gradients(dtype, D, M):
+                                       (torch.bfloat16, 128, 96)])      # tcgen05 or clusters, mma.sync, general, general
+@pytest.mark.parametrize("pieces", [-1, 3])
+def test_causal_ragged_batch_from_a_state_with_state_gradients(plan_override, pieces, dtype, D, M):
     """The ragged calls with every state argument: the sequences continue from S_0, Z_0, the upstream gradient
-    of the state at each sequence's own end comes in, the gradient of the initial state goes out."""
+    of the state at each sequence's own end comes in, the gradient of the initial state goes out (pieces: the bf16 problem on
+    the tcgen05 kernels, not on clusters)."""
     B, H, N = 3, 2, 512
+    plan_override(causal_pieces=pieces)
     lengths = [512, 200, 77]
     Q, K, V, G = draw_qkvg(B, H, N, D, M, seed=410, dtype=dtype)
     g = torch.Generator().manual_seed(411)

@@ -137,6 +137,53 @@ def test_training_step_replayed_from_a_cuda_graph(name):
     la.la_last_device_status()
 
 
+@pytest.mark.parametrize("kind,H,N,D", [("causal", 8, 1100, 64), ("causal", 4, 500, 64), ("causal", 8, 1100, 32), ("linear", 8, 1000, 64),
+                                        ("linear", 3, 300, 32)])
+def test_short_training_step_replayed_from_a_cuda_graph(kind, H, N, D):
+    """Steps of a cluster per sequence, captured with the copies that write their inputs just before them: with a saved buffer the
+    cluster kernel starts beside the pre-pass in front of it and waits for it at its own end, and what follows needs both.  Two
+    sets of values in turn, so that stale data would be the other set's; the replays give the bits of a synchronised run."""
+    if os.environ.get("LA_DEBUG"):
+        pytest.skip("checked mode synchronises after every call, which a stream capture does not allow")
+    fwd, bwd, make_saved = _calls(kind)
+    g = torch.Generator().manual_seed(3)
+    set_a = [torch.randn((1, H, N, D), generator=g).bfloat16().to(DEV) for _ in range(4)]
+    sets = [set_a, [(t.flip(2) * 0.75).contiguous() for t in set_a]]
+    src = [torch.empty_like(t) for t in set_a]
+    Q, K, V, G = (torch.empty_like(t) for t in set_a)
+    O, dQ, dK, dV = torch.empty_like(V), torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
+    saved = make_saved(Q, V)
+
+    def step(gap=lambda: None):
+        Q.copy_(src[0]); K.copy_(src[1]); V.copy_(src[2]); G.copy_(src[3]); gap()
+        fwd(Q, K, V, O=O, saved=saved); gap()
+        bwd(Q, K, V, G, dQ=dQ, dK=dK, dV=dV, saved=saved); gap()
+
+    want = []
+    for values in sets:
+        for a, b in zip(src, values):
+            a.copy_(b)
+        step(torch.cuda.synchronize)
+        want.append([t.clone() for t in (O, dQ, dK, dV)])
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            for _ in range(3):
+                step()
+    torch.cuda.current_stream().wait_stream(side)
+    for i in range(6):
+        for a, b in zip(src, sets[i % 2]):
+            a.copy_(b)
+        for t in (O, dQ, dK, dV):
+            t.fill_(7.0)
+        graph.replay()
+        for a, b, nm in zip(want[i % 2], (O, dQ, dK, dV), ("O", "dQ", "dK", "dV")):
+            assert torch.equal(a, b), f"replay {i}: {nm} differs from the synchronised run"
+    la.la_last_device_status()
+
+
 @pytest.mark.parametrize("D,H", [(32, 2), (64, 4)])
 def test_small_fp32_calls_that_feed_each_other(D, H):
     """The kernels of small fp32 problems start as programmatic dependents of whatever is in front of them, another call's
