@@ -29,10 +29,15 @@
  *    problem with M <= 64 runs on mma.sync kernels that keep fp32 accuracy
  *    (products of numbers split into bf16 parts), everything else on the general
  *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.
- *    Few short sequences (D = M in {32, 64}, or 128 features to 64 values; some
- *    hundred positions to 2048) take one launch of a kernel with a thread-block
- *    cluster per sequence instead; sizes of buffers and plans are unaffected.
+ *    Few short sequences (D = M in {32, 64}, or 128 bf16 features to 64 values with
+ *    LA_PHI_IDENTITY) take one launch of a kernel with a thread-block cluster per sequence
+ *    instead, where the context of the stream has room for one: the causal forward up to 2048
+ *    positions in bf16 (from 257) and 1024 in fp32 and with 128 features (from 65), the causal
+ *    backward up to 1024 (from 65; bf16 D = 64 from 257), the bidirectional forward in bf16 up
+ *    to 1536 at D = 64 and 8192 at D = 32.  Sizes of buffers and plans are unaffected.
  *    Only the tcgen05 kernels have a la_causal_plan() and a causal saved buffer.
+ *    bf16 features of LA_PHI_ELU1 below 1.2e-38 (keys and queries below -87.3) are zero on the
+ *    tcgen05 kernels and in clusters, and what bf16 holds of them everywhere else.
  *    Finite numbers keep their value on these kernels; an infinity in Q, K, V or G acts like a NaN
  *    (its products with split numbers are sums of infinities of both signs), so that results that
  *    fp32 arithmetic would make infinite may be NaN.  Rows that a length excludes are never read.
@@ -219,6 +224,8 @@ int la_linear_attention_backward_kept(const la_problem* p, const void* Q, const 
  * per-segment sums of the forward pre-pass.  Its layout is private to the library; it is
  * valid for la_causal_backward() with the same problem, Q, K and V until overwritten.  The
  * size is 0 for problems that do not run the tcgen05 kernels (pass NULL, or any pointer).
+ * Whether it is given does not change O, except that a problem of more sequences than one
+ * wave of clusters holds may run another kernel with it (O then agrees to rounding).
  */
 int la_causal_forward(const la_problem* p, const void* Q, const void* K, const void* V,
                       void* O, float* den, float* S_out, float* Z_out,
@@ -252,7 +259,8 @@ int la_causal_forward_from(const la_problem* p, const void* Q, const void* K, co
  * No per-position state is stored.  G = dL/dO.  O and den may be NULL (recomputed).
  * saved (optional): the buffer a la_causal_forward() call on the same problem and inputs
  * filled.  With it the backward pass reads phi(Q), phi(K) instead of recomputing them from
- * Q and K and skips its forward pre-pass; without it (NULL) everything is recomputed.  The
+ * Q and K and skips its forward pre-pass; without it (NULL) everything is recomputed.  Problems
+ * whose backward pass a cluster per sequence does have no use for the buffer and ignore it.  The
  * gradients agree with the recomputing path to rounding (phi(Q)/den is rounded from the
  * saved bf16 phi(Q) instead of the fp32 value).
  */
@@ -394,8 +402,10 @@ int la_causal_plan(const la_problem* p, int32_t* out, int capacity);
  * choice automatic; la_plan_override(-1, -1, -1) restores the defaults.  The setting is process-wide and
  * read by every later call, la_workspace_bytes() and la_causal_plan() included: change it only between
  * steps, size workspaces and saved buffers after the change, and never between a forward pass that
- * fills a saved buffer and the backward pass that reads it (the backward pass notices: it computes
- * nothing and la_last_device_status() returns LA_ERR_INVALID_ARG).
+ * fills a saved buffer and the backward pass that reads it (a backward pass on the tcgen05 kernels
+ * notices: it computes nothing and la_last_device_status() returns LA_ERR_INVALID_ARG).  A given
+ * causal_pieces leaves out the causal kernels with a cluster per sequence, linear_splits the
+ * bidirectional one.
  */
 int la_plan_override(int32_t causal_pieces, int32_t causal_short, int32_t linear_splits);
 

@@ -243,7 +243,7 @@ struct Bf16Features {
 };
 // ... with one warp per strip, at twice the registers: where a machine full of CTAs keeps the schedulers busy anyway, the
 // hand-overs cost more than they give.  Forward + backward, us, one / two warps: fp32 B32 H8 N4096 D64 2690 / 2930,
-// B4 H8 N4096 477 / 472, B1 H8 N1024 122 / 94; Fourier B8 H8 N1000 C128 272 / 288, B1 H8 N4000 343 / 265.
+// B4 H8 N4096 477 / 472; Fourier B8 H8 N1000 C128 272 / 288.  (The smallest grids run the kernels that follow or clusters.)
 struct Fp32One : Fp32 { static constexpr int WPS = 1; };
 struct Bf16FeaturesOne : Bf16Features { static constexpr int WPS = 1; };
 // ... and with an SM to itself: a grid of at most 148 CTAs has that anyway, and the backward kernels then have 255 registers
