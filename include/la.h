@@ -24,8 +24,9 @@
  *  - Supported sizes: D and M multiples of 8 in [8, 128]; B, H >= 1; N >= 0
  *    (N == 0 is a successful no-op).  bf16 problems with D = M in {32, 64} run
  *    on the tcgen05 kernels (any N: a last chunk of fewer than 128 positions is
- *    handled as padding), but causal ones of many short sequences (D = M = 32,
- *    B*H >= 444, N <= 1024) on mma.sync kernels with bf16 operands; every other
+ *    handled as padding), but causal ones of D = M = 32 (more than 2048 positions, or
+ *    tiles of 128 positions, counted over all sequences, beyond 296, from eight tiles a
+ *    sequence on beyond 512) on mma.sync kernels with bf16 operands; every other
  *    problem with M <= 64 runs on mma.sync kernels that keep fp32 accuracy
  *    (products of numbers split into bf16 parts), everything else on the general
  *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.
@@ -35,15 +36,17 @@
  *    positions in bf16 (from 257) and 1024 in fp32 and with 128 features (from 65), the causal
  *    backward up to 1024 (from 65; bf16 D = 64 from 257), the bidirectional forward in bf16 up
  *    to 1536 at D = 64 and 8192 at D = 32.  Sizes of buffers and plans are unaffected.
- *    Only the tcgen05 kernels have a la_causal_plan() and a causal saved buffer.
+ *    Only the tcgen05 kernels have a la_causal_plan(), and only they and the bf16
+ *    mma.sync ones of D = M = 32 (unless B*H >= 444 and N <= 1024) a causal saved buffer.
  *    bf16 features of LA_PHI_ELU1 below 1.2e-38 (keys and queries below -87.3) are zero on the
  *    tcgen05 kernels and in clusters, and what bf16 holds of them everywhere else.
  *    Finite numbers keep their value on these kernels; an infinity in Q, K, V or G acts like a NaN
  *    (its products with split numbers are sums of infinities of both signs), so that results that
  *    fp32 arithmetic would make infinite may be NaN.  Rows that a length excludes are never read.
  *    Features of -Inf keys and queries under LA_PHI_ELU1 are zero as everywhere.
- *    The fp32-accurate causal forward takes ws as an option: with less than
- *    la_workspace_bytes() (or NULL) it does not cut sequences into pieces.
+ *    The fp32-accurate causal forward, and the bf16 one of D = M = 32 with B*H >= 444 and
+ *    N <= 1024, take ws as an option: with less than la_workspace_bytes() (or NULL)
+ *    they do not cut sequences into pieces.
  *  - Return value: LA_OK (0) or a negative la_status.  All argument checks run
  *    on the host before anything is enqueued; a failed check enqueues nothing.
  *    The library never aborts, throws or traps.  la_last_error() returns a
@@ -220,10 +223,10 @@ int la_linear_attention_backward_kept(const la_problem* p, const void* Q, const 
  * state S_N, Z_N, which continues the sequence through la_recurrent_step().
  * saved (optional, device, 128-byte aligned, la_workspace_bytes(p, LA_OP_CAUSAL_SAVED)
  * bytes, owned by the caller): what a training step keeps for the backward pass, as the
- * paper's autograd function keeps phi(Q), phi(K): the mapped queries and keys and the
- * per-segment sums of the forward pre-pass.  Its layout is private to the library; it is
+ * paper's autograd function keeps phi(Q), phi(K): the mapped queries and keys (D = M = 64)
+ * and the per-segment sums of the forward pre-pass.  Its layout is private to the library; it is
  * valid for la_causal_backward() with the same problem, Q, K and V until overwritten.  The
- * size is 0 for problems that do not run the tcgen05 kernels (pass NULL, or any pointer).
+ * size is 0 for problems that keep nothing (pass NULL, or any pointer).
  * Whether it is given does not change O, except that a problem of more sequences than one
  * wave of clusters holds may run another kernel with it (O then agrees to rounding).
  */

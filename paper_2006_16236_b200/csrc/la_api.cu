@@ -258,7 +258,8 @@ size_t la_workspace_bytes(const la_problem* p, int32_t op) {
     if (op == LA_OP_DECODE_LAYER) return decode_layer_supported(*p) ? decode_layer_workspace(*p) : 0;
     if (p->N == 0) return 0;
     if (op == LA_OP_LINEAR_SAVED) op = LA_OP_LINEAR_FORWARD;          // the saved buffer holds what the forward's workspace holds
-    if (op == LA_OP_CAUSAL_SAVED) return tc_supported(*p, LA_OP_CAUSAL_BACKWARD) ? tc::causal_saved_bytes(*p) : 0;
+    if (op == LA_OP_CAUSAL_SAVED)
+        return tc_supported(*p, LA_OP_CAUSAL_BACKWARD) ? tc::causal_saved_bytes(*p) : causal_mma_supported(*p) ? causal_mma_saved_bytes(*p) : 0;
     if (op == LA_OP_LINEAR_VARLEN_FORWARD) op = LA_OP_LINEAR_FORWARD;
     if (op == LA_OP_LINEAR_VARLEN_BACKWARD) op = LA_OP_LINEAR_BACKWARD;
     if (tc_supported(*p, op)) return tc_workspace_bytes(*p, op);
@@ -492,7 +493,7 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     LA_REQUIRE_PTR(Q); LA_REQUIRE_PTR(K); LA_REQUIRE_PTR(V); LA_REQUIRE_PTR(O);
     LA_OPTIONAL_PTR(saved);
     const bool tc_path = tc_supported(*p, LA_OP_CAUSAL_FORWARD);
-    if (tc_path)        // (the other kernels' workspace is optional: without it a sequence is not cut into pieces)
+    if (tc_path || causal_mma_needs_workspace(*p))        // (elsewhere it is optional: without it a sequence is not cut into pieces)
         if (int rc = check_ws(p, lengths ? LA_OP_CAUSAL_VARLEN_FORWARD : LA_OP_CAUSAL_FORWARD, ws, ws_bytes)) return rc;
     if (int rc = check_saved(p, saved, saved_bytes)) return rc;
     if (int rc = check_arch()) return rc;
@@ -506,7 +507,7 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     if (tc_path)
         return debug_finish(tc::causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, st), stream);
     if (causal_mma_supported(*p))
-        return debug_finish(causal_mma_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, ws, ws_bytes, st), stream);
+        return debug_finish(causal_mma_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, ws_bytes, st), stream);
     return debug_finish(general_causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, st), stream);
 }
 
@@ -585,7 +586,7 @@ static int causal_backward_common(const la_problem* p, const void* Q, const void
     if (tc_supported(*p, LA_OP_CAUSAL_BACKWARD))
         return debug_finish(tc::causal_backward(*p, Q, K, V, lengths, G, sa, causal_cluster_backward_size(*p) ? nullptr : saved, dQ, dK, dV, ws, st), stream);
     if (causal_mma_supported(*p))
-        return debug_finish(causal_mma_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, ws, st), stream);
+        return debug_finish(causal_mma_backward(*p, Q, K, V, lengths, G, sa, saved, dQ, dK, dV, ws, st), stream);
     return debug_finish(general_causal_backward(*p, Q, K, V, lengths, G, sa, dQ, dK, dV, ws, st), stream);
 }
 

@@ -1,6 +1,6 @@
 // Causal form (Eq. 8-15) at fp32 accuracy on mma.sync (la_mma.cuh): fp32 problems, and bf16 ones of shapes or feature
-// maps that the tcgen05 kernels do not take; M <= 64, any D.  Also, with single bf16 planes, many short sequences of
-// D = M = 32 (causal_mma_preferred).
+// maps that the tcgen05 kernels do not take; M <= 64, any D.  Also bf16 problems with D = M = 32, on kernels of
+// their own (la_causal_warp.cuh).
 //
 // A sequence is cut into pieces, one CTA each; a CTA walks its piece in chunks of T = 64 positions.  Per chunk a strip of
 // sixteen rows (queries in the forward sweeps, keys in the reverse one) belongs to a pair of warps, and so do sixteen
@@ -16,15 +16,16 @@
 // The two warps of a strip share the products: forward, one the state's part and one the scores' part; dQ, one G S^T and
 // L k, one the scores' part; reverse, one dV and one dK.  The partial sums of the first two are added through shared
 // memory (the state planes, once nobody reads them any more).  Two warps per strip at 128 registers keep four warps on
-// a scheduler; one warp per strip at 168 to 255 registers kept two, and the tensor pipe 45 % busy.  Problems with single
-// planes have too little work for that: one warp per strip takes both parts (WPS = 1).
+// a scheduler; one warp per strip at 168 to 255 registers kept two, and the tensor pipe 45 % busy.
 //
 // Pieces other than the first (last, for the reverse sweep) start from the sum of the records [S | Z] of the pieces
 // before (after) them, which a pre-pass writes to the workspace.
+#include <math.h>
 #include <stdlib.h>
 
 #include <type_traits>
 
+#include "la_causal_warp.cuh"
 #include "la_mma_sweep.cuh"
 
 namespace la {
@@ -95,13 +96,12 @@ __device__ __forceinline__ void mask_diagonal(float (&s0)[4], float (&s1)[4], in
 
 // ---- forward ---------------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<ForwardLayout<C, DP, MP>, C>()))
+__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<ForwardLayout<C, DP, MP>>()))
 causal_mma_forward_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = ForwardLayout<C, DP, MP>;
     constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, WPS = C::WPS, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const bool state_part = WPS == 1 || warp < STRIPS_T, score_part = WPS == 1 || warp >= STRIPS_T;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
@@ -119,10 +119,10 @@ causal_mma_forward_kernel(const Params p) {
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
-        const uint32_t sK = smem_u32(buf + Sh::X), sV = smem_u32(buf + Sh::Y), sS = smem_u32(buf + Sh::S);
-        float* sZ = reinterpret_cast<float*>(buf + Sh::Z);
-        uint16_t* sZp = reinterpret_cast<uint16_t*>(buf + Sh::ZP);
-        float* sden = reinterpret_cast<float*>(buf + Sh::W);
+        const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
+        float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
+        uint16_t* sZp = reinterpret_cast<uint16_t*>(smem + Sh::ZP);
+        float* sden = reinterpret_cast<float*>(smem + Sh::W);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         const int strip = strip_of(warp, (n0 / T) & 1), row0 = strip * 16;
         StripOperand<WPS, NQ, DP> q;
@@ -134,22 +134,22 @@ causal_mma_forward_kernel(const Params p) {
             rv.load(V + n0 * M, cn, M, 0.f);
             if constexpr (WPS == 1) rq.load(Q + n0 * D, row0, cn, D, pad);
             else rq.load(Q + n0 * D, cn, D, pad);
-            if constexpr (C::BUF == 1) __syncthreads();         // the planes of the chunk before are no longer read
-            st.template publish<NS>(buf + Sh::S, sZ, sZp);
-            rk.template features<NQ>(buf + Sh::X, phi);
-            rv.template values<NV>(buf + Sh::Y);
+            __syncthreads();         // the planes of the chunk before are no longer read
+            st.template publish<NS>(smem + Sh::S, sZ, sZp);
+            rk.template features<NQ>(smem + Sh::X, phi);
+            rv.template values<NV>(smem + Sh::Y);
             if constexpr (WPS == 1) {
                 RawStrip<typename FeatureType<NQ>::type, DP> fq;
                 rq.template map<NQ>(phi, fq);
                 fq.template planes<NQ>(q.a);
             } else {
-                rq.template features<NQ>(buf + Sh::R, phi);
-                q.tile = smem_u32(buf + Sh::R); q.row0 = row0; q.lane = lane;
+                rq.template features<NQ>(smem + Sh::R, phi);
+                q.tile = smem_u32(smem + Sh::R); q.row0 = row0; q.lane = lane;
             }
         }
-        prefetch_rows<C, DP>(Q, n0 + T, r.end, D);
-        prefetch_rows<C, DP>(K, n0 + T, r.end, D);
-        prefetch_rows<C, MP>(V, n0 + T, r.end, M);
+        prefetch_rows<C>(Q, n0 + T, r.end, D);
+        prefetch_rows<C>(K, n0 + T, r.end, D);
+        prefetch_rows<C>(V, n0 + T, r.end, M);
         __syncthreads();
         const bool real = row0 < cn;
         float o[MP / 8][4], d0 = 0.f, d1 = 0.f;         // rows g, g + 8 of [num | den]; d0, d1 spread over the four lanes
@@ -170,15 +170,8 @@ causal_mma_forward_kernel(const Params p) {
                 if (jb == strip) mask_diagonal<false>(s0, s1, g, t);
                 uint32_t pa[NP][4];
                 operand_of<NP>(pa, s0, s1);
-                if constexpr (NP == 1) {            // numerator and normaliser see the same rounded scores
-                    float u[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma16816(u, pa[0], 0x3f803f80u, 0x3f803f80u);
-                    d0 += t == 0 ? u[0] : 0.f;
-                    d1 += t == 0 ? u[2] : 0.f;
-                } else {
-                    d0 += (s0[0] + s0[1]) + (s1[0] + s1[1]);
-                    d1 += (s0[2] + s0[3]) + (s1[2] + s1[3]);
-                }
+                d0 += (s0[0] + s0[1]) + (s1[0] + s1[1]);
+                d1 += (s0[2] + s0[3]) + (s1[2] + s1[3]);
 #pragma unroll
                 for (int n = 0; n < MP / 16; ++n) {
                     uint32_t b[NV][4];
@@ -215,7 +208,7 @@ causal_mma_forward_kernel(const Params p) {
             if constexpr (WPS == 2) {
                 bar_sync(1, 128);
                 if (real) {
-                    put_part(buf + Sh::S, strip, o);
+                    put_part(smem + Sh::S, strip, o);
                     d0 = quad_sum(d0);
                     d1 = quad_sum(d1);
                     if (t == 0) {
@@ -233,7 +226,7 @@ causal_mma_forward_kernel(const Params p) {
             d1 = quad_sum(d1);
             if constexpr (WPS == 2) {
                 bar_sync(2 + strip, 64);
-                add_part(buf + Sh::S, strip, o);
+                add_part(smem + Sh::S, strip, o);
                 d0 += sden[row0 + g];
                 d1 += sden[row0 + g + 8];
             }
@@ -250,7 +243,6 @@ causal_mma_forward_kernel(const Params p) {
             }
         }
         st.template update<NQ, NV, true>(sK, sV, nullptr);
-        flip<C, Sh>(buf, smem);
     }
     zero_rows<THREADS>(O, r.end, r.hi, M);
     if (den) zero_rows<THREADS>(den, r.end, r.hi, 1);
@@ -259,13 +251,12 @@ causal_mma_forward_kernel(const Params p) {
 
 // ---- dQ sweep --------------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DqLayout<C, DP, MP>, C>()))
+__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DqLayout<C, DP, MP>>()))
 causal_mma_dq_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = DqLayout<C, DP, MP>;
     constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, WPS = C::WPS, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const bool state_part = WPS == 1 || warp < STRIPS_T, score_part = WPS == 1 || warp >= STRIPS_T;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
@@ -285,9 +276,9 @@ causal_mma_dq_kernel(const Params p) {
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
             p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
-        const uint32_t sK = smem_u32(buf + Sh::X), sV = smem_u32(buf + Sh::Y), sS = smem_u32(buf + Sh::S);
-        float* sZ = reinterpret_cast<float*>(buf + Sh::Z);
-        float* sgo = reinterpret_cast<float*>(buf + Sh::W);
+        const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
+        float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
+        float* sgo = reinterpret_cast<float*>(smem + Sh::W);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         const int strip = strip_of(warp, (n0 / T) & 1), row0 = strip * 16;
         StripOperand<WPS, NV, MP> ga;
@@ -299,21 +290,21 @@ causal_mma_dq_kernel(const Params p) {
             rv.load(V + n0 * M, cn, M, 0.f);
             if constexpr (WPS == 1) rg.load(G + n0 * M, row0, cn, M, 0.f);
             else rg.load(G + n0 * M, cn, M, 0.f);
-            if constexpr (C::BUF == 1) __syncthreads();
-            st.template publish<NS>(buf + Sh::S, sZ, reinterpret_cast<uint16_t*>(buf + Sh::ZP));
-            rk.template features<NQ>(buf + Sh::X, phi);
-            rv.template values<NV>(buf + Sh::Y);
+            __syncthreads();
+            st.template publish<NS>(smem + Sh::S, sZ, reinterpret_cast<uint16_t*>(smem + Sh::ZP));
+            rk.template features<NQ>(smem + Sh::X, phi);
+            rv.template values<NV>(smem + Sh::Y);
             if constexpr (WPS == 1) {
                 rg.template planes<NV>(ga.a);
             } else {
-                rg.template values<NV>(buf + Sh::R);
-                ga.tile = smem_u32(buf + Sh::R); ga.row0 = row0; ga.lane = lane;
+                rg.template values<NV>(smem + Sh::R);
+                ga.tile = smem_u32(smem + Sh::R); ga.row0 = row0; ga.lane = lane;
             }
         }
-        prefetch_rows<C, DP>(Q, n0 + T, r.end, D);
-        prefetch_rows<C, DP>(K, n0 + T, r.end, D);
-        prefetch_rows<C, MP>(V, n0 + T, r.end, M);
-        prefetch_rows<C, MP>(G, n0 + T, r.end, M);
+        prefetch_rows<C>(Q, n0 + T, r.end, D);
+        prefetch_rows<C>(K, n0 + T, r.end, D);
+        prefetch_rows<C>(V, n0 + T, r.end, M);
+        prefetch_rows<C>(G, n0 + T, r.end, M);
         __syncthreads();
         const bool real = row0 < cn;
         // The first chunk of a sequence goes through twice, the second time with the G_i . O_i it found taken off the
@@ -379,7 +370,7 @@ causal_mma_dq_kernel(const Params p) {
                 }
                 if (pass == first_pass) bar_sync(1, THREADS);
                 if (real) {
-                    put_part(buf + Sh::S, strip, h);
+                    put_part(smem + Sh::S, strip, h);
                     bar_arrive(2 + strip, 64);
                     if (pass == 0) {
                         bar_sync(6 + strip, 64);
@@ -438,7 +429,7 @@ causal_mma_dq_kernel(const Params p) {
                     if constexpr (WPS == 2) {
                         rq.load(Q + n0 * D, row0, cn, D, pad);
                         bar_sync(2 + strip, 64);
-                        add_part(buf + Sh::S, strip, h);
+                        add_part(smem + Sh::S, strip, h);
                     } else {
                         scores();
                         rq.load(Q + n0 * D, row0, cn, D, pad);
@@ -487,20 +478,18 @@ causal_mma_dq_kernel(const Params p) {
             }
         }
         st.template update<NQ, NV, true>(sK, sV, nullptr);
-        flip<C, Sh>(buf, smem);
     }
     zero_rows<THREADS>(dQ, r.end, r.hi, D);
 }
 
 // ---- dK, dV sweep ----------------------------------------------------------------------------------------------
 template <typename C, int DP, int MP, bool EXACT>
-__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DkvLayout<C, DP, MP>, C>(C::WPS == 1 ? 3 : 2)))
+__global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DkvLayout<C, DP, MP>>(C::WPS == 1 ? 3 : 2)))
 causal_mma_dkv_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = DkvLayout<C, DP, MP>;
     constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, NR = C::NR, WPS = C::WPS, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t* buf = smem;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const bool v_part = WPS == 1 || warp < STRIPS_T, k_part = WPS == 1 || warp >= STRIPS_T;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
@@ -522,25 +511,25 @@ causal_mma_dkv_kernel(const Params p) {
             p.rec + (r.bh * p.records + r.piece) * (int64_t)(D * M + D), p.pieces - 1 - r.piece);
     const int64_t chunks = (r.end - r.lo + T - 1) / T;
     for (int64_t c = chunks - 1; c >= 0; --c) {
-        const uint32_t sQ = smem_u32(buf + Sh::X), sG = smem_u32(buf + Sh::Y), sR = smem_u32(buf + Sh::S);
-        float* sr = reinterpret_cast<float*>(buf + Sh::Z);
-        float* sdl = reinterpret_cast<float*>(buf + Sh::W);
-        uint16_t* wpl = reinterpret_cast<uint16_t*>(buf + Sh::WP);
+        const uint32_t sQ = smem_u32(smem + Sh::X), sG = smem_u32(smem + Sh::Y), sR = smem_u32(smem + Sh::S);
+        float* sr = reinterpret_cast<float*>(smem + Sh::Z);
+        float* sdl = reinterpret_cast<float*>(smem + Sh::W);
+        uint16_t* wpl = reinterpret_cast<uint16_t*>(smem + Sh::WP);
         const int64_t n0 = r.lo + c * T;
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T), blocks = (cn + 15) / 16;
         const int strip = strip_of(warp, c & 1), row0 = strip * 16;
         {
             ReverseRows<IO, DP, MP, THREADS> rr;
             rr.load(Q, G, dn, delta, n0, cn, D, M, pad);
-            if constexpr (C::BUF == 1) __syncthreads();
-            st.template publish<NS>(buf + Sh::S, sr, reinterpret_cast<uint16_t*>(buf + Sh::ZP));
-            rr.template store<NR, NV>(buf + Sh::X, buf + Sh::Y, sdl, wpl, phi);
+            __syncthreads();
+            st.template publish<NS>(smem + Sh::S, sr, reinterpret_cast<uint16_t*>(smem + Sh::ZP));
+            rr.template store<NR, NV>(smem + Sh::X, smem + Sh::Y, sdl, wpl, phi);
         }
         if (c > 0) {
-            prefetch_rows<C, DP>(Q, n0 - T, r.end, D);
-            prefetch_rows<C, DP>(K, n0 - T, r.end, D);
-            prefetch_rows<C, MP>(V, n0 - T, r.end, M);
-            prefetch_rows<C, MP>(G, n0 - T, r.end, M);
+            prefetch_rows<C>(Q, n0 - T, r.end, D);
+            prefetch_rows<C>(K, n0 - T, r.end, D);
+            prefetch_rows<C>(V, n0 - T, r.end, M);
+            prefetch_rows<C>(G, n0 - T, r.end, M);
         }
         __syncthreads();
         if (v_part && row0 < cn) {
@@ -666,14 +655,46 @@ causal_mma_dkv_kernel(const Params p) {
             }
         }
         st.template update<NR, NV, false>(sQ, sG, wpl);
-        flip<C, Sh>(buf, smem);
     }
     zero_rows<THREADS>(dK, r.end, r.hi, D);
     zero_rows<THREADS>(dV, r.end, r.hi, M);
     if (r.piece == 0) st.write(p, p.S1 ? p.S1 + r.bh * D * M : nullptr, p.Z1 ? p.Z1 + r.bh * D : nullptr);
 }
 
+// ---- bf16, D = M = 32: a warp per piece (la_causal_warp.cuh) -----------------------------------------------------
+enum WarpPass { kWarpForward, kWarpSums, kWarpDq, kWarpDqReverse, kWarpReverseSums, kWarpDkv };
+constexpr int warp_ring(int pass) {
+    return pass == kWarpForward ? warp32::Ring<3, false>::BYTES : pass == kWarpSums ? warp32::Ring<2, false>::BYTES :
+           pass == kWarpReverseSums ? warp32::Ring<2, true>::BYTES : pass == kWarpDkv ? warp32::Ring<4, true>::BYTES : warp32::Ring<4, false>::BYTES;
+}
+// registers for twelve warps on an SM, eight where the dQ sweep keeps two kinds of sums
+constexpr int warp_resident(int pass) { return pass == kWarpDqReverse ? 8 : pass == kWarpSums || pass == kWarpReverseSums ? 16 : 12; }
+template <int PASS> constexpr int kWarpRing = warp_ring(PASS);
+template <int PASS, bool ELU>
+__global__ void __launch_bounds__(32, warp_resident(PASS)) causal_warp_kernel(const Params p) {
+    __shared__ __align__(128) uint8_t smem[kWarpRing<PASS>];
+    wait_for_stream();
+    release_next();
+    if constexpr (PASS == kWarpForward) warp32::forward<ELU>(p, smem);
+    if constexpr (PASS == kWarpSums) warp32::sums<ELU>(p, smem);
+    if constexpr (PASS == kWarpDq) warp32::dq<ELU, false>(p, smem);
+    if constexpr (PASS == kWarpDqReverse) warp32::dq<ELU, true>(p, smem);
+    if constexpr (PASS == kWarpReverseSums) warp32::reverse_sums<ELU>(p, smem);
+    if constexpr (PASS == kWarpDkv) warp32::dkv<ELU>(p, smem);
+}
+
 // ---- host ------------------------------------------------------------------------------------------------------
+// Which bf16 problems with D = M = 32 a warp per piece takes: all that the cluster kernels leave (la_cluster.cu: short sequences of
+// few heads; more than 296 tiles of 128 positions, 512 from eight tiles on, or more than sixteen tiles), whatever the context.
+// Forward + backward, us, tcgen05 kernels (128x8x784: the former ones of this file) / a warp per piece: 128x8x784 284 / 154, 16x8x3072 136 / 106,
+// 32x8x3072 262 / 187, 8x8x16384 376 / 251, 64x8x2048 363 / 234, 1x8x4096 73 / 51, 1x1x16384 156 / 77, 2x1x65536 355 / 154,
+// 1x8x65536 273 / 214, 16x8x700 47 / 44, 16x8x300 33 / 29, 20x8x256 41 / 31, 56x8x64 22.6 / 20.5.
+bool of_warps(const la_problem& p) {
+    if (p.dtype != LA_BF16 || p.D != 32 || p.M != 32 || p.N > (1 << 30)) return false;
+    const int64_t tiles = (p.N + 127) / 128, ctas = tiles * p.B * p.H;
+    return tiles > 16 || (ctas > 296 && (tiles < 8 || ctas > 512));
+}
+
 struct Plan { int pieces; int64_t len; };
 
 // The estimates of choose_plan() for kernels that leave an SM little to gain from a second CTA, in units of one chunk of the main
@@ -699,13 +720,25 @@ double wide_cost(const WideCosts& w, int64_t bh, int64_t chunks, int64_t n) {
     return t;
 }
 
+// A warp per piece: two of them on every scheduler (eight on an SM, the most that the dQ sweep with both sums has registers for), or
+// what comes closest; and no more than a piece's start makes good: it adds up the records before it, 0.45 us of a step for each,
+// where a chunk of 64 takes 7.7 us.  Forward + backward, us, B x H x N: number of pieces: 16x8x3072 4: 131, 8: 106, 12: 115; 8x8x16384
+// 8: 322, 16: 251, 24: 280; 32x8x3072 3: 232, 4: 187, 8: 200; 50x8x1000 2: 121, 3: 119, 4: 106; 64x8x2048 1: 257, 3: 234, 4: 250;
+// 100x8x2000 1: 360, 2: 353, 3: 375; 128x8x784 1: 154, 2: 190; few heads 1x8x16384 32: 106, 64: 88, 128: 113; 1x8x4096 16: 61,
+// 32: 51, 64: 59; 2x1x65536 64: 190, 128: 154.
+int64_t warp_pieces(int64_t bh, int64_t chunks) {
+    int64_t n = bh > 888 ? 1 : bh > 592 ? 2 : bh > 394 ? 3 : 1184 / bh;
+    const int64_t most = (int64_t)(4.0 * sqrt((double)chunks));
+    if (n > most) n = most;
+    return n < chunks ? n : chunks;
+}
+
 // Pieces per sequence, by the estimated time: fp32 D = M = 64 and Fourier features as above; the others in units of one chunk of a main
 // kernel (about 10 us alone on an SM):
 // an SM runs two CTAs in 1.25 times the time of one; a CTA's start costs about a chunk, and 0.2 for each record it sums, of
 // which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk (fp32 D = M = 32, B4 H8 N2000,
 // pieces 1 / 4 / 8 / 12 / 16: 353 / 141 / 113 / 131 / 119; B22 H8 N3316 903 / 732 / 749 / 733 / 757).  At most sixteen: the estimates
-// are checked up to N = 4096 only (for few sequences much longer than that they would want more), and they know nothing of the
-// single-plane kernels' four CTAs per SM.
+// are checked up to N = 4096 only (for few sequences much longer than that they would want more).
 Plan choose_plan(const la_problem& p, bool single) {
     const int64_t chunks = (p.N + T - 1) / T, bh = p.B * p.H;
     int64_t best = 1;
@@ -716,6 +749,8 @@ Plan choose_plan(const la_problem& p, bool single) {
     } else if (forced > 0) {
         best = forced < chunks ? forced : chunks;
         if (best > 1024) best = 1024;
+    } else if (of_warps(p)) {
+        best = warp_pieces(bh, chunks);
     } else if (!(wide && bh >= 222 && bh <= 296)) {          // (two CTAs on an SM as they are: one piece was the best of 112 measured sizes of 2 to 64 chunks)
         auto waves = [](int64_t ctas) {
             const int64_t sm = (ctas + 147) / 148;
@@ -752,25 +787,50 @@ Params make_params(const la_problem& p, const Plan& pl, const int* lengths) {
 }
 
 template <typename C, int DP, int MP, bool EXACT> struct Kernels {
-    static constexpr int THREADS = kThreads<C>, BUF = C::BUF;
+    static constexpr int THREADS = kThreads<C>;
     static int sums(const la_problem& p, const Params& a, bool reverse, cudaStream_t st) {
         if (a.pieces == 1) return LA_OK;
         const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)(a.pieces - 1);
         if (reverse)
-            return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, true>>(kProfMmaSum, THREADS, bh, y, BUF * SumLayout<C, DP, MP, true>::BYTES, a, st);
-        return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, false>>(kProfMmaSum, THREADS, bh, y, BUF * SumLayout<C, DP, MP, false>::BYTES, a, st);
+            return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, true>>(kProfMmaSum, THREADS, bh, y, SumLayout<C, DP, MP, true>::BYTES, a, st);
+        return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, false>>(kProfMmaSum, THREADS, bh, y, SumLayout<C, DP, MP, false>::BYTES, a, st);
     }
     static int forward(const la_problem& p, const Params& a, cudaStream_t st) {
         if (int rc = sums(p, a, false, st)) return rc;
         return launch<causal_mma_forward_kernel<C, DP, MP, EXACT>>(kProfMmaForward, THREADS, (unsigned)(p.B * p.H), (unsigned)a.pieces,
-                      BUF * ForwardLayout<C, DP, MP>::BYTES, a, st);
+                      ForwardLayout<C, DP, MP>::BYTES, a, st);
     }
     static int backward(const la_problem& p, const Params& fwd, const Params& rev, cudaStream_t st) {
         const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)fwd.pieces;
         if (int rc = sums(p, fwd, false, st)) return rc;
-        if (int rc = launch<causal_mma_dq_kernel<C, DP, MP, EXACT>>(kProfMmaDq, THREADS, bh, y, BUF * DqLayout<C, DP, MP>::BYTES, fwd, st)) return rc;
+        if (int rc = launch<causal_mma_dq_kernel<C, DP, MP, EXACT>>(kProfMmaDq, THREADS, bh, y, DqLayout<C, DP, MP>::BYTES, fwd, st)) return rc;
         if (int rc = sums(p, rev, true, st)) return rc;
-        return launch<causal_mma_dkv_kernel<C, DP, MP, EXACT>>(kProfMmaDkv, THREADS, bh, y, BUF * DkvLayout<C, DP, MP>::BYTES, rev, st);
+        return launch<causal_mma_dkv_kernel<C, DP, MP, EXACT>>(kProfMmaDkv, THREADS, bh, y, DkvLayout<C, DP, MP>::BYTES, rev, st);
+    }
+};
+
+struct WarpKernels {
+    template <int PASS> static int run(const la_problem& p, ProfKernel prof, int pieces, const Params& a, cudaStream_t st) {
+        if (p.phi == LA_PHI_IDENTITY) return launch<causal_warp_kernel<PASS, false>>(prof, 32, (unsigned)(p.B * p.H), (unsigned)pieces, 0, a, st);
+        return launch<causal_warp_kernel<PASS, true>>(prof, 32, (unsigned)(p.B * p.H), (unsigned)pieces, 0, a, st);
+    }
+    static int forward(const la_problem& p, const Params& a, cudaStream_t st) {
+        if (a.pieces > 1)
+            if (int rc = run<kWarpSums>(p, kProfMmaSum, a.pieces - 1, a, st)) return rc;
+        return run<kWarpForward>(p, kProfMmaForward, a.pieces, a, st);
+    }
+    // (with a stamp: the forward pass has left the sums)
+    static int backward(const la_problem& p, const Params& fwd, const Params& rev, cudaStream_t st) {
+        if (fwd.pieces > 1 && !fwd.stamp)
+            if (int rc = run<kWarpSums>(p, kProfMmaSum, fwd.pieces - 1, fwd, st)) return rc;
+        if (fwd.pieces > 2 || p.N > 128) {       // (two pieces of a chunk or two: the warps with both sums would set the time)
+            if (int rc = run<kWarpDqReverse>(p, kProfMmaDq, fwd.pieces, fwd, st)) return rc;
+        } else {
+            if (int rc = run<kWarpDq>(p, kProfMmaDq, fwd.pieces, fwd, st)) return rc;
+            if (fwd.pieces > 1)
+                if (int rc = run<kWarpReverseSums>(p, kProfMmaSum, fwd.pieces - 1, rev, st)) return rc;
+        }
+        return run<kWarpDkv>(p, kProfMmaDkv, fwd.pieces, rev, st);
     }
 };
 
@@ -787,7 +847,7 @@ template <typename F> int dispatch(const la_problem& p, int pieces, F f) {
         if (p.D <= 64) return exact ? f(Kernels<Fp32, 64, 64, true>()) : f(Kernels<Fp32, 64, 64, false>());
         return f(Kernels<Fp32, 128, 64, false>());
     }
-    if (p.D == 32 && p.M == 32) return f(Kernels<Bf16, 32, 32, true>());
+    if (of_warps(p)) return f(WarpKernels());
     if (p.phi == LA_PHI_IDENTITY) {
         if (p.D <= 64) return f(Kernels<Bf16Features, 64, 64, false>());
         if (exact && full) return f(Kernels<Bf16FeaturesOne, 128, 64, true>());
@@ -804,38 +864,50 @@ bool causal_mma_supported(const la_problem& p) {
     return !disabled && p.M <= 64;
 }
 
-// bf16, D = M = 32, many short sequences: the tcgen05 kernels run one CTA per SM and start up for about three chunks of
-// 128 positions in every sequence, and handle 128 scores per row where D is 32.  Forward + backward, us, tcgen05 /
-// mma.sync: 1024 heads N 784 373 / 287, 2048 x 300 442 / 234, 512 x 512 131 / 102, 512 x 1024 212 / 192; but
-// 512 x 2048 367 / 372, 256 x 512 66 / 70, 128 x 3072 138 / 195.  (D = M = 64: 512 x 512 161 / 265.)
-bool causal_mma_preferred(const la_problem& p) {
-    return p.dtype == LA_BF16 && p.D == 32 && p.M == 32 && p.B * p.H >= 3 * 148 && p.N <= 1024;
-}
+bool causal_mma_preferred(const la_problem& p) { return of_warps(p); }
+
+// The forward's workspace is optional for all problems of this file but those that a warp per piece took over from the tcgen05 kernels.
+bool causal_mma_needs_workspace(const la_problem& p) { return of_warps(p) && (p.B * p.H < 3 * 148 || p.N > 1024); }
 
 size_t causal_mma_workspace(const la_problem& p, bool backward) {
     const size_t rec = record_bytes(p, choose_plan(p, false));
-    return backward ? aux_bytes(p) + rec : rec;
+    return backward ? aux_bytes(p) + (of_warps(p) ? 2 * rec : rec) : rec;
+}
+// the records of a forward pass, and the plan they were written under
+size_t causal_mma_saved_bytes(const la_problem& p) {
+    const size_t rec = causal_mma_needs_workspace(p) ? record_bytes(p, choose_plan(p, false)) : 0;
+    return rec ? kStampBytes + rec : 0;
 }
 
 int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
-                       const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* ws, size_t ws_bytes, cudaStream_t st) {
+                       const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, void* ws, size_t ws_bytes, cudaStream_t st) {
     Plan pl = choose_plan(p, false);
-    if (!ws || !aligned16(ws) || ws_bytes < record_bytes(p, pl)) pl = choose_plan(p, true);       // no room for records: one piece per sequence
+    if (saved && causal_mma_saved_bytes(p)) {
+        ws = (char*)saved + kStampBytes;
+    } else if (saved = nullptr; !ws || !aligned16(ws) || ws_bytes < record_bytes(p, pl)) pl = choose_plan(p, true);       // no room for records: one piece per sequence
     Params a = make_params(p, pl, lengths);
     a.Q = Q; a.K = K; a.V = V; a.O = O; a.den = den;
     a.S0 = S_in; a.Z0 = Z_in; a.S1 = S_out; a.Z1 = Z_out;
     a.rec = (float*)ws;
+    a.stamp = (int*)saved;
     return dispatch(p, pl.pieces, [&](auto k) { return decltype(k)::forward(p, a, st); });
 }
 
 int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
-                        const StateArgs& sa, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st) {
+                        const StateArgs& sa, const void* saved, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st) {
     const Plan pl = choose_plan(p, false);
     Params f = make_params(p, pl, lengths);
     f.Q = Q; f.K = K; f.V = V; f.G = G; f.dQ = dQ; f.dK = dK; f.dV = dV;
     f.aux = (float*)ws;
     f.rec = (float*)((char*)ws + aux_bytes(p));
+    if (saved && causal_mma_saved_bytes(p)) {
+        f.stamp = (int*)saved;
+        f.status = device_status_ptr();
+        if (!f.status) return fail(LA_ERR_CUDA, "device status word unavailable");
+    }
     Params r = f;
+    if (of_warps(p)) r.rec = f.rec_out = (float*)((char*)f.rec + record_bytes(p, pl));
+    if (f.stamp) f.rec = (float*)((char*)saved + kStampBytes);
     f.S0 = sa.S_in; f.Z0 = sa.Z_in;
     r.first_record = 1;
     r.S0 = sa.dS_out; r.Z0 = sa.dZ_out; r.S1 = sa.dS_in; r.Z1 = sa.dZ_in;

@@ -306,7 +306,7 @@ size_t record_bytes(const la_problem& p) {
 template <typename C, int DP, int MP, bool EXACT> struct Kernels {
     template <bool REVERSE> static int sums(const la_problem& p, const Params& a, cudaStream_t st) {
         return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, REVERSE>>(kProfMmaSum, kThreads<C>, (unsigned)(p.B * p.H), (unsigned)a.pieces,
-                                                                        C::BUF * SumLayout<C, DP, MP, REVERSE>::BYTES, a, st);
+                                                                        SumLayout<C, DP, MP, REVERSE>::BYTES, a, st);
     }
     template <auto KERNEL> static int apply(const la_problem& p, const Params& a, cudaStream_t st) {
         return launch<KERNEL>(kProfMmaApply, THREADS, (unsigned)(p.B * p.H), (unsigned)a.pieces, ApplyLayout<C, DP, MP>::BYTES, a, st);

@@ -23,6 +23,7 @@ struct Params {
     const float *S0, *Z0;        // state the sweep starts from (forward: S_in, Z_in; reverse: dS_out, dZ_out), each or null
     float *S1, *Z1;              // where the state it ends with goes (S_out, Z_out / dS_in, dZ_in), each or null
     float* rec;                  // [bh][records][D * M + D]: sums of the pieces first_record .. first_record + records - 1
+    float* rec_out;              // where the dQ sweep leaves the reverse records, or null
     int records, first_record;
     float* aux;                  // [bh][2][N]: dn_i, -G_i . O_i
     const int* lengths;
@@ -228,17 +229,17 @@ struct State {
 // q / dn (NR).  Everything computed in fp32 has three planes; bf16 values, and features that are bf16 as given, one.
 struct Fp32 {
     using IO = float;
-    static constexpr int NQ = 3, NV = 3, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
+    static constexpr int NQ = 3, NV = 3, NP = 3, NS = 3, NR = 3, WPS = 2;
     static constexpr bool MAPPED = true, ALONE = false;
 };
 struct Bf16Wide {
     using IO = __nv_bfloat16;
-    static constexpr int NQ = 3, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
+    static constexpr int NQ = 3, NV = 1, NP = 3, NS = 3, NR = 3, WPS = 2;
     static constexpr bool MAPPED = true, ALONE = false;
 };
 struct Bf16Features {
     using IO = __nv_bfloat16;
-    static constexpr int NQ = 1, NV = 1, NP = 3, NS = 3, NR = 3, BUF = 1, WPS = 2;
+    static constexpr int NQ = 1, NV = 1, NP = 3, NS = 3, NR = 3, WPS = 2;
     static constexpr bool MAPPED = false, ALONE = false;
 };
 // ... with one warp per strip, at twice the registers: where a machine full of CTAs keeps the schedulers busy anyway, the
@@ -251,11 +252,10 @@ struct Bf16FeaturesOne : Bf16Features { static constexpr int WPS = 1; };
 // N2666 341 / 327; fp32 D = 64 B1 H8 N2000 110 / 100, B16 H8 N100 67 / 59 (but 160 CTAs, B20 H8 N99, 95 / 100).
 struct Fp32Alone : Fp32 { static constexpr bool ALONE = true; };
 struct Bf16FeaturesAlone : Bf16Features { static constexpr bool ALONE = true; };
-// bf16 operands throughout (with fp32 sums), as the tcgen05 kernels have them.  BUF = 2: the small tiles are there twice,
-// one barrier per chunk (the other set was last read before the barrier of this chunk).
+// bf16 operands throughout (with fp32 sums), as the tcgen05 kernels have them (la_cluster.cu)
 struct Bf16 {
     using IO = __nv_bfloat16;
-    static constexpr int NQ = 1, NV = 1, NP = 1, NS = 1, NR = 1, BUF = 2, WPS = 1;
+    static constexpr int NQ = 1, NV = 1, NP = 1, NS = 1, NR = 1, WPS = 1;
     static constexpr bool MAPPED = true, ALONE = false;
 };
 
@@ -271,16 +271,10 @@ template <typename C, int DP, int MP, bool REVERSE>
 using SumLayout = Layout<1, DP, MP, REVERSE ? C::NR : C::NQ, C::NV, 0, 0, 0, 0>;
 
 template <typename C> constexpr int kThreads = 128 * C::WPS;
-// CTAs of an SM that the registers are shared out for: as many as shared memory holds, at most two (or `three_planes`),
-// or four where operands have single planes (1024 sequences of 784: 287 us, five 300, six 330)
-template <typename Sh, typename C> constexpr int resident(int three_planes = 2) {
-    const int fit = 227 * 1024 / (C::BUF * Sh::BYTES + 1024), most = C::NP == 1 ? 4 : three_planes;
+// CTAs of an SM that the registers are shared out for: as many as shared memory holds, at most two (or `most`)
+template <typename Sh> constexpr int resident(int most = 2) {
+    const int fit = 227 * 1024 / (Sh::BYTES + 1024);
     return fit < most ? fit : most;
-}
-
-template <typename C, typename Sh>
-__device__ __forceinline__ void flip(uint8_t*& buf, uint8_t* smem) {
-    if constexpr (C::BUF == 2) buf = buf == smem ? smem + Sh::BYTES : smem;
 }
 
 template <int NT8> __device__ __forceinline__ void clear(float (&x)[NT8][4]) {
@@ -291,19 +285,13 @@ template <int NT8> __device__ __forceinline__ void clear(float (&x)[NT8][4]) {
 }
 
 // rows n0 .. n0 + T - 1, those before `end`, on their way to L2
-template <typename C, int COLS, typename IO>
+template <typename C, typename IO>
 __device__ __forceinline__ void prefetch_rows(const IO* x, int64_t n0, int64_t end, int cols) {
     constexpr int THREADS = kThreads<C>;
     if (n0 < 0 || n0 >= end) return;
     const int64_t rows = end - n0 < T ? end - n0 : T;
     const char* p = reinterpret_cast<const char*>(x + n0 * cols);
-    if constexpr (C::BUF == 2) {            // (few lines: no loop)
-        const int bytes = (int)rows * cols * (int)sizeof(IO), o = (int)threadIdx.x * 128;
-        static_assert(T * COLS * (int)sizeof(IO) <= THREADS * 128, "one line per thread");
-        if (o < bytes) prefetch_l2(p + o);
-    } else {
-        for (int64_t o = threadIdx.x * 128; o < rows * cols * (int64_t)sizeof(IO); o += THREADS * 128) prefetch_l2(p + o);
-    }
+    for (int64_t o = threadIdx.x * 128; o < rows * cols * (int64_t)sizeof(IO); o += THREADS * 128) prefetch_l2(p + o);
 }
 
 // feature-mapped pairs in registers: bf16 where features have one plane
@@ -346,13 +334,12 @@ struct ReverseRows {
 };
 
 template <typename C, int DP, int MP, bool EXACT, bool REVERSE>
-__global__ void __launch_bounds__(kThreads<C>, C::NP == 1 ? 4 : 2)
+__global__ void __launch_bounds__(kThreads<C>, 2)
 causal_mma_sum_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = SumLayout<C, DP, MP, REVERSE>;
     constexpr int NX = REVERSE ? C::NR : C::NQ, NY = C::NV, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t* buf = smem;
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
     wait_for_stream();
@@ -366,28 +353,27 @@ causal_mma_sum_kernel(const Params p) {
     State<DP, MP, 4 * C::WPS> st;
     st.init(p, nullptr, nullptr, nullptr, 0);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
-        float* w = reinterpret_cast<float*>(buf + Sh::W);
-        uint16_t* wpl = reinterpret_cast<uint16_t*>(buf + Sh::WP);
+        float* w = reinterpret_cast<float*>(smem + Sh::W);
+        uint16_t* wpl = reinterpret_cast<uint16_t*>(smem + Sh::WP);
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
         if constexpr (REVERSE) {
             ReverseRows<IO, DP, MP, THREADS> rr;
             rr.load(X, Y, dn, delta, n0, cn, D, M, pad);
-            if constexpr (C::BUF == 1) __syncthreads();
-            rr.template store<NX, NY>(buf + Sh::X, buf + Sh::Y, w, wpl, phi);
+            __syncthreads();
+            rr.template store<NX, NY>(smem + Sh::X, smem + Sh::Y, w, wpl, phi);
         } else {
             RawTile<IO, T, DP, THREADS> rx;
             RawTile<IO, T, MP, THREADS> ry;
             rx.load(X + n0 * D, cn, D, pad);
             ry.load(Y + n0 * M, cn, M, 0.f);
-            if constexpr (C::BUF == 1) __syncthreads();
-            rx.template features<NX>(buf + Sh::X, phi);
-            ry.template values<NY>(buf + Sh::Y);
+            __syncthreads();
+            rx.template features<NX>(smem + Sh::X, phi);
+            ry.template values<NY>(smem + Sh::Y);
         }
-        prefetch_rows<C, DP>(X, n0 + T, r.end, D);
-        prefetch_rows<C, MP>(Y, n0 + T, r.end, M);
+        prefetch_rows<C>(X, n0 + T, r.end, D);
+        prefetch_rows<C>(Y, n0 + T, r.end, M);
         __syncthreads();
-        st.template update<NX, NY, !REVERSE>(smem_u32(buf + Sh::X), smem_u32(buf + Sh::Y), wpl);
-        flip<C, Sh>(buf, smem);
+        st.template update<NX, NY, !REVERSE>(smem_u32(smem + Sh::X), smem_u32(smem + Sh::Y), wpl);
     }
     float* dst = p.rec + (r.bh * p.records + blockIdx.y) * (int64_t)(D * M + D);
     st.write(p, dst, dst + D * M);

@@ -11,15 +11,17 @@ size_t tc_workspace_bytes(const la_problem& p, int op);
 // pieces, parts, piece_begin[], piece_first_part[], part_begin[], launch_order[] (see la_causal_plan)
 int tc_causal_plan(const la_problem& p, int32_t* out, int capacity);
 
-// Causal form at fp32 accuracy on mma.sync (la_causal_mma.cu): M <= 64, any type and feature map.  The forward's
-// workspace is optional (without it a sequence is one piece).
+// Causal form on mma.sync (la_causal_mma.cu): at fp32 accuracy, M <= 64, any type and feature map; and bf16 problems with D = M = 32 by a
+// warp per piece.  The forward's workspace is optional (without it a sequence is one piece) but for some of the latter.
 bool causal_mma_supported(const la_problem& p);
 bool causal_mma_preferred(const la_problem& p);      // of the problems that both kinds of kernels take
+bool causal_mma_needs_workspace(const la_problem& p);
 size_t causal_mma_workspace(const la_problem& p, bool backward);
+size_t causal_mma_saved_bytes(const la_problem& p);  // what a forward pass leaves for the backward pass, or 0
 int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
-                       const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* ws, size_t ws_bytes, cudaStream_t st);
+                       const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, void* ws, size_t ws_bytes, cudaStream_t st);
 int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
-                        const StateArgs& sa, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
+                        const StateArgs& sa, const void* saved, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
 
 // Non-causal form at fp32 accuracy on mma.sync (la_linear_mma.cu): M <= 64, any type and feature map; saved (or null):
 // where the forward leaves its sums and the backward finds them.

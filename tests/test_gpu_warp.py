@@ -1,0 +1,115 @@
+"""bf16, D = M = 32: a warp per piece of a sequence, at the edges of its chunks of sixteen positions, whole and in pieces, ragged, from
+a state, with and without a saved buffer, against the fp64 oracle under the bf16 gates."""
+import os
+import re
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2006_16236_b200 as la
+from paper_2006_16236_b200.inputs import draw_qkvg
+from parity import assert_close
+
+DEV, BF, D = "cuda:0", torch.bfloat16, 32
+
+
+@pytest.fixture(autouse=True)
+def _automatic_plans():
+    yield
+    la.la_plan_override()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("pieces", [-1, 1, 2, 5])
+@pytest.mark.parametrize("B,H,N", [(38, 8, 1), (38, 8, 15), (38, 8, 17), (38, 8, 63), (38, 8, 64), (38, 8, 200), (1, 2, 2100), (2, 1, 2049 + 64)])
+def test_pieces_lengths_and_states(B, H, N, pieces):
+    Q, K, V, G = draw_qkvg(B, H, N, D, D, 7 + N, BF, 1.0)
+    g = torch.Generator().manual_seed(N)
+    S0, Z0 = torch.randn((B, H, D, D), generator=g) * 3.0, torch.rand((B, H, D), generator=g) * 4.0 + 1.0
+    dSN, dZN = torch.randn((B, H, D, D), generator=g) * 0.05, torch.randn((B, H, D), generator=g) * 0.05
+    lengths = [max(N - (7 * b) % (N + 1), 0) for b in range(B)]
+    lengths[0] = N
+    la.la_plan_override(pieces)
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    st = {"S_in": S0.to(DEV), "Z_in": Z0.to(DEV)}
+    ln = torch.tensor(lengths, dtype=torch.int32, device=DEV)
+    for phi in ("elu1", "identity"):
+        if phi == "identity":                           # features: positive, as the weights of a kernel are
+            Q, K = (Q.float().abs() + 0.1).to(BF), (K.float().abs() + 0.1).to(BF)
+            dev[:2] = Q.to(DEV), K.to(DEV)
+        S, Z, den = torch.empty_like(st["S_in"]), torch.empty_like(st["Z_in"]), torch.empty(B, H, N, device=DEV)
+        dS, dZ = torch.empty_like(S), torch.empty_like(Z)
+        saved = la.saved_buffer(dev[0], dev[2], phi=phi)
+        O = la.la_causal_forward(*dev[:3], phi=phi, lengths=ln, den=den, S_out=S, Z_out=Z, saved=saved, **st)
+        kw = {"phi": phi, "lengths": ln, "dS_out": dSN.to(DEV), "dZ_out": dZN.to(DEV), **st}
+        grads = la.la_causal_backward(*dev, saved=saved, dS_in=dS, dZ_in=dZ, **kw)
+        again = la.la_causal_backward(*dev, **kw)       # the kept sums are those that it would make itself
+        la.la_last_device_status()
+        assert all(torch.equal(a, b) for a, b in zip(grads, again))
+        for b in {0, min(1, B - 1), B - 1}:
+            n, h = lengths[b], b % H
+            assert not O[b, :, n:].any() and not den[b, :, n:].any() and not any(x[b, :, n:].any() for x in grads)
+            sl = (slice(b, b + 1), slice(h, h + 1))
+            s0, z0 = S0[sl].double().numpy(), Z0[sl].double().numpy()
+            if n == 0:
+                assert torch.equal(S[sl].cpu(), S0[sl]) and torch.equal(Z[sl].cpu(), Z0[sl])
+                continue
+            q, k, v, u = (t[sl][:, :, :n].double().numpy() for t in (Q, K, V, G))
+            Or, denr, Sr, Zr = oracle.causal_from_state(q, k, v, s0, z0, phi=phi)
+            for nm, x, ref in (("O", O[sl][:, :, :n], Or), ("den", den[sl][:, :, :n], denr), ("S_out", S[sl], Sr), ("Z_out", Z[sl], Zr)):
+                assert_close(x, ref, BF, nm)
+            refs = oracle.causal_backward_from_state(q, k, v, s0, z0, u, dSN[sl].double().numpy(), dZN[sl].double().numpy(), phi=phi)
+            for nm, x, ref in zip(("dQ", "dK", "dV", "dS_in", "dZ_in"), [x[sl][:, :, :n] for x in grads] + [dS[sl], dZ[sl]], refs):
+                assert_close(x, ref, BF, nm, grad=True)
+
+
+@pytest.mark.gpu
+def test_kept_sums_of_another_plan_are_refused():
+    if os.environ.get("LA_DEBUG"):
+        pytest.skip("in checked mode the call itself reads the status and raises; this test reads it afterwards")
+    dev = [t.to(DEV) for t in draw_qkvg(2, 4, 2200, D, D, 3, BF, 1.0)]
+    la.la_plan_override(3)
+    saved = torch.zeros(1 << 20, dtype=torch.uint8, device=DEV)
+    la.la_causal_forward(*dev[:3], saved=saved)
+    la.la_plan_override(4)
+    dQ, dK, dV = (torch.full_like(dev[0], 7.0) for _ in range(3))
+    la.la_causal_backward(*dev, saved=saved, dQ=dQ, dK=dK, dV=dV)
+    with pytest.raises(la.LaError) as e:
+        la.la_last_device_status()
+    assert e.value.status == -1 and "plan" in str(e.value)
+    assert torch.all(dQ == 7.0) and torch.all(dK == 7.0) and torch.all(dV == 7.0)
+
+
+@pytest.mark.gpu
+def test_steps_enqueued_behind_each_other():
+    """Forward and backward passes of small grids start as programmatic dependents of each other; inputs change in between."""
+    data = [[t.to(DEV) for t in draw_qkvg(1, 2, 2100, D, D, 20 + i, BF, 1.0)] for i in range(6)]
+    step = lambda x, s: (la.la_causal_forward(*x[:3], saved=s), *la.la_causal_backward(*x, saved=s))
+    want = []
+    for x in data:
+        want.append(step(x, la.saved_buffer(x[0], x[2])))
+        torch.cuda.synchronize()
+    buf, saved, got = [torch.empty_like(t) for t in data[0]], la.saved_buffer(data[0][0], data[0][2]), []
+    for x in data:
+        for a, b in zip(buf, x):
+            a.copy_(b)
+        got.append(step(buf, saved))
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for w, g in zip(want, got) for a, b in zip(w, g))
+
+
+def test_workspace_and_saved_sizes():
+    """Problems that kernels with a required workspace had before keep requiring one; others keep neither needing nor keeping one."""
+    p = lambda *s: la.make_problem(*s, 32, 32, la.LA_BF16)
+    size = lambda q, op: la.la_workspace_bytes(q, op)
+    assert size(p(16, 8, 3072), la.LA_OP_CAUSAL_FORWARD) > 0 and size(p(16, 8, 3072), la.LA_OP_CAUSAL_SAVED) > 0
+    assert size(p(128, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0 and size(p(60, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0
+
+
+def test_no_read_only_loads():
+    """As the other kernels that may start as programmatic dependents."""
+    path = os.path.join(os.path.dirname(la.__file__), "csrc", "la_causal_warp.cuh")
+    code = re.sub(r"//[^\n]*", "", open(path).read())
+    assert not re.findall(r"__ldg\s*\(|ld\.global\.nc|const \w+\s*\*\s*__restrict__", code)
