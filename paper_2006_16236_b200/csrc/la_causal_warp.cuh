@@ -3,10 +3,8 @@
 // The running sums of such a problem are 32 x 33 numbers: a warp holds them in its registers, walks its piece in chunks of
 // sixteen positions and needs no other warp.  Every product is mma.sync m16n8k16 (tcgen05 wants 128 rows: at D = 32 that is four
 // times as many scores as sums, and a start-up of three chunks per piece).  Nothing is exchanged through shared memory either:
-//   * A lane loads sixteen bytes of a row, columns 8 t .. 8 t + 7, and takes the four pairs as columns 2 t, 2 t + 1 of the four
-//     8-column tiles of an operand.  Tiles therefore hold the columns in another order (column 2 t + e of tile n is column
-//     8 t + 2 n + e of the tensor), the same one for every operand, so that all sums over columns agree and a result row
-//     leaves as sixteen bytes again.  With the fragments as they are, 2 bytes by 2, the L1 pipe was 70 % busy.
+//   * Rows arrive and leave in loads and stores of sixteen bytes, the columns in the order of la_warp.cuh.  With the fragments as they
+//     lie, pair by pair, the L1 pipe was 70 % busy.
 //   * The transposes that sums over positions need come from movmatrix.
 //   * The accumulators of the sums, rounded to bf16, are the operand of the next chunk's products as they lie.
 // Chunks of sixteen: one diagonal block of scores and no others, and a loop of 350 to 450 instructions (beyond some 500
@@ -24,69 +22,19 @@
 
 #include <type_traits>
 
-#include "la_mma_sweep.cuh"
+#include "la_warp.cuh"
 
 namespace la {
 namespace warp32 {
 
-using namespace mma;
+using namespace warp;
 using sweep::Params;
 using sweep::Range;
 
-constexpr int ROWS = 16;                    // positions of a chunk
 constexpr int C = 32, NT = C / 8;           // columns of a row, and their tiles
-constexpr int STAGES = 3;                   // the chunk at hand and those on their way
 constexpr int RECORD_FLOATS = C * C + C;
-
-// Sixteen rows: x[h][n] = columns 2 t, 2 t + 1 of tile n in row g + 8 h.  As an A operand (rows x columns) and as a B operand
-// (columns x rows) it serves as it lies; transposed, t[h][n] = rows 8 h + 2 t, 2 t + 1 of column g of tile n, it is
-// an A operand (columns x rows) and a B operand (rows x columns).
-struct Rows { uint32_t x[2][NT]; };
-
-__device__ __forceinline__ uint32_t transposed(uint32_t v) {
-    uint32_t r;
-    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
-    return r;
-}
-__device__ __forceinline__ Rows transposed(const Rows& r) {
-    Rows o;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int n = 0; n < NT; ++n) o.x[h][n] = transposed(r.x[h][n]);
-    return o;
-}
-
-__device__ __forceinline__ void mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_first(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
-        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
-}
-// c (rows of a x eight rows or columns) = or += the columns of a times b, b's operand pairs given by f(kk, half)
-template <bool FIRST, typename F>
-__device__ __forceinline__ void columns_mma(float (&c)[4], const Rows& a, F f) {
-#pragma unroll
-    for (int kk = 0; kk < NT / 2; ++kk) {
-        if (FIRST && kk == 0) mma_first(c, a.x[0][0], a.x[1][0], a.x[0][1], a.x[1][1], f(0, 0), f(0, 1));
-        else mma(c, a.x[0][2 * kk], a.x[1][2 * kk], a.x[0][2 * kk + 1], a.x[1][2 * kk + 1], f(kk, 0), f(kk, 1));
-    }
-}
-
-// two additions in one instruction
-__device__ __forceinline__ void add_pair(float& x, float& y, float a, float b) {
-    sm100::unpair(sm100::add2(sm100::pair(x, y), sm100::pair(a, b)), x, y);
-}
-// 1 / x to the last bit or two
-__device__ __forceinline__ float reciprocal(float x) {
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-constexpr uint32_t kOnes = 0x3f803f80u, kMinusInf = 0xff80ff80u;
+using Rows = warp::Rows<C>;
+template <int T, bool WEIGHTS> using Ring = warp::Ring<C, T, WEIGHTS>;
 
 // ---- the running sums -------------------------------------------------------------------------------------------
 // s[i][n]: rows 16 i + g (+ 8), columns 2 t, 2 t + 1 of tile n of the matrix X^T Y, rows and columns in the order of the tiles
@@ -136,7 +84,7 @@ struct Sums {
         for (int n = 0; n < NT; ++n) {
             float t[4];
             mma_first(t, p0[2], 0u, p1[2], 0u, b.x[0][n], b.x[1][n]);
-            mma(t, p0[0], p0[1], p1[0], p1[1], b.x[0][n], b.x[1][n]);
+            mma_add(t, p0[0], p0[1], p1[0], p1[1], b.x[0][n], b.x[1][n]);
             add_pair(t[0], t[1], t[2], t[3]);
             add_pair(v[n][0], v[n][1], t[0], t[1]);
         }
@@ -252,84 +200,6 @@ struct Span {
     }
 };
 
-// T tensors of sixteen rows each, a lane's own sixteen bytes of rows g and g + 8; WEIGHTS: and two fp32 numbers per row.
-template <int T, bool WEIGHTS>
-struct Ring {
-    static constexpr int STAGE_BYTES = T * 1024 + (WEIGHTS ? 128 : 0), BYTES = STAGES * STAGE_BYTES;
-    const uint8_t* src[T];          // the lane's bytes of the sequence's first chunk
-    const float* w;                 // the lane's weight of it: dn in lanes 0 .. 15, dl in lanes 16 .. 31
-    uint8_t* mine;                  // the lane's bytes of slot 0
-    int read, write;                // offsets of the slot at hand and of the next one to be filled
-    int end;                        // rows from `end` on are not there: zeros
-
-    __device__ __forceinline__ void start(uint8_t* smem, const Span& r, int64_t N, const void* const (&tensors)[T], const float* aux) {
-        const int lane = threadIdx.x & 31;
-#pragma unroll
-        for (int i = 0; i < T; ++i) src[i] = (const uint8_t*)tensors[i] + r.bh * N * (C * 2) + lane * 16;
-        if constexpr (WEIGHTS) w = aux + 2 * r.bh * N + (lane < 16 ? lane : N + lane - 16);
-        mine = smem + lane * 16;
-        end = r.end;
-        read = write = 0;
-    }
-    __device__ __forceinline__ void request(int n0) {
-        if constexpr (WEIGHTS) __syncwarp();            // every lane has read what is overwritten
-        if (n0 >= 0 && n0 < end) {
-            const int lane = threadIdx.x & 31, left = end - n0;
-            const uint32_t dst = smem_u32(mine + write);
-            const int64_t at = (int64_t)n0 * (C * 2);
-            if (left >= ROWS) {
-#pragma unroll
-                for (int i = 0; i < T; ++i)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 1024 + h * 512), "l"(src[i] + at + h * 512) : "memory");
-                if constexpr (WEIGHTS) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst - lane * 12 + T * 1024), "l"(w + n0) : "memory");
-            } else {                // (a size of zero reads nothing; the address stays inside the tensor)
-#pragma unroll
-                for (int i = 0; i < T; ++i)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const bool real = (lane >> 2) + 8 * h < left;
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + i * 1024 + h * 512),
-                                     "l"(real ? src[i] + at + h * 512 : src[i] - lane * 16), "r"(real ? 16 : 0) : "memory");
-                    }
-                if constexpr (WEIGHTS) {
-                    const bool real = (lane & 15) < left;
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst - lane * 12 + T * 1024), "l"(real ? w + n0 : w - (lane & 15)),
-                                 "r"(real ? 4 : 0) : "memory");
-                }
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        write = write == (STAGES - 1) * STAGE_BYTES ? 0 : write + STAGE_BYTES;
-    }
-    __device__ __forceinline__ void next() { read = read == (STAGES - 1) * STAGE_BYTES ? 0 : read + STAGE_BYTES; }
-    // The chunk STAGES - 1 behind the one that was just requested has arrived.  Of its `real` rows, if they are not all, the
-    // others of tensor `i` become what has no feature.
-    template <bool ELU> __device__ __forceinline__ void arrived(int i, int real) const {
-        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
-        if (real < ROWS) {
-            const int lane = threadIdx.x & 31;
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                if ((lane >> 2) + 8 * h >= real) *reinterpret_cast<uint4*>(mine + read + i * 1024 + h * 512) = ELU ? make_uint4(kMinusInf, kMinusInf, kMinusInf, kMinusInf) : make_uint4(0u, 0u, 0u, 0u);
-            if constexpr (WEIGHTS)
-                if (lane < 16 && lane >= real) *reinterpret_cast<float*>(mine + read - lane * 12 + T * 1024) = 1.f;
-        }
-        if constexpr (WEIGHTS) __syncwarp();
-    }
-    __device__ __forceinline__ Rows rows(int i) const {
-        Rows r;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint4 v = *reinterpret_cast<const uint4*>(mine + read + i * 1024 + h * 512);
-            r.x[h][0] = v.x; r.x[h][1] = v.y; r.x[h][2] = v.z; r.x[h][3] = v.w;
-        }
-        return r;
-    }
-    __device__ __forceinline__ const float* weights() const { return reinterpret_cast<const float*>(mine + read - (threadIdx.x & 31) * 16 + T * 1024); }
-};
-
 // features of sixteen rows, two at a time
 template <bool ELU> __device__ __forceinline__ void map_features(Rows& r) {
     if constexpr (ELU)
@@ -367,15 +237,7 @@ template <bool UPPER> __device__ __forceinline__ uint32_t diagonal_mask() {
     return (lo ? 0xffffu : 0u) | (hi ? 0xffff0000u : 0u);
 }
 
-// the lane's part of a row's dot product: a (bf16 pairs) with b (fp32 pairs at the same columns)
-template <typename F>
-__device__ __forceinline__ float row_part(const uint32_t (&a)[NT], F b) {
-    sm100::f32x2 d = sm100::mul2(sm100::pair_bf16(a[0]), b(0));
-#pragma unroll
-    for (int n = 1; n < NT; ++n) d = sm100::fma2(sm100::pair_bf16(a[n]), b(n), d);
-    return sm100::pair_sum(d);
-}
-
+template <typename F> __device__ __forceinline__ float row_sum(const uint32_t (&a)[NT], F b) { return sm100::pair_sum(row_part(a, b)); }
 // the lane's bytes of a result's row g; row g + 8 is 512 further
 __device__ __forceinline__ uint8_t* rows_at(void* tensor, const Span& r, int64_t N, int n0) {
     return (uint8_t*)tensor + (r.bh * N + n0) * (C * 2) + (threadIdx.x & 31) * 16;
@@ -395,8 +257,8 @@ __device__ __forceinline__ void forward(const Params& p, uint8_t* smem) {
     uint8_t* O = rows_at(p.O, r, p.N, r.lo);
     float* den = p.den ? p.den + r.bh * p.N : nullptr;
     Ring<3, false> in;
-    in.start(smem, r, p.N, {p.Q, p.K, p.V}, nullptr);
-    for (int i = 0; i < STAGES - 1; ++i) in.request(r.lo + i * ROWS);
+    in.start(smem, r.bh, p.N, r.end, {p.Q, p.K, p.V}, nullptr);
+    for (int i = 0; i < in.AHEAD; ++i) in.request(r.lo + i * ROWS);
 
     Sums st;                // S^T: rows are the columns of V
     st.clear();
@@ -406,8 +268,8 @@ __device__ __forceinline__ void forward(const Params& p, uint8_t* smem) {
 #pragma unroll 1
     for (int n0 = r.lo; n0 < r.end; n0 += ROWS) {
         const int cn = r.end - n0;              // (of them sixteen at most)
-        in.request(n0 + (STAGES - 1) * ROWS);
-        in.template arrived<ELU>(1, r.end - n0);
+        in.request(n0 + in.AHEAD * ROWS);
+        in.arrived(1, r.end - n0, ELU ? kMinusInf : 0u);
         Rows q = in.rows(0), k = in.rows(1);
         const Rows v = in.rows(2);
         map_features<ELU>(q);
@@ -427,9 +289,9 @@ __device__ __forceinline__ void forward(const Params& p, uint8_t* smem) {
             const uint32_t a0 = pack_rn(s0[0], s0[1]) & lower, a1 = pack_rn(s0[2], s0[3]), a3 = pack_rn(s1[2], s1[3]) & lower;
             mma_first(u, a0, a1, 0u, a3, kOnes, kOnes);            // numerator and normaliser see the same rounded scores
 #pragma unroll
-            for (int n = 0; n < NT; ++n) mma(o[n], a0, a1, 0u, a3, vt.x[0][n], vt.x[1][n]);
-            d0 = u[0] + quad_sum(row_part(q.x[0], [&](int n) { return sm100::pair(st.v[n][0], st.v[n][1]); }));
-            d1 = u[2] + quad_sum(row_part(q.x[1], [&](int n) { return sm100::pair(st.v[n][0], st.v[n][1]); }));
+            for (int n = 0; n < NT; ++n) mma_add(o[n], a0, a1, 0u, a3, vt.x[0][n], vt.x[1][n]);
+            d0 = u[0] + quad_sum(row_sum(q.x[0], [&](int n) { return sm100::pair(st.v[n][0], st.v[n][1]); }));
+            d1 = u[2] + quad_sum(row_sum(q.x[1], [&](int n) { return sm100::pair(st.v[n][0], st.v[n][1]); }));
         }
         {
             const Rows kt = transposed(k);
@@ -463,14 +325,14 @@ __device__ __forceinline__ void sums(const Params& p, uint8_t* smem) {
     const Span r(p, (int)blockIdx.y + p.first_record);
     if (p.stamp && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *reinterpret_cast<int4*>(p.stamp) = sweep::plan_stamp(p);
     Ring<2, false> in;
-    in.start(smem, r, p.N, {p.K, p.V}, nullptr);
-    for (int i = 0; i < STAGES - 1; ++i) in.request(r.lo + i * ROWS);
+    in.start(smem, r.bh, p.N, r.end, {p.K, p.V}, nullptr);
+    for (int i = 0; i < in.AHEAD; ++i) in.request(r.lo + i * ROWS);
     Sums st;
     st.clear();
 #pragma unroll 1
     for (int n0 = r.lo; n0 < r.end; n0 += ROWS) {
-        in.request(n0 + (STAGES - 1) * ROWS);
-        in.template arrived<ELU>(0, r.end - n0);
+        in.request(n0 + in.AHEAD * ROWS);
+        in.arrived(0, r.end - n0, ELU ? kMinusInf : 0u);
         Rows k = in.rows(0);
         const Rows v = in.rows(1);
         map_features<ELU>(k);
@@ -493,8 +355,8 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     float* dn_all = p.aux + 2 * r.bh * p.N;
     float* dl_all = dn_all + p.N;
     Ring<4, false> in;
-    in.start(smem, r, p.N, {p.Q, p.K, p.V, p.G}, nullptr);
-    for (int i = 0; i < STAGES - 1; ++i) in.request(r.lo + i * ROWS);
+    in.start(smem, r.bh, p.N, r.end, {p.Q, p.K, p.V, p.G}, nullptr);
+    for (int i = 0; i < in.AHEAD; ++i) in.request(r.lo + i * ROWS);
 
     Sums st;                // S: rows are features
     st.clear();
@@ -512,8 +374,8 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     // is then what it was with chunks of 64 positions (B128 H8 N784: 4.4e-3; with one chunk 4.6e-3).
     auto chunk = [&](int n0, auto first) {
         const int cn = r.end - n0;              // (of them sixteen at most)
-        in.request(n0 + (STAGES - 1) * ROWS);
-        in.template arrived<ELU>(1, cn);
+        in.request(n0 + in.AHEAD * ROWS);
+        in.arrived(1, cn, ELU ? kMinusInf : 0u);
         Rows q = in.rows(0), k = in.rows(1);
         const Rows v = in.rows(2), G = in.rows(3);
         in.next();
@@ -551,10 +413,10 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
             const uint32_t a0 = pack_rn(s0[0], s0[1]) & lower, a1 = pack_rn(s0[2], s0[3]), a3 = pack_rn(s1[2], s1[3]) & lower;
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
-                mma(h[n], a0, a1, 0u, a3, kt.x[0][n], kt.x[1][n]);
+                mma_add(h[n], a0, a1, 0u, a3, kt.x[0][n], kt.x[1][n]);
                 zc[n][0] = zc[n][2] = st.v[n][0];
                 zc[n][1] = zc[n][3] = st.v[n][1];
-                mma(zc[n], kOnes & lower, kOnes, 0u, kOnes & lower, kt.x[0][n], kt.x[1][n]);
+                mma_add(zc[n], kOnes & lower, kOnes, 0u, kOnes & lower, kt.x[0][n], kt.x[1][n]);
             }
             if (pass == 1) {            // (the sums are not needed any more; their products run beside the row sums)
                 st.add(kt, transposed(v));
@@ -563,8 +425,8 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
             float d[2], e[2];
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                d[b] = row_part(q.x[b], [&](int n) { return sm100::pair(zc[n][2 * b], zc[n][2 * b + 1]); });
-                e[b] = row_part(q.x[b], [&](int n) { return sm100::pair(h[n][2 * b], h[n][2 * b + 1]); });
+                d[b] = row_sum(q.x[b], [&](int n) { return sm100::pair(zc[n][2 * b], zc[n][2 * b + 1]); });
+                e[b] = row_sum(q.x[b], [&](int n) { return sm100::pair(h[n][2 * b], h[n][2 * b + 1]); });
             }
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
@@ -626,14 +488,14 @@ __device__ __forceinline__ void reverse_sums(const Params& p, uint8_t* smem) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const Span r(p, (int)blockIdx.y + p.first_record);
     Ring<2, true> in;
-    in.start(smem, r, p.N, {p.Q, p.G}, p.aux);
-    for (int i = 0; i < STAGES - 1; ++i) in.request(r.lo + i * ROWS);
+    in.start(smem, r.bh, p.N, r.end, {p.Q, p.G}, p.aux);
+    for (int i = 0; i < in.AHEAD; ++i) in.request(r.lo + i * ROWS);
     Sums st;
     st.clear();
 #pragma unroll 1
     for (int n0 = r.lo; n0 < r.end; n0 += ROWS) {
-        in.request(n0 + (STAGES - 1) * ROWS);
-        in.template arrived<ELU>(0, r.end - n0);
+        in.request(n0 + in.AHEAD * ROWS);
+        in.arrived(0, r.end - n0, ELU ? kMinusInf : 0u);
         Rows q = in.rows(0);
         const Rows G = in.rows(1);
         const float* w = in.weights();
@@ -656,9 +518,9 @@ __device__ __forceinline__ void dkv(const Params& p, uint8_t* smem) {
     const int last = r.lo + (r.end - r.lo - 1) / ROWS * ROWS;           // (an empty piece: its end is its start)
     uint8_t *dK = rows_at(p.dK, r, p.N, last), *dV = rows_at(p.dV, r, p.N, last);
     Ring<4, true> in;
-    in.start(smem, r, p.N, {p.Q, p.K, p.V, p.G}, p.aux);
+    in.start(smem, r.bh, p.N, r.end, {p.Q, p.K, p.V, p.G}, p.aux);
     auto at = [&](int n0) { return n0 >= r.lo ? n0 : -1; };
-    for (int i = 0; i < STAGES - 1; ++i) in.request(at(last - i * ROWS));
+    for (int i = 0; i < in.AHEAD; ++i) in.request(at(last - i * ROWS));
 
     Sums st;                // R: rows are features; record i is the sum of piece i + 1
     st.clear();
@@ -668,8 +530,8 @@ __device__ __forceinline__ void dkv(const Params& p, uint8_t* smem) {
 #pragma unroll 1
     for (int n0 = last; n0 >= r.lo && n0 < r.end; n0 -= ROWS) {
         const int cn = r.end - n0;              // (of them sixteen at most)
-        in.request(at(n0 - (STAGES - 1) * ROWS));
-        in.template arrived<ELU>(0, r.end - n0);
+        in.request(at(n0 - in.AHEAD * ROWS));
+        in.arrived(0, r.end - n0, ELU ? kMinusInf : 0u);
         Rows q = in.rows(0), k = in.rows(1);
         const Rows v = in.rows(2), G = in.rows(3);
         const float* w = in.weights();
@@ -687,7 +549,7 @@ __device__ __forceinline__ void dkv(const Params& p, uint8_t* smem) {
             columns_mma<true>(s1, k, [&](int kk, int h) { return q.x[1][2 * kk + h]; });
             const uint32_t a0 = pack_rn(s0[0], s0[1]) & upper, a2 = pack_rn(s1[0], s1[1]), a3 = pack_rn(s1[2], s1[3]) & upper;
 #pragma unroll
-            for (int n = 0; n < NT; ++n) mma(gv[n], a0, 0u, a2, a3, gt.x[0][n], gt.x[1][n]);
+            for (int n = 0; n < NT; ++n) mma_add(gv[n], a0, 0u, a2, a3, gt.x[0][n], gt.x[1][n]);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 uint32_t o[NT];
@@ -708,7 +570,7 @@ __device__ __forceinline__ void dkv(const Params& p, uint8_t* smem) {
             columns_mma<false>(s1, v, [&](int kk, int h) { return G.x[1][2 * kk + h]; });
             const uint32_t a0 = pack_rn(s0[0], s0[1]) & upper, a2 = pack_rn(s1[0], s1[1]), a3 = pack_rn(s1[2], s1[3]) & upper;
 #pragma unroll
-            for (int n = 0; n < NT; ++n) mma(gk[n], a0, 0u, a2, a3, qt.x[0][n], qt.x[1][n]);
+            for (int n = 0; n < NT; ++n) mma_add(gk[n], a0, 0u, a2, a3, qt.x[0][n], qt.x[1][n]);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 uint32_t o[NT];

@@ -1,4 +1,4 @@
-// Non-causal linear attention on the tensor cores (bf16, D = M = 64), Eq. 5-6 and the
+// Non-causal linear attention on the tensor cores (bf16, D = M = 32 or 64), Eq. 5-6 and the
 // gradient of Eq. 13-15 with full (unmasked) sums.
 //
 // The per-head sums are formed once (pre-pass: every sequence is cut into splits, each
@@ -23,9 +23,12 @@
 // with ysum = sum_j V_j, gsum = sum_i G_i / dn_i, rho0 = sum_i dl_i / dn_i, qh' = q' / dn.
 // The column sums of S'' and R'' vanish, so (1 + x')^T S'' = x'^T S''.
 //
+// Two kinds of kernels: tcgen05 ones, below, and those of la_linear_warp.cuh (of_warps).
+//
 // Sum kernel: 10 warps (0-7 apply elu to the X tile in place, half a row per thread; 8 TMA; 9 MMA issue).
 // Apply kernel: 14 warps (0-7 epilogue, two per TMEM quadrant, half a chunk row each; 8-11 apply elu to the
 // X tile in place; 12 TMA; 13 MMA issue).
+#include "la_linear_warp.cuh"
 #include "la_tc.cuh"
 #include "la_tc_common.cuh"
 
@@ -38,17 +41,9 @@ LA_TRACE_DECL(g_trace_lin)
 
 namespace {
 
-// Record of one split: [A' (64x64) | a' (64) | ysum (64) | w0 (1) | pad]:
-//   forward sums (sum kernel)            : A' = sum k'_j V_j^T, a' = sum k'_j, ysum = sum V_j,        w0 unused
-//   reverse sums (backward-Q apply pass) : A' = sum qh'_i G_i^T, a' = sum qh'_i dl_i, ysum = sum G_i / dn_i, w0 = sum dl_i / dn_i
-constexpr int kRecFloats = kDim * kDim + kDim + kDim + 8;
-// The last four words of a record: the split plan it was written under.  A backward pass that is given kept records and
-// would split the sequences in another way (la_plan_override() in between) reports that and writes nothing.  The CTAs of
-// sequence i look at record i, which every plan has: all of them at the first one took 0.5 us longer a step.
-constexpr int kRecStamp = kRecFloats - 4;
-__device__ __forceinline__ int4 split_stamp(int nseg, int chunks_per_seg, int dim) {
-    return make_int4(0x4c414c53, nseg, chunks_per_seg, dim);
-}
+using lin::kRecFloats;          // both kinds of kernels write and read the same records
+using lin::kRecStamp;
+using lin::split_stamp;
 
 __device__ __forceinline__ float elu_fast(float x) {      // elu(x) = phi(x) - 1
     float e;
@@ -119,7 +114,6 @@ struct LsParams {
     int64_t N;
     int chunks, chunks_per_seg, nseg;
     int phi;
-    int dim;
 };
 
 template <bool k3d>         // N is not a multiple of the chunk: the tiles are 3-D boxes that end with their sequence
@@ -170,7 +164,7 @@ linear_sum_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     LA_TRACE_CTA(g_trace_lin, 1);
     if (tid == kLsThreads - 1)
         *reinterpret_cast<int4*>(prm.records + (bh * prm.nseg + seg) * (int64_t)kRecFloats + kRecStamp) =
-            split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
+            split_stamp(prm.nseg, prm.chunks_per_seg, kDim);
     // Ragged batch: only `real` rows of this split exist; chunks behind them are skipped and the rows behind
     // them in the last chunk are zeroed after the load (at least one chunk runs, so that the record is written
     // from an accumulator that holds zeros and not from one that was never started).
@@ -233,7 +227,7 @@ linear_sum_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         const int t = tid & 127, hf = tid >> 7;
         const uint32_t r7 = t & 7;
         const bool elu = prm.phi == LA_PHI_ELU1;
-        const int nch = prm.dim >> 3;
+        const int nch = kDim >> 3;
         #pragma unroll 1
         for (int c = 0; c < L; ++c) {
             const int s = c % kLsStages;
@@ -336,7 +330,6 @@ struct ApParams {
     int chunks, chunks_per_seg, nseg;
     float eps;
     int phi;
-    int dim;                    // D = M: 64, or 32 (tiles zero-padded to 64 columns)
     int early;                  // a kernel of the same call runs in front: the first tiles are requested before the wait
 };
 
@@ -423,7 +416,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
     }
     bool mismatch = false;      // (the same for every thread)
     if (kHasY && prm.kept) {
-        const int4 a = *reinterpret_cast<const int4*>(prm.kept + bh * (int64_t)kRecFloats + kRecStamp), b = split_stamp(prm.nseg, prm.chunks_per_seg, prm.dim);
+        const int4 a = *reinterpret_cast<const int4*>(prm.kept + bh * (int64_t)kRecFloats + kRecStamp), b = split_stamp(prm.nseg, prm.chunks_per_seg, kDim);
         mismatch = a.x != b.x || a.y != b.y || a.z != b.z || a.w != b.w;
     }
     // state of this head: add the split records (fp32), remove the column means, round the
@@ -462,7 +455,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             else sScal[1] = z;
         }
         __syncthreads();
-        const int dim = prm.dim;
+        constexpr int dim = kDim;
         // column sums in two steps (a thread alone would walk its column for a microsecond): four threads per column
         // take every fourth row, in a fixed order, and leave their partial sums behind the matrix
         float* sPartial = sF + kDim * kDim + kDim;                                // fp32 [4][64]
@@ -591,7 +584,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             if (*abort_flag) break;
             if (t == 0) LA_TRACE(g_trace_lin, c, 14);
             uint8_t* rowX = smem + kApOffStage + s * 2 * kTileBytes + t * 128;
-            if (elu) elu_row_inplace<true>(rowX, r7, 1.f, prm.dim >> 3); else elu_row_inplace<false>(rowX, r7, 1.f, prm.dim >> 3);
+            if (elu) elu_row_inplace<true>(rowX, r7, 1.f, kDim >> 3); else elu_row_inplace<false>(rowX, r7, 1.f, kDim >> 3);
             fence_proxy_async_smem();
             mbar_arrive(&bars->mapped[s]);
             if (t == 0) LA_TRACE(g_trace_lin, c, 15);
@@ -606,7 +599,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         const uint32_t r7 = t & 7;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const bool elu = prm.phi == LA_PHI_ELU1;
-        const float fD = (float)prm.dim, fN = (float)len;
+        const float fD = (float)kDim, fN = (float)len;
         // (columns beyond a 32-wide problem are zero padding: they add nothing to the sums, and the store clips them)
         float* sX = reinterpret_cast<float*>(smem + kApOffX);
         float* mine = sX + (hf * 128 + t) * 8;
@@ -822,11 +815,11 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             const int e = hf * 128 + t;
             const int64_t r_lo = row0 + (int64_t)L * kChunk;
             const int64_t nrows = max((int64_t)0, min((int64_t)(L_all - L) * kChunk, prm.N - (int64_t)(c_begin + L) * kChunk));
-            const int64_t n16 = nrows * prm.dim * 2 / 16;
-            uint4* o0 = reinterpret_cast<uint4*>(prm.out0 + r_lo * prm.dim);
+            const int64_t n16 = nrows * kDim * 2 / 16;
+            uint4* o0 = reinterpret_cast<uint4*>(prm.out0 + r_lo * kDim);
             for (int64_t i = e; i < n16; i += 256) o0[i] = make_uint4(0u, 0u, 0u, 0u);
             if (kMode == kApplyBackwardKV) {
-                uint4* o1 = reinterpret_cast<uint4*>(prm.out1 + r_lo * prm.dim);
+                uint4* o1 = reinterpret_cast<uint4*>(prm.out1 + r_lo * kDim);
                 for (int64_t i = e; i < n16; i += 256) o1[i] = make_uint4(0u, 0u, 0u, 0u);
             }
             if (kMode == kApplyForward && prm.den)
@@ -874,7 +867,6 @@ int launch_sums_as(const la_problem& p, const Segmentation& sg, const CUtensorMa
     prm.chunks_per_seg = sg.chunks_per_seg;
     prm.nseg = sg.nseg;
     prm.phi = p.phi;
-    prm.dim = (int)p.D;
     prof_begin(kProfLinearSum, st);
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = chained_launch((unsigned)(sg.nseg * p.B * p.H), kLsThreads, kLsSmemBytes, st, &attr);
@@ -904,7 +896,6 @@ int launch_apply_as(const la_problem& p, const Segmentation& sg, const CUtensorM
     prm.nseg = sg.nseg;
     prm.eps = p.eps;
     prm.phi = p.phi;
-    prm.dim = (int)p.D;
     const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
     CUtensorMap mO0, mO1;                   // one warp's 32 rows per store
     if (int rc = encode_attention_map(&mO0, prm.out0, p.N % kChunk != 0, seqs, n, 32, (int)p.D)) return rc;
@@ -925,6 +916,105 @@ int launch_apply(const la_problem& p, const Segmentation& sg, const CUtensorMap&
                         : launch_apply_as<kMode, false>(p, sg, mX, mY, prm, st);
 }
 
+// ---- a warp per sixteen positions (la_linear_warp.cuh) ----------------------------------------------------------------
+struct StreamWait {
+    __device__ __forceinline__ void operator()() const {
+        grid_dependency_wait();
+        allow_dependent_launch();
+    }
+};
+template <int W, bool ELU>
+__global__ void __launch_bounds__(lin::THREADS, 1) linear_warp_sum_kernel(const lin::Params p) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    lin::sums<W, ELU>(p, smem, StreamWait());
+}
+template <int W, int MODE, bool ELU>
+__global__ void __launch_bounds__(lin::THREADS, 1) linear_warp_apply_kernel(const lin::Params p) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    lin::apply<W, MODE, ELU>(p, smem, StreamWait());
+}
+
+// Which problems: all with D = M = 32 (tcgen05 tiles of 64 columns are half empty), and of D = M = 64 those whose CTAs have little to do but
+// start: both forms and the passes alike.  Forward + backward with kept sums (forward alone), us, tcgen05 / a warp per sixteen
+// positions, B x H x N: D = 32 4x8x8192 117 / 64 (40 / 21), 64x8x512 176 / 100 (66 / 32), 8x8x1024 49 / 26 (18 / 9), 1x8x8000 64 / 41;
+// D = 64 1x8x2000 42 / 32 (16 / 12), 4x8x2000 53 / 47 (20 / 16), 8x8x1024 52 / 46 (19 / 16), 64x8x512 199 / 185 (73 / 64), 128x8x256
+// 262 / 222, 64x8x100 114 / 84, but 16x8x1024 75 / 77, 16x8x2048 128 / 137, 8x8x4096 129 / 138 (45 / 47).
+bool of_warps(const la_problem& p) { return p.D == 32 || p.N <= 512 || p.B * p.H * p.N <= 65536; }
+
+template <auto KERNEL>
+int launch_as(ProfKernel prof, const la_problem& p, int smem, const lin::Params& a, cudaStream_t st) {
+    static std::atomic<uint64_t> attr_done{0};          // one per instantiation
+    if (int rc = opt_in_smem_once(KERNEL, (uint32_t)smem, attr_done)) return rc;
+    prof_begin(prof, st);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = chained_launch((unsigned)(a.nseg * p.B * p.H), lin::THREADS, (uint32_t)smem, st, &attr);
+    LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, KERNEL, a));
+    note_launch();
+    prof_end(prof, st);
+    return LA_OK;
+}
+template <int W> int launch_warp_sums(const la_problem& p, const lin::Params& a, cudaStream_t st) {
+    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_sum_kernel<W, true>>(kProfLinearSum, p, lin::kSumSmem<W>, a, st);
+    return launch_as<linear_warp_sum_kernel<W, false>>(kProfLinearSum, p, lin::kSumSmem<W>, a, st);
+}
+template <int W, int MODE> int launch_warp_apply(const la_problem& p, const lin::Params& a, cudaStream_t st) {
+    constexpr int smem = lin::ApplyLayout<W, MODE>::BYTES;
+    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_apply_kernel<W, MODE, true>>(kProfLinearApply, p, smem, a, st);
+    return launch_as<linear_warp_apply_kernel<W, MODE, false>>(kProfLinearApply, p, smem, a, st);
+}
+
+int make_params(const la_problem& p, const int* lengths, lin::Params* a) {
+    const Segmentation sg = choose_splits(p);
+    *a = {};
+    a->lengths = lengths;
+    a->status = device_status_ptr();
+    if (!a->status) return fail(LA_ERR_CUDA, "device status word unavailable");
+    a->N = p.N;
+    a->heads = (int)p.H;
+    a->nseg = sg.nseg;
+    a->chunks_per_seg = sg.chunks_per_seg;
+    a->eps = p.eps;
+    return LA_OK;
+}
+
+template <int W> int warp_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O, float* den,
+                                  float* KV, float* Zs, float* rec, cudaStream_t st) {
+    lin::Params a;
+    if (int rc = make_params(p, lengths, &a)) return rc;
+    a.X = K; a.Y = V;
+    a.records = rec;
+    if (int rc = launch_warp_sums<W>(p, a, st)) return rc;
+    if (!O) return LA_OK;       // the sums are wanted alone
+    a.X = Q;
+    a.out0 = O;
+    a.den = den;
+    a.state_out = KV;
+    a.vec_out = Zs;
+    a.early = 1;                // behind the sum kernel
+    return launch_warp_apply<W, lin::kApplyForward>(p, a, st);
+}
+
+template <int W> int warp_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* saved,
+                                   const void* G, void* dQ, void* dK, void* dV, float* rec_s, float* rec_r, cudaStream_t st) {
+    lin::Params a;
+    if (int rc = make_params(p, lengths, &a)) return rc;
+    a.records = rec_s;
+    a.X = K; a.Y = V;
+    if (!saved)                 // (with a saved buffer rec_s are the forward's own records)
+        if (int rc = launch_warp_sums<W>(p, a, st)) return rc;
+    a.kept = (const float*)saved;
+    a.early = saved ? 0 : 1;    // the first kernel of the call with saved records, else behind the sum kernel
+    a.X = Q; a.Y = G;
+    a.out0 = dQ;
+    a.rec_out = rec_r;          // the reverse sums of Q / dn and G are formed by the same pass
+    if (int rc = launch_warp_apply<W, lin::kApplyBackwardQ>(p, a, st)) return rc;
+    a.records = rec_r;
+    a.X = K; a.Y = V;
+    a.out0 = dK; a.out1 = dV;
+    a.early = 1;                // behind the dQ pass
+    return launch_warp_apply<W, lin::kApplyBackwardKV>(p, a, st);
+}
+
 }  // namespace
 
 size_t linear_forward_workspace(const la_problem& p) {
@@ -936,6 +1026,7 @@ size_t linear_backward_workspace(const la_problem& p) {
 }
 
 int linear_keep_sums(const la_problem& p, const void* K, const void* V, const int* lengths, void* saved, cudaStream_t st) {
+    if (of_warps(p)) return (p.D == 32 ? warp_forward<32> : warp_forward<64>)(p, nullptr, K, V, lengths, nullptr, nullptr, nullptr, nullptr, (float*)saved, st);
     const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
     CUtensorMap mK, mV;
     if (int rc = encode_attention_map(&mK, K, p.N % kChunk != 0, seqs, n, kChunk, (int)p.D)) return rc;
@@ -945,6 +1036,7 @@ int linear_keep_sums(const la_problem& p, const void* K, const void* V, const in
 
 int linear_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, void* O,
                    float* den, float* KV, float* Zs, void* saved, void* ws, cudaStream_t st) {
+    if (of_warps(p)) return (p.D == 32 ? warp_forward<32> : warp_forward<64>)(p, Q, K, V, lengths, O, den, KV, Zs, saved ? (float*)saved : (float*)ws, st);
     const Segmentation sg = choose_splits(p);
     const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
     CUtensorMap mQ, mK, mV;
@@ -966,6 +1058,9 @@ int linear_forward(const la_problem& p, const void* Q, const void* K, const void
 
 int linear_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths,
                     const void* saved, const void* G, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st) {
+    if (of_warps(p))
+        return (p.D == 32 ? warp_backward<32> : warp_backward<64>)(p, Q, K, V, lengths, saved, G, dQ, dK, dV, saved ? const_cast<float*>((const float*)saved) : (float*)ws,
+                                 (float*)((uint8_t*)ws + linear_forward_workspace(p)), st);
     const Segmentation sg = choose_splits(p);
     const size_t bh = (size_t)(p.B * p.H);
     const uint64_t n = (uint64_t)p.N;

@@ -1,5 +1,6 @@
-"""bf16, D = M = 32: a warp per piece of a sequence, at the edges of its chunks of sixteen positions, whole and in pieces, ragged, from
-a state, with and without a saved buffer, against the fp64 oracle under the bf16 gates."""
+"""bf16 kernels whose warps take sixteen positions at a time, at the edges of their chunks, against the fp64 oracle under the bf16 gates:
+causal, D = M = 32, a warp per piece of a sequence (whole and in pieces, ragged, from a state, with and without a saved buffer), and
+non-causal, D = M = 32 and 64 (whole and split, ragged, with and without kept sums)."""
 import os
 import re
 
@@ -66,6 +67,47 @@ def test_pieces_lengths_and_states(B, H, N, pieces):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("splits", [-1, 1, 3])
+@pytest.mark.parametrize("W", [32, 64])
+@pytest.mark.parametrize("N", [1, 15, 17, 256, 257, 500, 900])
+def test_noncausal_chunks_and_splits(N, W, splits):
+    B, H = 5, 8
+    Q, K, V, G = draw_qkvg(B, H, N, W, W, 11 + N, BF, 0.5)
+    lengths = [N, 0, (N + 1) // 2, max(N - 1, 1), min(N, 16)]
+    la.la_plan_override(-1, -1, splits)
+    for phi in ("elu1", "identity"):
+        if phi == "identity":
+            Q, K = (Q.float().abs() + 0.1).to(BF), (K.float().abs() + 0.1).to(BF)
+        dev = [t.to(DEV) for t in (Q, K, V, G)]
+        for ln in (None, torch.tensor(lengths, dtype=torch.int32, device=DEV)):
+            saved = la.linear_saved_buffer(dev[0], dev[2], phi=phi)
+            den, KV, Zs = torch.empty(B, H, N, device=DEV), torch.empty(B, H, W, W, device=DEV), torch.empty(B, H, W, device=DEV)
+            # (a clustered forward pass is another kernel's matter: with forced splits it is this one)
+            O = la.la_linear_attention(*dev[:3], phi=phi, lengths=ln, saved=saved, den=den, KV=KV, Zs=Zs)
+            grads = la.la_linear_attention_backward(*dev, phi=phi, lengths=ln, saved=saved)
+            again = la.la_linear_attention_backward(*dev, phi=phi, lengths=ln)
+            la.la_last_device_status()
+            assert all(torch.equal(a, b) for a, b in zip(grads, again))
+            for b in range(B):
+                n, h = N if ln is None else lengths[b], b
+                assert not O[b, :, n:].any() and not den[b, :, n:].any() and not any(x[b, :, n:].any() for x in grads)
+                if n == 0:
+                    assert not KV[b].any() and not Zs[b].any()
+                    continue
+                sl = (slice(b, b + 1), slice(h, h + 1), slice(0, n))
+                q, k, v, u = (t[sl].double().numpy() for t in (Q, K, V, G))
+                Or, denr = oracle.linear_attention(q, k, v, causal=False, phi=phi)[:2]
+                fk = oracle.feature_map(k) if phi == "elu1" else k
+                for nm, x, ref in (("O", O[sl], Or), ("den", den[sl], denr), ("KV", KV[b, h], np.einsum("nd,nm->dm", fk[0, 0], v[0, 0])),
+                                   ("Zs", Zs[b, h][None], fk[0, 0].sum(0)[None])):
+                    assert_close(x, ref, BF, nm)
+                if n == 1:
+                    continue                            # dQ and dK are analytically zero
+                for nm, x, ref in zip(("dQ", "dK", "dV"), grads, oracle.linear_attention_backward(q, k, v, u, causal=False, phi=phi)):
+                    assert_close(x[sl], ref, BF, nm, grad=True)
+
+
+@pytest.mark.gpu
 def test_kept_sums_of_another_plan_are_refused():
     if os.environ.get("LA_DEBUG"):
         pytest.skip("in checked mode the call itself reads the status and raises; this test reads it afterwards")
@@ -110,6 +152,6 @@ def test_workspace_and_saved_sizes():
 
 def test_no_read_only_loads():
     """As the other kernels that may start as programmatic dependents."""
-    path = os.path.join(os.path.dirname(la.__file__), "csrc", "la_causal_warp.cuh")
-    code = re.sub(r"//[^\n]*", "", open(path).read())
-    assert not re.findall(r"__ldg\s*\(|ld\.global\.nc|const \w+\s*\*\s*__restrict__", code)
+    for name in ("la_warp.cuh", "la_causal_warp.cuh", "la_linear_warp.cuh"):
+        code = re.sub(r"//[^\n]*", "", open(os.path.join(os.path.dirname(la.__file__), "csrc", name)).read())
+        assert not re.findall(r"__ldg\s*\(|ld\.global\.nc|const \w+\s*\*\s*__restrict__", code)
