@@ -36,7 +36,11 @@ using namespace sweep;
 
 template <typename C, int DP, int MP> using ForwardLayout = Layout<C::WPS, DP, MP, C::NQ, C::NV, C::NQ, DP, C::NS, MP>;
 template <typename C, int DP, int MP> using DqLayout = Layout<C::WPS, DP, MP, C::NQ, C::NV, C::NV, MP, C::NS, DP>;
-template <typename C, int DP, int MP> using DkvLayout = Layout<C::WPS, DP, MP, C::NR, C::NV, 0, 0, C::NS, 0>;
+// (kScaled: after the vectors G / dn in three planes, and 1 / dn)
+template <typename C, int DP, int MP> struct DkvLayout : Layout<C::WPS, DP, MP, kScaled<C> ? 1 : C::NR, C::NV, 0, 0, C::NS, 0> {
+    using Base = Layout<C::WPS, DP, MP, kScaled<C> ? 1 : C::NR, C::NV, 0, 0, C::NS, 0>;
+    static constexpr int GH = Base::BYTES, INV = GH + 3 * T * MP * 2, BYTES = kScaled<C> ? INV + T * 4 : Base::BYTES;
+};
 
 // named barriers: 1 = the state planes are no longer read; 2 + strip, 6 + strip = hand-overs within a pair of warps
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
@@ -117,7 +121,7 @@ causal_mma_forward_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece);
+            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * p.parts);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
         float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
@@ -274,7 +278,7 @@ causal_mma_dq_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece);
+            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * p.parts);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
         float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
@@ -488,7 +492,9 @@ __global__ void __launch_bounds__(kThreads<C>, (C::ALONE ? 1 : resident<DkvLayou
 causal_mma_dkv_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = DkvLayout<C, DP, MP>;
-    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, NR = C::NR, WPS = C::WPS, THREADS = kThreads<C>;
+    constexpr int NQ = C::NQ, NV = C::NV, NP = C::NP, NS = C::NS, WPS = C::WPS, THREADS = kThreads<C>;
+    constexpr bool SCALED = kScaled<C>;
+    constexpr int NX = SCALED ? 1 : C::NR;          // planes of the queries' tile
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const bool v_part = WPS == 1 || warp < STRIPS_T, k_part = WPS == 1 || warp >= STRIPS_T;
@@ -508,7 +514,7 @@ causal_mma_dkv_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;           // record i is the sum of piece i + 1
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + (r.bh * p.records + r.piece) * (int64_t)(D * M + D), p.pieces - 1 - r.piece);
+            p.rec + (r.bh * p.records + r.piece * p.parts) * (int64_t)(D * M + D), (p.pieces - 1 - r.piece) * p.parts);
     const int64_t chunks = (r.end - r.lo + T - 1) / T;
     for (int64_t c = chunks - 1; c >= 0; --c) {
         const uint32_t sQ = smem_u32(smem + Sh::X), sG = smem_u32(smem + Sh::Y), sR = smem_u32(smem + Sh::S);
@@ -519,11 +525,12 @@ causal_mma_dkv_kernel(const Params p) {
         const int cn = (int)(r.end - n0 < T ? r.end - n0 : T), blocks = (cn + 15) / 16;
         const int strip = strip_of(warp, c & 1), row0 = strip * 16;
         {
-            ReverseRows<IO, DP, MP, THREADS> rr;
+            std::conditional_t<SCALED, ScaledRows<IO, DP, MP, THREADS>, ReverseRows<IO, DP, MP, THREADS>> rr;
             rr.load(Q, G, dn, delta, n0, cn, D, M, pad);
             __syncthreads();
             st.template publish<NS>(smem + Sh::S, sr, reinterpret_cast<uint16_t*>(smem + Sh::ZP));
-            rr.template store<NR, NV>(smem + Sh::X, smem + Sh::Y, sdl, wpl, phi);
+            if constexpr (SCALED) rr.store(smem + Sh::X, smem + Sh::Y, smem + Sh::GH, sdl, reinterpret_cast<float*>(smem + Sh::INV), wpl);
+            else rr.template store<C::NR, NV>(smem + Sh::X, smem + Sh::Y, sdl, wpl, phi);
         }
         if (c > 0) {
             prefetch_rows<C>(Q, n0 - T, r.end, D);
@@ -532,6 +539,15 @@ causal_mma_dkv_kernel(const Params p) {
             prefetch_rows<C>(G, n0 - T, r.end, M);
         }
         __syncthreads();
+        auto scale_columns = [&](int ib, float (&s0)[4], float (&s1)[4]) {       // the scores of queries 16 ib .. by their 1 / dn
+            const float* v = reinterpret_cast<const float*>(smem + Sh::INV) + ib * 16 + 2 * t;
+            const float2 i0 = load_pair(v), i1 = load_pair(v + 8);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                s0[2 * h] *= i0.x; s0[2 * h + 1] *= i0.y;
+                s1[2 * h] *= i1.x; s1[2 * h + 1] *= i1.y;
+            }
+        };
         if (v_part && row0 < cn) {
             uint32_t ka[DP / 16][NQ][4];
             {
@@ -560,12 +576,13 @@ causal_mma_dkv_kernel(const Params p) {
                     Chain c;
 #pragma unroll
                     for (int kk = 0; kk < DP / 16; ++kk) {
-                        uint32_t b[NR][4];
-                        load_rows<NR, DP>(b, sQ, T * DP * 2, ib * 16, kk * 2, lane);
-                        c.step<NQ, NR>(ka[kk], b);
+                        uint32_t b[NX][4];
+                        load_rows<NX, DP>(b, sQ, T * DP * 2, ib * 16, kk * 2, lane);
+                        c.step<NQ, NX>(ka[kk], b);
                     }
                     c.put(s0, s1);
                 }
+                if constexpr (SCALED) scale_columns(ib, s0, s1);
                 if (ib == strip) mask_diagonal<true>(s0, s1, g, t);
                 uint32_t pa[NP][4];
                 operand_of<NP>(pa, s0, s1);
@@ -626,14 +643,15 @@ causal_mma_dkv_kernel(const Params p) {
                     }
                     c.add_to(s0, s1);
                 }
+                if constexpr (SCALED) scale_columns(ib, s0, s1);
                 if (ib == strip) mask_diagonal<true>(s0, s1, g, t);
                 uint32_t pa[NP][4];
                 operand_of<NP>(pa, s0, s1);
 #pragma unroll
                 for (int n = 0; n < DP / 16; ++n) {
-                    uint32_t b[NR][4];
-                    load_cols_t<NR, DP>(b, sQ, T * DP * 2, ib * 16, n * 2, lane);
-                    block_mma<NP, NR>(gk[2 * n], gk[2 * n + 1], pa, b);
+                    uint32_t b[NX][4];
+                    load_cols_t<NX, DP>(b, sQ, T * DP * 2, ib * 16, n * 2, lane);
+                    block_mma<NP, NX>(gk[2 * n], gk[2 * n + 1], pa, b);
                 }
             }
             RawStrip<IO, DP> rk;
@@ -654,7 +672,8 @@ causal_mma_dkv_kernel(const Params p) {
                 }
             }
         }
-        st.template update<NR, NV, false>(sQ, sG, wpl);
+        if constexpr (SCALED) st.template update<1, 3, false>(sQ, smem_u32(smem + Sh::GH), wpl);
+        else st.template update<C::NR, NV, false>(sQ, sG, wpl);
     }
     zero_rows<THREADS>(dK, r.end, r.hi, D);
     zero_rows<THREADS>(dV, r.end, r.hi, M);
@@ -768,8 +787,16 @@ Plan choose_plan(const la_problem& p, bool single) {
     return Plan{(int)((p.N + len - 1) / len), len};
 }
 
+// Records of a piece: with bf16 features the sums of few pieces are shared out over the SMs that would have none (Fourier B8 H8 N1000, two
+// pieces of eight chunks, three passes over the sums: 14, 14 and 27 us with 64 CTAs that load a chunk when they need it, 10, 10 and 15
+// with 128 that load it ahead; fp32 D = 48 B3 H4 N1500 99.5 / 100.5 a step, D = 80 B1 H8 N2000 202 / 207).
+int record_parts(const la_problem& p, const Plan& pl) {
+    if (of_warps(p) || p.dtype != LA_BF16 || pl.pieces < 2) return 1;
+    const int64_t idle = 148 / (p.B * p.H * (pl.pieces - 1)), chunks = pl.len / T, most = chunks < 4 ? chunks : 4;
+    return (int)(idle < 1 ? 1 : idle < most ? idle : most);
+}
 size_t record_bytes(const la_problem& p, const Plan& pl) {
-    return (size_t)(p.B * p.H) * (size_t)(pl.pieces - 1) * (size_t)(p.D * p.M + p.D) * sizeof(float);
+    return (size_t)(p.B * p.H) * (size_t)(pl.pieces - 1) * (size_t)record_parts(p, pl) * (size_t)(p.D * p.M + p.D) * sizeof(float);
 }
 size_t aux_bytes(const la_problem& p) { return ((size_t)(p.B * p.H) * (size_t)p.N * 2 * sizeof(float) + 15) & ~(size_t)15; }
 
@@ -781,7 +808,8 @@ Params make_params(const la_problem& p, const Plan& pl, const int* lengths) {
     // us a step); otherwise CTAs that wait on the SMs with room leave the kernel unevenly spread (B32 H8 N4096 D64
     // backward 2007 -> 2862 us, released at the kernel's end B37 H8 N512 267 -> 328 us).
     a.chained = 2 * p.B * p.H * pl.pieces <= 148;
-    a.records = pl.pieces - 1;
+    a.parts = record_parts(p, pl);
+    a.records = (pl.pieces - 1) * a.parts;
     a.heads = (int)p.H; a.D = (int)p.D; a.M = (int)p.M; a.phi = p.phi; a.eps = p.eps;
     return a;
 }
@@ -790,7 +818,7 @@ template <typename C, int DP, int MP, bool EXACT> struct Kernels {
     static constexpr int THREADS = kThreads<C>;
     static int sums(const la_problem& p, const Params& a, bool reverse, cudaStream_t st) {
         if (a.pieces == 1) return LA_OK;
-        const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)(a.pieces - 1);
+        const unsigned bh = (unsigned)(p.B * p.H), y = (unsigned)a.records;
         if (reverse)
             return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, true>>(kProfMmaSum, THREADS, bh, y, SumLayout<C, DP, MP, true>::BYTES, a, st);
         return launch<causal_mma_sum_kernel<C, DP, MP, EXACT, false>>(kProfMmaSum, THREADS, bh, y, SumLayout<C, DP, MP, false>::BYTES, a, st);

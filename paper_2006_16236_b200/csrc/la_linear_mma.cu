@@ -340,7 +340,7 @@ Params make_params(const la_problem& p, const int* lengths) {
     const Plan pl = choose_plan(p);
     Params a = {};
     a.lengths = lengths;
-    a.N = p.N; a.piece_len = pl.len; a.pieces = pl.splits; a.records = pl.splits;
+    a.N = p.N; a.piece_len = pl.len; a.pieces = pl.splits; a.records = pl.splits; a.parts = 1;
     a.chained = 2 * p.B * p.H * pl.splits <= 148;       // (small grids only, as in la_causal_mma.cu)
     a.heads = (int)p.H; a.D = (int)p.D; a.M = (int)p.M; a.phi = p.phi; a.eps = p.eps;
     return a;

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 #include "la_mma.cuh"
 #include "la_tc.cuh"
@@ -25,6 +26,7 @@ struct Params {
     float* rec;                  // [bh][records][D * M + D]: sums of the pieces first_record .. first_record + records - 1
     float* rec_out;              // where the dQ sweep leaves the reverse records, or null
     int records, first_record;
+    int parts;                   // records of a piece (causal sums): its sums in that many ranges
     float* aux;                  // [bh][2][N]: dn_i, -G_i . O_i
     const int* lengths;
     int64_t N, piece_len;
@@ -267,8 +269,12 @@ template <int WPS, int DP, int MP, int NX, int NY, int NRW, int RC, int NS, int 
                          Z = S + (PLANES > PART ? PLANES : PART), ZP = Z + DP * 4, W = ZP + 3 * DP * 2, WP = W + T * 4,
                          BYTES = (WP + 3 * T * 2 + 127) / 128 * 128;
 };
+// Where q and G are bf16 and q / dn and G / dn need three planes, the division goes to G, of which there are fewer columns, and in the
+// reverse scores to their columns: (k q^T) / dn, ((G V^T + dl) / dn) q instead of k (q / dn)^T, (G V^T + dl) (q / dn).  Per sixteen
+// keys and queries that is 96 products where it was 176.  Fourier B8 H8 N1000 C128 dK and dV 84 -> 77 us.
+template <typename C> constexpr bool kScaled = C::NQ == 1 && C::NV == 1 && C::NR == 3;
 template <typename C, int DP, int MP, bool REVERSE>
-using SumLayout = Layout<1, DP, MP, REVERSE ? C::NR : C::NQ, C::NV, 0, 0, 0, 0>;
+using SumLayout = Layout<1, DP, MP, REVERSE && !kScaled<C> ? C::NR : C::NQ, REVERSE && kScaled<C> ? C::NR : C::NV, 0, 0, 0, 0>;
 
 template <typename C> constexpr int kThreads = 128 * C::WPS;
 // CTAs of an SM that the registers are shared out for: as many as shared memory holds, at most two (or `most`)
@@ -333,47 +339,110 @@ struct ReverseRows {
     }
 };
 
+// The same for kScaled: q and (tg, if given) G as they are, G / dn in three planes, the planes of dl / dn; dl and 1 / dn in fp32.
+template <typename IO, int DP, int MP, int THREADS>
+struct ScaledRows {
+    RawTile<IO, T, DP, THREADS> rq;
+    RawTile<IO, T, MP, THREADS> rg;
+    float inv[RawTile<IO, T, MP, THREADS>::GROUPS];
+    float dl, dn;
+    __device__ __forceinline__ void load(const IO* Q, const IO* G, const float* dns, const float* delta, int64_t n0, int cn, int D, int M, float) {
+        rq.load(Q + n0 * D, cn, D, 0.f);
+        rg.load(G + n0 * M, cn, M, 0.f);
+#pragma unroll
+        for (int u = 0; u < RawTile<IO, T, MP, THREADS>::GROUPS; ++u) {
+            const int row = ((int)threadIdx.x + u * THREADS) / (MP / 8);
+            inv[u] = row < cn ? dns[n0 + row] : 1.f;
+        }
+        dl = (int)threadIdx.x < cn ? delta[n0 + threadIdx.x] : 0.f;
+        dn = (int)threadIdx.x < cn ? dns[n0 + threadIdx.x] : 1.f;
+    }
+    __device__ __forceinline__ void store(uint8_t* tq, uint8_t* tg, uint8_t* th, float* w, float* winv, uint16_t* wpl) {
+#pragma unroll
+        for (int u = 0; u < RawTile<IO, T, MP, THREADS>::GROUPS; ++u) inv[u] = 1.f / inv[u];
+        rq.copy(tq);
+        if (tg) rg.copy(tg);
+        rg.template store<3>(th, [&](int u, float x) { return x * inv[u]; });
+        if (threadIdx.x < T) {
+            const float i = 1.f / dn;
+            w[threadIdx.x] = dl;
+            if (winv) winv[threadIdx.x] = i;
+            uint32_t o[3];
+            split2<3>(dl * i, 0.f, o);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) wpl[k * T + threadIdx.x] = (uint16_t)o[k];
+        }
+    }
+};
+
 template <typename C, int DP, int MP, bool EXACT, bool REVERSE>
 __global__ void __launch_bounds__(kThreads<C>, 2)
 causal_mma_sum_kernel(const Params p) {
     using IO = typename C::IO;
     using Sh = SumLayout<C, DP, MP, REVERSE>;
-    constexpr int NX = REVERSE ? C::NR : C::NQ, NY = C::NV, THREADS = kThreads<C>;
+    constexpr bool SCALED = REVERSE && kScaled<C>;
+    constexpr int NX = REVERSE && !SCALED ? C::NR : C::NQ, NY = SCALED ? C::NR : C::NV, THREADS = kThreads<C>;
     extern __shared__ __align__(128) uint8_t smem[];
     const int D = EXACT ? DP : p.D, M = EXACT ? MP : p.M, phi = C::MAPPED ? p.phi : (int)LA_PHI_IDENTITY;
     const float pad = pad_value(phi);
     wait_for_stream();
     release_next();
-    const Range r = range_of(p, (int)blockIdx.y + p.first_record);
+    Range r = range_of(p, (int)blockIdx.y / p.parts + p.first_record);
+    if (p.parts > 1) {          // the CTA's part of the piece
+        const int64_t chunks = (r.hi - r.lo + T - 1) / T, each = (chunks + p.parts - 1) / p.parts * T, lo = r.lo + (int)blockIdx.y % p.parts * each;
+        r.lo = lo < r.hi ? lo : r.hi;
+        if (r.lo + each < r.hi) r.hi = r.lo + each;
+        r.end = r.end < r.lo ? r.lo : r.end < r.hi ? r.end : r.hi;
+    }
     const IO* X = (const IO*)(REVERSE ? p.Q : p.K) + r.bh * p.N * D;
     const IO* Y = (const IO*)(REVERSE ? p.G : p.V) + r.bh * p.N * M;
     const float* dn = REVERSE ? p.aux + r.bh * 2 * p.N : nullptr;
     const float* delta = REVERSE ? dn + p.N : nullptr;
+    float* w = reinterpret_cast<float*>(smem + Sh::W);
+    uint16_t* wpl = reinterpret_cast<uint16_t*>(smem + Sh::WP);
     if (!REVERSE && p.stamp && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *reinterpret_cast<int4*>(p.stamp) = plan_stamp(p);
+    struct ForwardRows {
+        RawTile<IO, T, DP, THREADS> rx;
+        RawTile<IO, T, MP, THREADS> ry;
+    };
+    // bf16 rows of a chunk are requested before the products of the one before (fp32 ones have no registers for that)
+    constexpr bool AHEAD = sizeof(IO) == 2 && C::WPS == 2;
+    std::conditional_t<SCALED, ScaledRows<IO, DP, MP, THREADS>, std::conditional_t<REVERSE, ReverseRows<IO, DP, MP, THREADS>, ForwardRows>> rows;
+    auto load = [&](int64_t n0) {
+        const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
+        if constexpr (REVERSE) {
+            rows.load(X, Y, dn, delta, n0, cn, D, M, pad);
+        } else {
+            rows.rx.load(X + n0 * D, cn, D, pad);
+            rows.ry.load(Y + n0 * M, cn, M, 0.f);
+        }
+    };
+    if (AHEAD && r.lo < r.end) load(r.lo);
     State<DP, MP, 4 * C::WPS> st;
     st.init(p, nullptr, nullptr, nullptr, 0);
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
-        float* w = reinterpret_cast<float*>(smem + Sh::W);
-        uint16_t* wpl = reinterpret_cast<uint16_t*>(smem + Sh::WP);
-        const int cn = (int)(r.end - n0 < T ? r.end - n0 : T);
-        if constexpr (REVERSE) {
-            ReverseRows<IO, DP, MP, THREADS> rr;
-            rr.load(X, Y, dn, delta, n0, cn, D, M, pad);
-            __syncthreads();
-            rr.template store<NX, NY>(smem + Sh::X, smem + Sh::Y, w, wpl, phi);
-        } else {
-            RawTile<IO, T, DP, THREADS> rx;
-            RawTile<IO, T, MP, THREADS> ry;
-            rx.load(X + n0 * D, cn, D, pad);
-            ry.load(Y + n0 * M, cn, M, 0.f);
-            __syncthreads();
-            rx.template features<NX>(smem + Sh::X, phi);
-            ry.template values<NY>(smem + Sh::Y);
+        if constexpr (!AHEAD) {
+            load(n0);
+            __syncthreads();        // the planes of the chunk before are no longer read
         }
-        prefetch_rows<C>(X, n0 + T, r.end, D);
-        prefetch_rows<C>(Y, n0 + T, r.end, M);
+        if constexpr (SCALED) rows.store(smem + Sh::X, nullptr, smem + Sh::Y, w, nullptr, wpl);
+        else if constexpr (REVERSE) rows.template store<NX, NY>(smem + Sh::X, smem + Sh::Y, w, wpl, phi);
+        else {
+            rows.rx.template features<NX>(smem + Sh::X, phi);
+            rows.ry.template values<NY>(smem + Sh::Y);
+        }
+        if constexpr (!AHEAD) {
+            prefetch_rows<C>(X, n0 + T, r.end, D);
+            prefetch_rows<C>(Y, n0 + T, r.end, M);
+        }
         __syncthreads();
+        if constexpr (AHEAD) {
+            if (n0 + T < r.end) load(n0 + T);
+            prefetch_rows<C>(X, n0 + 2 * T, r.end, D);
+            prefetch_rows<C>(Y, n0 + 2 * T, r.end, M);
+        }
         st.template update<NX, NY, !REVERSE>(smem_u32(smem + Sh::X), smem_u32(smem + Sh::Y), wpl);
+        if constexpr (AHEAD) __syncthreads();
     }
     float* dst = p.rec + (r.bh * p.records + blockIdx.y) * (int64_t)(D * M + D);
     st.write(p, dst, dst + D * M);
