@@ -1,5 +1,5 @@
 // Non-causal form (Eq. 5-6 and its gradient) of bf16 problems with D = M = 32 or 64 on mma.sync: the kernels of la_tc_linear.cu, where
-// the formulas and the centred operands are.  A CTA of sixteen warps per split of a sequence; a warp takes sixteen positions at a time
+// the formulas and the centred operands are.  A CTA of sixteen warps per split of a sequence (or eight, two on an SM, where nothing is summed); a warp takes sixteen positions at a time
 // past the sums of the whole sequence, with its next positions on their way (la_warp.cuh).  Where sums over the positions are formed,
 // every warp has sixteen rows and sixteen columns of them (W = 64) and adds up over the chunks of all warps, which lie in shared memory
 // as they came or were mapped: a barrier per 256 positions.  (All of the sums in the registers of every warp, transposes by movmatrix and
@@ -44,7 +44,8 @@ struct Params {
     const int* lengths;         // [B] real positions per batch element (right-padded ragged batch), or null
     int* status;
     int64_t N;
-    int heads, nseg, chunks_per_seg;            // nseg CTAs per sequence
+    int heads, nseg, chunks_per_seg;            // records of a sequence, written by a CTA each
+    int parts;                  // CTAs of a sequence
     float eps;
     int early;                  // a kernel of the same call runs in front: the first positions are requested before the wait
 };
@@ -54,7 +55,7 @@ struct Params {
 struct Span { int64_t bh; int lo, end, zero_lo, zero_hi, len; };
 __device__ __forceinline__ Span span_of(const Params& p) {
     Span s;
-    const int parts = p.nseg, part = (int)(blockIdx.x % parts);
+    const int parts = p.parts, part = (int)(blockIdx.x % parts);
     s.bh = blockIdx.x / parts;
     s.len = (int)(p.lengths ? min((int64_t)max(p.lengths[s.bh / p.heads], 0), p.N) : p.N);
     const int chunks = (s.len + ROWS - 1) / ROWS, each = (chunks + parts - 1) / parts;
@@ -111,7 +112,7 @@ template <int W> __device__ __forceinline__ void put_row(void* tensor, int64_t r
 #pragma unroll
     for (int q = 0; q < W / 32; ++q) *reinterpret_cast<uint4*>(at + q * 64) = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
 }
-template <int W> __device__ __forceinline__ void zero_rows(void* tensor, int64_t from, int64_t to) {
+template <int W, int THREADS> __device__ __forceinline__ void zero_rows(void* tensor, int64_t from, int64_t to) {
     uint4* x = reinterpret_cast<uint4*>((uint8_t*)tensor + from * (W * 2));
     for (int64_t i = threadIdx.x; i < (to - from) * (W / 8); i += THREADS) x[i] = make_uint4(0u, 0u, 0u, 0u);
 }
@@ -247,7 +248,7 @@ enum ApplyMode { kApplyForward = 0, kApplyBackwardQ = 1, kApplyBackwardKV = 2 };
 
 // Shared memory: the centred matrix S'' as B operands in the order of the lanes ([kk][n / 2][lane], sixteen bytes), as it lies (rows
 // summed over) and / or transposed; the vectors a' and nu; scratch for their making, later the chunks on their way
-template <int W, int MODE> struct ApplyLayout {
+template <int W, int MODE, int WARPS> struct ApplyLayout {
     static constexpr int TENSORS = MODE == kApplyForward ? 1 : 2;
     using Chunks = Ring<W, TENSORS, false, MODE == kApplyForward ? 3 : 2>;          // (three of two tensors do not fit)
     static constexpr int OPERAND = W * W * 2;
@@ -277,10 +278,11 @@ template <int W> __device__ __forceinline__ void product(float (&c)[W / 8][4], c
         }
 }
 
-template <int W, int MODE, bool ELU, typename Wait>
+template <int W, int MODE, int WARPS, bool ELU, typename Wait>
 __device__ __forceinline__ void apply(const Params& p, uint8_t* smem, Wait wait) {
-    using L = ApplyLayout<W, MODE>;
-    constexpr int NT = W / 8;
+    using L = ApplyLayout<W, MODE, WARPS>;
+    constexpr int NT = W / 8, THREADS = 32 * WARPS, CHUNK = WARPS * ROWS;
+    static_assert(MODE != kApplyBackwardQ || WARPS == lin::WARPS, "the sums are shared out over that many");
     constexpr bool kHasY = MODE != kApplyForward;
     float* sA = reinterpret_cast<float*>(smem + L::VEC);         // a': Z' (forward, backward Q) or r' (backward K/V)
     float* sNu = sA + kDim;                                      // rank-one part along 1: ysum + mu  /  gsum + rho
@@ -334,23 +336,24 @@ __device__ __forceinline__ void apply(const Params& p, uint8_t* smem, Wait wait)
             else sScal[1] = z;
         }
         __syncthreads();
-        {                               // column sums: eight threads a column take every eighth row
+        constexpr int PARTS = THREADS / kDim;
+        {                               // column sums: every PARTS-th row a thread
             const int col = tid & (kDim - 1), part = tid >> 6;
             float m = 0.f;
             if (col < W)
-                for (int d = part; d < W; d += 8) m += sF[d * kDim + col];
+                for (int d = part; d < W; d += PARTS) m += sF[d * kDim + col];
             sMu[kDim + part * kDim + col] = m;
         }
         __syncthreads();
         if (tid < W) {                  // column tid: mean over the rows; nu = ysum + mu
             float m = 0.f;
 #pragma unroll
-            for (int k = 1; k <= 8; ++k) m += sMu[k * kDim + tid];
+            for (int k = 1; k <= PARTS; ++k) m += sMu[k * kDim + tid];
             m *= 1.f / W;
             const float ysum = sNu[tid];
             sNu[tid] = ysum + m;
             sMu[tid] = m;
-            if (MODE == kApplyForward && blockIdx.x % p.nseg == 0) {
+            if (MODE == kApplyForward && blockIdx.x % p.parts == 0) {
                 // true sums for the caller: S = 1 ysum^T + A', Z = N 1 + a'
                 if (p.vec_out) p.vec_out[r.bh * W + tid] = (float)r.len + sA[tid];
                 if (p.state_out)
@@ -549,8 +552,8 @@ __device__ __forceinline__ void apply(const Params& p, uint8_t* smem, Wait wait)
         for (int k = 0; k < WARPS; ++k) w_sum += sScal[4 + k];
         st.put_record(reinterpret_cast<float*>(smem + L::RING), rec_out, w_sum);
     }
-    zero_rows<W>(p.out0, base + r.zero_lo, base + r.zero_hi);
-    if (MODE == kApplyBackwardKV) zero_rows<W>(p.out1, base + r.zero_lo, base + r.zero_hi);
+    zero_rows<W, THREADS>(p.out0, base + r.zero_lo, base + r.zero_hi);
+    if (MODE == kApplyBackwardKV) zero_rows<W, THREADS>(p.out1, base + r.zero_lo, base + r.zero_hi);
     if (MODE == kApplyForward && p.den)
         for (int64_t i = base + r.zero_lo + tid; i < base + r.zero_hi; i += THREADS) p.den[i] = 0.f;
 }

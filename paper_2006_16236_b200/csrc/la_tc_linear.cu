@@ -23,10 +23,10 @@
 // with ysum = sum_j V_j, gsum = sum_i G_i / dn_i, rho0 = sum_i dl_i / dn_i, qh' = q' / dn.
 // The column sums of S'' and R'' vanish, so (1 + x')^T S'' = x'^T S''.
 //
-// Two kinds of kernels: tcgen05 ones, below, and those of la_linear_warp.cuh (of_warps).
-//
+// The passes that form no sums are kernels of la_linear_warp.cuh; so are the sums and the backward Q pass where of_warps() says so, and
+// elsewhere the two tcgen05 kernels below:
 // Sum kernel: 10 warps (0-7 apply elu to the X tile in place, half a row per thread; 8 TMA; 9 MMA issue).
-// Apply kernel: 14 warps (0-7 epilogue, two per TMEM quadrant, half a chunk row each; 8-11 apply elu to the
+// dQ kernel: 14 warps (0-7 epilogue, two per TMEM quadrant, half a chunk row each; 8-11 apply elu to the
 // X tile in place; 12 TMA; 13 MMA issue).
 #include "la_linear_warp.cuh"
 #include "la_tc.cuh"
@@ -287,17 +287,15 @@ linear_sum_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
 }
 
 // ===========================================================================
-// Apply passes.
+// The backward Q pass, with the reverse sums on the side.
 // ===========================================================================
-enum ApplyMode { kApplyForward = 0, kApplyBackwardQ = 1, kApplyBackwardKV = 2 };
-
 constexpr int kApStages = 4;
 constexpr int kApThreads = 448;
 constexpr uint32_t kApOffStage = 0;                                   // kApStages x {X, Y}
 constexpr uint32_t kApOffState = kApOffStage + kApStages * 2 * kTileBytes;   // bf16 centred state tile [64][64]
 constexpr uint32_t kApOffVec = kApOffState + kDim * 128;              // fp32 [3][64]: a' (Z' or r'), nu, scratch
 constexpr uint32_t kApOffBar = kApOffVec + 1024;
-constexpr uint32_t kApOffOut = (kApOffBar + 256 + 1023) & ~1023u;      // two result tiles on their way out
+constexpr uint32_t kApOffOut = (kApOffBar + 256 + 1023) & ~1023u;      // result tile on its way out (before that: scratch)
 constexpr uint32_t kApOffX = kApOffOut + 2 * kTileBytes;               // fp32 [2 halves][128 rows][8]: partial sums exchanged
 // backward Q only: the chunk's weighted queries x' / dn and its aux tile (columns 0..15: dl_i, 16..23: 1 / dn_i),
 // operands of the reverse sums that this pass forms on the side (see the sum kernel for the product)
@@ -316,12 +314,8 @@ struct ApBarriers {
 
 struct ApParams {
     const float* records;       // [BH][nseg][kRecFloats]: summed by every CTA
-    __nv_bfloat16* out0;        // forward: O;  backward Q: dQ;  backward K/V: dK
-    __nv_bfloat16* out1;        // backward K/V: dV
-    float* den;                 // forward: q.Z (optional)
-    float* rec_out;             // backward Q: [BH][nseg][kRecFloats] reverse sums of this pass's rows (out)
-    float* state_out;           // forward: KV [BH][64][64] (optional)
-    float* vec_out;             // forward: Zs [BH][64] (optional)
+    __nv_bfloat16* out;         // dQ
+    float* rec_out;             // [BH][nseg][kRecFloats] reverse sums of this pass's rows (out)
     const int* lengths;         // [B] real positions per batch element (right-padded ragged batch), or null
     const float* kept;          // backward: the forward's kept records, whose stamp has to be this plan's, or null
     int heads;
@@ -333,20 +327,18 @@ struct ApParams {
     int early;                  // a kernel of the same call runs in front: the first tiles are requested before the wait
 };
 
-template <int kMode, bool k3d>
+template <bool k3d>
 __global__ void __launch_bounds__(kApThreads, 1)
-linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
-                    const __grid_constant__ CUtensorMap mapOut0, const __grid_constant__ CUtensorMap mapOut1,
-                    const ApParams prm) {
+linear_dq_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
+                 const __grid_constant__ CUtensorMap mapOut, const ApParams prm) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
     ApBarriers* bars = reinterpret_cast<ApBarriers*>(smem + kApOffBar);
-    float* sA = reinterpret_cast<float*>(smem + kApOffVec);      // a': Z' (forward, backward Q) or r' (backward K/V)
-    float* sNu = sA + 64;                                        // rank-one part along 1: ysum + mu  /  gsum + rho
-    float* sScal = sA + 128;                                     // [0] = sum_d a'_d, [1] = w0
-    constexpr bool kHasY = kMode != kApplyForward;
-    constexpr uint32_t kTiles = kHasY ? 2 : 1;
+    float* sA = reinterpret_cast<float*>(smem + kApOffVec);      // a': Z'
+    float* sNu = sA + 64;                                        // rank-one part along 1: ysum + mu
+    float* sScal = sA + 128;                                     // [0] = sum_d a'_d
+    constexpr uint32_t kTiles = 2;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int seg = blockIdx.x % prm.nseg;
@@ -359,8 +351,8 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
     if (tid == 0) {
         for (int s = 0; s < kApStages; ++s) {
             mbar_init(&bars->full[s], 1);
-            // MMA commit + epilogue threads (they read the X and Y rows) (+ the commit of the reverse sums, which read Y)
-            mbar_init(&bars->empty[s], 1 + 256 + (kMode == kApplyBackwardQ ? 1 : 0));
+            // MMA commit + epilogue threads (they read the X and Y rows) + the commit of the reverse sums, which read Y
+            mbar_init(&bars->empty[s], 1 + 256 + 1);
             mbar_init(&bars->mapped[s], 128);
         }
         for (int b = 0; b < 2; ++b) {
@@ -403,11 +395,11 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         const int y = (c_begin + c) * kChunk, z = (int)bh;          // position in the sequence; sequence
         mbar_arrive_expect_tx(&bars->full[s], kTiles * kTileBytes);
         tile_load<k3d>(st, &mapX, y, z, prm.N, &bars->full[s]);
-        if (kHasY) tile_load<k3d>(st + kTileBytes, &mapY, y, z, prm.N, &bars->full[s]);
+        tile_load<k3d>(st + kTileBytes, &mapY, y, z, prm.N, &bars->full[s]);
     };
     if (warp == 8 && lane == 0) {
         prefetch_tensormap(&mapX);
-        if (kHasY) prefetch_tensormap(&mapY);
+        prefetch_tensormap(&mapY);
         for (int c = 0; c < min(L, kApStages); ++c) issue_load(c);
     }
     if (early) {
@@ -415,7 +407,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         allow_dependent_launch();
     }
     bool mismatch = false;      // (the same for every thread)
-    if (kHasY && prm.kept) {
+    if (prm.kept) {
         const int4 a = *reinterpret_cast<const int4*>(prm.kept + bh * (int64_t)kRecFloats + kRecStamp), b = split_stamp(prm.nseg, prm.chunks_per_seg, kDim);
         mismatch = a.x != b.x || a.y != b.y || a.z != b.z || a.w != b.w;
     }
@@ -472,13 +464,6 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             const float ysum = sNu[tid];
             sNu[tid] = ysum + m;
             sF[kDim * kDim + tid] = m;                                            // mu, just past the matrix
-            if (kMode == kApplyForward && seg == 0 && tid < dim) {
-                // true sums for the caller: S = 1 ysum^T + A', Z = N 1 + a'
-                if (prm.vec_out) prm.vec_out[bh * dim + tid] = (float)len + sA[tid];
-                if (prm.state_out)
-                    for (int d = 0; d < dim; ++d)
-                        prm.state_out[bh * (int64_t)(dim * dim) + d * dim + tid] = sF[d * kDim + tid] + ysum;
-            }
         }
         if (warp == 2) {                // sum of a' (64 values, two per lane, then a butterfly: the same order in every CTA)
             float z = sA[lane] + sA[lane + 32];
@@ -504,7 +489,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
     volatile int* abort_flag = &bars->abort_flag;
     LA_TRACE_CTA(g_trace_lin, 5);
 
-    if (kHasY && mismatch) {    // nothing is started; the tiles requested above have to arrive before the CTA may leave
+    if (mismatch) {    // nothing is started; the tiles requested above have to arrive before the CTA may leave
         if (tid == 0) atomicOr(prm.status, kStatusPlanMismatch);
         if (warp == 8 && lane == 0)
             for (int c = 0; c < min(L, kApStages); ++c) mbar_wait(&bars->full[c], 0, prm.status, kStatusTmaTimeout);
@@ -524,7 +509,6 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         {
             const bool leader = elect_one();
             const uint32_t idesc_kk = umma_idesc_bf16(128, 64, 0, 0);
-            const uint32_t idesc_kmn = umma_idesc_bf16(128, 64, 0, 1);
             const uint32_t aSt = sbase + kApOffState;
             bool ok = true;
             // backward Q: the reverse sums of chunk c, [A' | a'] += (x' / dn)^T [G | dl] and (row 80) the sums weighted by
@@ -547,30 +531,19 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             #pragma unroll 1
             for (int c = 0; c < L && ok; ++c) {
                 const int s = c % kApStages, b = c & 1;
-                const uint32_t aX = sbase + kApOffStage + s * 2 * kTileBytes, aY = aX + kTileBytes;
+                const uint32_t aY = sbase + kApOffStage + s * 2 * kTileBytes + kTileBytes;
                 ok = mbar_wait_warp(&bars->mapped[s], (c / kApStages) & 1, prm.status, kStatusPipeTimeout);
                 if (ok && c >= 2) ok = mbar_wait_warp(&bars->acc_free[b], ((c >> 1) - 1) & 1, prm.status, kStatusPipeTimeout);
                 if (!ok || __any_sync(0xFFFFFFFFu, *abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
-                const uint32_t d0 = tmem + b * 128, d1 = d0 + 64;
-                if (kMode == kApplyForward) {
-                    for (int k = 0; k < 4; ++k)      // q' S''
-                        umma_bf16(leader, d0, desc_k(aX + k * 32), desc_mn(aSt + k * 2048), idesc_kmn, k > 0);
-                } else if (kMode == kApplyBackwardQ) {
-                    for (int k = 0; k < 4; ++k)      // h'' = G S''^T
-                        umma_bf16(leader, d0, desc_k(aY + k * 32), desc_k(aSt + k * 32), idesc_kk, k > 0);
-                } else {
-                    for (int k = 0; k < 4; ++k)      // V R''^T
-                        umma_bf16(leader, d0, desc_k(aY + k * 32), desc_k(aSt + k * 32), idesc_kk, k > 0);
-                    for (int k = 0; k < 4; ++k)      // k' R''
-                        umma_bf16(leader, d1, desc_k(aX + k * 32), desc_mn(aSt + k * 2048), idesc_kmn, k > 0);
-                }
+                for (int k = 0; k < 4; ++k)          // h'' = G S''^T
+                    umma_bf16(leader, tmem + b * 128, desc_k(aY + k * 32), desc_k(aSt + k * 32), idesc_kk, k > 0);
                 umma_commit(leader, &bars->acc_full[b]);
                 umma_commit(leader, &bars->empty[s]);
-                if (kMode == kApplyBackwardQ && c >= 1) ok = issue_sums(c - 1);
+                if (c >= 1) ok = issue_sums(c - 1);
             }
-            if (kMode == kApplyBackwardQ && ok && L >= 1) ok = issue_sums(L - 1);
-            if (kMode == kApplyBackwardQ) umma_commit(leader, &bars->sums_done);
+            if (ok && L >= 1) ok = issue_sums(L - 1);
+            umma_commit(leader, &bars->sums_done);
             if (!ok) *abort_flag = 1;
         }
     } else if (warp >= 4 && warp < 8) {
@@ -609,7 +582,6 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         #pragma unroll 1
         for (int c = 0; c < L; ++c) {
             const int s = c % kApStages, b = c & 1;
-            const int64_t row = row0 + (int64_t)c * kChunk + t;
             const bool padded = (int64_t)c * kChunk + t >= real;      // a row behind the sequence's end: zeros go out
             if (!mbar_wait(&bars->mapped[s], (c / kApStages) & 1, prm.status, kStatusPipeTimeout)) { *abort_flag = 1; break; }
             if (*abort_flag) break;
@@ -619,7 +591,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) lds128(rowX + (((hf * 4 + cc) ^ r7) << 4), xv[cc]);
             float ynu_h = 0.f;                       // this half of Y_i . nu (backward)
-            if (kHasY) {
+            {
                 uint32_t yv[4][4];
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) lds128(rowX + kTileBytes + (((hf * 4 + cc) ^ r7) << 4), yv[cc]);
@@ -648,7 +620,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             tmem_ld32(tmem + lane_base + b * 128 + hf * 32, acc);
             tmem_ld_wait();
             float sh_h = 0.f, qh_h = 0.f;
-            if (kMode == kApplyBackwardQ) {
+            {
                 f32x2 sh4[4] = {0, 0, 0, 0}, qh4[4] = {0, 0, 0, 0};
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc)
@@ -678,27 +650,10 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             if (tid == 0) LA_TRACE(g_trace_lin, c, 11);
             const float x1sum = fD + sx;             // (1 + x') . 1
             uint8_t* out_row = smem + kApOffOut + t * 128;
-            if (kMode == kApplyForward) {
-                // den = (1 + q') . (N 1 + Z');  num = (1 + q').1 nu + q' S''
-                const float den = fN * x1sum + sScal[0] + xa;
-                const float inv = 1.f / (den + prm.eps);
-                const float w = x1sum * inv;
-                if (hf == 0 && prm.den && (!k3d || (int64_t)(c_begin + c) * kChunk + t < prm.N)) prm.den[row] = padded ? 0.f : den;
-                const f32x2 inv2 = pair(inv, inv), w2 = pair(w, w);
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
-                    uint32_t outp[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)     // acc * inv + w * nu
-                        outp[j] = pack_bf16x2(fma2(pair(acc[cc * 8 + 2 * j], acc[cc * 8 + 2 * j + 1]), inv2,
-                                                   mul2(w2, pair_ld(nuH + cc * 8 + 2 * j))));
-                    sts128(out_row + (((hf * 4 + cc) ^ r7) << 4), outp[0], outp[1], outp[2], outp[3]);
-                }
-            } else {
+            {
                 // backward Q:  h = (G.nu) 1 + h'',  Z = N 1 + Z',  gq = (h - (q.h / dn) Z) / dn
-                // backward KV: gk = (V.nu_R + w0) 1 + V R''^T + r'
                 float c1 = 0.f, cz = 0.f, scale = 1.f;          // out_d = scale * (acc_d + c1 + cz * a'_d)
-                if (kMode == kApplyBackwardQ) {
+                {
                     const float den = fN * x1sum + sScal[0] + xa;
                     const float dn = den + prm.eps;
                     scale = 1.f / dn;
@@ -731,9 +686,6 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
                     }
                     fence_proxy_async_smem();
                     mbar_arrive(&bars->xs_ready);
-                } else {
-                    c1 = ynu + sScal[1];
-                    cz = 1.f;
                 }
                 const f32x2 scale2 = pair(scale, scale), cz2 = pair(cz, cz), c12 = pair(c1, c1), one2 = pair(1.f, 1.f);
 #pragma unroll
@@ -749,25 +701,11 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
                     }
                     sts128(out_row + (((hf * 4 + cc) ^ r7) << 4), outp[0], outp[1], outp[2], outp[3]);
                 }
-                if (kMode == kApplyBackwardKV) {
-                    tmem_ld32(tmem + lane_base + b * 128 + 64 + hf * 32, acc);
-                    tmem_ld_wait();
-                    const f32x2 xs2 = pair(x1sum, x1sum);
-#pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {       // gV = (1 + k').1 nu_R + k' R''
-                        uint32_t outp[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            outp[j] = pack_bf16x2(fma2(xs2, pair_ld(nuH + cc * 8 + 2 * j), pair(acc[cc * 8 + 2 * j], acc[cc * 8 + 2 * j + 1])));
-                        sts128(out_row + kTileBytes + (((hf * 4 + cc) ^ r7) << 4), outp[0], outp[1], outp[2], outp[3]);
-                    }
-                }
             }
             if (padded) {
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) {
                     sts128(out_row + (((hf * 4 + cc) ^ r7) << 4), 0u, 0u, 0u, 0u);
-                    if (kMode == kApplyBackwardKV) sts128(out_row + kTileBytes + (((hf * 4 + cc) ^ r7) << 4), 0u, 0u, 0u, 0u);
                 }
             }
             if (tid == 0) LA_TRACE(g_trace_lin, c, 12);
@@ -778,8 +716,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             if (hf == 0 && lane == 0) {
                 const int y = (c_begin + c) * kChunk + quad * 32;       // rows at positions >= N are clipped by the store
                 if (!k3d || y < prm.N) {
-                    tile_store<k3d>(&mapOut0, smem + kApOffOut + quad * 32 * 128, y, (int)bh, prm.N);
-                    if (kMode == kApplyBackwardKV) tile_store<k3d>(&mapOut1, smem + kApOffOut + kTileBytes + quad * 32 * 128, y, (int)bh, prm.N);
+                    tile_store<k3d>(&mapOut, smem + kApOffOut + quad * 32 * 128, y, (int)bh, prm.N);
                 }
                 tma_store_commit();
             }
@@ -787,7 +724,7 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
         }
         if (hf == 0 && lane == 0) tma_store_wait_all<0>();
         LA_TRACE_CTA(g_trace_lin, 6);
-        if (kMode == kApplyBackwardQ && warp < 3) {
+        if (warp < 3) {
             // this split's record of the reverse sums: accumulator rows 0..63 (warps 0, 1) and row 80 (warp 2, lane 16),
             // zeros if the split holds no real row
             const bool ok = mbar_wait(&bars->sums_done, 0, prm.status, kStatusMmaTimeout) && !*abort_flag;
@@ -816,14 +753,8 @@ linear_apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             const int64_t r_lo = row0 + (int64_t)L * kChunk;
             const int64_t nrows = max((int64_t)0, min((int64_t)(L_all - L) * kChunk, prm.N - (int64_t)(c_begin + L) * kChunk));
             const int64_t n16 = nrows * kDim * 2 / 16;
-            uint4* o0 = reinterpret_cast<uint4*>(prm.out0 + r_lo * kDim);
+            uint4* o0 = reinterpret_cast<uint4*>(prm.out + r_lo * kDim);
             for (int64_t i = e; i < n16; i += 256) o0[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (kMode == kApplyBackwardKV) {
-                uint4* o1 = reinterpret_cast<uint4*>(prm.out1 + r_lo * kDim);
-                for (int64_t i = e; i < n16; i += 256) o1[i] = make_uint4(0u, 0u, 0u, 0u);
-            }
-            if (kMode == kApplyForward && prm.den)
-                for (int64_t i = e; i < nrows; i += 256) prm.den[r_lo + i] = 0.f;
         }
     }
 
@@ -882,11 +813,11 @@ int launch_sums(const la_problem& p, const Segmentation& sg, const CUtensorMap& 
                         : launch_sums_as<false>(p, sg, mX, mY, lengths, records, st);
 }
 
-template <int kMode, bool k3d>
-int launch_apply_as(const la_problem& p, const Segmentation& sg, const CUtensorMap& mX, const CUtensorMap& mY,
+template <bool k3d>
+int launch_dq_as(const la_problem& p, const Segmentation& sg, const CUtensorMap& mX, const CUtensorMap& mY,
                     ApParams prm, cudaStream_t st) {
     static std::atomic<uint64_t> attr_done{0};          // one per instantiation
-    if (int rc = opt_in_smem_once(linear_apply_kernel<kMode, k3d>, kApSmemBytes, attr_done)) return rc;
+    if (int rc = opt_in_smem_once(linear_dq_kernel<k3d>, kApSmemBytes, attr_done)) return rc;
     prm.status = device_status_ptr();
     if (!prm.status) return fail(LA_ERR_CUDA, "device status word unavailable");
     prm.heads = (int)p.H;
@@ -897,23 +828,19 @@ int launch_apply_as(const la_problem& p, const Segmentation& sg, const CUtensorM
     prm.eps = p.eps;
     prm.phi = p.phi;
     const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
-    CUtensorMap mO0, mO1;                   // one warp's 32 rows per store
-    if (int rc = encode_attention_map(&mO0, prm.out0, p.N % kChunk != 0, seqs, n, 32, (int)p.D)) return rc;
-    if (int rc = encode_attention_map(&mO1, prm.out1 ? prm.out1 : prm.out0, p.N % kChunk != 0, seqs, n, 32, (int)p.D)) return rc;
+    CUtensorMap mO;                         // one warp's 32 rows per store
+    if (int rc = encode_attention_map(&mO, prm.out, p.N % kChunk != 0, seqs, n, 32, (int)p.D)) return rc;
     prof_begin(kProfLinearApply, st);
     cudaLaunchAttribute attr;
     const cudaLaunchConfig_t cfg = chained_launch((unsigned)(sg.nseg * p.B * p.H), kApThreads, kApSmemBytes, st, &attr);
-    LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, linear_apply_kernel<kMode, k3d>, mX, mY, mO0, mO1, prm));
+    LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, linear_dq_kernel<k3d>, mX, mY, mO, prm));
     note_launch();
     prof_end(kProfLinearApply, st);
     return LA_OK;
 }
 
-template <int kMode>
-int launch_apply(const la_problem& p, const Segmentation& sg, const CUtensorMap& mX, const CUtensorMap& mY,
-                 const ApParams& prm, cudaStream_t st) {
-    return p.N % kChunk ? launch_apply_as<kMode, true>(p, sg, mX, mY, prm, st)
-                        : launch_apply_as<kMode, false>(p, sg, mX, mY, prm, st);
+int launch_dq(const la_problem& p, const Segmentation& sg, const CUtensorMap& mX, const CUtensorMap& mY, const ApParams& prm, cudaStream_t st) {
+    return p.N % kChunk ? launch_dq_as<true>(p, sg, mX, mY, prm, st) : launch_dq_as<false>(p, sg, mX, mY, prm, st);
 }
 
 // ---- a warp per sixteen positions (la_linear_warp.cuh) ----------------------------------------------------------------
@@ -928,39 +855,46 @@ __global__ void __launch_bounds__(lin::THREADS, 1) linear_warp_sum_kernel(const 
     extern __shared__ __align__(128) uint8_t smem[];
     lin::sums<W, ELU>(p, smem, StreamWait());
 }
+// warps of a CTA of the apply passes: sixteen where they form sums as well, else eight, two CTAs on an SM
+template <int MODE> constexpr int kApplyWarps = MODE == lin::kApplyBackwardQ ? lin::WARPS : 8;
 template <int W, int MODE, bool ELU>
-__global__ void __launch_bounds__(lin::THREADS, 1) linear_warp_apply_kernel(const lin::Params p) {
+__global__ void __launch_bounds__(32 * kApplyWarps<MODE>, lin::WARPS / kApplyWarps<MODE>) linear_warp_apply_kernel(const lin::Params p) {
     extern __shared__ __align__(128) uint8_t smem[];
-    lin::apply<W, MODE, ELU>(p, smem, StreamWait());
+    lin::apply<W, MODE, kApplyWarps<MODE>, ELU>(p, smem, StreamWait());
 }
 
-// Which problems: all with D = M = 32 (tcgen05 tiles of 64 columns are half empty), and of D = M = 64 those whose CTAs have little to do but
-// start: both forms and the passes alike.  Forward + backward with kept sums (forward alone), us, tcgen05 / a warp per sixteen
-// positions, B x H x N: D = 32 4x8x8192 117 / 64 (40 / 21), 64x8x512 176 / 100 (66 / 32), 8x8x1024 49 / 26 (18 / 9), 1x8x8000 64 / 41;
-// D = 64 1x8x2000 42 / 32 (16 / 12), 4x8x2000 53 / 47 (20 / 16), 8x8x1024 52 / 46 (19 / 16), 64x8x512 199 / 185 (73 / 64), 128x8x256
-// 262 / 222, 64x8x100 114 / 84, but 16x8x1024 75 / 77, 16x8x2048 128 / 137, 8x8x4096 129 / 138 (45 / 47).
+// Which sums and backward Q passes: all with D = M = 32 (tcgen05 tiles of 64 columns are half empty), and of D = M = 64 those whose CTAs
+// have little to do but start.  Forward + backward with kept sums (forward alone), us, all on tcgen05 / as it is now, B x H x N:
+// D = 32 4x8x8192 118 / 63 (41 / 23), 64x8x512 176 / 83 (66 / 27), 8x8x1024 49 / 26 (18 / 10), 1x8x8000 64 / 40; D = 64 1x8x2000
+// 42 / 33 (16 / 12), 8x8x1024 52 / 47 (19 / 16), 64x8x512 199 / 167 (73 / 56), 64x8x100 114 / 72 (48 / 24); with these two passes on tcgen05
+// 8x8x4096 130 / 120 (45 / 40), ragged 127 / 116, 32x8x1024 151 / 133 (55 / 46), 4x8x8192 131 / 115; with none 8x8x4096 138, 16x8x1024 77
+// where the two on tcgen05 make it 71.
 bool of_warps(const la_problem& p) { return p.D == 32 || p.N <= 512 || p.B * p.H * p.N <= 65536; }
 
 template <auto KERNEL>
-int launch_as(ProfKernel prof, const la_problem& p, int smem, const lin::Params& a, cudaStream_t st) {
+int launch_as(ProfKernel prof, const la_problem& p, int warps, int smem, const lin::Params& a, cudaStream_t st) {
     static std::atomic<uint64_t> attr_done{0};          // one per instantiation
     if (int rc = opt_in_smem_once(KERNEL, (uint32_t)smem, attr_done)) return rc;
     prof_begin(prof, st);
     cudaLaunchAttribute attr;
-    const cudaLaunchConfig_t cfg = chained_launch((unsigned)(a.nseg * p.B * p.H), lin::THREADS, (uint32_t)smem, st, &attr);
+    const cudaLaunchConfig_t cfg = chained_launch((unsigned)(a.parts * p.B * p.H), 32 * (unsigned)warps, (uint32_t)smem, st, &attr);
     LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, KERNEL, a));
     note_launch();
     prof_end(prof, st);
     return LA_OK;
 }
 template <int W> int launch_warp_sums(const la_problem& p, const lin::Params& a, cudaStream_t st) {
-    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_sum_kernel<W, true>>(kProfLinearSum, p, lin::kSumSmem<W>, a, st);
-    return launch_as<linear_warp_sum_kernel<W, false>>(kProfLinearSum, p, lin::kSumSmem<W>, a, st);
+    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_sum_kernel<W, true>>(kProfLinearSum, p, lin::WARPS, lin::kSumSmem<W>, a, st);
+    return launch_as<linear_warp_sum_kernel<W, false>>(kProfLinearSum, p, lin::WARPS, lin::kSumSmem<W>, a, st);
 }
-template <int W, int MODE> int launch_warp_apply(const la_problem& p, const lin::Params& a, cudaStream_t st) {
-    constexpr int smem = lin::ApplyLayout<W, MODE>::BYTES;
-    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_apply_kernel<W, MODE, true>>(kProfLinearApply, p, smem, a, st);
-    return launch_as<linear_warp_apply_kernel<W, MODE, false>>(kProfLinearApply, p, smem, a, st);
+template <int W, int MODE> int launch_warp_apply(const la_problem& p, lin::Params a, cudaStream_t st) {
+    constexpr int warps = kApplyWarps<MODE>, smem = lin::ApplyLayout<W, MODE, warps>::BYTES;
+    if (warps < lin::WARPS) {       // two CTAs on every SM over all heads, at least 128 positions each
+        const int64_t most = chunks_of(p.N), want = 2 * sm_count() / (p.B * p.H);
+        a.parts = (int)(want < 1 ? 1 : want < most ? want : most);
+    }
+    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_apply_kernel<W, MODE, true>>(kProfLinearApply, p, warps, smem, a, st);
+    return launch_as<linear_warp_apply_kernel<W, MODE, false>>(kProfLinearApply, p, warps, smem, a, st);
 }
 
 int make_params(const la_problem& p, const int* lengths, lin::Params* a) {
@@ -971,7 +905,7 @@ int make_params(const la_problem& p, const int* lengths, lin::Params* a) {
     if (!a->status) return fail(LA_ERR_CUDA, "device status word unavailable");
     a->N = p.N;
     a->heads = (int)p.H;
-    a->nseg = sg.nseg;
+    a->nseg = a->parts = sg.nseg;
     a->chunks_per_seg = sg.chunks_per_seg;
     a->eps = p.eps;
     return LA_OK;
@@ -1039,21 +973,21 @@ int linear_forward(const la_problem& p, const void* Q, const void* K, const void
     if (of_warps(p)) return (p.D == 32 ? warp_forward<32> : warp_forward<64>)(p, Q, K, V, lengths, O, den, KV, Zs, saved ? (float*)saved : (float*)ws, st);
     const Segmentation sg = choose_splits(p);
     const uint64_t seqs = (uint64_t)(p.B * p.H), n = (uint64_t)p.N;
-    CUtensorMap mQ, mK, mV;
-    if (int rc = encode_attention_map(&mQ, Q, p.N % kChunk != 0, seqs, n, kChunk, (int)p.D)) return rc;
+    CUtensorMap mK, mV;
     if (int rc = encode_attention_map(&mK, K, p.N % kChunk != 0, seqs, n, kChunk, (int)p.D)) return rc;
     if (int rc = encode_attention_map(&mV, V, p.N % kChunk != 0, seqs, n, kChunk, (int)p.D)) return rc;
     float* rec = saved ? (float*)saved : (float*)ws;      // the split records, kept for the backward pass if asked
     if (int rc = launch_sums(p, sg, mK, mV, lengths, rec, st)) return rc;
-    ApParams a = {};
-    a.lengths = lengths;
+    lin::Params a;
+    if (int rc = make_params(p, lengths, &a)) return rc;
     a.records = rec;
-    a.out0 = (__nv_bfloat16*)O;
+    a.X = Q;
+    a.out0 = O;
     a.den = den;
     a.state_out = KV;
     a.vec_out = Zs;
     a.early = 1;                // behind the sum kernel
-    return launch_apply<kApplyForward>(p, sg, mQ, mQ, a, st);
+    return launch_warp_apply<64, lin::kApplyForward>(p, a, st);
 }
 
 int linear_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths,
@@ -1064,33 +998,31 @@ int linear_backward(const la_problem& p, const void* Q, const void* K, const voi
     const Segmentation sg = choose_splits(p);
     const size_t bh = (size_t)(p.B * p.H);
     const uint64_t n = (uint64_t)p.N;
-    CUtensorMap mQ, mK, mV, mG;
+    CUtensorMap mQ, mG;
     if (int rc = encode_attention_map(&mQ, Q, p.N % kChunk != 0, bh, n, kChunk, (int)p.D)) return rc;
-    if (int rc = encode_attention_map(&mK, K, p.N % kChunk != 0, bh, n, kChunk, (int)p.D)) return rc;
-    if (int rc = encode_attention_map(&mV, V, p.N % kChunk != 0, bh, n, kChunk, (int)p.D)) return rc;
     if (int rc = encode_attention_map(&mG, G, p.N % kChunk != 0, bh, n, kChunk, (int)p.D)) return rc;
     uint8_t* w = (uint8_t*)ws;
     float* rec_s = (float*)w;   w += bh * sg.nseg * kRecFloats * sizeof(float);
     float* rec_r = (float*)w;   w += bh * sg.nseg * kRecFloats * sizeof(float);
 
     if (saved) rec_s = (float*)saved;         // the forward's own records: nothing to recompute
-    else if (int rc = launch_sums(p, sg, mK, mV, lengths, rec_s, st)) return rc;
+    else if (int rc = linear_keep_sums(p, K, V, lengths, rec_s, st)) return rc;
     ApParams a = {};
     a.early = saved ? 0 : 1;    // the first kernel of the call with saved records, else behind the sum kernel
     a.lengths = lengths;
     a.kept = (const float*)saved;
     a.records = rec_s;
-    a.out0 = (__nv_bfloat16*)dQ;
+    a.out = (__nv_bfloat16*)dQ;
     a.rec_out = rec_r;          // the reverse sums of Q / dn and G are formed by the same pass
-    if (int rc = launch_apply<kApplyBackwardQ>(p, sg, mQ, mG, a, st)) return rc;
-    ApParams b = {};
-    b.lengths = lengths;
+    if (int rc = launch_dq(p, sg, mQ, mG, a, st)) return rc;
+    lin::Params b;
+    if (int rc = make_params(p, lengths, &b)) return rc;
     b.kept = (const float*)saved;
     b.records = rec_r;
-    b.out0 = (__nv_bfloat16*)dK;
-    b.out1 = (__nv_bfloat16*)dV;
+    b.X = K; b.Y = V;
+    b.out0 = dK; b.out1 = dV;
     b.early = 1;                // behind the dQ pass
-    return launch_apply<kApplyBackwardKV>(p, sg, mK, mV, b, st);
+    return launch_warp_apply<64, lin::kApplyBackwardKV>(p, b, st);
 }
 
 }  // namespace tc
