@@ -121,7 +121,7 @@ causal_mma_forward_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * p.parts);
+            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * parts_of<C>(p));
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
         float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
@@ -278,7 +278,7 @@ causal_mma_dq_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * p.parts);
+            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * parts_of<C>(p));
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
         float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
@@ -514,7 +514,7 @@ causal_mma_dkv_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;           // record i is the sum of piece i + 1
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + (r.bh * p.records + r.piece * p.parts) * (int64_t)(D * M + D), (p.pieces - 1 - r.piece) * p.parts);
+            p.rec + (r.bh * p.records + r.piece * parts_of<C>(p)) * (int64_t)(D * M + D), (p.pieces - 1 - r.piece) * parts_of<C>(p));
     const int64_t chunks = (r.end - r.lo + T - 1) / T;
     for (int64_t c = chunks - 1; c >= 0; --c) {
         const uint32_t sQ = smem_u32(smem + Sh::X), sG = smem_u32(smem + Sh::Y), sR = smem_u32(smem + Sh::S);
@@ -792,9 +792,9 @@ Plan choose_plan(const la_problem& p, bool single) {
 
 // Records of a piece: with bf16 features the sums of few pieces are shared out over the SMs that would have none (Fourier B8 H8 N1000, two
 // pieces of eight chunks, three passes over the sums: 14, 14 and 27 us with 64 CTAs that load a chunk when they need it, 10, 10 and 15
-// with 128 that load it ahead; fp32 D = 48 B3 H4 N1500 99.5 / 100.5 a step, D = 80 B1 H8 N2000 202 / 207).
+// with 128 that load it ahead; no gain in fp32).
 int record_parts(const la_problem& p, const Plan& pl) {
-    if (of_warps(p) || p.dtype != LA_BF16 || pl.pieces < 2) return 1;
+    if (of_warps(p) || p.dtype != LA_BF16 || p.phi != LA_PHI_IDENTITY || pl.pieces < 2) return 1;        // (kScaled, see dispatch())
     const int64_t idle = 148 / (p.B * p.H * (pl.pieces - 1)), chunks = pl.len / T, most = chunks < 4 ? chunks : 4;
     return (int)(idle < 1 ? 1 : idle < most ? idle : most);
 }

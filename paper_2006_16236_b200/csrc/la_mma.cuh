@@ -203,8 +203,8 @@ __device__ __forceinline__ void with_phi(int phi, F f) {
     else f([](float x) { const float e = expf(x); return x > 0.f ? x + 1.f : e; });
 }
 
-// Whole tiles without a predicate and padding per group: where tiles are never wider than the problem and the kernels small,
-// that is bf16 with 32 columns (D = M = 32, la_causal_mma.cu); the others lost 5 to 8 % to the second copy of their loads.
+// Whole strips without a predicate and padding per group: where they are never wider than the problem and the kernels small,
+// that is bf16 with 32 columns (D = M = 32, la_cluster.cu); the others lost 5 to 8 % to the second copy of their loads.
 template <typename IO, int C> constexpr bool kPlainLoads = sizeof(IO) == 2 && C == 32;
 
 // T rows of `cols` columns (padded to C), contiguous in global memory; rows cn.. and columns cols.. hold `pad`.
@@ -213,14 +213,6 @@ struct RawTile {
     static constexpr int GROUPS = T * (C / 8) / THREADS;
     Group8<IO> r[GROUPS];
     __device__ __forceinline__ void load(const IO* src, int cn, int cols, float pad) {
-        if constexpr (kPlainLoads<IO, C>) {
-            if (cn >= T) {
-                src += threadIdx.x * 8;
-#pragma unroll
-                for (int u = 0; u < GROUPS; ++u) r[u].load(src + u * (THREADS * 8));
-                return;
-            }
-        }
 #pragma unroll
         for (int u = 0; u < GROUPS; ++u) {
             const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), c = idx % (C / 8) * 8;
@@ -240,18 +232,8 @@ struct RawTile {
     // planes of the features
     template <int NP>
     __device__ __forceinline__ void features(uint8_t* tile, int phi) const {
-        // One plane: two values at a time, from bf16 to bf16, five and a half instructions a value instead of ten.  These kernels
-        // are bound by instruction issue: with this, loads without predicates and one prefetch per thread, B128 H8 N784 D32
-        // forward + backward 298.9 -> 283 us.
-        if constexpr (NP == 1) {
-            static_assert(sizeof(IO) == 2, "one plane");
-            if (phi == LA_PHI_IDENTITY) return copy(tile);
-#pragma unroll
-            for (int u = 0; u < GROUPS; ++u) {
-                const int idx = (int)threadIdx.x + u * THREADS, row = idx / (C / 8), g = idx % (C / 8);
-                *reinterpret_cast<uint4*>(tile + tile_at<C>(row, g)) =
-                    make_uint4(tc::phi_pair<true>(r[u].a.x), tc::phi_pair<true>(r[u].a.y), tc::phi_pair<true>(r[u].a.z), tc::phi_pair<true>(r[u].a.w));
-            }
+        if constexpr (NP == 1) {            // features as they are given
+            copy(tile);
         } else {
             with_phi<NP>(phi, [&](auto f) { store<NP>(tile, [&](int, float x) { return f(x); }); });
         }
