@@ -24,9 +24,7 @@ struct Params {
     const float *S0, *Z0;        // state the sweep starts from (forward: S_in, Z_in; reverse: dS_out, dZ_out), each or null
     float *S1, *Z1;              // where the state it ends with goes (S_out, Z_out / dS_in, dZ_in), each or null
     float* rec;                  // [bh][records][D * M + D]: sums of the pieces first_record .. first_record + records - 1
-    float* rec_out;              // where the dQ sweep leaves the reverse records, or null
     int records, first_record;
-    int parts;                   // records of a piece (causal sums): its sums in that many ranges
     float* aux;                  // [bh][2][N]: dn_i, -G_i . O_i
     const int* lengths;
     int64_t N, piece_len;
@@ -35,6 +33,8 @@ struct Params {
     int* stamp;                  // kept sums (or null): the plan they were written under, see plan_stamp()
     int* status;                 // device status word (with stamp)
     float eps;
+    int parts;                   // records of a piece (causal sums): its sums in that many ranges
+    float* rec_out;              // where the dQ sweep leaves the reverse records, or null
 };
 
 // positions [lo, hi) of this CTA's piece, of them [lo, end) real
