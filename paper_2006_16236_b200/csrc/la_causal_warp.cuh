@@ -301,7 +301,7 @@ __device__ __forceinline__ void forward(const Params& p, uint8_t* smem) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int row = g + 8 * h;
-            const float d = h ? d1 : d0, i = reciprocal(d + p.eps);
+            const float d = h ? d1 : d0, i = 1.f / (d + p.eps);
             const sm100::f32x2 inv = sm100::pair(i, i);
             uint32_t w[NT];
 #pragma unroll
@@ -352,8 +352,8 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     if (p.stamp && sweep::other_plan(p, *reinterpret_cast<const int4*>(p.stamp))) return;
     const Span r(p, blockIdx.y);
     uint8_t* dQ = rows_at(p.dQ, r, p.N, r.lo);
-    float* dn_all = p.aux + 2 * r.bh * p.N;
-    float* dl_all = dn_all + p.N;
+    float* inv_all = p.aux + 2 * r.bh * p.N;         // 1 / dn_i, which every later use of it takes
+    float* dl_all = inv_all + p.N;
     Ring<4, false> in;
     in.start(smem, r.bh, p.N, r.end, {p.Q, p.K, p.V, p.G}, nullptr);
     for (int i = 0; i < in.AHEAD; ++i) in.request(r.lo + i * ROWS);
@@ -431,7 +431,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
                 dn[b] = quad_sum(d[b]) + p.eps;
-                inv[b] = reciprocal(dn[b]);
+                inv[b] = 1.f / dn[b];
                 go[b] = (quad_sum(e[b]) - c[b] * p.eps) * inv[b];        // what is left of G_i . O_i
                 c[b] += go[b];
             }
@@ -466,7 +466,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
             if (g + 8 * b < cn) {
                 put_row(dQ, b, w);
                 if (t == 0) {
-                    dn_all[n0 + g + 8 * b] = dn[b];
+                    inv_all[n0 + g + 8 * b] = inv[b];
                     dl_all[n0 + g + 8 * b] = -c[b];
                 }
             }
@@ -500,7 +500,7 @@ __device__ __forceinline__ void reverse_sums(const Params& p, uint8_t* smem) {
         const Rows G = in.rows(1);
         const float* w = in.weights();
         const float2 l0 = load_pair(w + 16 + 2 * t), l1 = load_pair(w + 24 + 2 * t);
-        map_weighted<ELU>(q, reciprocal(w[g]), reciprocal(w[g + 8]));
+        map_weighted<ELU>(q, w[g], w[g + 8]);
         const Rows qt = transposed(q);
         st.add(qt, transposed(G));
         st.add_weighted(qt, l0, l1);
@@ -536,7 +536,7 @@ __device__ __forceinline__ void dkv(const Params& p, uint8_t* smem) {
         const Rows v = in.rows(2), G = in.rows(3);
         const float* w = in.weights();
         const float2 l0 = load_pair(w + 16 + 2 * t), l1 = load_pair(w + 24 + 2 * t);
-        map_weighted<ELU>(q, reciprocal(w[g]), reciprocal(w[g + 8]));
+        map_weighted<ELU>(q, w[g], w[g + 8]);
         map_features<ELU>(k);
         const Rows qt = transposed(q), gt = transposed(G);
         uint32_t rb[4][NT];

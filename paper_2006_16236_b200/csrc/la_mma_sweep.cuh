@@ -25,7 +25,7 @@ struct Params {
     float *S1, *Z1;              // where the state it ends with goes (S_out, Z_out / dS_in, dZ_in), each or null
     float* rec;                  // [bh][records][D * M + D]: sums of the pieces first_record .. first_record + records - 1
     int records, first_record;
-    float* aux;                  // [bh][2][N]: dn_i, -G_i . O_i
+    float* aux;                  // [bh][2][N]: dn_i (a warp per piece: 1 / dn_i), -G_i . O_i
     const int* lengths;
     int64_t N, piece_len;
     int pieces, heads, D, M, phi;

@@ -57,12 +57,6 @@ __device__ __forceinline__ void columns_mma(float (&c)[4], const Rows<W>& a, F f
 __device__ __forceinline__ void add_pair(float& x, float& y, float a, float b) {
     sm100::unpair(sm100::add2(sm100::pair(x, y), sm100::pair(a, b)), x, y);
 }
-// 1 / x to the last bit or two
-__device__ __forceinline__ float reciprocal(float x) {
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 
 // the lane's part of a row's dot product: a (bf16 pairs) with b (fp32 pairs at the same columns)
 template <int NT, typename F>
@@ -82,7 +76,7 @@ struct Ring {
     static constexpr int AHEAD = STAGES - 1, TILE = ROWS * W * 2, PARTS = W / 32;        // a row's parts of 64 bytes
     static constexpr int STAGE_BYTES = T * TILE + (WEIGHTS ? 128 : 0), BYTES = STAGES * STAGE_BYTES;
     const uint8_t* src[T];          // the lane's bytes of the sequence's first chunk
-    const float* w;                 // the lane's weight of it: dn in lanes 0 .. 15, dl in lanes 16 .. 31
+    const float* w;                 // the lane's weight of it: 1 / dn in lanes 0 .. 15, dl in lanes 16 .. 31
     uint8_t* base;                  // slot 0
     uint8_t* mine;                  // the lane's bytes of it (rows of 64 bytes, the four sixteens of row g in another order: an
                                     // ldmatrix that reads one of eight rows finds them in different banks)

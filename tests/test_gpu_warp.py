@@ -67,6 +67,33 @@ def test_pieces_lengths_and_states(B, H, N, pieces):
 
 
 @pytest.mark.gpu
+def test_the_normaliser_divides_to_the_last_bit():
+    """Features a, b along one axis and values chosen so that (a v0 + b v1) / (a + b) lies halfway between two bf16 numbers: all sums are
+    exact, so the output is that of one correctly rounded fp32 reciprocal, a product and the rounding to bf16, to the bit.  (A
+    reciprocal that is one fp32 bit off leaves the middle and may round the other way.)"""
+    rng, heads = np.random.default_rng(0), 512
+    a, b, v0, v1 = (np.zeros(s, np.float32) for s in ((heads,), (heads,), (heads, D), (heads, D)))
+    n0, n1 = np.meshgrid(np.arange(129, 256, 2), np.arange(128, 256))           # v0 = n0 / 256, v1 = n1 / 128
+    for h in range(heads):
+        found = np.zeros(0, np.int64)
+        while len(found) < D:
+            a[h], b[h] = 2 * rng.integers(64) + 1, 2 * rng.integers(1, 256)
+            total = (a[h] * n0 + 2 * b[h] * n1).astype(np.int64).ravel()
+            r, rest = np.divmod(total, int(a[h] + b[h]))
+            found = np.nonzero((rest == 0) & (r % 2 == 1) & (r > 256) & (r < 512))[0]       # an odd number of 1/256, between 1 and 2
+        at = rng.permutation(found)[:D]
+        v0[h], v1[h] = n0.ravel()[at] / 256, n1.ravel()[at] / 128
+    Q, K, V = (torch.zeros(1, heads, 2, D) for _ in range(3))
+    Q[..., 0], K[0, :, 0, 0], K[0, :, 1, 0], V[0, :, 0], V[0, :, 1] = 1.0, *map(torch.from_numpy, (a, b, v0, v1))
+    Qd, Kd, Vd = (t.to(DEV, BF) for t in (Q, K, V))
+    assert all(torch.equal(x.cpu().float(), t) for x, t in zip((Qd, Kd, Vd), (Q, K, V)))
+    O = la.la_causal_forward(Qd, Kd, Vd, phi="identity", eps=0.0)
+    inv = np.float32(1.0) / (a + b)
+    want = torch.from_numpy((a[:, None] * v0 + b[:, None] * v1) * inv[:, None]).to(BF)
+    assert torch.equal(O[0, :, 1].cpu(), want)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("splits", [-1, 1, 3])
 @pytest.mark.parametrize("W", [32, 64])
 @pytest.mark.parametrize("N", [1, 15, 17, 256, 257, 500, 900])
