@@ -208,6 +208,12 @@ template <bool ELU> __device__ __forceinline__ void map_features(Rows& r) {
 #pragma unroll
             for (int n = 0; n < NT; ++n) r.x[h][n] = tc::phi_pair<true>(r.x[h][n]);
 }
+// the larger of two bf16 pairs, NaN where one of them is
+__device__ __forceinline__ uint32_t max_nan_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.NaN.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
 // phi(q) / dn, rounded once
 template <bool ELU> __device__ __forceinline__ void map_weighted(Rows& r, float inv0, float inv1) {
 #pragma unroll
@@ -216,16 +222,16 @@ template <bool ELU> __device__ __forceinline__ void map_weighted(Rows& r, float 
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
             const uint32_t w = r.x[h][n];
-            float x = sm100::bf16_lo(w), y = sm100::bf16_hi(w);
-            if constexpr (ELU) {          // (the square of the exponential of half the number, as phi_pair: the smallest features are kept)
+            sm100::f32x2 x = sm100::pair_bf16(w);
+            if constexpr (ELU) {          // exp(min(x, 0)) + max(x, 0); the square of the exponential of half the number, as phi_pair: the smallest features are kept
                 float t0, t1, e0, e1;
-                sm100::unpair(sm100::mul2(sm100::pair(x, y), sm100::pair(0.72134752044448170f, 0.72134752044448170f)), t0, t1);
+                sm100::unpair(sm100::mul2(sm100::pair_bf16(sm100::min_bf16x2(w, 0u)), sm100::pair(0.72134752044448170f, 0.72134752044448170f)), t0, t1);
                 asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(t0));
                 asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(t1));
-                x = x > 0.f ? x + 1.f : e0 * e0;
-                y = y > 0.f ? y + 1.f : e1 * e1;
+                const sm100::f32x2 e = sm100::pair(e0, e1);
+                x = sm100::fma2(e, e, sm100::pair_bf16(max_nan_bf16x2(w, 0u)));
             }
-            r.x[h][n] = sm100::pack_bf16x2(sm100::mul2(sm100::pair(x, y), inv));
+            r.x[h][n] = sm100::pack_bf16x2(sm100::mul2(x, inv));
         }
     }
 }
@@ -345,7 +351,7 @@ __device__ __forceinline__ void sums(const Params& p, uint8_t* smem) {
 }
 
 // ---- dQ sweep -----------------------------------------------------------------------------------------------------
-// REVERSE: and the sums q^^T [G | dl] of the piece, q^ = phi(q) / dn from the rounded features, for the sweep that follows.
+// REVERSE: and the sums q^^T [G | dl] of the piece, q^ = phi(q) / dn, for the sweep that follows.
 template <bool ELU, bool REVERSE>
 __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -378,7 +384,6 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
         in.arrived(1, cn, ELU ? kMinusInf : 0u);
         Rows q = in.rows(0), k = in.rows(1);
         const Rows v = in.rows(2), G = in.rows(3);
-        in.next();
         map_features<ELU>(q);
         map_features<ELU>(k);
         const Rows kt = transposed(k);
@@ -437,16 +442,15 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
             }
         }
         if (REVERSE && r.piece > 0) {
-            Rows w;
-            float dl[2];
+            Rows w = in.rows(0);            // (again: rounded once, as the sweep that takes these sums has its own)
+            float i[2], dl[2];
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
                 const bool real = g + 8 * b < cn;           // (rows that are not there may have a normaliser of zero)
-                const float i = real ? inv[b] : 0.f;
+                i[b] = real ? inv[b] : 0.f;
                 dl[b] = real ? -c[b] : 0.f;
-#pragma unroll
-                for (int n = 0; n < NT; ++n) w.x[b][n] = sm100::pack_bf16x2(sm100::mul2(sm100::pair_bf16(q.x[b][n]), sm100::pair(i, i)));
             }
+            map_weighted<ELU>(w, i[0], i[1]);
             w = transposed(w);
             back.add(w, transposed(G));
             auto of_row = [&](float x, int row) { return __shfl_sync(0xffffffffu, x, row * 4); };
@@ -471,6 +475,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
                 }
             }
         }
+        in.next();
         dQ += ROWS * C * 2;
     };
     int n0 = r.lo;

@@ -94,6 +94,28 @@ def test_the_normaliser_divides_to_the_last_bit():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("pieces,N", [(2, 128), (2, 512), (5, 512)])
+@pytest.mark.parametrize("phi", ["elu1", "identity"])
+def test_sums_of_pieces_are_those_of_the_sweep(phi, pieces, N):
+    """The gradient of the initial state is the sum of phi(q) / dn G over all positions: what the reverse sweep adds up itself where a
+    sequence is one piece, and what records of the pieces hold where it is several.  Both round phi(q) / dn to bf16 once, so that they
+    differ by the order of fp32 additions, and by the few operands that an fp32 bit of dn takes over a rounding boundary: 2^-24 of
+    2^-8, one in 2^16, each off by 2^-8 of itself, 2^-16 of the whole.  Rounded twice they are 2^-9 apart."""
+    B, H = 38, 8
+    Q, K, V, G = draw_qkvg(B, H, N, D, D, 3, BF, 1.0)
+    if phi == "identity":
+        Q, K = (Q.float().abs() + 0.1).to(BF), (K.float().abs() + 0.1).to(BF)
+    dev = [t.to(DEV) for t in (Q, K, V, G)]
+    S0, Z0, got = torch.ones(B, H, D, D, device=DEV), torch.full((B, H, D), 3.0, device=DEV), []
+    for n in (1, pieces):
+        la.la_plan_override(n)
+        dS, dZ = torch.empty_like(S0), torch.empty_like(Z0)
+        la.la_causal_backward(*dev, phi=phi, S_in=S0, Z_in=Z0, dS_in=dS, dZ_in=dZ)
+        got.append(dS)
+    assert float((got[1] - got[0]).norm() / got[0].norm()) < 2.0 ** -14
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("splits", [-1, 1, 3])
 @pytest.mark.parametrize("W", [32, 64])
 @pytest.mark.parametrize("N", [1, 15, 17, 256, 257, 500, 900])
