@@ -374,11 +374,15 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     if constexpr (REVERSE) back.clear();
     st.add_state<false>(p.S0 ? p.S0 + r.bh * C * C : nullptr, p.Z0 ? p.Z0 + r.bh * C : nullptr);
     const uint32_t lower = diagonal_mask<false>();
-    // The first chunks of a sequence go through twice, the second time with the G_i . O_i it found taken off the scores
-    // and off the sums' part, and have the sums in two bf16 parts: where few terms make up a row, h and (q . h / dn) Zc cancel
-    // almost entirely (in row 0 completely).  Four chunks: dQ's error against 64 bits, which its first rows have the largest part in,
-    // is then what it was with chunks of 64 positions (B128 H8 N784: 4.4e-3; with one chunk 4.6e-3).
+    // The first 64 positions of a sequence go through twice, the second time with the G_i . O_i they found taken off the scores
+    // and off the sums' part: where few terms make up a row, h and (q . h / dn) Zc cancel almost entirely (in row 0 completely).  The first
+    // 256 have the sums in two bf16 parts: their rounding, once for sixteen positions, is what dQ loses most by where the weights are
+    // near-uniform.  dQ's error against 64 bits with 64 / 128 / 256 positions, inputs scaled by 1/8: B16 H8 N3072 1.83e-2 / 1.79e-2 / 1.73e-2,
+    // where tcgen05 chunks of 128 positions have 1.76e-2; B38 H8 N200 1.68e-2 / 1.59e-2 / 1.52e-2 for 1.59e-2 (the features' own rounding:
+    // 1.5e-2).  A step of B128 H8 N784 159.7 / 160.1 / 162.3 us.
+    constexpr int TWICE = 4 * ROWS, PRECISE = 16 * ROWS;
     auto chunk = [&](int n0, auto first) {
+        const bool twice = decltype(first)::value && n0 < TWICE;
         const int cn = r.end - n0;              // (of them sixteen at most)
         in.request(n0 + in.AHEAD * ROWS);
         in.arrived(1, cn, ELU ? kMinusInf : 0u);
@@ -390,7 +394,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
         float c[2] = {0.f, 0.f}, dn[2], inv[2], go[2];          // c: G_i . O_i of rows g, g + 8, as far as it is known
         float h[NT][4], zc[NT][4];
 #pragma unroll 1
-        for (int pass = decltype(first)::value ? 0 : 1; pass < 2; ++pass) {
+        for (int pass = twice ? 0 : 1; pass < 2; ++pass) {
             {
                 uint32_t sb[4][NT];
                 st.rounded(sb);
@@ -406,7 +410,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
 #pragma unroll
                 for (int n = 0; n < NT; ++n) columns_mma<false>(h[n], G, [&](int kk, int i) { return sb[n][2 * kk + i]; });
             }
-            if (decltype(first)::value && pass == 1) {
+            if (twice && pass == 1) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     s0[j] -= c[j >> 1];
@@ -480,7 +484,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     };
     int n0 = r.lo;
 #pragma unroll 1
-    for (; n0 < 4 * ROWS && n0 < r.end; n0 += ROWS) chunk(n0, std::true_type());
+    for (; n0 < PRECISE && n0 < r.end; n0 += ROWS) chunk(n0, std::true_type());
 #pragma unroll 1
     for (; n0 < r.end; n0 += ROWS) chunk(n0, std::false_type());
     if (REVERSE && r.piece > 0) back.put_record(p.rec_out + (r.bh * p.records + r.piece - 1) * (int64_t)RECORD_FLOATS);
