@@ -121,7 +121,7 @@ causal_mma_forward_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * parts_of<C>(p));
+            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * parts_of<C, EXACT>(p));
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
         float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
@@ -278,7 +278,7 @@ causal_mma_dq_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * parts_of<C>(p));
+            p.rec + r.bh * p.records * (int64_t)(D * M + D), r.piece * parts_of<C, EXACT>(p));
     for (int64_t n0 = r.lo; n0 < r.end; n0 += T) {
         const uint32_t sK = smem_u32(smem + Sh::X), sV = smem_u32(smem + Sh::Y), sS = smem_u32(smem + Sh::S);
         float* sZ = reinterpret_cast<float*>(smem + Sh::Z);
@@ -514,7 +514,7 @@ causal_mma_dkv_kernel(const Params p) {
 
     State<DP, MP, 4 * WPS> st;           // record i is the sum of piece i + 1
     st.init(p, p.S0 ? p.S0 + r.bh * D * M : nullptr, p.Z0 ? p.Z0 + r.bh * D : nullptr,
-            p.rec + (r.bh * p.records + r.piece * parts_of<C>(p)) * (int64_t)(D * M + D), (p.pieces - 1 - r.piece) * parts_of<C>(p));
+            p.rec + (r.bh * p.records + r.piece * parts_of<C, EXACT>(p)) * (int64_t)(D * M + D), (p.pieces - 1 - r.piece) * parts_of<C, EXACT>(p));
     const int64_t chunks = (r.end - r.lo + T - 1) / T;
     for (int64_t c = chunks - 1; c >= 0; --c) {
         const uint32_t sQ = smem_u32(smem + Sh::X), sG = smem_u32(smem + Sh::Y), sR = smem_u32(smem + Sh::S);
@@ -790,13 +790,14 @@ Plan choose_plan(const la_problem& p, bool single) {
     return Plan{(int)((p.N + len - 1) / len), len};
 }
 
-// Records of a piece: with bf16 features the sums of few pieces are shared out over the SMs that would have none (Fourier B8 H8 N1000, two
-// pieces of eight chunks, three passes over the sums: 14, 14 and 27 us with 64 CTAs that load a chunk when they need it, 10, 10 and 15
-// with 128 that load it ahead; no gain in fp32).
+// Records of a piece: where sequences are two pieces of 128 bf16 features, their sums are shared out over the SMs that would have none
+// (Fourier B8 H8 N1000, pieces of eight chunks, three passes over the sums: 14, 14 and 27 us with 64 CTAs that load a chunk when they
+// need it, 10, 10 and 15 with 128 that load it ahead; pieces of three chunks B8 H8 N300 fwd 19.5 / 18.7, of two N256 20.6 / 22.3).  Not where
+// there are more pieces: each adds up all records before its own, and four for one took B1 H1 N4000 (16 pieces) from 179 to 382 us.
 int record_parts(const la_problem& p, const Plan& pl) {
-    if (of_warps(p) || p.dtype != LA_BF16 || p.phi != LA_PHI_IDENTITY || pl.pieces < 2) return 1;        // (kScaled, see dispatch())
-    const int64_t idle = 148 / (p.B * p.H * (pl.pieces - 1)), chunks = pl.len / T, most = chunks < 4 ? chunks : 4;
-    return (int)(idle < 1 ? 1 : idle < most ? idle : most);
+    if (p.dtype != LA_BF16 || p.phi != LA_PHI_IDENTITY || p.D != 128 || p.M != 64 || pl.pieces != 2 || pl.len < 3 * T) return 1;     // (see parts_of())
+    const int64_t idle = 148 / (p.B * p.H);
+    return (int)(idle < 1 ? 1 : idle < 4 ? idle : 4);
 }
 size_t record_bytes(const la_problem& p, const Plan& pl) {
     return (size_t)(p.B * p.H) * (size_t)(pl.pieces - 1) * (size_t)record_parts(p, pl) * (size_t)(p.D * p.M + p.D) * sizeof(float);

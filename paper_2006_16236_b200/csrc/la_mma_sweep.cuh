@@ -273,8 +273,8 @@ template <int WPS, int DP, int MP, int NX, int NY, int NRW, int RC, int NS, int 
 // reverse scores to their columns: (k q^T) / dn, ((G V^T + dl) / dn) q instead of k (q / dn)^T, (G V^T + dl) (q / dn).  Per sixteen
 // keys and queries that is 96 products where it was 176.  Fourier B8 H8 N1000 C128 dK and dV 84 -> 77 us.
 template <typename C> constexpr bool kScaled = C::NQ == 1 && C::NV == 1 && C::NR == 3;
-// (the other configurations have one record of a piece: known when compiled, it is 1 % of a step of a small grid)
-template <typename C> __device__ __forceinline__ int parts_of(const Params& p) { return kScaled<C> ? p.parts : 1; }
+// (all but 128 features by 64 columns have one record of a piece: known when compiled, it is 1 to 4 % of a step of a small grid)
+template <typename C, bool EXACT> __device__ __forceinline__ int parts_of(const Params& p) { return kScaled<C> && EXACT ? p.parts : 1; }
 template <typename C, int DP, int MP, bool REVERSE>
 using SumLayout = Layout<1, DP, MP, REVERSE && !kScaled<C> ? C::NR : C::NQ, REVERSE && kScaled<C> ? C::NR : C::NV, 0, 0, 0, 0>;
 
@@ -389,7 +389,7 @@ causal_mma_sum_kernel(const Params p) {
     const float pad = pad_value(phi);
     wait_for_stream();
     release_next();
-    const int parts = parts_of<C>(p);
+    const int parts = parts_of<C, EXACT>(p);
     Range r = range_of(p, (int)blockIdx.y / parts + p.first_record);
     if (parts > 1) {            // the CTA's part of the piece
         const int64_t chunks = (r.hi - r.lo + T - 1) / T, each = (chunks + parts - 1) / parts * T, lo = r.lo + (int)blockIdx.y % parts * each;

@@ -60,6 +60,19 @@ def test_pieces_of_the_fp32_accurate_causal_kernels(L, dt, phi, D, BHN, pieces):
     assert la.la_workspace_bytes(p, binding.LA_OP_CAUSAL_FORWARD) == BHN[0] * BHN[1] * (pieces - 1) * D * 65 * 4
 
 
+@pytest.mark.parametrize("D,M", [(128, 64), (64, 32), (96, 48)])
+@pytest.mark.parametrize("BH,N", [(1, 2000), (1, 4000), (3, 1500), (4, 2000), (4, 4000), (20, 2000), (64, 1000), (64, 300), (64, 200)])
+def test_pieces_of_bf16_features_add_up_few_records(L, BH, N, D, M):
+    """Every piece starts by adding up the records of all pieces before it: one each, or up to four where there is one piece before."""
+    p = la.make_problem(BH, 1, N, D, M, binding.LA_BF16, phi="identity")
+    size = BH * (D * M + D) * 4
+    records, rest = divmod(la.la_workspace_bytes(p, binding.LA_OP_CAUSAL_FORWARD), size)
+    la.la_plan_override(causal_pieces=1)
+    one = la.la_workspace_bytes(p, binding.LA_OP_CAUSAL_FORWARD)
+    la.la_plan_override()
+    assert one == 0 and rest == 0 and records <= 15
+
+
 def _p(**kw):
     base = dict(B=1, H=1, N=128, D=64, M=64, dtype_code=binding.LA_F32)
     base.update(kw)
