@@ -1,6 +1,7 @@
 // Feature map (Eq. 7) as a stand-alone elementwise kernel, and the one-token
 // recurrent step (Eq. 16-20, attention part).
 #include "la_common.cuh"
+#include "la_tc_common.cuh"
 
 namespace la {
 
@@ -280,8 +281,9 @@ int launch_poly2_map_backward(const void* x, const void* dy, void* dx, int64_t r
 // front is then the projection of the same call, which never touches the state, waited for everything before it
 // and only then let this kernel be scheduled, so the last writer of the state has completed: the state, which
 // is all the traffic of this kernel, streams in while that projection runs.
+constexpr int kEarlyCtas = 10;        // of the step with an early state, on an SM: 48 registers each
 template <typename T, int D, int M, bool kEarlyState = false>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, kEarlyState ? kEarlyCtas : 0)
 recurrent_step_kernel(const T* q, const T* k, const T* v,       // (written by the kernel in front, see load_global())
                       float* __restrict__ S, float* __restrict__ Z, T* __restrict__ out,
                       float eps, int phi, int resident) {
@@ -306,8 +308,8 @@ recurrent_step_kernel(const T* q, const T* k, const T* v,       // (written by t
     if (kEarlyState) {
 #pragma unroll
         for (int p = 0; p < PASSES; ++p) s[p] = Sp[(r0 + p * RPP) * TPR + c4];
-        // The CTAs that find no room beside these (48 registers: ten on an SM) find their state in L2, one line per thread:
-        // a decode layer of B256 H8 21.5 -> 20.5 us, B512 31.4 -> 29.2, B1000 54.6 / 54.7 (HBM is busy throughout).
+        // The CTAs that find no room beside these find their state in L2, one line per thread (how many these are, and when not: see
+        // recurrent_dispatch()).
         if (bh + resident < gridDim.x && tid * 128 < D * M * 4)
             asm volatile("prefetch.global.L2 [%0];" ::"l"((const char*)(Sp + (int64_t)resident * (D * M / 4)) + tid * 128));
     }
@@ -591,7 +593,13 @@ static int recurrent_dispatch(const la_problem& p, const void* q, const void* k,
         cfg.stream = st;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        if (early_state) LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, recurrent_step_kernel<T, 64, 64, true>, qq, kk, vv, S, Z, oo, p.eps, p.phi, 10 * 148));
+        // The first `resident` CTAs ask for the states of those behind them while the projection in front runs, up to three and a half
+        // times as many: with more HBM is busy throughout and they only come in its way.  A decode layer, us, without / with, by number of
+        // states: 2048 21.2 / 20.2, 4096 31.3 / 29.2, 5000 33.9 / 33.0, 5120 36.6 / 35.8, 6000 39.4 / 40.0, 6144 42.0 / 42.6 and 44.2 / 44.8,
+        // 8000 54.6 / 54.9, 12000 78.3 / 82.9, 24000 153.8 / 166.7.
+        const int resident = kEarlyCtas * tc::sm_count(), none = 1 << 30;
+        const bool ahead = 2 * (int64_t)grid <= 7 * (int64_t)resident;
+        if (early_state) LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, recurrent_step_kernel<T, 64, 64, true>, qq, kk, vv, S, Z, oo, p.eps, p.phi, ahead ? resident : none));
         else LA_CUDA_TRY(cudaLaunchKernelEx(&cfg, recurrent_step_kernel<T, 64, 64>, qq, kk, vv, S, Z, oo, p.eps, p.phi, 0));
         note_launch();
         return LA_OK;
