@@ -159,32 +159,67 @@ struct Sums {
                 for (int j = 0; j < 4; ++j) s[i][n][j] = buf[at(8 * n + 2 * t + (j & 1), 16 * i + 8 * (j >> 1) + g)];
         __syncwarp();
     }
-    // The caller's matrix [D][M] and vector [D]; TURNED: s holds the matrix transposed.  f(element of s, element of the matrix)
-    template <bool TURNED, typename F> static __device__ __forceinline__ void each(F f) {
-        const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int r = 8 * (g >> 1) + 2 * (2 * i + (j >> 1)) + (g & 1), c = 8 * t + 2 * n + (j & 1);
-                    f(i, n, j, TURNED ? c * C + r : r * C + c);
-                }
-    }
+    // The caller's matrix [D][M] and vector [D], in loads and stores of sixteen bytes.  A lane has of s every
+    // second one of eight rows, and of the matrix its own two columns of each tile: columns 8 t .. 8 t + 7 of rows 8 (g / 2) + g % 2 + 2 k.
+    // TURNED (s holds the matrix transposed): rows and columns change places, and lanes g and g ^ 1 load (store) half a row each and
+    // exchange what the other wants.
+    static __device__ __forceinline__ int first_row() { const int g = (threadIdx.x & 31) >> 2; return 8 * (g >> 1) + (g & 1); }
     template <bool TURNED> __device__ __forceinline__ void add_state(const float* S, const float* z) {
-        const int t = threadIdx.x & 3;
-        if (S) each<TURNED>([&](int i, int n, int j, int at) { s[i][n][j] += S[at]; });
+        const int lane = threadIdx.x & 31, t = lane & 3;
+        const bool odd = lane & 4;
+        if (S && !TURNED)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float4* q = reinterpret_cast<const float4*>(S + (first_row() + 2 * k) * C + 8 * t);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float4 v = q[u];
+                    float (&a)[4] = s[k >> 1][2 * u], (&b)[4] = s[k >> 1][2 * u + 1];
+                    const int e = (k & 1) * 2;
+                    a[e] += v.x; a[e + 1] += v.y; b[e] += v.z; b[e + 1] += v.w;
+                }
+            }
+        if (S && TURNED)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {           // element u & 1 of tile u / 2
+                const float4 v = *reinterpret_cast<const float4*>(S + (8 * t + u) * C + 8 * (lane >> 3) + (odd ? 4 : 0));
+                const float x = __shfl_xor_sync(0xffffffffu, odd ? v.x : v.y, 4), y = __shfl_xor_sync(0xffffffffu, odd ? v.z : v.w, 4);
+                const int n = u >> 1, e = u & 1;
+                s[0][n][e] += odd ? x : v.x;
+                s[0][n][2 + e] += odd ? y : v.z;
+                s[1][n][e] += odd ? v.y : x;
+                s[1][n][2 + e] += odd ? v.w : y;
+            }
         if (z)
 #pragma unroll
-            for (int n = 0; n < NT; ++n) { v[n][0] += z[8 * t + 2 * n]; v[n][1] += z[8 * t + 2 * n + 1]; }
+            for (int u = 0; u < 2; ++u) {
+                const float4 w = reinterpret_cast<const float4*>(z + 8 * t)[u];
+                v[2 * u][0] += w.x; v[2 * u][1] += w.y; v[2 * u + 1][0] += w.z; v[2 * u + 1][1] += w.w;
+            }
     }
     template <bool TURNED> __device__ __forceinline__ void put_state(float* S, float* z) const {
         const int lane = threadIdx.x & 31, t = lane & 3;
-        if (S) each<TURNED>([&](int i, int n, int j, int at) { S[at] = s[i][n][j]; });
+        const bool odd = lane & 4;
+        if (S && !TURNED)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float (&a)[4] = s[k >> 1][2 * u], (&b)[4] = s[k >> 1][2 * u + 1];
+                    const int e = (k & 1) * 2;
+                    reinterpret_cast<float4*>(S + (first_row() + 2 * k) * C + 8 * t)[u] = make_float4(a[e], a[e + 1], b[e], b[e + 1]);
+                }
+        if (S && TURNED)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int n = u >> 1, e = u & 1;
+                const float a0 = s[0][n][e], a1 = s[0][n][2 + e], a2 = s[1][n][e], a3 = s[1][n][2 + e];
+                const float x = __shfl_xor_sync(0xffffffffu, odd ? a0 : a2, 4), y = __shfl_xor_sync(0xffffffffu, odd ? a1 : a3, 4);
+                *reinterpret_cast<float4*>(S + (8 * t + u) * C + 8 * (lane >> 3) + (odd ? 4 : 0)) = odd ? make_float4(x, a2, y, a3) : make_float4(a0, x, a1, y);
+            }
         if (z && lane < 4)
 #pragma unroll
-            for (int n = 0; n < NT; ++n) { z[8 * t + 2 * n] = v[n][0]; z[8 * t + 2 * n + 1] = v[n][1]; }
+            for (int u = 0; u < 2; ++u) reinterpret_cast<float4*>(z + 8 * t)[u] = make_float4(v[2 * u][0], v[2 * u][1], v[2 * u + 1][0], v[2 * u + 1][1]);
     }
 };
 
