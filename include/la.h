@@ -38,7 +38,7 @@
  *    backward up to 1024 (from 65; bf16 D = 64 from 257), the bidirectional forward in bf16 up
  *    to 1536 at D = 64 and 8192 at D = 32.  Sizes of buffers and plans are unaffected.
  *    Only the tcgen05 kernels have a la_causal_plan(), and only they and the bf16
- *    mma.sync ones of D = M = 32 (unless B*H >= 444 and N <= 1024) a causal saved buffer.
+ *    mma.sync ones of D = M = 32 (where they cut sequences into pieces) a causal saved buffer.
  *    bf16 features of LA_PHI_ELU1 below 1.2e-38 (keys and queries below -87.3) are zero on the
  *    tcgen05 kernels and in clusters, and what bf16 holds of them everywhere else.
  *    Finite numbers keep their value on these kernels; an infinity in Q, K, V or G acts like a NaN

@@ -911,7 +911,7 @@ size_t causal_mma_workspace(const la_problem& p, bool backward) {
 }
 // the records of a forward pass, and the plan they were written under
 size_t causal_mma_saved_bytes(const la_problem& p) {
-    const size_t rec = causal_mma_needs_workspace(p) ? record_bytes(p, choose_plan(p, false)) : 0;
+    const size_t rec = of_warps(p) ? record_bytes(p, choose_plan(p, false)) : 0;
     return rec ? kStampBytes + rec : 0;
 }
 

@@ -24,7 +24,8 @@ def _automatic_plans():
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("pieces", [-1, 1, 2, 5])
-@pytest.mark.parametrize("B,H,N", [(38, 8, 1), (38, 8, 15), (38, 8, 17), (38, 8, 63), (38, 8, 64), (38, 8, 200), (1, 2, 2100), (2, 1, 2049 + 64)])
+@pytest.mark.parametrize("B,H,N", [(38, 8, 1), (38, 8, 15), (38, 8, 17), (38, 8, 63), (38, 8, 64), (38, 8, 65), (38, 8, 100), (38, 8, 128), (38, 8, 200),
+                                   (56, 8, 200), (150, 8, 40), (1, 2, 2100), (2, 1, 2049 + 64)])
 def test_pieces_lengths_and_states(B, H, N, pieces):
     Q, K, V, G = draw_qkvg(B, H, N, D, D, 7 + N, BF, 1.0)
     g = torch.Generator().manual_seed(N)
@@ -207,11 +208,11 @@ def test_steps_enqueued_behind_each_other():
 
 
 def test_workspace_and_saved_sizes():
-    """Problems that kernels with a required workspace had before keep requiring one; others keep neither needing nor keeping one."""
+    """Problems that kernels with a required workspace had before keep requiring one; sequences in pieces keep their sums, whole ones nothing."""
     p = lambda *s: la.make_problem(*s, 32, 32, la.LA_BF16)
     size = lambda q, op: la.la_workspace_bytes(q, op)
     assert size(p(16, 8, 3072), la.LA_OP_CAUSAL_FORWARD) > 0 and size(p(16, 8, 3072), la.LA_OP_CAUSAL_SAVED) > 0
-    assert size(p(128, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0 and size(p(60, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0
+    assert size(p(128, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0 and size(p(60, 8, 784), la.LA_OP_CAUSAL_SAVED) > 0
 
 
 def test_no_read_only_loads():
