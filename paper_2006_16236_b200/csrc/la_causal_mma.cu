@@ -742,17 +742,44 @@ double wide_cost(const WideCosts& w, int64_t bh, int64_t chunks, int64_t n) {
     return t;
 }
 
-// A warp per piece: two of them on every scheduler (eight on an SM, the most that the dQ sweep with both sums has registers for), or
-// what comes closest; and no more than a piece's start makes good: it adds up the records before it, 0.45 us of a step for each,
-// where a chunk of 64 takes 7.7 us.  Forward + backward, us, B x H x N: number of pieces: 16x8x3072 4: 131, 8: 106, 12: 115; 8x8x16384
-// 8: 322, 16: 251, 24: 280; 32x8x3072 3: 232, 4: 187, 8: 200; 50x8x1000 2: 121, 3: 119, 4: 106; 64x8x2048 1: 257, 3: 234, 4: 250;
-// 100x8x2000 1: 360, 2: 353, 3: 375; 128x8x784 1: 154, 2: 190; few heads 1x8x16384 32: 106, 64: 88, 128: 113; 1x8x4096 16: 61,
-// 32: 51, 64: 59; 2x1x65536 64: 190, 128: 154.
-int64_t warp_pieces(int64_t bh, int64_t chunks) {
-    int64_t n = bh > 888 ? 1 : bh > 592 ? 2 : bh > 394 ? 3 : 1184 / bh;
-    const int64_t most = (int64_t)(4.0 * sqrt((double)chunks));
-    if (n > most) n = most;
-    return n < chunks ? n : chunks;
+// What n pieces of a sequence cost a warp per piece, in us: warps in waves of as many as an SM holds, each a little slower the more of
+// them share it; the records that a piece adds up; the kernels' starts.  (The first 64 positions go through the dQ sweep twice.)  Fitted to
+// 2500 measured numbers of pieces for 450 sizes, B*H 150 to 900, N 192 to 4096: 7 % off in the mean.
+double warp_wave(int64_t warps, double sixteens, int64_t most, double alone, double each) {
+    const int64_t wave = 148 * most, rest = (warps % wave + 147) / 148;
+    return sixteens * ((double)(warps / wave) * (alone + each * (double)most) + (rest ? alone + each * (double)rest : 0.0));
+}
+double warp_cost(int64_t bh, int64_t N, int64_t n, bool forward_alone) {
+    const int64_t chunks = (N + T - 1) / T, per = (chunks + n - 1) / n;
+    n = (chunks + per - 1) / per;
+    const int64_t warps = bh * n;
+    const double r = (double)(((per * T < N ? per * T : N) + 15) / 16), records = (double)(n - 1) * (double)warps / 148.0;
+    double t = warp_wave(warps, r, 12, 0.44, 0.06) + 0.025 * records + 2.5;
+    if (n > 1) t += warp_wave(bh * (n - 1), r, 16, 0.2, 0.035) + 1.2;
+    if (forward_alone) return t;
+    return t + warp_wave(warps, r + 0.5 * (r < 4.0 ? r : 4.0), 8, 0.74, 0.03) + warp_wave(warps, r, warps <= 8 * 148 ? 8 : 12, 0.25, 0.15) + 0.05 * records + 6.9;
+}
+
+// Pieces for a warp each, of a training step or of a forward pass that keeps no sums: eight warps on an SM, the most that the dQ sweep with
+// both sums has registers for, and no more than a piece's start makes good (forward + backward, us, B x H x N: number of pieces: 16x8x3072
+// 4: 131, 8: 106, 12: 115; 8x8x16384 8: 322, 16: 251, 24: 280; 1x8x16384 32: 106, 64: 88, 128: 113; 1x8x4096 16: 61, 32: 51, 64: 59; 2x1x65536
+// 64: 190, 128: 154).  Beyond 148 sequences another number where the estimate above finds it faster by its own error (just past a full wave
+// above all: 400x1x2048 3: 235, 8: 201; 444x1x512 3: 73, 4: 58; 592x1x784 3: 114, 2: 104; forward alone 400x1x2048 3: 71, 4: 59): 2 % off the best of the measured numbers in the mean where the first rule alone is 4 % (forward alone 2 and 6).  One piece: two
+// chunks (500x1x100 1: 25.1, 2: 28.2), three of as many sequences as run one on a scheduler (530x1x192 1: 36.1, 3: 38.4; but 640x1x192 1: 46.1,
+// 2: 44.2 and 180x1x192 1: 35.7, 3: 22.6), and more than 888 sequences (900x1x784 1: 155, 2: 181, 3: 164).
+int64_t warp_pieces(int64_t bh, int64_t N, bool forward_alone) {
+    const int64_t chunks = (N + T - 1) / T, most = (int64_t)(4.0 * sqrt((double)chunks));
+    if (bh > 888 || chunks <= 2 || (chunks == 3 && bh >= 444 && bh <= 592)) return 1;
+    int64_t best = bh > 592 ? 2 : bh > 394 ? 3 : 1184 / bh;
+    if (best > most) best = most;
+    if (best > chunks) best = chunks;
+    if (bh <= 148) return best;
+    double least = 0.93 * warp_cost(bh, N, best, forward_alone);
+    for (int64_t n = 1; n <= 16 && n <= chunks && n * bh <= 4000; ++n) {        // (as far as it was measured)
+        const double t = warp_cost(bh, N, n, forward_alone);
+        if (t < least) { least = t; best = n; }
+    }
+    return best;
 }
 
 // Pieces per sequence, by the estimated time: fp32 D = M = 64 and Fourier features as above; the others in units of one chunk of a main
@@ -761,18 +788,19 @@ int64_t warp_pieces(int64_t bh, int64_t chunks) {
 // which it has half of them on average; the pre-pass does 0.35 of a main kernel's work per chunk (fp32 D = M = 32, B4 H8 N2000,
 // pieces 1 / 4 / 8 / 12 / 16: 353 / 141 / 113 / 131 / 119; B22 H8 N3316 903 / 732 / 749 / 733 / 757).  At most sixteen: the estimates
 // are checked up to N = 4096 only (for few sequences much longer than that they would want more).
-Plan choose_plan(const la_problem& p, bool single) {
+enum PlanFor { kStep, kForwardAlone, kNoRecords };        // a training step; a forward pass that keeps no sums; no room for records
+Plan choose_plan(const la_problem& p, PlanFor what) {
     const int64_t chunks = (p.N + T - 1) / T, bh = p.B * p.H;
     int64_t best = 1;
     const int forced = tc::causal_pieces_override();
     const bool wide = p.dtype == LA_F32 ? p.D == 64 && p.M == 64 : p.phi == LA_PHI_IDENTITY && p.D == 128 && p.M == 64;
-    if (single) {
+    if (what == kNoRecords) {
         best = 1;
     } else if (forced > 0) {
         best = forced < chunks ? forced : chunks;
         if (best > 1024) best = 1024;
     } else if (of_warps(p)) {
-        best = warp_pieces(bh, chunks);
+        best = warp_pieces(bh, p.N, what == kForwardAlone);
     } else if (!(wide && bh >= 222 && bh <= 296)) {          // (two CTAs on an SM as they are: one piece was the best of 112 measured sizes of 2 to 64 chunks)
         auto waves = [](int64_t ctas) {
             const int64_t sm = (ctas + 147) / 148;
@@ -906,21 +934,21 @@ bool causal_mma_preferred(const la_problem& p) { return of_warps(p); }
 bool causal_mma_needs_workspace(const la_problem& p) { return of_warps(p) && (p.B * p.H < 3 * 148 || p.N > 1024); }
 
 size_t causal_mma_workspace(const la_problem& p, bool backward) {
-    const size_t rec = record_bytes(p, choose_plan(p, false));
+    const size_t rec = record_bytes(p, choose_plan(p, backward ? kStep : kForwardAlone));
     return backward ? aux_bytes(p) + (of_warps(p) ? 2 * rec : rec) : rec;
 }
 // the records of a forward pass, and the plan they were written under
 size_t causal_mma_saved_bytes(const la_problem& p) {
-    const size_t rec = of_warps(p) ? record_bytes(p, choose_plan(p, false)) : 0;
+    const size_t rec = of_warps(p) ? record_bytes(p, choose_plan(p, kStep)) : 0;
     return rec ? kStampBytes + rec : 0;
 }
 
 int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,
                        const float* Z_in, void* O, float* den, float* S_out, float* Z_out, void* saved, void* ws, size_t ws_bytes, cudaStream_t st) {
-    Plan pl = choose_plan(p, false);
-    if (saved && causal_mma_saved_bytes(p)) {
-        ws = (char*)saved + kStampBytes;
-    } else if (saved = nullptr; !ws || !aligned16(ws) || ws_bytes < record_bytes(p, pl)) pl = choose_plan(p, true);       // no room for records: one piece per sequence
+    if (saved && !causal_mma_saved_bytes(p)) saved = nullptr;
+    Plan pl = choose_plan(p, saved ? kStep : kForwardAlone);
+    if (saved) ws = (char*)saved + kStampBytes;
+    else if (!ws || !aligned16(ws) || ws_bytes < record_bytes(p, pl)) pl = choose_plan(p, kNoRecords);        // one piece per sequence
     Params a = make_params(p, pl, lengths);
     a.Q = Q; a.K = K; a.V = V; a.O = O; a.den = den;
     a.S0 = S_in; a.Z0 = Z_in; a.S1 = S_out; a.Z1 = Z_out;
@@ -931,7 +959,7 @@ int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const 
 
 int causal_mma_backward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const void* G,
                         const StateArgs& sa, const void* saved, void* dQ, void* dK, void* dV, void* ws, cudaStream_t st) {
-    const Plan pl = choose_plan(p, false);
+    const Plan pl = choose_plan(p, kStep);
     Params f = make_params(p, pl, lengths);
     f.Q = Q; f.K = K; f.V = V; f.G = G; f.dQ = dQ; f.dK = dK; f.dV = dV;
     f.aux = (float*)ws;

@@ -215,6 +215,15 @@ def test_workspace_and_saved_sizes():
     assert size(p(128, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0 and size(p(60, 8, 784), la.LA_OP_CAUSAL_SAVED) > 0
 
 
+@pytest.mark.parametrize("BHN,pieces", [((50, 8, 2048), 8), ((444, 1, 512), 4), ((592, 1, 784), 2), ((500, 1, 100), 1), ((560, 1, 128), 1), ((180, 1, 192), 3),
+                                        ((900, 1, 784), 1), ((128, 1, 3072), 8), ((4, 1, 4096), 32)], ids=str)
+def test_numbers_of_pieces(BHN, pieces):
+    """What was measured best, or within 3 % of it: just past a full wave of warps, two chunks, many sequences, few."""
+    p = la.make_problem(*BHN, 32, 32, la.LA_BF16)
+    kept = la.la_workspace_bytes(p, la.LA_OP_CAUSAL_SAVED)
+    assert (kept - 16 if kept else 0) == BHN[0] * BHN[1] * (pieces - 1) * 32 * 33 * 4
+
+
 def test_no_read_only_loads():
     """As the other kernels that may start as programmatic dependents."""
     for name in ("la_warp.cuh", "la_causal_warp.cuh", "la_linear_warp.cuh"):
