@@ -229,7 +229,8 @@ int la_linear_attention_backward_kept(const la_problem* p, const void* Q, const 
  * valid for la_causal_backward() with the same problem, Q, K and V until overwritten.  The
  * size is 0 for problems that keep nothing (pass NULL, or any pointer).
  * Whether it is given does not change O, except that a problem of more sequences than one
- * wave of clusters holds may run another kernel with it (O then agrees to rounding).
+ * wave of clusters holds, and bf16 ones of D = M = 32 that a warp per piece takes, may run
+ * another kernel or be cut in another way with it (O then agrees to rounding).
  */
 int la_causal_forward(const la_problem* p, const void* Q, const void* K, const void* V,
                       void* O, float* den, float* S_out, float* Z_out,

@@ -504,8 +504,9 @@ static int causal_forward_common(const la_problem* p, const void* Q, const void*
     LA_DEBUG_SPAN(saved, saved_bytes);
     if (causal_cluster_forward_preferred(*p, tc_path && saved, S_in != nullptr, st))
         return debug_finish(causal_cluster_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, tc_path ? saved : nullptr, st), stream);
-    if (tc_path)
-        return debug_finish(tc::causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, st), stream);
+    const bool left = causal_mma_supported(*p) && causal_mma_leaves_forward(*p) && !(saved && causal_mma_saved_bytes(*p));
+    if (tc_path || left)
+        return debug_finish(tc::causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, left ? nullptr : saved, ws, st), stream);
     if (causal_mma_supported(*p))
         return debug_finish(causal_mma_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, saved, ws, ws_bytes, st), stream);
     return debug_finish(general_causal_forward(*p, Q, K, V, lengths, S_in, Z_in, O, den, S_out, Z_out, st), stream);

@@ -930,11 +930,23 @@ bool causal_mma_supported(const la_problem& p) {
 
 bool causal_mma_preferred(const la_problem& p) { return of_warps(p); }
 
+// Of a warp per piece, which forward passes that keep no sums run on the tcgen05 kernels all the same: where one CTA of those per
+// sequence is a wave of its own, well filled, the more of them the longer the sequences (their plan makes two pieces up to 74 sequences, and 149
+// are two waves).  us, tcgen05 / a warp per piece, from a state in brackets, B*H x N: 90x512 8.2 / 9.8, 100x512 8.2 / 10.0 (9.5 / 10.8), 128x512 8.2 /
+// 10.5 (9.5 / 11.3), 112x1024 12.9 / 14.9, 128x1024 13.1 / 15.2, 140x1280 15.4 / 18.7, 128x4096 42.0 / 45.3; at the edges 112x1500 0.98 of the
+// time, 128x1500 1.00, 148x900 0.93, 100x1000 0.98, 90x784 0.96, 74x640 0.67, 150x512 0.74.  A training step is faster on warps.
+bool causal_mma_leaves_forward(const la_problem& p) {
+    if (!of_warps(p) || tc::causal_pieces_override() >= 0 || p.B * p.H * p.N >= (1LL << 31)) return false;        // (32-bit TMA coordinates)
+    const int64_t bh = p.B * p.H, tiles = (p.N + 127) / 128, from = 56 + 6 * tiles;
+    return bh <= 148 && bh > (from < 112 ? from : 112);
+}
+
 // The forward's workspace is optional for all problems of this file but those that a warp per piece took over from the tcgen05 kernels.
 bool causal_mma_needs_workspace(const la_problem& p) { return of_warps(p) && (p.B * p.H < 3 * 148 || p.N > 1024); }
 
 size_t causal_mma_workspace(const la_problem& p, bool backward) {
     const size_t rec = record_bytes(p, choose_plan(p, backward ? kStep : kForwardAlone));
+    if (!backward && causal_mma_leaves_forward(p)) return tc::causal_forward_workspace(p);
     return backward ? aux_bytes(p) + (of_warps(p) ? 2 * rec : rec) : rec;
 }
 // the records of a forward pass, and the plan they were written under

@@ -16,6 +16,7 @@ int tc_causal_plan(const la_problem& p, int32_t* out, int capacity);
 bool causal_mma_supported(const la_problem& p);
 bool causal_mma_preferred(const la_problem& p);      // of the problems that both kinds of kernels take
 bool causal_mma_needs_workspace(const la_problem& p);
+bool causal_mma_leaves_forward(const la_problem& p); // a forward pass that keeps no sums, of the latter: to the tcgen05 kernels
 size_t causal_mma_workspace(const la_problem& p, bool backward);
 size_t causal_mma_saved_bytes(const la_problem& p);  // what a forward pass leaves for the backward pass, or 0
 int causal_mma_forward(const la_problem& p, const void* Q, const void* K, const void* V, const int* lengths, const float* S_in,

@@ -208,11 +208,39 @@ def test_steps_enqueued_behind_each_other():
 
 
 def test_workspace_and_saved_sizes():
-    """Problems that kernels with a required workspace had before keep requiring one; sequences in pieces keep their sums, whole ones nothing."""
+    """Sequences in pieces need room for their sums, and keep them for a training step; whole ones, and forward passes that are one kernel,
+    nothing."""
     p = lambda *s: la.make_problem(*s, 32, 32, la.LA_BF16)
     size = lambda q, op: la.la_workspace_bytes(q, op)
-    assert size(p(16, 8, 3072), la.LA_OP_CAUSAL_FORWARD) > 0 and size(p(16, 8, 3072), la.LA_OP_CAUSAL_SAVED) > 0
+    assert size(p(8, 8, 3072), la.LA_OP_CAUSAL_FORWARD) > 0 and size(p(8, 8, 3072), la.LA_OP_CAUSAL_SAVED) > 0
+    assert size(p(16, 8, 3072), la.LA_OP_CAUSAL_FORWARD) == 0 and size(p(16, 8, 3072), la.LA_OP_CAUSAL_SAVED) > 0
     assert size(p(128, 8, 784), la.LA_OP_CAUSAL_SAVED) == 0 and size(p(60, 8, 784), la.LA_OP_CAUSAL_SAVED) > 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("BH,N,tcgen05", [(128, 512, True), (112, 1000, True), (100, 1000, False), (148, 300, True), (149, 512, False), (90, 512, True),
+                                          (76, 1024, False)], ids=str)
+def test_forward_passes_that_keep_no_sums(BH, N, tcgen05):
+    """A wave of one tcgen05 CTA per sequence takes them; training steps, which keep sums, stay on warps.  Both to the same gates, from a
+    state too."""
+    B, H = BH, 1
+    Q, K, V, _ = draw_qkvg(B, H, N, D, D, 3, BF, 1.0, with_grad=False)
+    g = torch.Generator().manual_seed(1)
+    S0, Z0 = torch.randn((B, H, D, D), generator=g) * 3.0, torch.rand((B, H, D), generator=g) * 4.0 + 1.0
+    dev, st = [t.to(DEV) for t in (Q, K, V)], {"S_in": S0.to(DEV), "Z_in": Z0.to(DEV)}
+    for saved in (None, la.saved_buffer(dev[0], dev[2])):
+        S, Z = torch.empty_like(st["S_in"]), torch.empty_like(st["Z_in"])
+        la.la_profile_enable(True)
+        O = la.la_causal_forward(*dev, S_out=S, Z_out=Z, saved=saved, **st)
+        la.la_last_device_status()
+        names = set(la.la_profile_read())
+        la.la_profile_enable(False)
+        assert ("causal_fwd_kernel" in names) == (tcgen05 and saved is None) and ("causal_mma_forward_kernel" in names) != ("causal_fwd_kernel" in names)
+        for b in (0, B - 1):
+            q, k, v = (t[b:b + 1].double().numpy() for t in (Q, K, V))
+            ref = oracle.causal_from_state(q, k, v, S0[b:b + 1].double().numpy(), Z0[b:b + 1].double().numpy())
+            for nm, x, r in (("O", O, ref[0]), ("S_out", S, ref[2]), ("Z_out", Z, ref[3])):
+                assert_close(x[b:b + 1], r, BF, nm)
 
 
 @pytest.mark.parametrize("BHN,pieces", [((50, 8, 2048), 8), ((444, 1, 512), 4), ((592, 1, 784), 2), ((500, 1, 100), 1), ((560, 1, 128), 1), ((180, 1, 192), 3),
