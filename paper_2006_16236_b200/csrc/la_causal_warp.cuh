@@ -342,7 +342,7 @@ __device__ __forceinline__ void forward(const Params& p, uint8_t* smem) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int row = g + 8 * h;
-            const float d = h ? d1 : d0, i = 1.f / (d + p.eps);
+            const float d = h ? d1 : d0, i = reciprocal(d + p.eps);
             const sm100::f32x2 inv = sm100::pair(i, i);
             uint32_t w[NT];
 #pragma unroll
@@ -475,7 +475,7 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
                 dn[b] = quad_sum(d[b]) + p.eps;
-                inv[b] = 1.f / dn[b];
+                inv[b] = reciprocal(dn[b]);
                 go[b] = (quad_sum(e[b]) - c[b] * p.eps) * inv[b];        // what is left of G_i . O_i
                 c[b] += go[b];
             }

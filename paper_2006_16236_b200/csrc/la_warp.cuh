@@ -58,6 +58,18 @@ __device__ __forceinline__ void add_pair(float& x, float& y, float a, float b) {
     sm100::unpair(sm100::add2(sm100::pair(x, y), sm100::pair(a, b)), x, y);
 }
 
+// 1 / x as a division gives it, without the branch of one, at which these loops would be cut in two (B128 H8 N784 161.7 -> 155.7 us a
+// step): the approximation and one Newton-Raphson step in fused multiply-adds, which rounds correctly but for mantissas of all ones
+// (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990); of all 2^32 numbers ten, with reciprocals
+// below 1.2e-38, differ from 1.f / x, of the approximation alone 13 %.  Where the residual is no small number (x zero, infinite, NaN, or its
+// reciprocal too large) the approximation is the answer.
+__device__ __forceinline__ float reciprocal(float x) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    const float e = fmaf(-x, r, 1.f);
+    return fabsf(e) < 0.5f ? fmaf(r, e, r) : r;
+}
+
 // the lane's part of a row's dot product: a (bf16 pairs) with b (fp32 pairs at the same columns)
 template <int NT, typename F>
 __device__ __forceinline__ sm100::f32x2 row_part(const uint32_t (&a)[NT], F b) {
