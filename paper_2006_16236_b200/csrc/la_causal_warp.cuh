@@ -411,11 +411,11 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     const uint32_t lower = diagonal_mask<false>();
     // The first 64 positions of a sequence go through twice, the second time with the G_i . O_i they found taken off the scores
     // and off the sums' part: where few terms make up a row, h and (q . h / dn) Zc cancel almost entirely (in row 0 completely).  The first
-    // 256 have the sums in two bf16 parts: their rounding, once for sixteen positions, is what dQ loses most by where the weights are
-    // near-uniform.  dQ's error against 64 bits with 64 / 128 / 256 positions, inputs scaled by 1/8: B16 H8 N3072 1.83e-2 / 1.79e-2 / 1.73e-2,
-    // where tcgen05 chunks of 128 positions have 1.76e-2; B38 H8 N200 1.68e-2 / 1.59e-2 / 1.52e-2 for 1.59e-2 (the features' own rounding:
-    // 1.5e-2).  A step of B128 H8 N784 159.7 / 160.1 / 162.3 us.
-    constexpr int TWICE = 4 * ROWS, PRECISE = 16 * ROWS;
+    // 192 have the sums in two bf16 parts: their rounding, once for sixteen positions, is what dQ loses most by where the weights are
+    // near-uniform.  dQ's error against 64 bits with 64 / 128 / 192 / 256 positions, inputs scaled by 1/8: B16 H8 N3072 1.83e-2 / 1.79e-2 /
+    // 1.76e-2 / 1.73e-2, where tcgen05 chunks of 128 positions have 1.76e-2; B50 H8 N1000 1.79e-2 / 1.73e-2 / 1.69e-2 / 1.66e-2 for 1.71e-2 (the
+    // features' own rounding: 1.5e-2).  A step of B128 H8 N784 159.7 / 160.1 / 161.7 / 162.3 us when it was measured.
+    constexpr int TWICE = 4 * ROWS, PRECISE = 12 * ROWS;
     auto chunk = [&](int n0, auto first) {
         const bool twice = decltype(first)::value && n0 < TWICE;
         const int cn = r.end - n0;              // (of them sixteen at most)
