@@ -287,7 +287,7 @@ KERNEL_ALG_BYTES = {
     "causal_fwd_kernel": lambda d, e: 4 * d * e + 4,            # Q, K, V in; O, den out
     "causal_bwd_dq_kernel": lambda d, e: 5 * d * e + 8,         # Q, K, V, G in; dQ, dn, dl out
     "causal_bwd_dkv_kernel": lambda d, e: 6 * d * e + 8,        # Q, K, V, G, dn, dl in; dK, dV out
-    "linear_apply_kernel": None,                                # three variants share the name: not ranked
+    "linear_warp_apply_kernel": None,                           # two variants share the name: not ranked
 }
 for _tc, _mma in (("fwd", "forward"), ("bwd_dq", "dq"), ("bwd_dkv", "dkv")):       # the same work on mma.sync
     KERNEL_ALG_BYTES[f"causal_mma_{_mma}_kernel"] = KERNEL_ALG_BYTES[f"causal_{_tc}_kernel"]

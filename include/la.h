@@ -487,7 +487,8 @@ long long la_kernel_launches(void);
  * the kernels on mma.sync 8 causal_mma_forward_kernel, 9 causal_mma_dq_kernel, 10 causal_mma_dkv_kernel,
  * 11 causal_mma_sum_kernel (both forms), 12 linear_mma_apply_kernel (three variants), and of those with a
  * thread-block cluster per sequence 13 causal_cluster_forward_kernel, 14 causal_cluster_backward_kernel (all
- * gradients), 15 linear_cluster_forward_kernel.
+ * gradients), 15 linear_cluster_forward_kernel, and of the bf16 non-causal ones on mma.sync 16 linear_warp_sum_kernel,
+ * 17 linear_warp_apply_kernel (forward; dK, dV), 18 linear_warp_dq_kernel (5 and 6 are the tcgen05 ones, 6 dQ alone).
  * Not thread-safe; meant for a benchmark's single launching thread.
  */
 int la_profile_enable(int on);

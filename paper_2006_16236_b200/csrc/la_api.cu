@@ -246,7 +246,8 @@ const char* la_profile_kernel_name(int kernel) {
                                             "linear_apply_kernel", "recurrent_step_kernel", "causal_mma_forward_kernel",
                                             "causal_mma_dq_kernel", "causal_mma_dkv_kernel", "causal_mma_sum_kernel",
                                             "linear_mma_apply_kernel", "causal_cluster_forward_kernel", "causal_cluster_backward_kernel",
-                                            "linear_cluster_forward_kernel"};
+                                            "linear_cluster_forward_kernel", "linear_warp_sum_kernel", "linear_warp_apply_kernel",
+                                            "linear_warp_dq_kernel"};
     return kernel >= 0 && kernel < kProfCount ? names[kernel] : "";
 }
 

@@ -45,7 +45,8 @@ void note_launch();
 enum ProfKernel {
     kProfCausalFwd = 0, kProfCausalBwdDq = 1, kProfCausalBwdDkv = 2, kProfSegmentSum = 3, kProfProjection = 4,
     kProfLinearSum = 5, kProfLinearApply = 6, kProfRecurrent = 7, kProfMmaForward = 8, kProfMmaDq = 9, kProfMmaDkv = 10,
-    kProfMmaSum = 11, kProfMmaApply = 12, kProfClusterForward = 13, kProfClusterBackward = 14, kProfClusterLinear = 15, kProfCount = 16
+    kProfMmaSum = 11, kProfMmaApply = 12, kProfClusterForward = 13, kProfClusterBackward = 14, kProfClusterLinear = 15,
+    kProfLinearWarpSum = 16, kProfLinearWarpApply = 17, kProfLinearWarpDq = 18, kProfCount = 19
 };
 void prof_begin(int kernel, cudaStream_t st);
 void prof_end(int kernel, cudaStream_t st);

@@ -884,8 +884,8 @@ int launch_as(ProfKernel prof, const la_problem& p, int warps, int smem, const l
     return LA_OK;
 }
 template <int W> int launch_warp_sums(const la_problem& p, const lin::Params& a, cudaStream_t st) {
-    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_sum_kernel<W, true>>(kProfLinearSum, p, lin::WARPS, lin::kSumSmem<W>, a, st);
-    return launch_as<linear_warp_sum_kernel<W, false>>(kProfLinearSum, p, lin::WARPS, lin::kSumSmem<W>, a, st);
+    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_sum_kernel<W, true>>(kProfLinearWarpSum, p, lin::WARPS, lin::kSumSmem<W>, a, st);
+    return launch_as<linear_warp_sum_kernel<W, false>>(kProfLinearWarpSum, p, lin::WARPS, lin::kSumSmem<W>, a, st);
 }
 template <int W, int MODE> int launch_warp_apply(const la_problem& p, lin::Params a, cudaStream_t st) {
     constexpr int warps = kApplyWarps<MODE>, smem = lin::ApplyLayout<W, MODE, warps>::BYTES;
@@ -893,8 +893,9 @@ template <int W, int MODE> int launch_warp_apply(const la_problem& p, lin::Param
         const int64_t most = chunks_of(p.N), want = 2 * sm_count() / (p.B * p.H);
         a.parts = (int)(want < 1 ? 1 : want < most ? want : most);
     }
-    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_apply_kernel<W, MODE, true>>(kProfLinearApply, p, warps, smem, a, st);
-    return launch_as<linear_warp_apply_kernel<W, MODE, false>>(kProfLinearApply, p, warps, smem, a, st);
+    constexpr ProfKernel prof = MODE == lin::kApplyBackwardQ ? kProfLinearWarpDq : kProfLinearWarpApply;
+    if (p.phi == LA_PHI_ELU1) return launch_as<linear_warp_apply_kernel<W, MODE, true>>(prof, p, warps, smem, a, st);
+    return launch_as<linear_warp_apply_kernel<W, MODE, false>>(prof, p, warps, smem, a, st);
 }
 
 int make_params(const la_problem& p, const int* lengths, lin::Params* a) {

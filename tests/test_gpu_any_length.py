@@ -6,6 +6,8 @@ these tests sits at the front of a larger buffer filled with a marker, so that a
 tensor's end would be seen (and would be harmless); stores into the next sequence show up in the
 comparison with the oracle.
 """
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -40,8 +42,8 @@ def _untouched(tails):
 
 @pytest.fixture
 def tcgen05(request):
-    """Whether the calls are kept to the tcgen05 kernels: plans that are forced, to pieces and splits as the automatic ones
-    choose about, leave out the kernels with a cluster per sequence that would take short problems."""
+    """Whether the calls are kept to the tcgen05 kernels (non-causal: to those with a warp per sixteen positions): plans that are forced, to
+    pieces and splits as the automatic ones choose about, leave out the kernels with a cluster per sequence that would take short problems."""
     yield request.param
     la.la_plan_override()
 
@@ -114,7 +116,7 @@ def test_noncausal_any_length(tcgen05, shape):
     la.la_last_device_status()
     names = set(la.la_profile_read())
     la.la_profile_enable(False)
-    assert names == {"linear_sum_kernel", "linear_apply_kernel"} | (set() if tcgen05 else {"linear_cluster_forward_kernel"}), names
+    assert names == {"linear_warp_sum_kernel", "linear_warp_apply_kernel", "linear_warp_dq_kernel"} | (set() if tcgen05 else {"linear_cluster_forward_kernel"}), names
     _untouched(tails)
     q, k, v, g = (t.double().numpy() for t in (Q, K, V, G))
     O_ref, den_ref = oracle.linear_attention(q, k, v, causal=False)[:2]
@@ -122,6 +124,82 @@ def test_noncausal_any_length(tcgen05, shape):
     assert_close(den, den_ref, torch.bfloat16, "den")
     for nm, ref in zip(("dQ", "dK", "dV"), oracle.linear_attention_backward(q, k, v, g, causal=False)):
         assert_close(outs[nm], ref, torch.bfloat16, nm, grad=True)
+
+
+SUMS_AND_DQ = {"linear_sum_kernel", "linear_apply_kernel"}         # the non-causal kernels on tcgen05: D = 64, more than 512 and 65536 positions
+
+
+@pytest.mark.parametrize("ragged", [False, True])
+@pytest.mark.parametrize("phi", ["elu1", "identity"])
+@pytest.mark.parametrize("N", [1000, 1001, 1024])
+def test_noncausal_of_many_positions(N, phi, ragged):
+    B, H, D = 9, 8, 64
+    lengths = [N, 0, N - 1, 513, 128, 1, 640, N // 2, 999] if ragged else [N] * B
+    Q, K, V, G = draw_qkvg(B, H, N, D, D, 13 + N, torch.bfloat16, 0.5)
+    if phi == "identity":                               # features: positive, as the weights of a kernel are
+        Q, K = ((t.float().abs() + 0.1).to(torch.bfloat16) for t in (Q, K))
+    tails, dev, outs = {}, {}, {}
+    for nm, t in zip("QKVG", (Q, K, V, G)):
+        dev[nm], tails[nm] = _place(t.to(DEV))
+    for nm, like in (("O", V), ("dQ", Q), ("dK", K), ("dV", V)):
+        outs[nm], tails[nm] = _front(tuple(like.shape), torch.bfloat16)
+    den, tails["den"] = _front((B, H, N), torch.float32)
+    KV, tails["KV"] = _front((B, H, D, D), torch.float32)
+    Zs, tails["Zs"] = _front((B, H, D), torch.float32)
+    saved = la.linear_saved_buffer(dev["Q"], dev["V"], phi=phi)
+    kw = {"phi": phi, "lengths": torch.tensor(lengths, dtype=torch.int32, device=DEV) if ragged else None}
+    la.la_profile_enable(True)
+    la.la_linear_attention(dev["Q"], dev["K"], dev["V"], O=outs["O"], den=den, KV=KV, Zs=Zs, saved=saved, **kw)
+    la.la_linear_attention_backward(dev["Q"], dev["K"], dev["V"], dev["G"], saved=saved, dQ=outs["dQ"], dK=outs["dK"], dV=outs["dV"], **kw)
+    la.la_last_device_status()
+    names = set(la.la_profile_read())
+    la.la_profile_enable(False)
+    assert names == SUMS_AND_DQ | {"linear_warp_apply_kernel"}, names
+    _untouched(tails)
+    again = la.la_linear_attention_backward(dev["Q"], dev["K"], dev["V"], dev["G"], **kw)      # the sums that it would make itself
+    assert all(torch.equal(outs[nm], x) for nm, x in zip(("dQ", "dK", "dV"), again))
+    for b, n in enumerate(lengths):
+        for nm in ("O", "dQ", "dK", "dV"):
+            assert not outs[nm][b, :, n:].any(), f"{nm}: padding of sequence {b} is not zero"
+        h = b % H
+        sl = (slice(b, b + 1), slice(h, h + 1), slice(0, n))
+        if n == 0:
+            assert not KV[b].any() and not Zs[b].any()
+            continue
+        q, k, v, g = (t[sl].double().numpy() for t in (Q, K, V, G))
+        O_ref, den_ref = oracle.linear_attention(q, k, v, causal=False, phi=phi)[:2]
+        assert_close(outs["O"][sl], O_ref, torch.bfloat16, f"O of sequence {b}")
+        assert_close(den[sl], den_ref, torch.bfloat16, f"den of sequence {b}")
+        fk = oracle.feature_map(k) if phi == "elu1" else k
+        assert_close(KV[b:b + 1, h:h + 1], np.einsum("bhnd,bhnm->bhdm", fk, v), torch.bfloat16, f"KV of sequence {b}")
+        assert_close(Zs[b:b + 1, h:h + 1], fk.sum(2), torch.bfloat16, f"Zs of sequence {b}")
+        if n > 1:                                       # (of one position dQ and dK are analytically zero)
+            for nm, ref in zip(("dQ", "dK", "dV"), oracle.linear_attention_backward(q, k, v, g, causal=False, phi=phi)):
+                assert_close(outs[nm][sl], ref, torch.bfloat16, f"{nm} of sequence {b}", grad=True)
+
+
+def test_noncausal_of_many_positions_refuses_sums_of_another_plan():
+    if os.environ.get("LA_DEBUG"):
+        pytest.skip("in checked mode the call itself reads the status and raises; this test reads it afterwards")
+    dev = [t.to(DEV) for t in draw_qkvg(9, 8, 1000, 64, 64, 5, torch.bfloat16, 0.5)]
+    try:
+        la.la_plan_override(linear_splits=4)
+        saved = la.linear_saved_buffer(dev[0], dev[2])
+        la.la_linear_attention(*dev[:3], saved=saved)
+        for splits in (2, 3, -1):
+            la.la_plan_override(linear_splits=splits)
+            outs = [torch.full_like(dev[0], 7.0) for _ in range(3)]
+            la.la_profile_enable(True)
+            la.la_linear_attention_backward(*dev, saved=saved, dQ=outs[0], dK=outs[1], dV=outs[2])
+            with pytest.raises(la.LaError) as e:
+                la.la_last_device_status()
+            names = set(la.la_profile_read())
+            la.la_profile_enable(False)
+            assert e.value.status == -1 and "plan" in str(e.value) and names == {"linear_apply_kernel", "linear_warp_apply_kernel"}
+            assert all(torch.all(t == 7.0) for t in outs)           # nothing was written
+            la.la_last_device_status()
+    finally:
+        la.la_plan_override()
 
 
 @pytest.mark.parametrize("causal", [False, True])

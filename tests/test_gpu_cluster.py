@@ -193,7 +193,7 @@ def test_these_kernels_are_profiled_under_their_own_names():
     assert kernels_of(lambda: la.la_causal_backward(Q, K, V, G)) == {"causal_cluster_backward_kernel": 1}
     assert kernels_of(lambda: la.la_linear_attention(Q, K, V)) == {"linear_cluster_forward_kernel": 1}
     saved = la.linear_saved_buffer(Q, V)
-    assert kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved)) == {"linear_sum_kernel": 1, "linear_cluster_forward_kernel": 1}
+    assert kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved)) == {"linear_warp_sum_kernel": 1, "linear_cluster_forward_kernel": 1}
 
 
 @pytest.fixture(scope="module")
@@ -295,10 +295,10 @@ def test_which_kernel_takes_a_backward_pass(dtype, D, BHN, cluster):
                                            (32, (1, 8, 8192), True), (32, (1, 8, 8193), False), (32, (2, 8, 2049), False)], ids=str)
 def test_which_kernel_takes_a_bidirectional_forward_pass(D, BHN, cluster):
     Q, K, V = (torch.zeros(*BHN, D, dtype=torch.bfloat16, device=DEV) for _ in range(3))
-    want = {"linear_cluster_forward_kernel"} if cluster else {"linear_sum_kernel", "linear_apply_kernel"}
+    want = {"linear_cluster_forward_kernel"} if cluster else {"linear_warp_sum_kernel", "linear_warp_apply_kernel"}
     assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V))) == want
     saved = la.linear_saved_buffer(Q, V)
-    assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved))) == want | {"linear_sum_kernel"}
+    assert set(kernels_of(lambda: la.la_linear_attention(Q, K, V, saved=saved))) == want | {"linear_warp_sum_kernel"}
 
 
 @pytest.mark.parametrize("dtype,phi,D,M", CAUSAL)
