@@ -439,28 +439,26 @@ linear_dq_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant
                 if (idx < kDim * kDim / 4) reinterpret_cast<float4*>(sF)[idx] = acc[u];
             }
         }
-        if (tid < 2 * kDim + 1) {       // a' (64), ysum (64), w0 (1)
+        if (tid < 2 * kDim) {           // a' (64), ysum (64)
             float z = 0.f;
             for (int n = 0; n < prm.nseg; ++n) z += load_global(rec + (int64_t)n * kRecFloats + kDim * kDim + tid);
             if (tid < kDim) sA[tid] = z;
-            else if (tid < 2 * kDim) sNu[tid - kDim] = z;
-            else sScal[1] = z;
+            else sNu[tid - kDim] = z;
         }
         __syncthreads();
-        constexpr int dim = kDim;
         // column sums in two steps (a thread alone would walk its column for a microsecond): four threads per column
         // take every fourth row, in a fixed order, and leave their partial sums behind the matrix
         float* sPartial = sF + kDim * kDim + kDim;                                // fp32 [4][64]
         if (tid < 4 * kDim) {
             const int col = tid & (kDim - 1), part = tid >> 6;
             float m = 0.f;
-            for (int d = part; d < dim; d += 4) m += sF[d * kDim + col];
+            for (int d = part; d < kDim; d += 4) m += sF[d * kDim + col];
             sPartial[part * kDim + col] = m;
         }
         __syncthreads();
-        if (tid < kDim) {               // column tid: mean over the dim real rows; nu = ysum + mu
+        if (tid < kDim) {               // column tid: mean over the rows; nu = ysum + mu
             float m = (sPartial[tid] + sPartial[kDim + tid]) + (sPartial[2 * kDim + tid] + sPartial[3 * kDim + tid]);
-            m *= 1.f / dim;
+            m *= 1.f / kDim;
             const float ysum = sNu[tid];
             sNu[tid] = ysum + m;
             sF[kDim * kDim + tid] = m;                                            // mu, just past the matrix
@@ -476,7 +474,7 @@ linear_dq_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant
             const int d = idx >> 3, c8 = idx & 7;
             float v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = d < dim ? sF[d * kDim + c8 * 8 + j] - sF[kDim * kDim + c8 * 8 + j] : 0.f;
+            for (int j = 0; j < 8; ++j) v[j] = sF[d * kDim + c8 * 8 + j] - sF[kDim * kDim + c8 * 8 + j];
             sts128(smem + kApOffState + d * 128 + ((c8 ^ (d & 7)) << 4), pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]),
                    pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
         }
@@ -573,7 +571,6 @@ linear_dq_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const bool elu = prm.phi == LA_PHI_ELU1;
         const float fD = (float)kDim, fN = (float)len;
-        // (columns beyond a 32-wide problem are zero padding: they add nothing to the sums, and the store clips them)
         float* sX = reinterpret_cast<float*>(smem + kApOffX);
         float* mine = sX + (hf * 128 + t) * 8;
         const float* other = sX + ((hf ^ 1) * 128 + t) * 8;
