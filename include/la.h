@@ -26,8 +26,9 @@
  *    on the tcgen05 kernels (any N: a last chunk of fewer than 128 positions is
  *    handled as padding), but causal ones of D = M = 32 (more than 2048 positions, or
  *    tiles of 128 positions, counted over all sequences, beyond 296, from eight tiles a
- *    sequence on beyond 512) and the non-causal ones (but two passes of those of
- *    D = M = 64 beyond 65536 positions in all) on mma.sync kernels with bf16 operands; every other
+ *    sequence on beyond 512; but not forward passes that keep no sums of some 80 to 148
+ *    sequences) and the non-causal ones (but two passes of those of D = M = 64 with N > 512 and
+ *    more than 65536 positions in all) on mma.sync kernels with bf16 operands; every other
  *    problem with M <= 64 runs on mma.sync kernels that keep fp32 accuracy
  *    (products of numbers split into bf16 parts), everything else on the general
  *    fp32-arithmetic kernels; results agree within the rounding of the I/O type.

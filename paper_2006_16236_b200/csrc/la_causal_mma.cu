@@ -707,9 +707,11 @@ __global__ void __launch_bounds__(32, warp_resident(PASS)) causal_warp_kernel(co
 // ---- host ------------------------------------------------------------------------------------------------------
 // Which bf16 problems with D = M = 32 a warp per piece takes: all that the cluster kernels leave (la_cluster.cu: short sequences of
 // few heads; more than 296 tiles of 128 positions, 512 from eight tiles on, or more than sixteen tiles), whatever the context.
-// Forward + backward, us, tcgen05 kernels (128x8x784: the former ones of this file) / a warp per piece: 128x8x784 284 / 154, 16x8x3072 136 / 106,
-// 32x8x3072 262 / 187, 8x8x16384 376 / 251, 64x8x2048 363 / 234, 1x8x4096 73 / 51, 1x1x16384 156 / 77, 2x1x65536 355 / 154,
-// 1x8x65536 273 / 214, 16x8x700 47 / 44, 16x8x300 33 / 29, 20x8x256 41 / 31, 56x8x64 22.6 / 20.5.
+// Forward + backward, us, tcgen05 kernels (128x8x784, 60x8x300, 56x8x64: former ones of this file) / a warp per piece, in bursts of the same
+// step: 128x8x784 282 / 156, 60x8x300 65 / 57, 16x8x3072 136 / 112, 32x8x3072 263 / 195, 8x8x16384 378 / 254, 64x8x2048 365 / 254, 1x8x4096
+// 73 / 51, 1x1x16384 153 / 78, 2x1x65536 355 / 159, 1x8x65536 273 / 218, 16x8x700 48.5 / 46.3, 16x8x300 33.0 / 31.3, 20x8x256 40.6 / 32.8,
+// 56x8x64 22.5 / 21.5; of 401 sizes, in captured graphs, four are slower by more than 1 % (B*H 444 N 64 16.1 / 17.2, N 128 24.9 / 25.4; five whole
+// chunks of one wave of tcgen05 CTAs, B*H 128 N 640 37.3 / 39.9, 148 38.3 / 39.8).  Forward passes alone: causal_mma_leaves_forward().
 bool of_warps(const la_problem& p) {
     if (p.dtype != LA_BF16 || p.D != 32 || p.M != 32 || p.N > (1 << 30)) return false;
     const int64_t tiles = (p.N + 127) / 128, ctas = tiles * p.B * p.H;

@@ -2,22 +2,23 @@
 //
 // The running sums of such a problem are 32 x 33 numbers: a warp holds them in its registers, walks its piece in chunks of
 // sixteen positions and needs no other warp.  Every product is mma.sync m16n8k16 (tcgen05 wants 128 rows: at D = 32 that is four
-// times as many scores as sums, and a start-up of three chunks per piece).  Nothing is exchanged through shared memory either:
+// times as many scores as sums, and a start-up of three chunks per piece).  Operands do not pass through shared memory from lane to lane
+// (of the rows only their two weights do, and once per piece the sums are turned there):
 //   * Rows arrive and leave in loads and stores of sixteen bytes, the columns in the order of la_warp.cuh.  With the fragments as they
 //     lie, pair by pair, the L1 pipe was 70 % busy.
 //   * The transposes that sums over positions need come from movmatrix.
 //   * The accumulators of the sums, rounded to bf16, are the operand of the next chunk's products as they lie.
-// Chunks of sixteen: one diagonal block of scores and no others, and a loop of 350 to 450 instructions (beyond some 500
-// the fetch of the loop, not its issue, sets the pace).
+// Chunks of sixteen: one diagonal block of scores and no others, and loops of 440 to 620 instructions (twice as many, in chunks of 32, made
+// the fetch of the loop, not its issue, set the pace).
 //
-// What is rounded: features, scores and the copy of the sums that a chunk reads are bf16 operands; the sums, the normaliser
+// What is rounded: features, phi(q) / dn, scores and the copy of the sums that a chunk reads are bf16 operands, each rounded once; the sums, the normaliser
 // (its state in fp32 throughout) and everything per row are fp32.  A chunk's sums start from zero and are added with rounding:
 // the tensor cores truncate.
 //
 // What bounds it: two warps on a scheduler and what they wait for of their own instructions (0.56 issued per cycle), then HBM.  The next
 // two chunks are on their way to shared memory (cp.async, each lane its own bytes), so that no load is waited for.
-// Measured, B128 H8 N784, forward / dQ / dK, dV, us: 47 / 60 / 59 where the kernels with a CTA of four warps per sequence, a chunk of 64
-// and tiles in shared memory took 72 / 95 / 129; instructions of a warp per sixteen rows 430 / 590 / 570 for 660 / 950 / 1140.
+// Measured, B128 H8 N784, forward / dQ / dK, dV, us: 45 / 62 / 57 where the kernels with a CTA of four warps per sequence, a chunk of 64
+// and tiles in shared memory took 72 / 95 / 129; instructions of a warp per sixteen rows 440 / 620 / 555 for 660 / 950 / 1140.
 #pragma once
 
 #include <type_traits>
