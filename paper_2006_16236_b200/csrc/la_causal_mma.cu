@@ -765,9 +765,10 @@ double warp_cost(int64_t bh, int64_t N, int64_t n, bool forward_alone) {
 // both sums has registers for, and no more than a piece's start makes good (forward + backward, us, B x H x N: number of pieces: 16x8x3072
 // 4: 131, 8: 106, 12: 115; 8x8x16384 8: 322, 16: 251, 24: 280; 1x8x16384 32: 106, 64: 88, 128: 113; 1x8x4096 16: 61, 32: 51, 64: 59; 2x1x65536
 // 64: 190, 128: 154).  Beyond 148 sequences another number where the estimate above finds it faster by its own error (just past a full wave
-// above all: 400x1x2048 3: 235, 8: 201; 444x1x512 3: 73, 4: 58; 592x1x784 3: 114, 2: 104; forward alone 400x1x2048 3: 71, 4: 59): 2 % off the best of the measured numbers in the mean where the first rule alone is 4 % (forward alone 2 and 6).  One piece: two
-// chunks (500x1x100 1: 25.1, 2: 28.2), three of as many sequences as run one on a scheduler (530x1x192 1: 36.1, 3: 38.4; but 640x1x192 1: 46.1,
-// 2: 44.2 and 180x1x192 1: 35.7, 3: 22.6), and more than 888 sequences (900x1x784 1: 155, 2: 181, 3: 164).
+// above all: 400x1x2048 3: 235, 8: 201; 444x1x512 3: 73, 4: 58; 592x1x784 3: 114, 2: 104; forward alone 400x1x2048 3: 71, 4: 59): 2 % off the
+// best of the measured numbers in the mean, where the first rule alone is 4 % off (forward alone 2 and 6).  One piece: two chunks (500x1x100
+// 1: 25.1, 2: 28.2), three of as many sequences as run one on a scheduler (530x1x192 1: 36.1, 3: 38.4; but 640x1x192 1: 46.1, 2: 44.2, and
+// 180x1x192 1: 35.7, 3: 22.6), and more than 888 sequences (900x1x784 1: 155, 2: 181, 3: 164).
 int64_t warp_pieces(int64_t bh, int64_t N, bool forward_alone) {
     const int64_t chunks = (N + T - 1) / T, most = (int64_t)(4.0 * sqrt((double)chunks));
     if (bh > 888 || chunks <= 2 || (chunks == 3 && bh >= 444 && bh <= 592)) return 1;
