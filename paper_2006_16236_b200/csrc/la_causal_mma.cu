@@ -681,15 +681,15 @@ causal_mma_dkv_kernel(const Params p) {
 }
 
 // ---- bf16, D = M = 32: a warp per piece (la_causal_warp.cuh) -----------------------------------------------------
-enum WarpPass { kWarpForward, kWarpSums, kWarpDq, kWarpDqReverse, kWarpDkv, kWarpDkvFew };
+enum WarpPass { kWarpForward, kWarpSums, kWarpDq, kWarpDqReverse, kWarpReverseSums, kWarpDkv, kWarpDkvFew };
 constexpr int warp_ring(int pass) {
     return pass == kWarpForward ? warp32::Ring<3, false>::BYTES : pass == kWarpSums ? warp32::Ring<2, false>::BYTES :
-           pass >= kWarpDkv ? warp32::Ring<4, true>::BYTES : warp32::Ring<4, false>::BYTES;
+           pass == kWarpReverseSums ? warp32::Ring<2, true>::BYTES : pass >= kWarpDkv ? warp32::Ring<4, true>::BYTES : warp32::Ring<4, false>::BYTES;
 }
 // Registers for twelve warps on an SM; for eight in the dQ sweep that keeps two kinds of sums, and in the dK, dV sweep where all warps find
-// room that way too (128x8x784 157.5 -> 155.7 us a step, 111x8x300 73.1 -> 71.7, but 200x8x640 190 -> 200).
+// room that way too (128x8x784 158 -> 154 us a step, 16x8x3072 110 -> 108, but 200x8x640 190 -> 200).
 constexpr int warp_resident(int pass) {
-    return pass == kWarpDqReverse || pass == kWarpDkvFew ? 8 : pass == kWarpSums ? 16 : 12;
+    return pass == kWarpDqReverse || pass == kWarpDkvFew ? 8 : pass == kWarpSums || pass == kWarpReverseSums ? 16 : 12;
 }
 template <int PASS> constexpr int kWarpRing = warp_ring(PASS);
 template <int PASS, bool ELU>
@@ -701,6 +701,7 @@ __global__ void __launch_bounds__(32, warp_resident(PASS)) causal_warp_kernel(co
     if constexpr (PASS == kWarpSums) warp32::sums<ELU>(p, smem);
     if constexpr (PASS == kWarpDq) warp32::dq<ELU, false>(p, smem);
     if constexpr (PASS == kWarpDqReverse) warp32::dq<ELU, true>(p, smem);
+    if constexpr (PASS == kWarpReverseSums) warp32::reverse_sums<ELU>(p, smem);
     if constexpr (PASS >= kWarpDkv) warp32::dkv<ELU>(p, smem);
 }
 
@@ -886,11 +887,16 @@ struct WarpKernels {
         if (fwd.pieces > 1 && !fwd.stamp)
             if (int rc = run<kWarpSums>(p, kProfMmaSum, fwd.pieces - 1, fwd, st)) return rc;
         // The dQ sweep that can form both kinds of sums, eight warps on an SM with all registers they want, also where one kind is enough
-        // (128x8x784 155.7 us a step, with the other 158; 256x8x500 210 / 213), unless twelve make one wave of what eight would make two
-        // (160x8x512 159.8 / 151.6, 200x8x640 193.5 / 184.9).
+        // (128x8x784 158 us a step, with the other 160; 256x8x500 206 / 209), unless twelve make one wave of what eight would make two
+        // (160x8x512 150 / 157, 200x8x640 181 / 191).  Two pieces of one chunk or two: the warps with both sums would set the time.
         const int64_t warps = p.B * p.H * fwd.pieces;
-        const bool both = fwd.pieces > 1 || warps <= 8 * 148 || warps > 12 * 148;
-        if (int rc = both ? run<kWarpDqReverse>(p, kProfMmaDq, fwd.pieces, fwd, st) : run<kWarpDq>(p, kProfMmaDq, fwd.pieces, fwd, st)) return rc;
+        if (fwd.pieces > 2 || (fwd.pieces == 2 && p.N > 128) || (fwd.pieces == 1 && (warps <= 8 * 148 || warps > 12 * 148))) {
+            if (int rc = run<kWarpDqReverse>(p, kProfMmaDq, fwd.pieces, fwd, st)) return rc;
+        } else {
+            if (int rc = run<kWarpDq>(p, kProfMmaDq, fwd.pieces, fwd, st)) return rc;
+            if (fwd.pieces > 1)
+                if (int rc = run<kWarpReverseSums>(p, kProfMmaSum, fwd.pieces - 1, rev, st)) return rc;
+        }
         return warps <= 8 * 148 ? run<kWarpDkvFew>(p, kProfMmaDkv, fwd.pieces, rev, st) : run<kWarpDkv>(p, kProfMmaDkv, fwd.pieces, rev, st);
     }
 };

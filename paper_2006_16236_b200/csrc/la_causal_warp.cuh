@@ -527,6 +527,33 @@ __device__ __forceinline__ void dq(const Params& p, uint8_t* smem) {
     zero_rows(p.dQ, r, p.N);
 }
 
+// ---- sums of a piece: q^^T [G | dl], q^ = phi(q) / dn -----------------------------------------------------------------------
+template <bool ELU>
+__device__ __forceinline__ void reverse_sums(const Params& p, uint8_t* smem) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const Span r(p, (int)blockIdx.y + p.first_record);
+    Ring<2, true> in;
+    in.start(smem, r.bh, p.N, r.end, {p.Q, p.G}, p.aux);
+    for (int i = 0; i < in.AHEAD; ++i) in.request(r.lo + i * ROWS);
+    Sums st;
+    st.clear();
+#pragma unroll 1
+    for (int n0 = r.lo; n0 < r.end; n0 += ROWS) {
+        in.request(n0 + in.AHEAD * ROWS);
+        in.arrived(0, r.end - n0, ELU ? kMinusInf : 0u);
+        Rows q = in.rows(0);
+        const Rows G = in.rows(1);
+        const float* w = in.weights();
+        const float2 l0 = load_pair(w + 16 + 2 * t), l1 = load_pair(w + 24 + 2 * t);
+        map_weighted<ELU>(q, w[g], w[g + 8]);
+        const Rows qt = transposed(q);
+        st.add(qt, transposed(G));
+        st.add_weighted(qt, l0, l1);
+        in.next();
+    }
+    st.put_record(p.rec + (r.bh * p.records + blockIdx.y) * (int64_t)RECORD_FLOATS);
+}
+
 // ---- dK, dV sweep ---------------------------------------------------------------------------------------------------
 template <bool ELU>
 __device__ __forceinline__ void dkv(const Params& p, uint8_t* smem) {
