@@ -687,7 +687,7 @@ constexpr int warp_ring(int pass) {
            pass == kWarpReverseSums ? warp32::Ring<2, true>::BYTES : pass >= kWarpDkv ? warp32::Ring<4, true>::BYTES : warp32::Ring<4, false>::BYTES;
 }
 // Registers for twelve warps on an SM; for eight in the dQ sweep that keeps two kinds of sums, and in the dK, dV sweep where all warps find
-// room that way too (128x8x784 158 -> 154 us a step, 16x8x3072 110 -> 108, but 200x8x640 190 -> 200).
+// room that way too (128x8x784 157.5 -> 155.7 us a step, 111x8x300 73.1 -> 71.7, but 200x8x640 190 -> 200).
 constexpr int warp_resident(int pass) {
     return pass == kWarpDqReverse || pass == kWarpDkvFew ? 8 : pass == kWarpSums || pass == kWarpReverseSums ? 16 : 12;
 }
@@ -887,8 +887,9 @@ struct WarpKernels {
         if (fwd.pieces > 1 && !fwd.stamp)
             if (int rc = run<kWarpSums>(p, kProfMmaSum, fwd.pieces - 1, fwd, st)) return rc;
         // The dQ sweep that can form both kinds of sums, eight warps on an SM with all registers they want, also where one kind is enough
-        // (128x8x784 158 us a step, with the other 160; 256x8x500 206 / 209), unless twelve make one wave of what eight would make two
-        // (160x8x512 150 / 157, 200x8x640 181 / 191).  Two pieces of one chunk or two: the warps with both sums would set the time.
+        // (128x8x784 155.7 us a step, with the other 158; 256x8x500 210 / 213), unless twelve make one wave of what eight would make two
+        // (160x8x512 159.8 / 151.6, 200x8x640 193.5 / 184.9).  Two pieces of one chunk, which only a forced plan makes, have a kernel for the
+        // reverse sums (100x8x128 34.9 / 37.1 us a step; 50x8x128 28.1 / 25.0).
         const int64_t warps = p.B * p.H * fwd.pieces;
         if (fwd.pieces > 2 || (fwd.pieces == 2 && p.N > 128) || (fwd.pieces == 1 && (warps <= 8 * 148 || warps > 12 * 148))) {
             if (int rc = run<kWarpDqReverse>(p, kProfMmaDq, fwd.pieces, fwd, st)) return rc;
