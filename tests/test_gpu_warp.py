@@ -220,27 +220,34 @@ def test_workspace_and_saved_sizes():
 @pytest.mark.gpu
 @pytest.mark.parametrize("BH,N,tcgen05", [(128, 512, True), (112, 1000, True), (100, 1000, False), (148, 300, True), (149, 512, False), (90, 512, True),
                                           (76, 1024, False)], ids=str)
-def test_forward_passes_that_keep_no_sums(BH, N, tcgen05):
+@pytest.mark.parametrize("phi", ["elu1", "identity"])
+def test_forward_passes_that_keep_no_sums(BH, N, tcgen05, phi):
     """A wave of one tcgen05 CTA per sequence takes them; training steps, which keep sums, stay on warps.  Both to the same gates, from a
-    state too."""
+    state; the identity map with lengths."""
     B, H = BH, 1
     Q, K, V, _ = draw_qkvg(B, H, N, D, D, 3, BF, 1.0, with_grad=False)
+    if phi == "identity":
+        Q, K = (Q.float().abs() + 0.1).to(BF), (K.float().abs() + 0.1).to(BF)
     g = torch.Generator().manual_seed(1)
     S0, Z0 = torch.randn((B, H, D, D), generator=g) * 3.0, torch.rand((B, H, D), generator=g) * 4.0 + 1.0
     dev, st = [t.to(DEV) for t in (Q, K, V)], {"S_in": S0.to(DEV), "Z_in": Z0.to(DEV)}
-    for saved in (None, la.saved_buffer(dev[0], dev[2])):
-        S, Z = torch.empty_like(st["S_in"]), torch.empty_like(st["Z_in"])
+    lengths = [N] * B if phi == "elu1" else [(N - 37 * b) % (N + 1) for b in range(B)]
+    ln = None if phi == "elu1" else torch.tensor(lengths, dtype=torch.int32, device=DEV)
+    for saved in (None, la.saved_buffer(dev[0], dev[2], phi=phi)):
+        S, Z, den = torch.empty_like(st["S_in"]), torch.empty_like(st["Z_in"]), torch.empty(B, H, N, device=DEV)
         la.la_profile_enable(True)
-        O = la.la_causal_forward(*dev, S_out=S, Z_out=Z, saved=saved, **st)
+        O = la.la_causal_forward(*dev, phi=phi, lengths=ln, den=den, S_out=S, Z_out=Z, saved=saved, **st)
         la.la_last_device_status()
         names = set(la.la_profile_read())
         la.la_profile_enable(False)
         assert ("causal_fwd_kernel" in names) == (tcgen05 and saved is None) and ("causal_mma_forward_kernel" in names) != ("causal_fwd_kernel" in names)
-        for b in (0, B - 1):
-            q, k, v = (t[b:b + 1].double().numpy() for t in (Q, K, V))
-            ref = oracle.causal_from_state(q, k, v, S0[b:b + 1].double().numpy(), Z0[b:b + 1].double().numpy())
-            for nm, x, r in (("O", O, ref[0]), ("S_out", S, ref[2]), ("Z_out", Z, ref[3])):
-                assert_close(x[b:b + 1], r, BF, nm)
+        for b in (0, 1, B - 1):
+            n = lengths[b]
+            q, k, v = (t[b:b + 1, :, :n].double().numpy() for t in (Q, K, V))
+            ref = oracle.causal_from_state(q, k, v, S0[b:b + 1].double().numpy(), Z0[b:b + 1].double().numpy(), phi=phi)
+            assert not O[b, :, n:].any() and not den[b, :, n:].any()
+            for nm, x, r in (("O", O[b:b + 1, :, :n], ref[0]), ("den", den[b:b + 1, :, :n], ref[1]), ("S_out", S[b:b + 1], ref[2]), ("Z_out", Z[b:b + 1], ref[3])):
+                assert_close(x, r, BF, nm)
 
 
 @pytest.mark.parametrize("BHN,pieces", [((50, 8, 2048), 8), ((444, 1, 512), 4), ((592, 1, 784), 2), ((500, 1, 100), 1), ((560, 1, 128), 1), ((180, 1, 192), 3),
